@@ -5,7 +5,14 @@
 // must be known in advance, which is what this predicts.
 //
 // Everything is plain FP32 FFMA with shared-memory tiles: the matrices are at
-// most 128 wide, so tensor cores would idle on the operand staging.
+// most 128 wide, so tensor cores would idle on the operand staging (and TF32
+// would drop mantissa bits that the FP32 interface keeps).
+//
+// Nets whose weights fit one CTA's shared memory (hidden and input width up to
+// 128, outputs up to 8: every capacity predictor) run fused: k_rows takes a
+// slab of rows through all layers and back, k_wgrad turns the activations it
+// leaves into weight gradients and applies Adam. Wider nets take one GEMM per
+// matrix product (k_gemm).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -187,6 +194,402 @@ __global__ void k_mlp_init(float* p, long long n, const long long* off, const in
   }
 }
 
+// ---------------------------------------------------------------------------
+// Fused path. A training step is two launches instead of 23: the layers are so
+// small (0.2 GFLOP a step at 1024 rows of the 12-128-128-128-2 predictor) that
+// the chain of separate kernels costs launches and drained pipelines, not
+// arithmetic.
+//
+// Between the two kernels (and for the backward pass) activations and their
+// gradients live in row-slab blocks: layer l's block is [slab][unit][R], R rows
+// of one unit contiguous, the same image that k_rows keeps in shared memory,
+// so that both kernels move it in whole 16-byte runs and k_wgrad reads four
+// rows of a unit per load.
+constexpr int kMaxLin = 9;       // linear maps: up to 8 hidden layers + the output
+constexpr int kFusedWidth = 128; // widest layer of the fused path
+constexpr int kFusedOut = 8;     // most outputs
+constexpr int kRowThreads = 512;
+constexpr int kRedLd = 132;      // row stride of the partial sums: 4 words past 128, so that the (row, unit) reads
+                                 // of the reduction fall into different banks
+
+struct FusedNet {
+  int nlin;
+  int din[kMaxLin], dout[kMaxLin];
+  int offW[kMaxLin], offb[kMaxLin];      // in the flat parameters
+  int sW[kMaxLin], sB[kMaxLin], ld[kMaxLin];  // shared memory: weights [din][ld] (columns past dout zero), biases
+  int sA[kMaxLin + 1];                   // shared memory: activations [width][R]
+  int sRed;                              // shared memory: partial sums [splits][R][kRedLd]
+  long long offA[kMaxLin + 1];           // global row-slab blocks
+  int nparams;
+};
+
+struct RowArgs {
+  FusedNet net;
+  const float* p;
+  const float* x;
+  const float* y;   // training: targets
+  float* act;       // training: activations for k_wgrad
+  float* dact;      // training: gradients of the layers' outputs
+  float* out;       // forward: yhat
+  float* lossp;     // training: one partial sum per CTA
+  int B;
+  float tau, scale;
+  long long grows, ga, gc, gm0;  // row permutation (grows = 0: none)
+};
+
+// One CTA takes R rows at a time through the net, weights resident in shared
+// memory. A layer's [R x 128] output is tiled 4 columns x 4 rows per thread
+// (two 16-byte shared loads for 16 FMAs); the threads left over split the sum
+// over the inputs, and the partial sums meet in shared memory (fixed order:
+// the result does not depend on the launch). Weight rows are padded to 4 words
+// past the layer's width, so that the backward pass, whose lanes walk the
+// rows, reads 16 bytes per lane without bank conflicts.
+// R: 8 rows give every SM work at the usual batch of 1024; 16 (training) and 32
+// (inference) rows load the weights for fewer slabs once there are more than
+// 16 rows per SM.
+template <int R, bool TRAIN>
+__global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__ RowArgs a) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ long long s_row[R];
+  __shared__ float s_loss[R * kFusedOut];
+  constexpr int RG = R / 4;                     // row groups of a tile row
+  constexpr int KS = kRowThreads / (32 * RG);   // splits of a sum
+  const FusedNet& net = a.net;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int L = net.nlin, n_in = net.din[0], n_out = net.dout[L - 1];
+  griddep_wait();  // the parameters (and, on a reused handle, the blocks) belong to the previous launch until here
+  for (int l = 0; l < L; ++l) {
+    const int din = net.din[l], dout = net.dout[l], ld = net.ld[l];
+    const float* W = a.p + net.offW[l];
+    float* s = sm + net.sW[l];
+    if ((dout & 3) == 0 && (net.offW[l] & 3) == 0) {
+      const int q = dout >> 2;
+      for (int i = tid; i < din * q; i += kRowThreads) cp_async16(s + (i / q) * ld + 4 * (i % q), W + 4 * i);
+    } else {
+      const int wd = (dout + 3) & ~3;
+      for (int i = tid; i < din * wd; i += kRowThreads) {
+        const int k = i / wd, c = i % wd;
+        s[k * ld + c] = c < dout ? W[k * dout + c] : 0.f;
+      }
+    }
+    for (int i = tid; i < dout; i += kRowThreads) sm[net.sB[l] + i] = a.p[net.offb[l] + i];
+  }
+  cp_async_commit();
+  const int nslab = (a.B + R - 1) / R;
+  float loss = 0.f;
+  for (int slab = blockIdx.x; slab < nslab; slab += gridDim.x) {
+    const int r0 = slab * R;
+    const int nr = min(R, a.B - r0);  // rows of this slab; the others stay zero in every block
+    if (tid < nr) {
+      long long row = r0 + tid;
+      if (a.grows) row = (a.ga * (a.gm0 + row) + a.gc) % a.grows;
+      s_row[tid] = row;
+    }
+    __syncthreads();
+    {
+      float* s = sm + net.sA[0];
+      for (int i = tid; i < n_in * R; i += kRowThreads) {
+        const int r = i % R, k = i / R;
+        const float v = r < nr ? a.x[(size_t)s_row[r] * n_in + k] : 0.f;
+        s[i] = v;
+        if (TRAIN) a.act[net.offA[0] + (long long)slab * n_in * R + i] = v;
+      }
+    }
+    cp_async_wait_0();
+    __syncthreads();
+    // forward through the hidden layers
+    float* red = sm + net.sRed;
+    const int rg = warp % RG, ks = warp / RG;
+    for (int l = 0; l + 1 < L; ++l) {
+      const int din = net.din[l], dout = net.dout[l], ld = net.ld[l];
+      const float* W = sm + net.sW[l];
+      const float* X = sm + net.sA[l];
+      const int c0 = 4 * lane;
+      if (c0 < dout) {
+        const int per = (din + KS - 1) / KS, k0 = ks * per, k1 = min(din, k0 + per);
+        float acc[4][4] = {};
+#pragma unroll 8
+        for (int k = k0; k < k1; ++k) {
+          const float4 wv = *reinterpret_cast<const float4*>(W + k * ld + c0);
+          const float4 xv = *reinterpret_cast<const float4*>(X + k * R + 4 * rg);
+          const float w4[4] = {wv.x, wv.y, wv.z, wv.w}, x4[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(x4[r], w4[c], acc[r][c]);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          *reinterpret_cast<float4*>(red + (ks * R + 4 * rg + r) * kRedLd + c0) =
+              make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+      }
+      __syncthreads();
+      float* Y = sm + net.sA[l + 1];
+      for (int i = tid; i < dout * R; i += kRowThreads) {
+        const int r = i % R, c = i / R;
+        float v = 0.f;
+#pragma unroll
+        for (int z = 0; z < KS; ++z) v += red[(z * R + r) * kRedLd + c];
+        v = r < nr ? fmaxf(v + sm[net.sB[l] + c], 0.f) : 0.f;
+        Y[i] = v;
+        if (TRAIN) a.act[net.offA[l + 1] + (long long)slab * dout * R + i] = v;
+      }
+      __syncthreads();
+    }
+    // output layer: one warp per (row, output), lanes over the inputs
+    {
+      const int l = L - 1, din = net.din[l], ld = net.ld[l];
+      const float* W = sm + net.sW[l];
+      const float* X = sm + net.sA[l];
+      float* D = sm + net.sA[L];
+      for (int e = warp; e < R * n_out; e += kRowThreads / 32) {
+        const int r = e % R, o = e / R;
+        float v = 0.f;
+        for (int k = lane; k < din; k += 32) v = fmaf(X[k * R + r], W[k * ld + o], v);
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, m);
+        if (lane == 0) {
+          v += sm[net.sB[l] + o];
+          if (!TRAIN) {
+            if (r < nr) a.out[(size_t)(r0 + r) * n_out + o] = v;
+          } else {
+            // pinball loss at quantile tau: e = y - yhat, max(tau e, (tau - 1) e), averaged over all entries
+            float d = 0.f, le = 0.f;
+            if (r < nr) {
+              const float er = a.y[(size_t)s_row[r] * n_out + o] - v;
+              le = er > 0.f ? a.tau * er : (a.tau - 1.f) * er;
+              d = (er > 0.f ? -a.tau : 1.f - a.tau) * a.scale;
+            }
+            s_loss[e] = le;
+            D[e] = d;
+            a.dact[net.offA[L] + (long long)slab * n_out * R + e] = d;
+          }
+        }
+      }
+    }
+    if (!TRAIN) continue;  // (the next slab's first barrier keeps its row list apart)
+    __syncthreads();
+    if (warp == 0) {
+      float v = 0.f;
+      for (int e = lane; e < R * n_out; e += 32) v += s_loss[e];
+#pragma unroll
+      for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, m);
+      loss += v;
+    }
+    // backward: the gradient of layer l's input replaces that input in shared memory
+    for (int l = L - 1; l > 0; --l) {
+      const int din = net.din[l], dout = net.dout[l], ld = net.ld[l];
+      const float* W = sm + net.sW[l];
+      const float* D = sm + net.sA[l + 1];
+      float* X = sm + net.sA[l];
+      float* dst = a.dact + net.offA[l] + (long long)slab * din * R;
+      if (l == L - 1) {  // at most 8 outputs: one thread per (input, row)
+        for (int i = tid; i < din * R; i += kRowThreads) {
+          const int r = i % R, k = i / R;
+          float v = 0.f;
+          for (int o = 0; o < dout; ++o) v = fmaf(D[o * R + r], W[k * ld + o], v);
+          v = X[i] > 0.f ? v : 0.f;
+          X[i] = v;
+          dst[i] = v;
+        }
+        __syncthreads();
+        continue;
+      }
+      // lanes take the inputs lane, lane + 32, ...; the outputs are taken four at a time and split over the warps
+      const int nq = (dout + 3) >> 2, per = (nq + KS - 1) / KS, q0 = ks * per, q1 = min(nq, q0 + per);
+      float acc[4][4] = {};  // [input][row]
+#pragma unroll 2
+      for (int q = q0; q < q1; ++q) {
+        float dv[4][4], wv[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          // columns past the width are zero in W; their rows of D are not read
+          const float4 t = 4 * q + j < dout ? *reinterpret_cast<const float4*>(D + (4 * q + j) * R + 4 * rg)
+                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+          dv[j][0] = t.x; dv[j][1] = t.y; dv[j][2] = t.z; dv[j][3] = t.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int k = min(lane + 32 * i, din - 1);
+          const float4 t = *reinterpret_cast<const float4*>(W + k * ld + 4 * q);
+          wv[i][0] = t.x; wv[i][1] = t.y; wv[i][2] = t.z; wv[i][3] = t.w;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[i][r] = fmaf(dv[j][r], wv[i][j], acc[i][r]);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (lane + 32 * i < din)
+#pragma unroll
+          for (int r = 0; r < 4; ++r) red[(ks * R + 4 * rg + r) * kRedLd + lane + 32 * i] = acc[i][r];
+      __syncthreads();
+      for (int i = tid; i < din * R; i += kRowThreads) {
+        const int r = i % R, k = i / R;
+        float v = 0.f;
+#pragma unroll
+        for (int z = 0; z < KS; ++z) v += red[(z * R + r) * kRedLd + k];
+        v = X[i] > 0.f ? v : 0.f;
+        X[i] = v;
+        dst[i] = v;
+      }
+      __syncthreads();
+    }
+  }
+  if (TRAIN && tid == 0) a.lossp[blockIdx.x] = loss;
+}
+
+struct WgradArgs {
+  FusedNet net;
+  const float* act;
+  const float* dact;
+  float* part;      // [splits][nparams]
+  unsigned* done;   // [tiles], zero between launches
+  float *g, *p, *m, *v;
+  int nslab, slabs_per_split;
+  const float* lossp;
+  int nloss;
+  float loss_scale;
+  float* loss_out;  // nullable
+  int adam;
+  float lr, b1, b2, eps, c1, c2;
+};
+
+constexpr int kWT = 32;         // inputs and outputs of a weight-gradient tile
+constexpr int kWRows = 128;     // rows staged at a time
+constexpr int kWThreads = 256;
+
+__host__ __device__ inline int wgrad_tiles(const FusedNet& net, int l) {
+  return ((net.din[l] + kWT - 1) / kWT) * ((net.dout[l] + kWT - 1) / kWT);
+}
+
+// Weight gradients X^T dY of every layer in one launch: a CTA owns a 32 x 32
+// tile of one layer's gradient and a run of rows. 64 threads cover the tile
+// with 4 x 4 outputs each and four such groups take a quarter of the staged rows
+// each (128 rows a stage: 32 KB of shared memory). The tiles of the first
+// inputs also sum the bias gradients. The last CTA of a tile to finish adds the
+// runs' partial gradients in run order (so the sums do not depend on timing)
+// and applies Adam to the tile's parameters.
+template <int R>
+__global__ void __launch_bounds__(kWThreads) k_wgrad(const __grid_constant__ WgradArgs a) {
+  __shared__ __align__(16) float s_x[kWRows / 4][kWT][4];   // [row quad][unit][row]
+  __shared__ __align__(16) float s_d[kWRows / 4][kWT][4];
+  __shared__ float s_b[8][kWT];
+  __shared__ bool s_last;
+  const FusedNet& net = a.net;
+  const int tid = threadIdx.x;
+  int l = 0, tile = blockIdx.x;
+  while (tile >= wgrad_tiles(net, l)) tile -= wgrad_tiles(net, l++);
+  const int din = net.din[l], dout = net.dout[l];
+  const int tn = (dout + kWT - 1) / kWT;
+  const int k0 = (tile / tn) * kWT, n0 = (tile % tn) * kWT;
+  const int nk = min(kWT, din - k0), nn = min(kWT, dout - n0);
+  const int s0 = blockIdx.y * a.slabs_per_split, s1 = min(a.nslab, s0 + a.slabs_per_split);
+  constexpr int SS = kWRows / R;  // slabs per stage
+  constexpr int RQ = R / 4;
+  const int grp = tid >> 6, kg = (tid & 63) >> 3, ng = tid & 7;
+  float acc[4][4] = {}, bacc = 0.f;
+  griddep_wait();
+  const float* X = a.act + net.offA[l];
+  const float* D = a.dact + net.offA[l + 1];
+  for (int s = s0; s < s1; s += SS) {
+    // [slab][unit][R] -> [row quad][unit][4]; missing units and slabs are zero
+    for (int i = tid; i < SS * kWT * RQ; i += kWThreads) {
+      const int q = i % RQ, u = (i / RQ) % kWT, j = i / (RQ * kWT);
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f), d = x;
+      if (s + j < s1) {
+        if (u < nk) x = *reinterpret_cast<const float4*>(X + ((long long)(s + j) * din + k0 + u) * R + 4 * q);
+        if (u < nn) d = *reinterpret_cast<const float4*>(D + ((long long)(s + j) * dout + n0 + u) * R + 4 * q);
+      }
+      *reinterpret_cast<float4*>(s_x[j * RQ + q][u]) = x;
+      *reinterpret_cast<float4*>(s_d[j * RQ + q][u]) = d;
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int q = 8 * grp; q < 8 * grp + 8; ++q) {
+      float4 x[4], d[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(s_x[q][kg + 8 * i]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) d[i] = *reinterpret_cast<const float4*>(s_d[q][ng + 8 * i]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          acc[i][j] = fmaf(x[i].x, d[j].x, acc[i][j]);
+          acc[i][j] = fmaf(x[i].y, d[j].y, acc[i][j]);
+          acc[i][j] = fmaf(x[i].z, d[j].z, acc[i][j]);
+          acc[i][j] = fmaf(x[i].w, d[j].w, acc[i][j]);
+        }
+    }
+    if (k0 == 0) {  // bias: output tid % 32, every eighth quad
+      for (int q = tid >> 5; q < kWRows / 4; q += 8) {
+        const float4 d = *reinterpret_cast<const float4*>(s_d[q][tid & 31]);
+        bacc += (d.x + d.y) + (d.z + d.w);
+      }
+    }
+    __syncthreads();
+  }
+  // the four row groups' tiles meet in shared memory (the staging arrays, 1024 floats each)
+  float* s_t = &s_x[0][0][0];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s_t[grp * kWT * kWT + (kg + 8 * i) * kWT + ng + 8 * j] = acc[i][j];
+  s_b[tid >> 5][tid & 31] = bacc;
+  __syncthreads();
+  float* part = a.part + (long long)blockIdx.y * net.nparams;
+  for (int i = tid; i < kWT * kWT; i += kWThreads) {
+    const int k = i / kWT, n = i % kWT;
+    if (k < nk && n < nn)
+      part[net.offW[l] + (k0 + k) * dout + n0 + n] =
+          (s_t[i] + s_t[i + kWT * kWT]) + (s_t[i + 2 * kWT * kWT] + s_t[i + 3 * kWT * kWT]);
+  }
+  if (k0 == 0 && tid < nn) {
+    float b = 0.f;
+#pragma unroll
+    for (int z = 0; z < 8; ++z) b += s_b[z][tid];
+    part[net.offb[l] + n0 + tid] = b;
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) {
+    const unsigned n = atomicAdd(&a.done[blockIdx.x], 1u);
+    s_last = n == gridDim.y - 1;
+    if (s_last) a.done[blockIdx.x] = 0u;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_last) return;
+  const int S = gridDim.y;
+  const int entries = kWT * kWT + (k0 == 0 ? kWT : 0);
+  for (int i = tid; i < entries; i += kWThreads) {
+    const int k = i / kWT, n = i % kWT;  // k = 32: the bias row
+    if (n >= nn || (k < kWT && k >= nk)) continue;
+    const int e = k < kWT ? net.offW[l] + (k0 + k) * dout + n0 + n : net.offb[l] + n0 + n;
+    float gi = 0.f;
+    for (int z = 0; z < S; ++z) gi += __ldcg(a.part + (long long)z * net.nparams + e);
+    a.g[e] = gi;
+    if (a.adam) {  // Adam (Kingma & Ba, 2015) with bias correction
+      const float mi = a.b1 * a.m[e] + (1.f - a.b1) * gi;
+      const float vi = a.b2 * a.v[e] + (1.f - a.b2) * gi * gi;
+      a.m[e] = mi;
+      a.v[e] = vi;
+      a.p[e] -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+    }
+  }
+  if (blockIdx.x == 0 && a.loss_out && tid < 32) {
+    float v = 0.f;
+    for (int i = tid; i < a.nloss; i += 32) v += a.lossp[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    if (tid == 0) *a.loss_out = v * a.loss_scale;
+  }
+}
+
 // features of a model: log1p(side), log1p(n0 sheep), log1p(n0 wolves), the 8
 // rule params over their nominal values, horizon / 500
 __global__ void k_features(const int32_t* tab, int B, const int32_t* nominal, float* x) {
@@ -236,6 +639,11 @@ struct abm_mlp {
   long long* d_off;
   int* d_fan;
   int adam_t;
+  // fused path (fused = 0: a GEMM per product)
+  int fused;
+  FusedNet net;          // shared-memory offsets filled in per launch shape
+  float* wpart;          // [kSplits][nparams] partial weight gradients
+  unsigned* wdone;       // [tiles] arrivals per weight-gradient tile
 };
 
 static void mlp_free(abm_mlp* n) {
@@ -249,10 +657,52 @@ static void mlp_free(abm_mlp* n) {
   cudaFree(n->lossp);
   cudaFree(n->d_off);
   cudaFree(n->d_fan);
+  cudaFree(n->wpart);
+  cudaFree(n->wdone);
   delete n;
 }
 
 static const int kSplits = 32;
+constexpr size_t kMaxSmem = 227 * 1024 - 2048;  // dynamic shared memory of a CTA, less the static arrays
+
+// Shared-memory layout of k_rows<R, train>: weights, biases, activations
+// (training keeps every layer's, inference two that take turns), partial sums.
+// Returns the bytes.
+static size_t fused_layout(FusedNet& f, int R, bool train) {
+  int at = 0;
+  for (int l = 0; l < f.nlin; ++l) {
+    f.sW[l] = at;
+    at += f.din[l] * f.ld[l];
+  }
+  for (int l = 0; l < f.nlin; ++l) {
+    f.sB[l] = at;
+    at += (f.dout[l] + 3) & ~3;
+  }
+  int w[2] = {f.din[0], f.dout[0]};  // widest even and odd layer
+  for (int l = 2; l <= f.nlin; ++l) w[l & 1] = std::max(w[l & 1], f.dout[l - 1]);
+  const int base = at;
+  for (int l = 0; l <= f.nlin; ++l) {
+    if (train) {
+      f.sA[l] = at;
+      at += (l == 0 ? f.din[0] : f.dout[l - 1]) * R;
+    } else {
+      f.sA[l] = base + (l & 1) * w[0] * R;
+    }
+  }
+  if (!train) at = base + (w[0] + w[1]) * R;
+  f.sRed = at;
+  at += (kRowThreads / (32 * (R / 4))) * R * kRedLd;
+  return (size_t)at * sizeof(float);
+}
+
+// nets whose widths the fused tiles cover and whose shared memory fits with
+// the largest slabs (16 rows in training, 32 in inference)
+static bool fused_fits(FusedNet f) {
+  for (int l = 0; l < f.nlin; ++l)
+    if (f.din[l] > kFusedWidth || f.dout[l] > kFusedWidth) return false;
+  return f.dout[f.nlin - 1] <= kFusedOut && fused_layout(f, 16, true) <= kMaxSmem &&
+         fused_layout(f, 32, false) <= kMaxSmem;
+}
 
 extern "C" abm_status abm_mlp_destroy(abm_mlp* n) {
   if (!n) return ABM_ERR_ARG;
@@ -289,12 +739,27 @@ extern "C" abm_status abm_mlp_create(int32_t n_in, int32_t hidden, int32_t layer
     fan.push_back(di);
   }
   n->nparams = off;
+  const long long rows_pad = ((long long)max_batch + 31) / 32 * 32;  // whole row slabs
   long long aoff = 0;
   for (int l = 0; l <= n->nlin; ++l) {
     n->offA.push_back(aoff);
     const int w = l == 0 ? n_in : n->dout[l - 1];
-    aoff += (long long)max_batch * w;
+    aoff += rows_pad * w;
   }
+  int wtiles = 1;
+  n->net.nlin = n->nlin;
+  n->net.nparams = (int)n->nparams;
+  for (int l = 0; l < n->nlin; ++l) {
+    n->net.din[l] = n->din[l];
+    n->net.dout[l] = n->dout[l];
+    n->net.offW[l] = (int)n->offW[l];
+    n->net.offb[l] = (int)n->offb[l];
+    n->net.ld[l] = ((n->dout[l] + 3) & ~3) + (l == n->nlin - 1 ? 0 : 4);
+    n->net.offA[l] = n->offA[l];
+    wtiles += wgrad_tiles(n->net, l);
+  }
+  n->net.offA[n->nlin] = n->offA[n->nlin];
+  n->fused = fused_fits(n->net);
   const size_t P = (size_t)n->nparams;
   bool ok = cudaMalloc(&n->p, P * 4) == cudaSuccess && cudaMalloc(&n->g, P * 4) == cudaSuccess &&
             cudaMalloc(&n->m, P * 4) == cudaSuccess && cudaMalloc(&n->v, P * 4) == cudaSuccess &&
@@ -302,7 +767,9 @@ extern "C" abm_status abm_mlp_create(int32_t n_in, int32_t hidden, int32_t layer
             cudaMalloc(&n->part, (size_t)kSplits * std::max(hidden, n_in) * std::max(hidden, n_out) * 4) == cudaSuccess &&
             cudaMalloc(&n->lossp, 1024 * 4) == cudaSuccess &&
             cudaMalloc(&n->d_off, offs.size() * sizeof(long long)) == cudaSuccess &&
-            cudaMalloc(&n->d_fan, fan.size() * sizeof(int)) == cudaSuccess;
+            cudaMalloc(&n->d_fan, fan.size() * sizeof(int)) == cudaSuccess &&
+            (!n->fused || (cudaMalloc(&n->wpart, (size_t)kSplits * P * 4) == cudaSuccess &&
+                           cudaMalloc(&n->wdone, (size_t)wtiles * 4) == cudaSuccess));
   if (!ok) {
     cudaGetLastError();
     mlp_free(n);
@@ -311,7 +778,8 @@ extern "C" abm_status abm_mlp_create(int32_t n_in, int32_t hidden, int32_t layer
   cudaStream_t st = (cudaStream_t)stream;
   if (cudaMemcpyAsync(n->d_off, offs.data(), offs.size() * sizeof(long long), cudaMemcpyHostToDevice, st) != cudaSuccess ||
       cudaMemcpyAsync(n->d_fan, fan.data(), fan.size() * sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemsetAsync(n->m, 0, P * 4, st) != cudaSuccess || cudaMemsetAsync(n->v, 0, P * 4, st) != cudaSuccess) {
+      cudaMemsetAsync(n->m, 0, P * 4, st) != cudaSuccess || cudaMemsetAsync(n->v, 0, P * 4, st) != cudaSuccess ||
+      (n->fused && cudaMemsetAsync(n->wdone, 0, (size_t)wtiles * 4, st) != cudaSuccess)) {
     mlp_free(n);
     return ABM_ERR_CUDA;
   }
@@ -436,9 +904,121 @@ static Perm make_perm(int64_t rows, int64_t a, int64_t c, int64_t m0) {
   return p;
 }
 
+// ---- fused path, host side
+static int slab_rows(int B, bool train) {
+  // more than 16 rows per SM: larger slabs, so that a CTA goes through the resident weights with fewer barriers
+  return B <= 16 * num_sms() ? 8 : (train ? 16 : 32);
+}
+
+template <int R, bool TRAIN>
+static abm_status rows_launch(abm_mlp* n, RowArgs& ra, cudaStream_t st, int& grid) {
+  static std::atomic<unsigned long long> attr{0};
+  ra.net = n->net;
+  const size_t smem = fused_layout(ra.net, R, TRAIN);
+  ABM_CUDA_TRY(smem_attr_once(k_rows<R, TRAIN>, (int)kMaxSmem, attr));
+  grid = std::min((ra.B + R - 1) / R, num_sms());
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kRowThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  ABM_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_rows<R, TRAIN>, ra));
+  return ABM_OK;
+}
+
+struct AdamStep {
+  int on;
+  float lr, b1, b2, eps, c1, c2;
+};
+
+template <int R>
+static abm_status fused_train(abm_mlp* n, RowArgs& ra, const AdamStep& ad, float* loss_out, cudaStream_t st) {
+  int grid = 0;
+  abm_status e = rows_launch<R, true>(n, ra, st, grid);
+  if (e != ABM_OK) return e;
+  WgradArgs wa;
+  std::memset(&wa, 0, sizeof(wa));
+  wa.net = ra.net;
+  wa.act = n->act;
+  wa.dact = n->dact;
+  wa.part = n->wpart;
+  wa.done = n->wdone;
+  wa.g = n->g;
+  wa.p = n->p;
+  wa.m = n->m;
+  wa.v = n->v;
+  wa.nslab = (ra.B + R - 1) / R;
+  // runs of whole stages: 128 rows each while that gives at most kSplits runs
+  const int stages = (wa.nslab * R + kWRows - 1) / kWRows;
+  const int per = (stages + kSplits - 1) / kSplits;
+  wa.slabs_per_split = per * (kWRows / R);
+  wa.lossp = n->lossp;
+  wa.nloss = grid;
+  wa.loss_scale = ra.scale;
+  wa.loss_out = loss_out;
+  wa.adam = ad.on;
+  wa.lr = ad.lr;
+  wa.b1 = ad.b1;
+  wa.b2 = ad.b2;
+  wa.eps = ad.eps;
+  wa.c1 = ad.c1;
+  wa.c2 = ad.c2;
+  int tiles = 0;
+  for (int l = 0; l < n->nlin; ++l) tiles += wgrad_tiles(n->net, l);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)tiles, (unsigned)((stages + per - 1) / per));
+  cfg.blockDim = dim3(kWThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  ABM_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_wgrad<R>, wa));
+  return ABM_OK;
+}
+
+static abm_status fused_gradients(abm_mlp* n, const float* x, const float* y, int B, float tau, const Perm& pm,
+                                  const AdamStep& ad, float* loss_out, cudaStream_t st) {
+  RowArgs ra;
+  std::memset(&ra, 0, sizeof(ra));
+  ra.p = n->p;
+  ra.x = x;
+  ra.y = y;
+  ra.act = n->act;
+  ra.dact = n->dact;
+  ra.lossp = n->lossp;
+  ra.B = B;
+  ra.tau = tau;
+  ra.scale = 1.f / (float)(B * n->n_out);
+  ra.grows = pm.rows;
+  ra.ga = pm.a;
+  ra.gc = pm.c;
+  ra.gm0 = pm.m0;
+  return slab_rows(B, true) == 8 ? fused_train<8>(n, ra, ad, loss_out, st)
+                                 : fused_train<16>(n, ra, ad, loss_out, st);
+}
+
+static abm_status fused_forward(abm_mlp* n, const float* x, int B, float* y, cudaStream_t st) {
+  RowArgs ra;
+  std::memset(&ra, 0, sizeof(ra));
+  ra.p = n->p;
+  ra.x = x;
+  ra.out = y;
+  ra.B = B;
+  int grid;
+  return slab_rows(B, false) == 8 ? rows_launch<8, false>(n, ra, st, grid) : rows_launch<32, false>(n, ra, st, grid);
+}
+
 extern "C" abm_status abm_mlp_forward(abm_mlp* n, const float* x, int32_t B, float* y, void* stream) {
   if (!n || !x || !y || B < 1 || B > n->max_batch) return ABM_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
+  if (n->fused) return fused_forward(n, x, B, y, st);
   abm_status e = mlp_forward(n, x, B, make_perm(0, 0, 0, 0), st);
   if (e != ABM_OK) return e;
   ABM_CUDA_TRY(cudaMemcpyAsync(y, n->act + n->offA[n->nlin], sizeof(float) * (size_t)B * n->n_out,
@@ -446,12 +1026,12 @@ extern "C" abm_status abm_mlp_forward(abm_mlp* n, const float* x, int32_t B, flo
   return ABM_OK;
 }
 
-extern "C" abm_status abm_mlp_gradients(abm_mlp* n, const float* x, const float* y, int32_t B, float tau,
-                                        int64_t perm_rows, int64_t perm_a, int64_t perm_c, int64_t perm_m0,
-                                        float* loss_out, void* stream) {
-  if (!n || !x || !y || B < 1 || B > n->max_batch || perm_rows < 0 || (perm_rows > 0 && perm_a < 1)) return ABM_ERR_ARG;
-  cudaStream_t st = (cudaStream_t)stream;
-  const Perm pm = make_perm(perm_rows, perm_a, perm_c, perm_m0);
+static bool grad_args_ok(abm_mlp* n, const float* x, const float* y, int32_t B, int64_t perm_rows, int64_t perm_a) {
+  return n && x && y && B >= 1 && B <= n->max_batch && perm_rows >= 0 && (perm_rows == 0 || perm_a >= 1);
+}
+
+static abm_status gemm_gradients(abm_mlp* n, const float* x, const float* y, int B, float tau, const Perm& pm,
+                                 float* loss_out, cudaStream_t st) {
   abm_status e = mlp_forward(n, x, B, pm, st);
   if (e != ABM_OK) return e;
   k_gather_rows<<<std::max(1, std::min(1024, (B * n->n_in + 255) / 256)), 256, 0, st>>>(
@@ -459,15 +1039,33 @@ extern "C" abm_status abm_mlp_gradients(abm_mlp* n, const float* x, const float*
   return mlp_backward(n, x, y, B, tau, pm, loss_out, st);
 }
 
+extern "C" abm_status abm_mlp_gradients(abm_mlp* n, const float* x, const float* y, int32_t B, float tau,
+                                        int64_t perm_rows, int64_t perm_a, int64_t perm_c, int64_t perm_m0,
+                                        float* loss_out, void* stream) {
+  if (!grad_args_ok(n, x, y, B, perm_rows, perm_a)) return ABM_ERR_ARG;
+  const Perm pm = make_perm(perm_rows, perm_a, perm_c, perm_m0);
+  if (n->fused) return fused_gradients(n, x, y, B, tau, pm, AdamStep{}, loss_out, (cudaStream_t)stream);
+  return gemm_gradients(n, x, y, B, tau, pm, loss_out, (cudaStream_t)stream);
+}
+
 extern "C" abm_status abm_mlp_train_step(abm_mlp* n, const float* x, const float* y, int32_t B, float tau, float lr,
                                          int64_t perm_rows, int64_t perm_a, int64_t perm_c, int64_t perm_m0,
                                          float* loss_out, void* stream) {
-  abm_status e = abm_mlp_gradients(n, x, y, B, tau, perm_rows, perm_a, perm_c, perm_m0, loss_out, stream);
-  if (e != ABM_OK) return e;
-  n->adam_t += 1;
+  if (!grad_args_ok(n, x, y, B, perm_rows, perm_a)) return ABM_ERR_ARG;
+  const Perm pm = make_perm(perm_rows, perm_a, perm_c, perm_m0);
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  const float c1 = (float)(1.0 - std::pow((double)b1, n->adam_t));
-  const float c2 = (float)(1.0 - std::pow((double)b2, n->adam_t));
+  const int t = n->adam_t + 1;
+  const float c1 = (float)(1.0 - std::pow((double)b1, t));
+  const float c2 = (float)(1.0 - std::pow((double)b2, t));
+  if (n->fused) {
+    const abm_status e =
+        fused_gradients(n, x, y, B, tau, pm, AdamStep{1, lr, b1, b2, eps, c1, c2}, loss_out, (cudaStream_t)stream);
+    if (e == ABM_OK) n->adam_t = t;
+    return e;
+  }
+  const abm_status e = gemm_gradients(n, x, y, B, tau, pm, loss_out, (cudaStream_t)stream);
+  if (e != ABM_OK) return e;
+  n->adam_t = t;
   k_adam<<<std::max(1, std::min(1024, (int)((n->nparams + 255) / 256))), 256, 0, (cudaStream_t)stream>>>(
       n->p, n->g, n->m, n->v, (int)n->nparams, lr, b1, b2, eps, c1, c2);
   ABM_LAUNCH_CHECK();

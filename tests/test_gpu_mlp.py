@@ -164,3 +164,41 @@ def test_trained_predictor_gain(cap):
     np.testing.assert_array_equal(res["digest"], want)
     assert learned.sum() < 0.5 * fixed.sum()
     assert len(res["overflowed"]) <= 0.05 * n
+
+
+@pytest.mark.parametrize("n_in,hidden,layers,n_out,B", [
+    (12, 128, 3, 2, 1), (12, 37, 1, 2, 7), (1, 100, 2, 1, 9), (128, 64, 8, 8, 129), (12, 128, 3, 2, 2433),
+    (13, 127, 2, 5, 5001), (12, 128, 4, 2, 300), (12, 130, 2, 2, 77), (12, 64, 2, 9, 260)])
+def test_net_shapes_vs_float64(cap, n_in, hidden, layers, n_out, B):
+    """Both training paths (weights resident in shared memory; one GEMM per product) at the edges of their slabs,
+    tiles and widths: gradients, forward and loss. Tolerance: float32 sums of up to 5001 x 128 terms, 1e-4 of the
+    largest entry."""
+    import ctypes as C
+    from paper_2508_16508_gb300 import abm
+    rng = np.random.default_rng(B)
+    h = C.c_void_p()
+    abm.call("abm_mlp_create", n_in, hidden, layers, n_out, 3, B, abm.stream_handle(), C.byref(h))
+    try:
+        cnt = C.c_int64()
+        abm.call("abm_mlp_params", h, None, None, C.byref(cnt))
+        dims = [n_in] + [hidden] * layers + [n_out]
+        p = (rng.normal(size=cnt.value) * (2.0 / hidden) ** 0.5).astype(np.float32)  # biases too
+        x = rng.normal(size=(B, n_in)).astype(np.float32)
+        y = rng.normal(size=(B, n_out)).astype(np.float32) * 2
+        pd, xd, yd = (torch.from_numpy(v).cuda() for v in (p, x, y))
+        abm.call("abm_mlp_set_params", h, abm.ptr(pd), cnt.value, abm.stream_handle())
+        out, loss, g = torch.empty(B, n_out).cuda(), torch.zeros(1).cuda(), torch.empty(cnt.value).cuda()
+        abm.call("abm_mlp_forward", h, abm.ptr(xd), B, abm.ptr(out), abm.stream_handle())
+        abm.call("abm_mlp_gradients", h, abm.ptr(xd), abm.ptr(yd), B, 0.9, 0, 0, 0, 0, abm.ptr(loss),
+                 abm.stream_handle())
+        abm.call("abm_mlp_get_grads", h, abm.ptr(g), cnt.value, abm.stream_handle())
+        torch.cuda.synchronize()
+        net = omlp.unflatten(p, dims)
+        ref = omlp.forward(net, x.astype(np.float64))[-1]
+        ol, og = omlp.loss_and_grads(net, x.astype(np.float64), y.astype(np.float64), 0.9)
+        og = omlp.flatten(og)
+        np.testing.assert_allclose(out.cpu().numpy(), ref, rtol=1e-4, atol=1e-4 * np.abs(ref).max())
+        np.testing.assert_allclose(g.cpu().numpy(), og, rtol=1e-4, atol=1e-4 * np.abs(og).max())
+        assert abs(float(loss.item()) - ol) <= 1e-4 * abs(ol) + 1e-6
+    finally:
+        abm.call("abm_mlp_destroy", h)
