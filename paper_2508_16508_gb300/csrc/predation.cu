@@ -670,8 +670,7 @@ extern "C" abm_status abm_read_agents(abm_world* w, int32_t species, int32_t whi
     ABM_CUDA_TRY(cudaMemcpyAsync(dst, w->d.sp[species].active, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, st));
   } else {
     const int32_t* src = reinterpret_cast<const int32_t*>(w->d.sp[species].agent) + (which - 1);
-    ABM_CUDA_TRY(cudaMemcpy2DAsync(dst, sizeof(int32_t), src, sizeof(int4), sizeof(int32_t), n,
-                                   cudaMemcpyDeviceToDevice, st));
+    return strided_copy(dst, 1, src, 4, n, st);
   }
   return ABM_OK;
 }
