@@ -2,14 +2,20 @@
 // agents come first, ascending by one int32 field with ties kept in slot
 // order, and the placeholders after them in slot order.
 //
-// LSD radix sort of (key, value) pairs, key = the field with its sign bit
-// flipped (so unsigned order is signed order), value = the slot with the
-// placeholder flag in bit 31: four passes over the key bytes, then one pass
-// over the flag. Each pass: per-tile digit histograms -> one exclusive scan
-// over (digit, tile) -> each tile ranks its items stably per digit in shared
-// memory (warp match + per-warp digit counts) and writes them at their global
-// positions. Finally every agent's row (fields + live flag) is gathered into
-// spare arrays, which then become the slab's arrays.
+// The live slots are first packed, in slot order, as (key, slot) pairs, key =
+// the field with its sign bit flipped (so unsigned order is signed order);
+// placeholders need no sorting, so they are only listed. The packing pass also
+// counts all four key bytes, which gives every digit's first position and shows
+// which bytes hold one value only (the high bytes of cells, ids and ages):
+// their passes are left out. An LSD radix sort of the pairs then runs one pass
+// per byte that is left: per-chunk digit counts, a scan over the chunks, and a
+// stable scatter. Finally every agent's row (fields + live flag) is gathered
+// into spare arrays, which then become the slab's arrays.
+//
+// Every pass splits the pairs over the same number of CTAs, a contiguous chunk
+// each, so a position is a prefix over chunk counts: no CTA waits for another,
+// and the passes are chained with programmatic dependent launch. The number of
+// pairs is known on the device only; nothing is read back.
 #include <algorithm>
 #include <new>
 
@@ -19,23 +25,22 @@ namespace abm {
 
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortItems = 8;
+constexpr int kSortItems = 16;
 constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr int kWarpItems = 32 * kSortItems;
 constexpr int kBins = 256;
-constexpr int kScanThreads = 1024;
-constexpr int kScanItems = 4;
-constexpr int kScanBlock = kScanThreads * kScanItems;
-constexpr u32 kPlaceholder = 0x80000000u;  // value bit: the slot holds no agent
+constexpr int kPasses = 4;
+constexpr int kSortCtasPerSm = 4;  // resident scatter CTAs (45 KB of shared memory, at most 64 registers a thread)
 
 struct SortScratch {
-  int cap, n_pad, Fp, G;
+  int cap, n_pad, Fp, G;  // G: CTAs (= chunks) of every pass
   u32* key[2];
   u32* val[2];
-  u32* hist;        // [kBins * G], scanned in place
-  u32* sums;        // per scan block
+  u32* hist;        // [kBins][G]: a pass's digit counts per chunk, then its positions
+  u32* counts;      // [G] live slots per chunk
+  u32* digits;      // [kPasses][kBins] digit counts over all pairs, then [1] the nonbinary flag
   int32_t* fields;  // [n_pad * Fp]: the next fields array
   int32_t* active;  // [n_pad]: the next live-flag array
-  int* nonbinary;   // set when a live flag is neither 0 nor 1 (the gather then copies them)
 };
 
 void sort_scratch_free(SortScratch* p) {
@@ -45,174 +50,366 @@ void sort_scratch_free(SortScratch* p) {
     cudaFree(p->val[b]);
   }
   cudaFree(p->hist);
-  cudaFree(p->sums);
+  cudaFree(p->counts);
+  cudaFree(p->digits);
   cudaFree(p->fields);
   cudaFree(p->active);
-  cudaFree(p->nonbinary);
   delete p;
 }
 
-__global__ void k_sort_init(SlabDev s, int field, u32* key, u32* val, int* nonbinary) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.cap; i += gridDim.x * blockDim.x) {
-    const int a = s.active[i];
-    if (a != 0 && a != 1) *nonbinary = 1;
-    const bool live = a != 0;
-    key[i] = live ? ((u32)s.fields[(size_t)i * s.Fp + field] ^ 0x80000000u) : 0u;
-    val[i] = (u32)i | (live ? 0u : kPlaceholder);
-  }
+// chunk length of n items over G CTAs: whole tiles
+__device__ __forceinline__ int chunk_of(int n, int G) {
+  return (int)(((long long)n + (long long)G * kSortTile - 1) / ((long long)G * kSortTile)) * kSortTile;
 }
 
-__device__ __forceinline__ u32 digit_of(u32 key, u32 val, int pass) {
-  return pass < 4 ? (key >> (8 * pass)) & 0xFFu : val >> 31;
-}
-
-// per-tile digit counts, digit-major: hist[d * G + tile]
-__global__ void __launch_bounds__(kSortThreads) k_sort_hist(const u32* __restrict__ key, const u32* __restrict__ val,
-                                                            int n, int pass, int G, u32* hist) {
-  __shared__ u32 s_cnt[kBins];
-  s_cnt[threadIdx.x] = 0u;
+// sum over the block of one value per thread, in every thread (s: kSortWarps words)
+__device__ __forceinline__ u32 block_total(u32 v, u32* s) {
+  v = __reduce_add_sync(0xFFFFFFFFu, v);
   __syncthreads();
-  const int t = blockIdx.x;
-#pragma unroll
-  for (int r = 0; r < kSortItems; ++r) {
-    const int i = t * kSortTile + r * kSortThreads + threadIdx.x;
-    if (i < n) atomicAdd(&s_cnt[pass < 4 ? digit_of(key[i], 0u, pass) : digit_of(0u, val[i], pass)], 1u);
-  }
+  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
   __syncthreads();
-  hist[(size_t)threadIdx.x * G + t] = s_cnt[threadIdx.x];
-}
-
-// exclusive scan of a[0..n): blocks of kScanBlock, their sums, the offsets
-__global__ void __launch_bounds__(kScanThreads) k_scan_blocks(u32* a, int n, u32* sums) {
-  __shared__ u64 s_warp[kScanThreads / 32 + 1];
-  const int b0 = blockIdx.x * kScanBlock + threadIdx.x * kScanItems;
-  u32 v[kScanItems];
-  u32 local = 0;
+  u32 t = 0;
 #pragma unroll
-  for (int j = 0; j < kScanItems; ++j) {
-    v[j] = b0 + j < n ? a[b0 + j] : 0u;
-    local += v[j];
-  }
-  u32 ex, ex2, tot, tot2;
-  block_scan2<kScanThreads>(local, 0u, ex, ex2, tot, tot2, s_warp);
-#pragma unroll
-  for (int j = 0; j < kScanItems; ++j) {
-    if (b0 + j < n) a[b0 + j] = ex;
-    ex += v[j];
-  }
-  if (threadIdx.x == 0) sums[blockIdx.x] = tot;
+  for (int w = 0; w < kSortWarps; ++w) t += s[w];
+  return t;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_sums(u32* sums, int nb) {
-  __shared__ u64 s_warp[kScanThreads / 32 + 1];
-  u32 carry = 0;
-  for (int c0 = 0; c0 < nb; c0 += kScanThreads) {
-    const int i = c0 + threadIdx.x;
-    const u32 v = i < nb ? sums[i] : 0u;
-    u32 ex, ex2, tot, tot2;
-    block_scan2<kScanThreads>(v, 0u, ex, ex2, tot, tot2, s_warp);
-    if (i < nb) sums[i] = carry + ex;
-    carry += tot;
-    __syncthreads();
+// live slots per chunk; also empties the digit counts and notes flags other
+// than 0 and 1 (the gather then copies the flags)
+__global__ void __launch_bounds__(kSortThreads) k_sort_count(SlabDev s, SortScratch p) {
+  __shared__ u32 s_red[kSortWarps];
+  const int chunk = chunk_of(s.cap, gridDim.x);
+  const long long lo = (long long)blockIdx.x * chunk;
+  const int hi = (int)min((long long)s.cap, lo + chunk);
+  u32 n = 0;
+  bool other = false;
+  // flags are padded to whole tiles, with zeros
+  for (int i = (int)min(lo, (long long)s.cap) + 4 * (int)threadIdx.x; i < hi; i += 4 * kSortThreads) {
+    const int4 f = *reinterpret_cast<const int4*>(s.active + i);
+    n += (f.x != 0) + (f.y != 0) + (f.z != 0) + (f.w != 0);
+    other |= ((f.x | f.y | f.z | f.w) & ~1) != 0;
   }
+  const u32 t = block_total(n, s_red);
+  if (threadIdx.x == 0) p.counts[blockIdx.x] = t;
+  if (other) p.digits[kPasses * kBins] = 1u;  // (emptied by the memset before this launch)
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_add(u32* a, int n, const u32* sums) {
-  const u32 add = sums[blockIdx.x];
-  const int b0 = blockIdx.x * kScanBlock;
-  for (int j = threadIdx.x; j < kScanBlock; j += kScanThreads)
-    if (b0 + j < n) a[b0 + j] += add;
+// live slots before this chunk, and in all, in every thread
+__device__ __forceinline__ void live_prefix(const SortScratch& p, u32& before, u32& total, u32* s_red) {
+  u32 b = 0, t = 0;
+  for (int j = threadIdx.x; j < (int)gridDim.x; j += kSortThreads) {
+    const u32 c = p.counts[j];
+    t += c;
+    if (j < (int)blockIdx.x) b += c;
+  }
+  before = block_total(b, s_red);
+  total = block_total(t, s_red);
 }
 
-// Stable scatter of one pass. The tile's items are taken in rounds of 256
-// (slot order within the tile = round, warp, lane); an item's rank among the
-// tile's items with its digit = the count from earlier rounds + the counts of
-// lower warps in this round + the lower lanes of its warp with that digit.
-// The items are first placed in shared memory in (digit, rank) order, then
-// written out in that order, so that consecutive threads write consecutive
-// addresses of one digit's run.
-__global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const u32* __restrict__ key, const u32* __restrict__ val,
-                                                               int n, int pass, int G, const u32* __restrict__ off,
-                                                               u32* key_out, u32* val_out) {
-  __shared__ u32 s_key[kSortTile], s_val[kSortTile];  // the tile in (digit, rank) order
-  __shared__ u32 s_run[kBins];                // items of each digit in earlier rounds
-  __shared__ u32 s_off[kBins];                // the tile's global offset of each digit
-  __shared__ u32 s_start[kBins];              // a digit's first position in the tile order
-  __shared__ unsigned short s_wc[kSortWarps][kBins];  // this round's count per warp and digit
-  __shared__ u64 s_warp[kSortWarps + 1];
-  const int t = blockIdx.x;
+// Pack the live slots' (key, slot) pairs in slot order; placeholder r goes to
+// entry cap - 1 - r of the same list (the pairs never reach it). The keys of a
+// tile are strided loads of one sector each, 16 in flight per thread.
+__global__ void __launch_bounds__(kSortThreads, kSortCtasPerSm) k_sort_pack(SlabDev s, SortScratch p, int field) {
+  __shared__ u32 s_red[kSortWarps];
+  __shared__ u32 s_hist[kPasses][kBins];
+  __shared__ u32 s_wcnt[kSortWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_tile = min(kSortTile, n - t * kSortTile);
-  {
-    // the tile's count of digit d: the next (digit, tile) entry's offset minus its own
-    const size_t e = (size_t)threadIdx.x * G + t;
-    const u32 o = off[e];
-    const u32 next = e + 1 < (size_t)kBins * G ? off[e + 1] : (u32)n;
-    u32 ex, ex2, tot, tot2;
-    block_scan2<kSortThreads>(next - o, 0u, ex, ex2, tot, tot2, s_warp);
-    s_off[threadIdx.x] = o;
-    s_start[threadIdx.x] = ex;
-    s_run[threadIdx.x] = 0u;
-  }
-  for (int w = 0; w < kSortWarps; ++w) s_wc[w][threadIdx.x] = 0;
-  __syncthreads();
+  for (int b = 0; b < kPasses; ++b) s_hist[b][threadIdx.x] = 0u;
+  griddep_wait();
+  u32 before, total;
+  live_prefix(p, before, total, s_red);
+  const int chunk = chunk_of(s.cap, gridDim.x);
+  const long long lo = (long long)blockIdx.x * chunk;
   const u32 lt = (1u << lane) - 1u;
-  u32 kr[kSortItems], vr[kSortItems];  // all of the thread's items in flight at once
+  for (long long t0 = lo; t0 < lo + chunk && t0 < s.cap; t0 += kSortTile) {
+    const int w0 = (int)t0 + warp * kWarpItems;
+    u32 live[kSortItems], key[kSortItems];
 #pragma unroll
-  for (int r = 0; r < kSortItems; ++r) {
-    const int j = r * kSortThreads + threadIdx.x;
-    kr[r] = j < n_tile ? key[t * kSortTile + j] : 0u;
-    vr[r] = j < n_tile ? val[t * kSortTile + j] : 0u;
-  }
-#pragma unroll
-  for (int r = 0; r < kSortItems; ++r) {
-    const int j = r * kSortThreads + threadIdx.x;
-    const bool ok = j < n_tile;
-    const u32 k = kr[r], v = vr[r];
-    const u32 d = ok ? digit_of(k, v, pass) : (u32)kBins;  // kBins: no item
-    const u32 peers = __match_any_sync(0xFFFFFFFFu, d);
-    const u32 below = (u32)__popc(peers & lt);
-    if (ok && below == 0) s_wc[warp][d] = (unsigned short)__popc(peers);
-    __syncthreads();
-    if (ok) {
-      u32 pos = s_start[d] + s_run[d] + below;
-      for (int w = 0; w < warp; ++w) pos += s_wc[w][d];
-      s_key[pos] = k;
-      s_val[pos] = v;
+    for (int j = 0; j < kSortItems; ++j) {
+      const int i = w0 + 32 * j + lane;
+      live[j] = i < s.cap && s.active[i] != 0;
     }
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+      const int i = w0 + 32 * j + lane;
+      key[j] = live[j] ? (u32)s.fields[(size_t)i * s.Fp + field] ^ 0x80000000u : 0u;
+    }
+    u32 n = 0;
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+      live[j] = __ballot_sync(0xFFFFFFFFu, live[j]);
+      n += __popc(live[j]);
+    }
+    __syncthreads();  // s_wcnt of the previous tile is read
+    if (lane == 0) s_wcnt[warp] = n;
     __syncthreads();
-    {
-      u32 add = 0;
-      for (int w = 0; w < kSortWarps; ++w) {
-        add += s_wc[w][threadIdx.x];
-        s_wc[w][threadIdx.x] = 0;
+    u32 rank = before;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) {
+      if (w < warp) rank += s_wcnt[w];
+      before += s_wcnt[w];
+    }
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+      const int i = w0 + 32 * j + lane;
+      const u32 r = rank + __popc(live[j] & lt);
+      const bool on = (live[j] >> lane) & 1u;
+      if (on) {
+        p.key[0][r] = key[j];
+        p.val[0][r] = (u32)i;
+      } else if (i < s.cap) {
+        p.val[0][s.cap - 1 - (i - (int)r)] = (u32)i;
       }
-      s_run[threadIdx.x] += add;
+      rank += __popc(live[j]);
+      // digit counts; a byte that is the same in the whole warp costs one atomic
+      if (live[j]) {
+        const int first = __ffs(live[j]) - 1;
+#pragma unroll
+        for (int b = 0; b < kPasses; ++b) {
+          const u32 d = (key[j] >> (8 * b)) & 0xFFu;
+          const u32 d0 = __shfl_sync(0xFFFFFFFFu, d, first);
+          if (__all_sync(0xFFFFFFFFu, !on || d == d0)) {
+            if (lane == first) atomicAdd(&s_hist[b][d0], (u32)__popc(live[j]));
+          } else if (on) {
+            atomicAdd(&s_hist[b][d], 1u);
+          }
+        }
+      }
     }
-    __syncthreads();
   }
-  for (int j = threadIdx.x; j < n_tile; j += kSortThreads) {
-    const u32 k = s_key[j], v = s_val[j];
-    const u32 d = digit_of(k, v, pass);
-    const u32 pos = s_off[d] + ((u32)j - s_start[d]);
-    key_out[pos] = k;
-    val_out[pos] = v;
+  __syncthreads();
+  for (int b = 0; b < kPasses; ++b)
+    if (s_hist[b][threadIdx.x]) atomicAdd(&p.digits[b * kBins + threadIdx.x], s_hist[b][threadIdx.x]);
+}
+
+// What a pass has to know, from the digit counts (every thread of a block of
+// kSortThreads): the number of pairs, whether the pass's byte varies, which of
+// the two buffers holds the pairs before it, and whether a later byte varies.
+struct PassInfo {
+  int n;
+  bool run, last;
+  bool odd;  // the pairs lie in the second buffer
+  __device__ __forceinline__ u32* in(u32* const (&b)[2]) const { return odd ? b[1] : b[0]; }
+  __device__ __forceinline__ u32* out(u32* const (&b)[2]) const { return odd ? b[0] : b[1]; }
+};
+
+__device__ __forceinline__ PassInfo pass_info(const SortScratch& p, int pass, u32* s_red) {
+  u32 c[kPasses];
+#pragma unroll
+  for (int b = 0; b < kPasses; ++b) c[b] = p.digits[b * kBins + threadIdx.x];
+  PassInfo f;
+  f.n = (int)block_total(c[0], s_red);
+  u32 varies = 0;
+#pragma unroll
+  for (int b = 0; b < kPasses; ++b)
+    if (!__syncthreads_or(c[b] == (u32)f.n)) varies |= 1u << b;  // (also true of no pairs at all: nothing runs)
+  f.odd = __popc(varies & ((1u << pass) - 1u)) & 1;
+  f.run = (varies >> pass) & 1u;
+  f.last = (varies >> pass) == 1u;
+  return f;
+}
+
+// a pass's digit counts per chunk
+__global__ void __launch_bounds__(kSortThreads) k_sort_hist(SortScratch p, int pass) {
+  __shared__ u32 s_cnt[kBins];
+  __shared__ u32 s_red[kSortWarps];
+  s_cnt[threadIdx.x] = 0u;
+  griddep_wait();
+  const PassInfo f = pass_info(p, pass, s_red);
+  if (!f.run) return;
+  const int chunk = chunk_of(f.n, gridDim.x);
+  const long long lo = (long long)blockIdx.x * chunk;
+  const u32* key = f.in(p.key);
+  __syncthreads();
+  for (long long t0 = lo; t0 < lo + chunk && t0 < f.n; t0 += kSortTile) {
+    u32 k[kSortItems];
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+      const long long i = t0 + j * kSortThreads + threadIdx.x;
+      k[j] = i < f.n ? key[i] : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+      const long long i = t0 + j * kSortThreads + threadIdx.x;
+      if (i < f.n) atomicAdd(&s_cnt[(k[j] >> (8 * pass)) & 0xFFu], 1u);
+    }
+  }
+  __syncthreads();
+  p.hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = s_cnt[threadIdx.x];
+}
+
+// digit counts per chunk -> positions: a digit's first position (a scan of the
+// digit counts, in every CTA) plus the counts of the chunks before; one warp
+// per digit
+__global__ void __launch_bounds__(kSortThreads) k_sort_scan(SortScratch p, int pass, int G) {
+  __shared__ u32 s_red[kSortWarps];
+  __shared__ u64 s_warp[kSortWarps + 1];
+  __shared__ u32 s_first[kBins];
+  griddep_wait();
+  const PassInfo f = pass_info(p, pass, s_red);
+  if (!f.run) return;
+  u32 ex, ex2, tot, tot2;
+  block_scan2<kSortThreads>(p.digits[pass * kBins + threadIdx.x], 0u, ex, ex2, tot, tot2, s_warp);
+  s_first[threadIdx.x] = ex;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, d = blockIdx.x * kSortWarps + (threadIdx.x >> 5);
+  u32* row = p.hist + (size_t)d * G;
+  u32 carry = s_first[d];
+  for (int j0 = 0; j0 < G; j0 += 128) {  // four chunks per lane at a time
+    u32 v[4], sum = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = j0 + 4 * lane + u;
+      v[u] = j < G ? row[j] : 0u;
+      sum += v[u];
+    }
+    u32 inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u32 x = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += x;
+    }
+    u32 at = carry + inc - sum;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = j0 + 4 * lane + u;
+      if (j < G) row[j] = at;
+      at += v[u];
+    }
+    carry += __shfl_sync(0xFFFFFFFFu, inc, 31);
   }
 }
 
-// row i of the sorted slab <- row (val[i] without the flag) of the old one
-__global__ void k_sort_gather(SlabDev s, const u32* __restrict__ val, int32_t* fields_out, int32_t* active_out,
-                              int32_t* perm_out, const int* nonbinary) {
-  const bool exact = *nonbinary != 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.cap; i += gridDim.x * blockDim.x) {
-    const u32 v = val[i];
-    const int src = (int)(v & ~kPlaceholder);
-    // the flag travels with the value; only other nonzero live values need the old array
-    active_out[i] = exact ? s.active[src] : ((v & kPlaceholder) ? 0 : 1);
-    const int32_t* a = s.fields + (size_t)src * s.Fp;
-    int32_t* b = fields_out + (size_t)i * s.Fp;
-    for (int f = 0; f < s.Fp; f += 4) *reinterpret_cast<int4*>(b + f) = *reinterpret_cast<const int4*>(a + f);
-    if (perm_out) perm_out[i] = src;
+// Stable scatter of one pass, tile by tile of the CTA's chunk. Each warp ranks
+// its 512 consecutive pairs on its own (warp match; its digit counts in shared
+// memory), without block barriers; the warps' counts then give every pair its
+// place in the tile's (digit, rank) order. The pairs are placed there in shared
+// memory and written out in that order, so that consecutive threads write
+// consecutive addresses of one digit's run.
+__global__ void __launch_bounds__(kSortThreads, kSortCtasPerSm) k_sort_scatter(SortScratch p, int pass) {
+  __shared__ u32 s_key[kSortTile], s_val[kSortTile];
+  __shared__ u32 s_wc[kSortWarps][kBins];  // per warp: pairs of each digit, then its first place in the tile order
+  __shared__ u32 s_off[kBins];             // global position of a digit's place 0 of the tile order
+  __shared__ u64 s_warp[kSortWarps + 1];
+  __shared__ u32 s_red[kSortWarps];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  griddep_wait();
+  const PassInfo f = pass_info(p, pass, s_red);
+  if (!f.run) return;
+  const u32 *key = f.in(p.key), *val = f.in(p.val);
+  u32 *key_out = f.out(p.key), *val_out = f.out(p.val);
+  const int chunk = chunk_of(f.n, gridDim.x);
+  const long long lo = (long long)blockIdx.x * chunk;
+  const u32 lt = (1u << lane) - 1u;
+  u32 pos = p.hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x];  // digit threadIdx.x's next position
+  for (long long t0 = lo; t0 < lo + chunk && t0 < f.n; t0 += kSortTile) {
+    const int n_tile = (int)min((long long)kSortTile, f.n - t0);
+    u32 k[kSortItems], rank[kSortItems / 2];  // ranks below 512: two to a register
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+      const int i = warp * kWarpItems + 32 * j + lane;
+      k[j] = i < n_tile ? key[t0 + i] : 0u;
+    }
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) s_wc[w][threadIdx.x] = 0u;
+    __syncthreads();
+    u32* wc = s_wc[warp];
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+      const bool ok = warp * kWarpItems + 32 * j + lane < n_tile;
+      const u32 d = ok ? (k[j] >> (8 * pass)) & 0xFFu : (u32)kBins;  // kBins: no pair
+      const u32 peers = __match_any_sync(0xFFFFFFFFu, d);
+      const u32 below = (u32)__popc(peers & lt);
+      const u32 c = ok ? wc[d] : 0u;
+      __syncwarp();
+      if (ok && below == 0) wc[d] = c + (u32)__popc(peers);
+      __syncwarp();
+      if (j & 1) rank[j >> 1] |= (c + below) << 16;
+      else rank[j >> 1] = c + below;
+    }
+    __syncthreads();
+    u32 cnt = 0;
+    {
+      u32 c[kSortWarps];
+#pragma unroll
+      for (int w = 0; w < kSortWarps; ++w) {
+        c[w] = s_wc[w][threadIdx.x];
+        cnt += c[w];
+      }
+      u32 ex, ex2, tot, tot2;
+      block_scan2<kSortThreads>(cnt, 0u, ex, ex2, tot, tot2, s_warp);
+      s_off[threadIdx.x] = pos - ex;
+      pos += cnt;
+#pragma unroll
+      for (int w = 0; w < kSortWarps; ++w) {
+        s_wc[w][threadIdx.x] = ex;
+        ex += c[w];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+      const int i = warp * kWarpItems + 32 * j + lane;
+      if (i < n_tile) {
+        const u32 at = wc[(k[j] >> (8 * pass)) & 0xFFu] + ((rank[j >> 1] >> (16 * (j & 1))) & 0xFFFFu);
+        s_key[at] = k[j];
+        s_val[at] = val[t0 + i];
+      }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n_tile; i += kSortThreads) {
+      const u32 kk = s_key[i];
+      const u32 at = s_off[(kk >> (8 * pass)) & 0xFFu] + (u32)i;
+      if (!f.last) key_out[at] = kk;
+      val_out[at] = s_val[i];
+    }
+    __syncthreads();
+  }
+}
+
+// Row i of the sorted slab <- its old row. A thread moves 16-byte quads of
+// rows, four in flight; the quads of one row go to neighbouring threads. Bound
+// by the random rows' DRAM bursts.
+__global__ void __launch_bounds__(kSortThreads) k_sort_gather(SlabDev s, SortScratch p, int32_t* perm_out) {
+  __shared__ u32 s_red[kSortWarps];
+  griddep_wait();
+  // after the last pass: the buffer that holds the pairs, and their number
+  const PassInfo f = pass_info(p, kPasses, s_red);
+  const u32* val = f.in(p.val);
+  const bool exact = p.digits[kPasses * kBins] != 0u;
+  constexpr int U = 4;
+  const u32 q = (u32)s.Fp >> 2, sh = q == 4 ? 2 : q - 1;  // 1 to 4 quads a row
+  const u32 n = (u32)s.cap * q, T = gridDim.x * kSortThreads;
+  for (u32 e0 = blockIdx.x * kSortThreads + threadIdx.x; e0 < n; e0 += U * T) {
+    int src[U];
+    u32 row[U];
+    int4 r[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const u32 e = e0 + u * T;
+      src[u] = -1;
+      row[u] = q == 3 ? e / 3u : e >> sh;
+      if (e < n) {
+        const int i = (int)row[u];
+        src[u] = (int)(i < f.n ? val[i] : p.val[0][s.cap - 1 - (i - f.n)]);
+        if (!in_range(src[u], s.cap, s.err)) src[u] = -1;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (src[u] >= 0)
+        r[u] = __ldcs(reinterpret_cast<const int4*>(s.fields) + (u32)src[u] * q + (e0 + u * T - row[u] * q));
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (src[u] < 0) continue;
+      const u32 e = e0 + u * T;
+      reinterpret_cast<int4*>(p.fields)[e] = r[u];
+      if (e == row[u] * q) {
+        p.active[row[u]] = exact ? s.active[src[u]] : ((int)row[u] < f.n ? 1 : 0);
+        if (perm_out) perm_out[row[u]] = src[u];
+      }
+    }
   }
 }
 
@@ -226,18 +423,16 @@ static abm_status sort_scratch(abm_slab* s, SortScratch** out) {
   p->cap = s->d.cap;
   p->n_pad = s->n_pad;
   p->Fp = s->d.Fp;
-  p->G = (s->d.cap + kSortTile - 1) / kSortTile;
-  const size_t nh = (size_t)kBins * p->G;
-  const size_t nb = (nh + kScanBlock - 1) / kScanBlock;
+  p->G = std::min((s->d.cap + kSortTile - 1) / kSortTile, num_sms() * kSortCtasPerSm);
   bool ok = true;
   for (int b = 0; b < 2 && ok; ++b)
     ok = cudaMalloc(&p->key[b], sizeof(u32) * (size_t)p->cap) == cudaSuccess &&
          cudaMalloc(&p->val[b], sizeof(u32) * (size_t)p->cap) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->hist, sizeof(u32) * nh) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->sums, sizeof(u32) * nb) == cudaSuccess;
+  ok = ok && cudaMalloc(&p->hist, sizeof(u32) * (size_t)kBins * p->G) == cudaSuccess;
+  ok = ok && cudaMalloc(&p->counts, sizeof(u32) * (size_t)p->G) == cudaSuccess;
+  ok = ok && cudaMalloc(&p->digits, sizeof(u32) * (kPasses * kBins + 1)) == cudaSuccess;
   ok = ok && cudaMalloc(&p->fields, sizeof(int32_t) * (size_t)p->n_pad * p->Fp) == cudaSuccess;
   ok = ok && cudaMalloc(&p->active, sizeof(int32_t) * (size_t)p->n_pad) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->nonbinary, sizeof(int)) == cudaSuccess;
   // rows past the capacity are never gathered: keep them as the slab keeps its own
   ok = ok && cudaMemset(p->fields, 0, sizeof(int32_t) * (size_t)p->n_pad * p->Fp) == cudaSuccess;
   ok = ok && cudaMemset(p->active, 0, sizeof(int32_t) * (size_t)p->n_pad) == cudaSuccess;
@@ -264,30 +459,19 @@ extern "C" abm_status abm_sort(abm_slab* s, int32_t field, int32_t* out_perm, vo
   abm_status e = sort_scratch(s, &p);
   if (e != ABM_OK) return e;
   cudaStream_t st = (cudaStream_t)stream;
-  const int n = s->d.cap, G = p->G;
-  const int nh = kBins * G;
-  const int nb = (nh + kScanBlock - 1) / kScanBlock;
-  const int grid = std::max(1, std::min((n + 255) / 256, num_sms() * 8));
-  ABM_CUDA_TRY(cudaMemsetAsync(p->nonbinary, 0, sizeof(int), st));
-  k_sort_init<<<grid, 256, 0, st>>>(s->d, field, p->key[0], p->val[0], p->nonbinary);
+  const int G = p->G;
+  ABM_CUDA_TRY(cudaMemsetAsync(p->digits, 0, sizeof(u32) * (kPasses * kBins + 1), st));
+  k_sort_count<<<G, kSortThreads, 0, st>>>(s->d, *p);
   ABM_LAUNCH_CHECK();
-  int cur = 0;
-  for (int pass = 0; pass < 5; ++pass) {
-    k_sort_hist<<<G, kSortThreads, 0, st>>>(p->key[cur], p->val[cur], n, pass, G, p->hist);
-    ABM_LAUNCH_CHECK();
-    k_scan_blocks<<<nb, kScanThreads, 0, st>>>(p->hist, nh, p->sums);
-    ABM_LAUNCH_CHECK();
-    k_scan_sums<<<1, kScanThreads, 0, st>>>(p->sums, nb);
-    ABM_LAUNCH_CHECK();
-    k_scan_add<<<nb, kScanThreads, 0, st>>>(p->hist, nh, p->sums);
-    ABM_LAUNCH_CHECK();
-    k_sort_scatter<<<G, kSortThreads, 0, st>>>(p->key[cur], p->val[cur], n, pass, G, p->hist, p->key[cur ^ 1],
-                                               p->val[cur ^ 1]);
-    ABM_LAUNCH_CHECK();
-    cur ^= 1;
+  ABM_CUDA_TRY(launch_pdl(k_sort_pack, G, kSortThreads, st, s->d, *p, (int)field));
+  for (int pass = 0; pass < kPasses; ++pass) {
+    ABM_CUDA_TRY(launch_pdl(k_sort_hist, G, kSortThreads, st, *p, pass));
+    ABM_CUDA_TRY(launch_pdl(k_sort_scan, kBins / kSortWarps, kSortThreads, st, *p, pass, G));
+    ABM_CUDA_TRY(launch_pdl(k_sort_scatter, G, kSortThreads, st, *p, pass));
   }
-  k_sort_gather<<<grid, 256, 0, st>>>(s->d, p->val[cur], p->fields, p->active, out_perm, p->nonbinary);
-  ABM_LAUNCH_CHECK();
+  const long long quads = (long long)s->d.cap * (s->d.Fp >> 2);
+  const int grid = (int)std::min<long long>((quads + kSortThreads - 1) / kSortThreads, (long long)num_sms() * 8);
+  ABM_CUDA_TRY(launch_pdl(k_sort_gather, grid, kSortThreads, st, s->d, *p, out_perm));
   // the gathered arrays become the slab's; the old ones are the next sort's targets
   std::swap(s->d.fields, p->fields);
   std::swap(s->d.active, p->active);

@@ -446,3 +446,27 @@ def test_argument_errors(eng):
     assert L.abm_select(s.h, None, None, None, None) == abm.ERR_ARG
     p = abm.pred(abm.PRED_FIELD, field=2)
     assert L.abm_select(s.h, C.byref(p), None, None, None) == abm.ERR_ARG
+
+
+@pytest.mark.parametrize("n,F", [(1, 1), (4095, 4), (4096, 9), (4097, 16), (8193, 5), (700_001, 2)])
+@pytest.mark.parametrize("keys", ["equal", "byte2", "signed", "all_bits", "none_live", "all_live"])
+def test_sort_agents_key_ranges(eng, n, F, keys):
+    """Whole numbers, so exact: keys whose bytes are all alike (their passes are left out), in every position,
+    negative keys, all bits, and no or only live agents, at the edges of the sort's tiles."""
+    rng = np.random.default_rng(n + F)
+    k = {"equal": np.full(n, -7), "byte2": rng.integers(0, 40, n) << 16, "signed": rng.integers(-300, 300, n),
+         "all_bits": rng.integers(-2**31, 2**31, n)}.get(keys, rng.integers(0, 1000, n)).astype(np.int32)
+    live = {"none_live": np.zeros(n), "all_live": np.ones(n)}.get(keys, rng.random(n) < 0.6).astype(np.int32)
+    rest = rng.integers(-2**31, 2**31, (F, n)).astype(np.int32)
+    field = F - 1
+    rest[field] = k
+    s = eng.Slab(n, F)
+    for f in range(F):
+        s.write(f, torch.from_numpy(rest[f]).cuda())
+    s.write(-1, torch.from_numpy(live).cuda())
+    assert s.counters()["n_active"] == int(live.sum())
+    want = np.lexsort((np.arange(n), np.where(live, k, 0), live == 0))
+    np.testing.assert_array_equal(np_of(s.sort(field)), want)
+    np.testing.assert_array_equal(np_of(s.read(-1)), live[want])
+    for f in range(F):
+        np.testing.assert_array_equal(np_of(s.read(f)), rest[f][want])
