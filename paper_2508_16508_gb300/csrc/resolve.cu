@@ -39,26 +39,36 @@ __global__ void __launch_bounds__(kResThreads) k_claims(const int32_t* __restric
   }
   if (threadIdx.x == 0) s_used = 0;
   __syncthreads();
-  const int nchunks = (M + kResChunk - 1) / kResChunk;
-  for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    const int m0 = c * kResChunk;
+  // a contiguous run of claims per CTA, in chunks of kResChunk (the last one ragged)
+  const long long run = ((long long)M + gridDim.x - 1) / gridDim.x;
+  const int lo = (int)min((long long)M, run * blockIdx.x), hi = (int)min((long long)M, run * (blockIdx.x + 1));
+  for (int m0 = lo; m0 < hi; m0 += kResChunk) {
+    int rr[kResPerThread];
+    u32 pp[kResPerThread];
 #pragma unroll
     for (int j = 0; j < kResPerThread; ++j) {
-      const int m = m0 + j * kResThreads + threadIdx.x;  // coalesced
-      if (m >= M) continue;
-      const int r = res[m];
+      const int m = m0 + j * kResThreads + threadIdx.x;  // coalesced, all in flight
+      rr[j] = m < hi ? res[m] : -1;
+      pp[j] = m < hi ? prio[m] : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < kResPerThread; ++j) {
+      const int m = m0 + j * kResThreads + threadIdx.x;
+      const int r = rr[j];
       if (r < 0 || r >= R) continue;
-      const u64 key = ((u64)prio[m] << 32) | (u32)m;
+      const u64 key = ((u64)pp[j] << 32) | (u32)m;
       u32 h = ((u32)r * 2654435761u) >> (32 - kHashBits);
       bool done = false;
       for (int p = 0; p < kMaxProbe; ++p) {
-        int t = s_tag[h];
+        int t = *reinterpret_cast<volatile int*>(&s_tag[h]);
         if (t == -1) {
           t = atomicCAS(&s_tag[h], -1, r);
           if (t == -1) atomicAdd(&s_used, 1);
         }
         if (t == -1 || t == r) {
-          atomicMin(&s_best[h], key);
+          // most claims on a popular resource lose to one already seen: a plain
+          // read (keys only fall) spares them the contended 64-bit atomic
+          if (key < *reinterpret_cast<volatile u64*>(&s_best[h])) atomicMin(&s_best[h], key);
           done = true;
           break;
         }
@@ -68,9 +78,9 @@ __global__ void __launch_bounds__(kResThreads) k_claims(const int32_t* __restric
     }
     __syncthreads();
     // The table is folded into global memory only when it is half full or the
-    // CTA has no chunks left: skewed claims (a few hot resources) then cost
+    // CTA has no claims left: skewed claims (a few hot resources) then cost
     // one global atomic per distinct resource per CTA, not per chunk.
-    if (s_used > kHash / 2 || c + (int)gridDim.x >= nchunks) {
+    if (s_used > kHash / 2 || m0 + kResChunk >= hi) {
       for (int h = threadIdx.x; h < kHash; h += kResThreads) {
         const int t = s_tag[h];
         if (t >= 0) {
@@ -88,6 +98,7 @@ __global__ void __launch_bounds__(kResThreads) k_claims(const int32_t* __restric
 
 // winner per resource, then restore the table to "no claim"
 __global__ void k_winners(u64* table, int R, int32_t* winner) {
+  griddep_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < R; i += gridDim.x * blockDim.x) {
     const u64 v = table[i];
     winner[i] = v == kNoKey ? -1 : (int32_t)(u32)v;
@@ -97,6 +108,7 @@ __global__ void k_winners(u64* table, int R, int32_t* winner) {
 
 __global__ void k_is_winner(const int32_t* __restrict__ res, int M, int R, const int32_t* __restrict__ winner,
                             uint8_t* is_winner) {
+  griddep_wait();
   // 4 claims per thread: one 128-bit load of resource ids, one 32-bit store of flags
   const int n4 = M >> 2;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += gridDim.x * blockDim.x) {
@@ -118,6 +130,7 @@ __global__ void k_is_winner(const int32_t* __restrict__ res, int M, int R, const
 
 __global__ void k_is_winner_scalar(const int32_t* __restrict__ res, int M, int R,
                                    const int32_t* __restrict__ winner, uint8_t* is_winner) {
+  griddep_wait();
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
     const int r = res[m];
     is_winner[m] = (r >= 0 && r < R && winner[r] == m) ? 1 : 0;
@@ -137,17 +150,16 @@ abm_status resolve_launch(const int32_t* claim_res, const uint32_t* claim_prio, 
     k_claims<<<grid, kResThreads, smem, st>>>(claim_res, claim_prio, M, R, (u64*)table);
     ABM_LAUNCH_CHECK();
   }
-  k_winners<<<std::max(1, std::min((R + 255) / 256, sms * 8)), 256, 0, st>>>((u64*)table, R, out_winner);
-  ABM_LAUNCH_CHECK();
+  ABM_CUDA_TRY(launch_pdl(k_winners, std::max(1, std::min((R + 255) / 256, sms * 8)), 256, st, (u64*)table, (int)R,
+                          out_winner));
   if (out_is_winner && M > 0) {
     if ((((uintptr_t)claim_res) & 15) == 0 && (((uintptr_t)out_is_winner) & 3) == 0) {
-      k_is_winner<<<std::max(1, std::min((M / 4 + 255) / 256, sms * 8)), 256, 0, st>>>(
-          claim_res, M, R, out_winner, out_is_winner);
+      ABM_CUDA_TRY(launch_pdl(k_is_winner, std::max(1, std::min((M / 4 + 255) / 256, sms * 8)), 256, st, claim_res,
+                              (int)M, (int)R, (const int32_t*)out_winner, out_is_winner));
     } else {
-      k_is_winner_scalar<<<std::max(1, std::min((M + 255) / 256, sms * 8)), 256, 0, st>>>(
-          claim_res, M, R, out_winner, out_is_winner);
+      ABM_CUDA_TRY(launch_pdl(k_is_winner_scalar, std::max(1, std::min((M + 255) / 256, sms * 8)), 256, st, claim_res,
+                              (int)M, (int)R, (const int32_t*)out_winner, out_is_winner));
     }
-    ABM_LAUNCH_CHECK();
   }
   return ABM_OK;
 }
