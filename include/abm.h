@@ -400,7 +400,8 @@ abm_status abm_step_graph(abm_world* w, int32_t nsteps, int32_t reps, abm_step_s
 abm_status abm_step_profiled(abm_world* w, int32_t nsteps, abm_step_stats* stats, float* phase_ms,
                              void* stream);
 /* Execution engine of abm_step: ABM_ENGINE_PERSISTENT (default) runs all
- * requested steps in one cooperative launch of `ctas_per_sm` CTAs per SM
+ * requested steps in one cooperative launch of at most `ctas_per_sm` CTAs per
+ * SM (one while the sheep extent is small enough for that to be faster)
  * with bounded grid barriers between the phases; ABM_ENGINE_KERNELS runs six
  * kernels per step (and is what abm_step_profiled, energy statistics and
  * abm_step_graph use). Results are identical. */

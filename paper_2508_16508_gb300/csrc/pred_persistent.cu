@@ -1026,6 +1026,7 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
       c->hw[s] = s_book.hw[s];
       c->overflow[s] = s_book.ovf[s];
     }
+    note_class(w, ext[0], ext[1]);
   }
 }
 
@@ -1045,6 +1046,8 @@ int persistent_max_ctas() {
 }
 
 int persistent_warps() { return kPWarps; }
+
+int persistent_round_units() { return kQ * kSheepWarps; }
 
 abm_status launch_persistent(const WorldDev& d, u32* bar_next, int grid, int nsteps, abm_step_stats* stats,
                              cudaStream_t st, unsigned long long* phase_ns) {

@@ -352,6 +352,8 @@ __global__ void k_view_commit(WorldCtr* c, int sp, const int32_t* counters, cons
 // ============================================================================
 using namespace abm;
 
+constexpr int kResidentSlots = 3072;  // slots up to which one CTA is faster than the grid (see launch_steps)
+
 struct abm_world {
   WorldDev d;
   int cap_pad[2];
@@ -395,6 +397,7 @@ static void world_free(abm_world* w) {
   cudaFree(w->d.snext);
   cudaFree(w->d.wkey);
   cudaFree(w->d.wnext);
+  if (w->d.class_host) cudaFreeHost(w->d.class_host);  // (the frees above waited for every launch)
   if (w->gexec) cudaGraphExecDestroy(w->gexec);
   slab_free_view(w->view[0]);
   slab_free_view(w->view[1]);
@@ -452,6 +455,7 @@ extern "C" abm_status abm_create(const abm_config* cfg, void* stream, abm_world*
   ok = ok && cudaMalloc(&d.wclaim, sizeof(u64) * (size_t)d.ncells) == cudaSuccess;
   ok = ok && cudaMalloc(&d.ctr, sizeof(WorldCtr)) == cudaSuccess;
   ok = ok && cudaMalloc(&d.err, sizeof(int)) == cudaSuccess;
+  ok = ok && cudaHostAlloc(&d.class_host, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess;
   w->pgrid_max = persistent_max_ctas();
   if (w->pgrid_max < 1) ok = false;
   const int pmax = std::max(1, w->pgrid_max);
@@ -494,6 +498,9 @@ extern "C" abm_status abm_create(const abm_config* cfg, void* stream, abm_world*
   w->grid = num_sms() * 8;
   w->engine = ABM_ENGINE_PERSISTENT;
   w->pgrid = std::min(w->pgrid_max, num_sms() * 2);
+  d.class_small = resident_fits(d) ? kResidentSlots : -1;
+  d.class_round = num_sms() * persistent_round_units() * 128;
+  *d.class_host = extent_class(d, cfg->n0[0], cfg->n0[1]);
   k_world_init<<<num_sms() * 4, 256, 0, st>>>(d, cfg->n0[0], cfg->n0[1]);
   for (int s = 0; s < 2; ++s)  // check builds: canaries past the capacity
     if (slab_canary_fill(reinterpret_cast<int32_t*>(d.sp[s].agent), 4, d.sp[s].cap, w->cap_pad[s], st) != ABM_OK)
@@ -504,6 +511,26 @@ extern "C" abm_status abm_create(const abm_config* cfg, void* stream, abm_world*
   }
   *out = w;
   return ABM_OK;
+}
+
+// The launch of the next steps, by the size class of the extents that the last
+// finished launch left (a later one only costs speed, never results).
+// Class 0: one CTA with the state in its shared memory (launch_resident). A
+// step there costs 4 us for a few hundred agents and grows with the slots,
+// 12.8 us at 3441; the persistent kernel takes 14 us from 1 to 10,000.
+// Class 1: one persistent CTA per SM while that takes every sheep unit in one
+// round (then the moved agents stay in shared memory for the meals). A barrier
+// of fewer CTAs and twice the registers per thread are worth 2 us a step: 301 x
+// 301 cells 18.1 -> 15.8 us, 1400 x 1400 (3811 sheep units) 21.1 -> 18.9.
+// Class 2: the tuned number of CTAs; at 2048 x 2048 (two rounds of one CTA per
+// SM) the second CTA per SM wins, 33.7 us against 38.7.
+static abm_status launch_steps(abm_world* w, int nsteps, abm_step_stats* stats, cudaStream_t st,
+                               unsigned long long* phase_ns = nullptr) {
+  WorldDev d = w->d;
+  d.class_known = *reinterpret_cast<volatile int*>(d.class_host);
+  if (d.class_known == 0 && !phase_ns) return launch_resident(d, nsteps, stats, st);
+  const int grid = d.class_known < 2 ? std::min(w->pgrid, num_sms()) : w->pgrid;
+  return launch_persistent(d, &w->bar_next, grid, nsteps, stats, st, phase_ns);
 }
 
 // ev (nullable): 7 events recorded around the six kernels of the step
@@ -542,7 +569,7 @@ extern "C" abm_status abm_step_profiled(abm_world* w, int32_t nsteps, abm_step_s
     ABM_CUDA_TRY(cudaEventCreate(&e0));
     ABM_CUDA_TRY(cudaEventCreate(&e1));
     cudaEventRecord(e0, st);
-    abm_status rc = nsteps > 0 ? launch_persistent(w->d, &w->bar_next, w->pgrid, nsteps, stats, st, ns) : ABM_OK;
+    abm_status rc = nsteps > 0 ? launch_steps(w, nsteps, stats, st, ns) : ABM_OK;
     cudaEventRecord(e1, st);
     unsigned long long h[8] = {0};
     if (rc == ABM_OK) {
@@ -596,7 +623,7 @@ extern "C" abm_status abm_step(abm_world* w, int32_t nsteps, abm_step_stats* sta
   if (want_energy && w->d.variant != ABM_VARIANT_ONE_WOLF) return ABM_ERR_ARG;
   if (w->engine == ABM_ENGINE_PERSISTENT && !want_energy) {
     if (nsteps == 0) return ABM_OK;
-    abm_status e = launch_persistent(w->d, &w->bar_next, w->pgrid, nsteps, stats, (cudaStream_t)stream);
+    abm_status e = launch_steps(w, nsteps, stats, (cudaStream_t)stream);
     if (e == ABM_OK) w->steps_host += nsteps;
     return e;
   }
@@ -792,6 +819,7 @@ extern "C" abm_status abm_load(abm_world* w, const void* buf, size_t bytes, void
   ABM_CUDA_TRY(cudaMemsetAsync(w->d.ps.bar, 0, sizeof(u32) * 2, st));
   w->bar_next = 0;
   ABM_CUDA_TRY(cudaStreamSynchronize(st));
+  *w->d.class_host = extent_class(w->d, h.extent[0], h.extent[1]);
   w->steps_host = h.step;
   return ABM_OK;
 }

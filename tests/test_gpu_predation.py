@@ -352,3 +352,34 @@ def test_large_config_full_run_vs_stored_oracle(eng):
     st["grass.wait"] = gw.grass("wait").cpu().numpy()
     assert state_sha256(st) == want_sha
     gw.check()
+
+
+@pytest.mark.parametrize("side,cap,n0,kw", [
+    (40, (2048, 1024), (100, 25), {}),                                                   # stays small
+    (45, (7000, 1000), (1500, 300), dict(sheep_gain=40, regrowth=1, wolf_gain=1)),       # grows past 3072 slots
+    (1, (40, 5), (3, 2), dict(sheep_repro=0.9)), (7, (33, 32), (32, 31), dict(sheep_gain=20)),
+    (100, (32000, 700), (600, 90), dict(sheep_gain=30, regrowth=2))])                    # too large for one CTA
+def test_small_world_launches_agree(eng, side, cap, n0, kw):
+    """One CTA with the state in shared memory and the persistent grid (which step_profiled always takes) alternate
+    on one world and run alone on another; both equal the oracle, also where the population outgrows the one-CTA
+    launch, and for a world with several launches in flight."""
+    c = dict(side=side, n0=n0, cap=cap, seed=5, model=2, params=workloads.predation_params(**kw))
+    gw, ow = make(eng, c)
+    gp = eng.World(side, 5, 2, c["params"], cap, n0)
+    stats, pstats = gw.new_stats(28), gp.new_stats(28)
+    for k in range(4):
+        gw.step(1, stats[7 * k:7 * k + 1])
+        gw.step(3, stats[7 * k + 1:7 * k + 4])
+        if k % 2:
+            gw.step_profiled(3, stats[7 * k + 4:7 * k + 7])
+        else:
+            gw.step(3, stats[7 * k + 4:7 * k + 7])
+        gp.step_profiled(7, pstats[7 * k:7 * k + 7])
+    ost = ow.step(28)
+    for g, p, o in zip(eng.decode_stats(stats), eng.decode_stats(pstats), ost):
+        compare_stats(g, o, energy=False)
+        compare_stats(p, o, energy=False)
+    compare_state(gw, ow, "mixed")
+    compare_state(gp, ow, "persistent")
+    gw.check()
+    gp.check()
