@@ -48,25 +48,51 @@ struct PredDev {
   int field, cmp, and_mask, value;
 };
 
-__device__ __forceinline__ bool eval_pred(const PredDev& p, const SlabDev& s, int slot, int live) {
+// The N slots from `base` on (those below n) that satisfy the predicate, as a
+// bit mask. live: their live flags. The words of the live slots are all
+// requested before the first is used: fetched slot by slot behind a test of the
+// flag, sixteen fields a lane took 8 us of round trips.
+template <int N>
+__device__ __forceinline__ u32 pred_mask(const PredDev& p, const SlabDev& s, int base, int n, const int (&live)[N]) {
+  u32 on = 0;
+#pragma unroll
+  for (int j = 0; j < N; ++j) on |= (u32)(live[j] != 0) << j;
+  const u32 valid = n - base >= N ? (N == 32 ? 0xFFFFFFFFu : (1u << (N & 31)) - 1u) : (n > base ? (1u << (n - base)) - 1u : 0u);
+  if (p.kind == ABM_PRED_FREE) return ~on & valid;
+  on &= valid;
+  if (p.kind == ABM_PRED_LIVE || on == 0u) return on;
+  u32 m = 0;
   switch (p.kind) {
-    case ABM_PRED_LIVE: return live != 0;
-    case ABM_PRED_FREE: return live == 0;
     case ABM_PRED_BERNOULLI:
-      return live && draw(s.seed, s.model, p.step, (u32)slot, p.purpose, p.species) < p.threshold;
-    case ABM_PRED_MASK: return live && p.mask[slot] != 0;
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+        m |= (u32)(draw(s.seed, s.model, p.step, (u32)(base + j), p.purpose, p.species) < p.threshold) << j;
+      return m & on;
+    case ABM_PRED_MASK: {
+      int v[N];
+#pragma unroll
+      for (int j = 0; j < N; ++j) v[j] = (on >> j) & 1u ? p.mask[base + j] : 0;
+#pragma unroll
+      for (int j = 0; j < N; ++j) m |= (u32)(v[j] != 0) << j;
+      return m & on;
+    }
     case ABM_PRED_FIELD: {
-      if (!live) return false;
-      const int v = s.fields[(size_t)slot * s.Fp + p.field] & p.and_mask;
-      switch (p.cmp) {
-        case ABM_CMP_EQ: return v == p.value;
-        case ABM_CMP_NE: return v != p.value;
-        case ABM_CMP_LT: return v < p.value;
-        default: return v >= p.value;
+      int v[N];
+#pragma unroll
+      for (int j = 0; j < N; ++j) v[j] = (on >> j) & 1u ? s.fields[(size_t)(base + j) * s.Fp + p.field] : 0;
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const int x = v[j] & p.and_mask;
+        const bool f = p.cmp == ABM_CMP_EQ   ? x == p.value
+                       : p.cmp == ABM_CMP_NE ? x != p.value
+                       : p.cmp == ABM_CMP_LT ? x < p.value
+                                             : x >= p.value;
+        m |= (u32)f << j;
       }
+      return m & on;
     }
   }
-  return false;
+  return 0;
 }
 
 enum Op { OP_SELECT = 0, OP_REMOVE = 1, OP_ADD = 2, OP_UPDATE = 3, OP_FUSED = 4, OP_ARRAY = 5 };
@@ -196,17 +222,15 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count(ScanArgs a) {
       }
       live[4 * v + 0] = q.x; live[4 * v + 1] = q.y; live[4 * v + 2] = q.z; live[4 * v + 3] = q.w;
     }
-    u32 ma = 0, mb = 0, mr = 0;  // 16-bit masks over the lane's slots
+    const u32 valid = a.n - base >= kLaneSlots ? 0xFFFFu : (a.n > base ? (1u << (a.n - base)) - 1u : 0u);
+    u32 ma = 0, mr = 0;  // 16-bit masks over the lane's slots
+    if (OP == OP_ARRAY || OP == OP_ADD) {
 #pragma unroll
-    for (int j = 0; j < kLaneSlots; ++j) {
-      const int slot = base + j;
-      bool f = false;
-      if (slot < a.n) {
-        if (OP == OP_ARRAY) f = live[j] != 0;
-        else if (OP == OP_ADD) f = live[j] == 0;
-        else f = eval_pred(a.pred, s, slot, live[j]) != (a.negate != 0);
-      }
-      ma |= (u32)f << j;
+      for (int j = 0; j < kLaneSlots; ++j) ma |= (u32)((live[j] != 0) == (OP == OP_ARRAY)) << j;
+      ma &= valid;
+    } else {
+      ma = pred_mask<kLaneSlots>(a.pred, s, base, a.n, live);
+      if (a.negate) ma = ~ma & valid;
     }
     if (OP == OP_REMOVE) mr = ma;
     // removed slots become placeholders now: rewrite only the 4-slot groups
@@ -229,7 +253,6 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count(ScanArgs a) {
       }
     }
     ca += __popc(ma);
-    cb += __popc(mb);
     if (OP != OP_REMOVE) {
       const u32 na = __shfl_down_sync(0xFFFFFFFFu, ma, 1);
       if (!(lane & 1) && base < a.n) a.planeA[base >> 5] = ma | (na << 16);
@@ -248,12 +271,17 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count(ScanArgs a) {
     a.totals[2 * blockIdx.x + 1] = cb;
   }
   if (OP == OP_REMOVE) {
-    if (last_cta_out(a.ctrl)) {
-      int A = 0;
-      for (int b = 0; b < a.G; ++b) A += (int)a.totals[2 * b];
-      s.counters[0] -= A;
-      if (a.out_count) *a.out_count = A;
-      __threadfence();
+    __shared__ bool s_last;
+    const bool last = last_cta_out(a.ctrl);
+    if (threadIdx.x == 0) s_last = last;
+    __syncthreads();
+    if (!s_last) return;
+    u32 A = 0, B = 0;
+    for (int b = threadIdx.x; b < a.G; b += THREADS) A += ld_relaxed32(a.totals + 2 * b);
+    block_sum2<THREADS>(A, B, s_red);
+    if (threadIdx.x == 0) {
+      s.counters[0] -= (int)A;
+      if (a.out_count) *a.out_count = (int)A;
     }
   }
 }
@@ -761,6 +789,290 @@ __global__ void __launch_bounds__(256, 2) k_apply(ScanArgs a) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// Small sets: one launch per operation. Up to kSmallMax slots are held by one
+// thread-block cluster, LS consecutive slots per lane, so that flags, ranks and
+// record moves happen in one kernel: the CTAs' counts are exchanged through
+// distributed shared memory between two cluster barriers. Three launches that
+// each touch 0.4 MB cost their launches and round trips, not their bytes. GPU
+// time of a select / update / remove / add back to back, three launches against
+// one: 1000 slots 9.2 / 11.0 / 9.2 / 8.2 -> 2.2 / 2.8 / 2.1 / 1.8 us; 100,003
+// slots 10.2 / 14.3 / 10.3 / 8.2 -> 5.5 / 7.0 / 5.0 / 3.2; at 262,144 slots,
+// where 16 SMs do what 64 CTAs do above it, 8.4 / 11.0 / 7.7 / 4.2 (three
+// launches at 300,000: 8.2 / 12.3 / 8.2 / 8.2).
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallCtas = 16;  // cluster size, at most (above 8: opt-in)
+constexpr int kSmallMax = kSmallCtas * kSmallThreads * 16;
+
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// the 64-bit word at this CTA's shared address p, in the cluster's CTA `rank`
+__device__ __forceinline__ u64 ld_cluster(const u64* p, u32 rank) {
+  u32 at;
+  u64 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(at) : "memory");
+  return v;
+}
+
+// Records r0 .. r0 + n - 1 of a warp's staged slots (offsets from slot0): whole
+// rows, neighbouring lanes on neighbouring words of a record.
+// ADD: added to the row (wrapping); id_field >= 0: that field is id0 + r instead.
+__device__ __forceinline__ void move_small(const SlabDev& s, const unsigned short* stage, int slot0, u32 n, u32 r0,
+                                           const int32_t* rec, const int32_t* rec_idx, bool add, int id_field, int id0,
+                                           int lane) {
+  const u32 F = (u32)s.F;
+  if ((F & 3u) == 0u && ((uintptr_t)rec & 15) == 0) {
+    const u32 q = F >> 2;
+    for (u32 e = lane; e < n * q; e += 32) {
+      const u32 i = q == 1 ? e : (q == 2 ? e >> 1 : e / q), c = e - i * q;
+      const int slot = slot0 + stage[i];
+      if (!in_range(slot, s.cap, s.err)) continue;
+      const u32 j = rec_idx ? (u32)rec_idx[r0 + i] : r0 + i;
+      int4 r = __ldg(reinterpret_cast<const int4*>(rec) + (size_t)j * q + c);
+      int4* d = reinterpret_cast<int4*>(s.fields + (size_t)slot * s.Fp) + c;
+      if (add) {
+        const int4 o = *d;
+        r = make_int4((int)((u32)o.x + (u32)r.x), (int)((u32)o.y + (u32)r.y), (int)((u32)o.z + (u32)r.z),
+                      (int)((u32)o.w + (u32)r.w));
+      }
+      const int id = (int)((u32)id0 + r0 + i), f = id_field - 4 * (int)c;
+      if (f == 0) r.x = id;
+      if (f == 1) r.y = id;
+      if (f == 2) r.z = id;
+      if (f == 3) r.w = id;
+      *d = r;
+    }
+  } else {
+    for (u32 e = lane; e < n * F; e += 32) {
+      const u32 i = e / F, f = e - i * F;
+      const int slot = slot0 + stage[i];
+      if (!in_range(slot, s.cap, s.err)) continue;
+      const u32 j = rec_idx ? (u32)rec_idx[r0 + i] : r0 + i;
+      int v = rec[(size_t)j * F + f];
+      int32_t* d = s.fields + (size_t)slot * s.Fp + f;
+      if (add) v = (int)((u32)*d + (u32)v);
+      if ((int)f == id_field) v = (int)((u32)id0 + r0 + i);
+      *d = v;
+    }
+  }
+}
+
+template <int OP, int LS>
+__global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constant__ ScanArgs a) {
+  constexpr int STEP = 32 * LS;  // slots of a warp
+  __shared__ u64 s_w[kSmallWarps];
+  __shared__ u64 s_tot;     // this CTA's counts: A << 32 | B
+  __shared__ u64 s_pre[2];  // the CTAs before, all
+  __shared__ unsigned short s_stage[kSmallWarps * STEP];
+  const SlabDev& s = a.s;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int slot0 = ((int)blockIdx.x * kSmallWarps + warp) * STEP;
+  const int base = slot0 + LS * lane;
+  griddep_wait();
+  const int32_t* flag_src = OP == OP_ARRAY ? a.src : s.active;
+  int live[LS];
+  if (base + LS <= a.n && (((uintptr_t)flag_src) & 15) == 0) {
+#pragma unroll
+    for (int v = 0; v < LS / 4; ++v) {
+      const int4 q = *reinterpret_cast<const int4*>(flag_src + base + 4 * v);
+      live[4 * v] = q.x; live[4 * v + 1] = q.y; live[4 * v + 2] = q.z; live[4 * v + 3] = q.w;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < LS; ++j) live[j] = base + j < a.n ? flag_src[base + j] : 0;
+  }
+  // read before the barrier after which CTA 0 changes them
+  const int id0 = s.counters[1];
+  const int nrec = (OP == OP_UPDATE && a.use_rec_idx) ? s.counters[3] : a.k;
+  const u32 valid = a.n - base >= LS ? (1u << LS) - 1u : (a.n > base ? (1u << (a.n - base)) - 1u : 0u);
+  u32 on = 0, ma = 0, mb = 0, mr = 0;  // live; selected / free; chosen; removed
+#pragma unroll
+  for (int j = 0; j < LS; ++j) on |= (u32)(live[j] != 0) << j;
+  on &= valid;
+  if (OP == OP_ARRAY) {
+    ma = on;
+  } else if (OP == OP_ADD) {
+    ma = ~on & valid;
+  } else if (OP == OP_FUSED) {
+    u32 dr = 0, dc = 0;
+#pragma unroll
+    for (int m = 0; m < LS / 2; ++m) {
+      const uint4 u = mask_pair_draw((u32)(base >> 1) + m, a.mk, a.rk);
+      dr |= (u.x < a.threshold ? 1u << (2 * m) : 0u) | (u.z < a.threshold ? 2u << (2 * m) : 0u);
+      dc |= (u.y < a.threshold ? 1u << (2 * m) : 0u) | (u.w < a.threshold ? 2u << (2 * m) : 0u);
+    }
+    mr = on & dr;
+    on &= ~dr;
+    ma = ~on & valid;
+    mb = on & dc;
+  } else {
+    ma = pred_mask<LS>(a.pred, s, base, a.n, live);
+    if (a.negate) ma = ~ma & valid;
+    if (OP == OP_REMOVE) mr = ma;
+  }
+  // ranks: lanes, warps, CTAs
+  const u32 c = (u32)__popc(ma) | ((u32)__popc(mb) << 16);
+  u32 inc = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const u32 t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  const u32 ex = inc - c, tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+  if (lane == 0) s_w[warp] = ((u64)(tot & 0xFFFFu) << 32) | (tot >> 16);
+  __syncthreads();
+  u64 wv = s_w[lane], wpre = lane < warp ? wv : 0ull;  // kSmallWarps == 32
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    wv += __shfl_xor_sync(0xFFFFFFFFu, wv, o);
+    wpre += __shfl_xor_sync(0xFFFFFFFFu, wpre, o);
+  }
+  u64 pre = 0, all = wv;
+  if (gridDim.x > 1) {
+    if (threadIdx.x == 0) s_tot = wv;
+    cluster_arrive();
+    cluster_wait();
+    if (warp == 0) {
+      u64 t = lane < (int)gridDim.x ? ld_cluster(&s_tot, (u32)lane) : 0ull;
+      u64 p = lane < (int)blockIdx.x ? t : 0ull;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+        p += __shfl_xor_sync(0xFFFFFFFFu, p, o);
+      }
+      if (lane == 0) {
+        s_pre[0] = p;
+        s_pre[1] = t;
+      }
+    }
+    __syncthreads();
+    cluster_arrive();  // the others' counts are read; waited for before leaving
+    pre = s_pre[0];
+    all = s_pre[1];
+  } else {
+    __syncthreads();  // every thread has read the counters that are changed below
+  }
+  pre += wpre;
+  const u32 sa = (u32)(pre >> 32), sb = (u32)pre;
+  const int A = (int)(all >> 32), B = (int)all;
+  // removed slots become placeholders: k_count's (4-slot groups, other flags kept) and k_count_fused's (8-slot groups
+  // as 0/1) writes
+  if (OP == OP_REMOVE) {
+#pragma unroll
+    for (int v = 0; v < LS / 4; ++v) {
+      const u32 g = (mr >> (4 * v)) & 0xFu;
+      if (!g) continue;
+      const int b = base + 4 * v;
+      const int4 q = make_int4((g & 1u) ? 0 : live[4 * v], (g & 2u) ? 0 : live[4 * v + 1],
+                               (g & 4u) ? 0 : live[4 * v + 2], (g & 8u) ? 0 : live[4 * v + 3]);
+      if (b + 3 < a.n) {
+        *reinterpret_cast<int4*>(s.active + b) = q;
+      } else {
+        if (b + 0 < a.n) s.active[b + 0] = q.x;
+        if (b + 1 < a.n) s.active[b + 1] = q.y;
+        if (b + 2 < a.n) s.active[b + 2] = q.z;
+      }
+    }
+  }
+  const u32 limit = (u32)(OP == OP_UPDATE ? nrec : (OP == OP_SELECT || OP == OP_ARRAY ? 0x7FFFFFFF : a.k));
+  u32 na = 0;
+  if (OP != OP_REMOVE && sa < limit) na = min(tot & 0xFFFFu, limit - sa);
+  if (OP == OP_ADD || OP == OP_FUSED) {
+    // final flags: live, or free with a rank below the limit. Written as 0/1 in whole groups: the 16 slots around an
+    // added agent, the 8 around a removed one
+    const u32 e0 = ex & 0xFFFFu;
+    const u32 mine = e0 < na ? min((u32)__popc(ma), na - e0) : 0u;
+    const u32 added = mine == (u32)__popc(ma) ? ma : (mine ? ma & ((1u << __fns(ma, 0, (int)mine + 1)) - 1u) : 0u);
+    const u32 nl = on | added;
+    const u32 ab = __ballot_sync(0xFFFFFFFFu, added != 0u);
+    u32 wr = LS == 16 ? (added ? valid : 0u)
+                      : (((ab >> (lane & ~(16 / LS - 1))) & ((1u << (16 / LS)) - 1u)) ? valid : 0u);
+    if (OP == OP_FUSED) {
+      if (LS >= 8) {
+#pragma unroll
+        for (int h = 0; h < LS / 8; ++h)
+          if ((mr >> (8 * h)) & 0xFFu) wr |= valid & (0xFFu << (8 * h));
+      } else {
+        const u32 rb = __ballot_sync(0xFFFFFFFFu, mr != 0u);
+        if ((rb >> (lane & ~1)) & 3u) wr = valid;
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < LS / 4; ++v) {
+      if (!((wr >> (4 * v)) & 0xFu)) continue;
+      const u32 g = nl >> (4 * v);
+      const int b = base + 4 * v;
+      if (b + 3 < a.n) {
+        *reinterpret_cast<int4*>(s.active + b) =
+            make_int4((int)(g & 1u), (int)((g >> 1) & 1u), (int)((g >> 2) & 1u), (int)((g >> 3) & 1u));
+      } else {
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          if (b + j < a.n) s.active[b + j] = (int)((g >> j) & 1u);
+      }
+    }
+  }
+  // the selected slots in rank order, then lists and records
+  unsigned short* stage = s_stage + warp * STEP;
+  if (OP != OP_REMOVE && na) {
+    u32 pos = ex & 0xFFFFu;
+#pragma unroll
+    for (int j = 0; j < LS; ++j)
+      if ((ma >> j) & 1u) stage[pos++] = (unsigned short)(LS * lane + j);
+    __syncwarp();
+    int32_t* const list = a.list_a + (OP == OP_SELECT && a.list_base ? *a.list_base : 0);
+    if (OP != OP_FUSED)  // (the selective-update call hands no list out)
+      for (u32 i = lane; i < na; i += 32) list[sa + i] = slot0 + stage[i];
+    if (OP == OP_ADD || OP == OP_FUSED)
+      move_small(s, stage, slot0, na, sa, a.rec, nullptr, false, OP == OP_ADD ? a.id_field : -1, id0, lane);
+    if (OP == OP_UPDATE)
+      move_small(s, stage, slot0, na, sa, a.rec, a.use_rec_idx ? s.rec_idx : nullptr, a.op_kind == ABM_OP_ADD, -1, 0,
+                 lane);
+    __syncwarp();
+  }
+  if (OP == OP_FUSED && sb < (u32)a.k && (tot >> 16)) {
+    const u32 nb = min(tot >> 16, (u32)a.k - sb);
+    u32 pos = ex >> 16;
+#pragma unroll
+    for (int j = 0; j < LS; ++j)
+      if ((mb >> j) & 1u) stage[pos++] = (unsigned short)(LS * lane + j);
+    __syncwarp();
+    move_small(s, stage, slot0, nb, sb, a.rec2, nullptr, true, -1, 0, lane);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (OP == OP_SELECT || OP == OP_ARRAY) {
+      if (a.out_count) *a.out_count = A;
+      if (OP == OP_ARRAY) s.counters[3] = A;
+    } else if (OP == OP_REMOVE) {
+      s.counters[0] -= A;
+      if (a.out_count) *a.out_count = A;
+    } else if (OP == OP_ADD) {
+      const int r = min(a.k, A);
+      s.counters[0] += r;
+      if (a.id_field >= 0) s.counters[1] = (int)((u32)id0 + (u32)r);
+      if (a.k > A) s.counters[2] = 1;
+      if (a.out_count) *a.out_count = r;
+    } else if (OP == OP_UPDATE) {
+      if (a.out_count) *a.out_count = min(A, nrec);
+    } else {  // A = free after removal, B = chosen survivors
+      const int n_before = s.counters[0];
+      const int added = min(a.k, A);
+      s.counters[0] = s.cap - A + added;
+      if (a.k > A) s.counters[2] = 1;
+      if (a.out_count) {
+        a.out_count[0] = A - (s.cap - n_before);
+        a.out_count[1] = added;
+        a.out_count[2] = min(a.k, B);
+      }
+    }
+  }
+  if (gridDim.x > 1) cluster_wait();
+}
+
 // --------------------------------------------------------------------------
 // check builds: the fields past the capacity hold the canary, the live flags
 // there stay 0; k_canary_check records kErrCheck if either changed
@@ -1157,6 +1469,36 @@ static int apply_grid() {
   return num_sms() * b;
 }
 
+// One cluster of as few CTAs as hold the slots, LS slots per lane.
+template <int OP, int LS>
+static abm_status launch_small(const ScanArgs& a, cudaStream_t st) {
+  static std::atomic<unsigned long long> wide{0};  // devices on which the kernel may use clusters above 8
+  const int ctas = (a.n + kSmallThreads * LS - 1) / (kSmallThreads * LS);
+  if (ctas > 8) {
+    int dev = 0;
+    ABM_CUDA_TRY(cudaGetDevice(&dev));
+    const unsigned long long bit = (dev >= 0 && dev < 64) ? 1ull << dev : 0ull;
+    if (!bit || !(wide.load(std::memory_order_acquire) & bit)) {
+      ABM_CUDA_TRY(cudaFuncSetAttribute(k_small<OP, LS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      wide.fetch_or(bit, std::memory_order_release);
+    }
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)ctas;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  ABM_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_small<OP, LS>, a));
+  return ABM_OK;
+}
+
 // Up to three launches per operation: flags + per-warp / per-CTA counts, then
 // ranks + slot lists, then the record moves. Each warp owns one static
 // segment of slots in the first two passes; no CTA waits for another.
@@ -1176,6 +1518,10 @@ static abm_status launch_scan(abm_slab* s, const ScanArgs& a, bool aux, cudaStre
     if (OP == OP_ARRAY) ABM_CUDA_TRY(cudaMemsetAsync(s->d.counters + 3, 0, sizeof(int32_t), st));
     return ABM_OK;
   }
+  // small sets: one launch (see k_small); few slots per lane while one cluster has the lanes
+  if (b.n <= kSmallThreads * kSmallCtas * 4) return launch_small<OP, 4>(b, st);
+  if (b.n <= kSmallThreads * kSmallCtas * 8) return launch_small<OP, 8>(b, st);
+  if (b.n <= kSmallMax) return launch_small<OP, 16>(b, st);
   const int target = std::max(1, std::min(num_sms() * ctas_per_sm, s->max_ctas));
   const long per = ((long)b.n + target - 1) / target;
   b.chunk = (int)(((per + SUB - 1) / SUB) * SUB);

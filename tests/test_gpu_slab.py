@@ -470,3 +470,78 @@ def test_sort_agents_key_ranges(eng, n, F, keys):
     np.testing.assert_array_equal(np_of(s.read(-1)), live[want])
     for f in range(F):
         np.testing.assert_array_equal(np_of(s.read(f)), rest[f][want])
+
+
+@pytest.mark.parametrize("n", [1, 31, 4097, 65_536, 65_537, 131_072, 131_073, 200_001, 262_144, 262_145])
+@pytest.mark.parametrize("F", [1, 3, 8, 12])
+def test_one_launch_sizes(eng, n, F):
+    """Whole numbers, so exact: every set operation at the sizes where the one-launch path changes its slots per lane
+    and its cluster, and one slot past it, against the operations written out with numpy; flags other than 0 and 1."""
+    from paper_2508_16508_gb300 import abm
+    rng = np.random.default_rng(n * 16 + F)
+    s = eng.Slab(n, F, seed=9)
+    act = np.where(rng.random(n) < 0.5, rng.choice([1, 1, 1, 7], n), 0).astype(np.int32)
+    fld = rng.integers(-50, 50, (F, n)).astype(np.int32)
+    s.write(-1, torch.from_numpy(act).cuda())
+    for f in range(F):
+        s.write(f, torch.from_numpy(fld[f]).cuda())
+    k = max(1, n // 7)
+    rec = rng.integers(-2**31, 2**31, (k, F)).astype(np.int32)
+    rmask = (rng.random(k) < 0.5).astype(np.int32)
+    dev = torch.from_numpy(rec).cuda()
+
+    def check(where):
+        np.testing.assert_array_equal(np_of(s.read(-1)) != 0, act != 0, err_msg=where)
+        for f in range(F):
+            np.testing.assert_array_equal(np_of(s.read(f)), fld[f], err_msg=where)
+        assert s.counters()["n_active"] == int((act != 0).sum()), where
+
+    p = abm.pred(abm.PRED_FIELD, field=F - 1, cmp=abm.CMP_LT, value=0)
+    idx, cnt = s.select(p)
+    want = np.flatnonzero((act != 0) & (fld[F - 1] < 0))
+    np.testing.assert_array_equal(np_of(idx)[:int(cnt)], want)
+    perm, cnt = s.select_permutation(p)
+    sel = (act != 0) & (fld[F - 1] < 0)
+    np.testing.assert_array_equal(np_of(perm), np.argsort(~sel, kind="stable"))
+    for masked, op in ((False, abm.OP_ADD), (True, abm.OP_SET)):
+        p = abm.pred(abm.PRED_FIELD, field=0, cmp=abm.CMP_GE, value=-10)
+        sel = np.flatnonzero((act != 0) & (fld[0] >= -10))
+        rows = rec[rmask != 0] if masked else rec
+        r = min(len(sel), len(rows))
+        slots, cnt = s.update_distinct(p, dev, torch.from_numpy(rmask).cuda() if masked else None, op=op)
+        assert int(cnt) == r
+        np.testing.assert_array_equal(np_of(slots)[:r], sel[:r])
+        for f in range(F):
+            fld[f][sel[:r]] = rows[:r, f] + (fld[f][sel[:r]] if op == abm.OP_ADD else 0)
+        check(f"update {masked}")
+    m = torch.from_numpy((rng.random(n + 1) < 0.3).astype(np.int32)).cuda()[1:]  # not 16-byte aligned
+    gone = (act != 0) & (np_of(m) != 0)
+    assert int(s.remove(abm.pred(abm.PRED_MASK, mask=m))) == int(gone.sum())
+    act[gone] = 0
+    check("remove")
+    for id_field in (-1, F - 1):
+        free = np.flatnonzero(act == 0)
+        r = min(k, len(free))
+        first = s.counters()["next_id"]
+        slots, cnt = s.add(dev, id_field=id_field)
+        assert int(cnt) == r
+        np.testing.assert_array_equal(np_of(slots)[:r], free[:r])
+        act[free[:r]] = 1
+        for f in range(F):
+            fld[f][free[:r]] = first + np.arange(r) if f == id_field else rec[:r, f]
+        check(f"add {id_field}")
+    # the fused call against remove, update and add of the oracle's draws
+    o = oracle.Slab(n, F)
+    o.active[:] = np_of(s.read(-1))
+    for f in range(F):
+        o.fields[f][:] = fld[f]
+    if F <= 8:
+        T, kk = workloads.threshold(0.3), max(1, n // 5)
+        a = s.philox_records(4, abm.P_NEWREC0, abm.P_NEWREC1, kk)
+        b = s.philox_records(4, abm.P_DELTA0, abm.P_DELTA1, kk)
+        s.selective_update(4, T, a, b)
+        o.c1_call(4, T, kk, seed=9)
+        np.testing.assert_array_equal(np_of(s.read(-1)) != 0, o.active != 0)
+        for f in range(F):
+            np.testing.assert_array_equal(np_of(s.read(f)), o.fields[f])
+    s.check()
