@@ -65,14 +65,14 @@ class Slab:
 
     def select(self, p: abm.abm_pred, stream=None):
         idx = torch.empty(self.capacity, **self._i32)
-        cnt = torch.zeros(1, **self._i32)
+        cnt = torch.empty(1, **self._i32)  # (counts are always written: no fill kernel)
         call("abm_select", self.h, C.byref(p), ptr(idx), ptr(cnt), _stream(stream))
         return idx, cnt
 
     def select_permutation(self, p: abm.abm_pred, stream=None):
         """All slots, those satisfying p first (ascending), then the rest (ascending)."""
         perm = torch.empty(self.capacity, **self._i32)
-        cnt = torch.zeros(1, **self._i32)
+        cnt = torch.empty(1, **self._i32)
         call("abm_select_permutation", self.h, C.byref(p), ptr(perm), ptr(cnt), _stream(stream))
         return perm, cnt
 
@@ -84,7 +84,7 @@ class Slab:
         return perm
 
     def remove(self, p: abm.abm_pred, stream=None) -> torch.Tensor:
-        cnt = torch.zeros(1, **self._i32)
+        cnt = torch.empty(1, **self._i32)
         call("abm_remove", self.h, C.byref(p), ptr(cnt), _stream(stream))
         return cnt
 
@@ -92,7 +92,7 @@ class Slab:
         rec = records.to(torch.int32).contiguous()
         k = rec.shape[0] if rec.numel() else 0
         slots = torch.empty(max(k, 1), **self._i32)
-        cnt = torch.zeros(1, **self._i32)
+        cnt = torch.empty(1, **self._i32)
         call("abm_add", self.h, ptr(rec) if k else None, k, id_field, ptr(slots), ptr(cnt),
              _stream(stream))
         return slots, cnt
@@ -103,7 +103,7 @@ class Slab:
         k = rec.shape[0] if rec.numel() else 0
         rm = None if record_mask is None else record_mask.to(torch.int32).contiguous()
         slots = torch.empty(max(min(k, self.capacity), 1), **self._i32)
-        cnt = torch.zeros(1, **self._i32)
+        cnt = torch.empty(1, **self._i32)
         call("abm_update_distinct", self.h, C.byref(p), ptr(rec) if k else None, ptr(rm), k, op,
              ptr(slots), ptr(cnt), _stream(stream))
         return slots, cnt
@@ -111,7 +111,7 @@ class Slab:
     def selective_update(self, step: int, threshold: int, records: torch.Tensor,
                          deltas: torch.Tensor, out_counts: torch.Tensor | None = None, stream=None):
         k = records.shape[0]
-        out = torch.zeros(3, **self._i32) if out_counts is None else out_counts
+        out = torch.empty(3, **self._i32) if out_counts is None else out_counts  # always written
         call("abm_selective_update", self.h, step & 0xFFFFFFFF, threshold & 0xFFFFFFFF,
              ptr(records), ptr(deltas), k, ptr(out), _stream(stream))
         return out
