@@ -244,7 +244,9 @@ abm_status abm_selective_update(abm_slab* s, uint32_t step, uint32_t threshold,
 
 /* Launch shape of abm_selective_update's passes: `threads` per CTA (128, 256
  * or 512) and `ctas_per_sm` CTAs per SM (threads * ctas_per_sm <= 2048).
- * Results never depend on it; the autotuner picks it. Default 256, 8. */
+ * Results never depend on it; the autotuner picks it. Default 256 threads and
+ * 4 or 8 CTAs per SM, by the number of records. Sets of up to 262,144 slots run
+ * in one launch of their own shape. */
 abm_status abm_slab_tune(abm_slab* s, int32_t threads, int32_t ctas_per_sm, void* stream);
 
 /* Fill out[k][F] (device int32) with record j field f = word f%4 of

@@ -103,6 +103,7 @@ struct ScanArgs {
   u32* ctrl;               // [1] CTAs finished, [2] epoch (last-CTA-out bookkeeping)
   u32* planeA;             // n/32 words each: selected / free
   u32* planeB;             // chosen (fused call)
+  u32* planeL;             // the flags in memory after pass 1 that are 1 (fused call)
   u32* totals;             // [2 * G] per-CTA counts
   u32* wtotals;            // [2 * G * warps] per-warp counts
   int n;                   // slots (or array entries for OP_ARRAY)
@@ -332,11 +333,14 @@ __device__ __forceinline__ uint4 mask_pair_draw(u32 j, const u32 (&mk)[5], const
 }
 
 // Pass 1 of the selective-update call: as k_count, with the live flags as a
-// 16-bit mask per lane (any nonzero flag is live) read by two 32-byte loads
-// and written back as 0/1 in whole 8-slot (32-byte) groups; the lane's eight
-// draws are independent and all in flight together. The pass is bound by the
-// Philox draws (one per pair of slots): fewer draws in flight at a higher
-// occupancy measured slower.
+// 16-bit mask per lane (any nonzero flag is live) read by two 32-byte loads;
+// the lane's eight draws are independent and all in flight together. The pass
+// is bound by the Philox draws (one per pair of slots): fewer draws in flight
+// at a higher occupancy measured slower.
+// The flags are not written here: most removed slots are refilled by the same
+// call, so the ranking pass, which knows every final flag, writes the groups
+// that end up different. It compares with plane L. Flags other than 0 and 1
+// are put right at once (whole 8-slot groups, as 0/1).
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count_fused(ScanArgs a) {
   constexpr int WARPS = THREADS / 32;
@@ -349,21 +353,25 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count_fused(ScanArg
   u32 ca = 0, cb = 0;
   for (int b0 = wlo; b0 < whi; b0 += kWarpStep) {
     const int base = b0 + lane * kLaneSlots;
-    // the selective-update call: live flags as a 16-bit mask (any nonzero
-    // flag is live), read with two 32-byte loads, written back as 0/1 in
-    // whole 8-slot (32-byte) groups
     u32 ml = 0;
+    int odd = 0;
     if (base + kLaneSlots <= a.n) {
       int f[8];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         ld_v8(s.active + base + 8 * h, f);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) ml |= (u32)(f[j] != 0) << (8 * h + j);
+        for (int j = 0; j < 8; ++j) {
+          ml |= (u32)(f[j] != 0) << (8 * h + j);
+          odd |= f[j];
+        }
       }
     } else {
       for (int j = 0; j < kLaneSlots; ++j)
-        if (base + j < a.n) ml |= (u32)(s.active[base + j] != 0) << j;
+        if (base + j < a.n) {
+          ml |= (u32)(s.active[base + j] != 0) << j;
+          odd |= s.active[base + j];
+        }
     }
     // the draws' outcomes as 16-bit masks (bit j: slot base + j), combined
     // with the live mask once per 16 slots
@@ -381,28 +389,29 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count_fused(ScanArg
     const u32 al = ml & ~dr;        // still live
     const u32 ma = valid & ~al;     // free after the removals
     const u32 mb = al & dc;         // chosen among the live
-    const u32 nl = ml & ~mr;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (!((mr >> (8 * h)) & 0xFFu)) continue;
-      const int b = base + 8 * h;
-      if (b + 8 <= a.n) {
-        int f[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) f[j] = (int)((nl >> (8 * h + j)) & 1u);
-        st_v8(s.active + b, f);
-      } else {
-        for (int j = 0; j < 8; ++j)
-          if (b + j < a.n) s.active[b + j] = (int)((nl >> (8 * h + j)) & 1u);
+    u32 fl = ml;  // flags that are 1 in memory
+    if (odd & ~1) {
+      const u32 nl = ml & ~mr;
+      fl = 0;
+      for (int j = 0; j < kLaneSlots; ++j) {
+        if (base + j >= a.n) break;
+        if ((mr >> (j & 8)) & 0xFFu) {
+          s.active[base + j] = (int)((nl >> j) & 1u);
+          fl |= nl & (1u << j);
+        } else if (s.active[base + j] == 1) {
+          fl |= 1u << j;
+        }
       }
     }
     ca += __popc(ma);
     cb += __popc(mb);
     const u32 na = __shfl_down_sync(0xFFFFFFFFu, ma, 1);
     const u32 nb = __shfl_down_sync(0xFFFFFFFFu, mb, 1);
+    const u32 nf = __shfl_down_sync(0xFFFFFFFFu, fl, 1);
     if (!(lane & 1) && base < a.n) {
       a.planeA[base >> 5] = ma | (na << 16);
       a.planeB[base >> 5] = mb | (nb << 16);
+      a.planeL[base >> 5] = fl | (nf << 16);
     }
   }
   u64 v = ((u64)ca << 32) | cb;
@@ -425,15 +434,19 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count_fused(ScanArg
 // them out coalesced; steps with no rank below the limit are skipped. The add
 // passes also write the final live flags of every 16-slot group that receives
 // a new agent, whole (0/1), so no flag sector is written in part.
-// The selective-update call's records moved by the pass that ranks them:
-// the staged slots [0, n) of a warp step take records r0 + i (ADDROW: added
-// to the row, wrapping), two 32-byte rows per lane in flight. With a slab
-// that is mostly live, free and chosen slots spread evenly over it, so the
-// static slot partition also balances the record moves.
+// The selective-update call's records moved by the pass that ranks them: the
+// staged slots (offsets from slot0) take records r0 + i, i < n (ADDROW: added to
+// the row, wrapping), U 32-byte rows per lane in flight. Ranks are consecutive
+// over a warp's steps, so a warp stages slots over several steps until it has
+// kMoveBatch of them: four rows per lane, also where few slots are touched (see
+// kMoveShare for what that is worth).
+constexpr int kMoveBatch = 128;
+constexpr int kMoveStage = kMoveBatch + kWarpStep;
+
 template <bool ADDROW>
-__device__ __forceinline__ void move_staged(const ScanArgs& a, const int* stage, u32 n, u32 r0, const int32_t* rec,
-                                            int lane) {
-  constexpr int U = 2;
+__device__ __forceinline__ void move_staged(const ScanArgs& a, const unsigned short* stage, int slot0, u32 n, u32 r0,
+                                            const int32_t* rec, int lane) {
+  constexpr int U = ADDROW ? 2 : 4;
   for (u32 i0 = lane; i0 < n; i0 += 32 * U) {
     int slot[U];
     int r[U][8];
@@ -442,7 +455,7 @@ __device__ __forceinline__ void move_staged(const ScanArgs& a, const int* stage,
       const u32 i = i0 + 32 * u;
       slot[u] = -1;
       if (i < n) {
-        slot[u] = stage[i];
+        slot[u] = slot0 + stage[i];
         if (!in_range(slot[u], a.s.cap, a.s.err)) slot[u] = -1;
         ld_v8_nc(rec + (size_t)(r0 + i) * 8, r[u]);
       }
@@ -463,14 +476,33 @@ __device__ __forceinline__ void move_staged(const ScanArgs& a, const int* stage,
   }
 }
 
+// a lane's flagged slots (bits of m, offsets from off0) to stage[pos ...), those below place `end`. Dense steps go
+// through all 16 places, sparse ones through the set bits only.
+template <typename S>
+__device__ __forceinline__ void stage_bits(S* stage, u32 m, u32 pos, u32 end, int off0, bool dense) {
+  if (dense) {
+#pragma unroll
+    for (int j = 0; j < kLaneSlots; ++j) {
+      const u32 at = pos + (u32)__popc(m & ((1u << j) - 1u));
+      if (((m >> j) & 1u) && at < end) stage[at] = (S)(off0 + j);
+    }
+  } else {
+    while (m && pos < end) {
+      stage[pos++] = (S)(off0 + __ffs(m) - 1);
+      m &= m - 1;
+    }
+  }
+}
+
 // MOVE (selective-update call, 8 fields, 32-byte aligned records): the pass
 // moves the records itself instead of writing the rank-ordered slot lists, and
 // no apply pass follows.
 template <int OP, int THREADS, bool MOVE = false>
-__global__ void __launch_bounds__(THREADS, MOVE ? (768 / THREADS > 0 ? 768 / THREADS : 1) : 1) k_scatter(ScanArgs a) {
+__global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(ScanArgs a) {
   constexpr int WARPS = THREADS / 32;
   __shared__ u64 s_red[WARPS];
-  __shared__ int s_stage[WARPS * kWarpStep];
+  __shared__ int s_stage[MOVE ? 1 : WARPS * kWarpStep];
+  __shared__ unsigned short s_move[MOVE ? WARPS * 2 * kMoveStage : 1];
   griddep_wait();
   const SlabDev& s = a.s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -480,12 +512,13 @@ __global__ void __launch_bounds__(THREADS, MOVE ? (768 / THREADS > 0 ? 768 / THR
   // the plane words of the warp's first step, requested ahead of the prefix
   // sums; each step then requests the next step's words before its own work,
   // so a warp waits for one round trip in all, not one per step
-  u32 wa_next = 0, wb_next = 0;
+  u32 wa_next = 0, wb_next = 0, wl_next = 0;
   {
     const int base = wlo + lane * kLaneSlots;
     if (wlo < whi && base < a.n) {
       wa_next = a.planeA[base >> 5];
       if (OP == OP_FUSED) wb_next = a.planeB[base >> 5];
+      if (OP == OP_FUSED) wl_next = a.planeL[base >> 5];
     }
   }
   u32 pa = 0, pb = 0, ta = 0, tb = 0;
@@ -517,16 +550,22 @@ __global__ void __launch_bounds__(THREADS, MOVE ? (768 / THREADS > 0 ? 768 / THR
   const u32 limit_b = (u32)a.k;
   // ranks land at list_a + *list_base (the permutation's second half)
   int32_t* const list_a = a.list_a + (OP == OP_SELECT && a.list_base ? *a.list_base : 0);
-  int* const stage = s_stage + warp * kWarpStep;
+  int* const stage = s_stage + (MOVE ? 0 : warp * kWarpStep);
+  // MOVE: the slots staged for adds (0) and updates (1): how many, the first one's step and rank
+  unsigned short* const mst[2] = {s_move + (MOVE ? warp * 2 * kMoveStage : 0),
+                                  s_move + (MOVE ? (warp * 2 + 1) * kMoveStage : 0)};
+  u32 mcnt[2] = {0, 0}, mrank[2] = {0, 0};
+  int mbase[2] = {0, 0};
   for (int b0 = wlo; b0 < whi; b0 += kWarpStep) {
     const int base = b0 + lane * kLaneSlots;
-    const u32 wa = wa_next, wb = wb_next;
+    const u32 wa = wa_next, wb = wb_next, wl = wl_next;
     {
       const int nbase = base + kWarpStep;
-      wa_next = wb_next = 0;
+      wa_next = wb_next = wl_next = 0;
       if (b0 + kWarpStep < whi && nbase < a.n) {
         wa_next = a.planeA[nbase >> 5];
         if (OP == OP_FUSED) wb_next = a.planeB[nbase >> 5];
+        if (OP == OP_FUSED) wl_next = a.planeL[nbase >> 5];
       }
     }
     u32 ma = 0, mb = 0;
@@ -547,58 +586,77 @@ __global__ void __launch_bounds__(THREADS, MOVE ? (768 / THREADS > 0 ? 768 / THR
     pa += tot & 0xFFFFu;
     pb += tot >> 16;
     // plane A: the step's ranks [sa, sa + na) are below the limit
-    if (sa < limit && (tot & 0xFFFFu)) {
-      const u32 na = min(tot & 0xFFFFu, limit - sa);
-      const u32 off = ex & 0xFFFFu;
-      // plane A is dense: every flagged slot of the lane goes to its place
-      // below na, unrolled (no loop over the set bits)
+    const u32 na = sa < limit ? min(tot & 0xFFFFu, limit - sa) : 0u;
+    const u32 nb = OP == OP_FUSED && sb < limit_b ? min(tot >> 16, limit_b - sb) : 0u;
+    if constexpr (MOVE) {
+      const u32 n2[2] = {na, nb}, r2[2] = {sa, sb}, m2[2] = {ma, mb}, o2[2] = {ex & 0xFFFFu, ex >> 16};
+      // staged offsets are 16 bits; the next step's must still fit
+      const bool last = b0 + kWarpStep >= whi;
 #pragma unroll
-      for (int j = 0; j < kLaneSlots; ++j) {
-        const u32 pos = off + (u32)__popc(ma & ((1u << j) - 1u));
-        if (((ma >> j) & 1u) && pos < na) stage[pos] = base + j;
-      }
-      __syncwarp();
-      if constexpr (MOVE) move_staged<false>(a, stage, na, sa, a.rec, lane);
-      else for (u32 i = lane; i < na; i += 32) list_a[sa + i] = stage[i];
-      if (OP == OP_ADD || OP == OP_FUSED) {
-        // flags of the lane's 16 slots after the adds: live 1, free 0, and the
-        // free slots with a rank below the limit 1
-        const u32 mine = (ex & 0xFFFFu) < na ? min((u32)__popc(ma), na - (ex & 0xFFFFu)) : 0u;
-        if (mine) {
-          const u32 added = mine == (u32)__popc(ma) ? ma : ma & ((1u << __fns(ma, 0, (int)mine + 1)) - 1u);
-          const u32 valid = base + kLaneSlots <= a.n ? 0xFFFFu : (1u << (a.n - base)) - 1u;
-          const u32 nl = ((~ma & valid) | added) & valid;
-          if (valid == 0xFFFFu) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              int f[8];
-#pragma unroll
-              for (int j = 0; j < 8; ++j) f[j] = (int)((nl >> (8 * h + j)) & 1u);
-              st_v8(s.active + base + 8 * h, f);
-            }
-          } else {
-            for (int j = 0; j < kLaneSlots; ++j)
-              if ((valid >> j) & 1u) s.active[base + j] = (int)((nl >> j) & 1u);
+      for (int k = 0; k < 2; ++k) {
+        if (n2[k]) {
+          if (mcnt[k] == 0) {
+            mbase[k] = b0;
+            mrank[k] = r2[k];
           }
+          stage_bits(mst[k], m2[k], mcnt[k] + o2[k], mcnt[k] + n2[k], base - mbase[k], n2[k] > kWarpStep / 4);
+          mcnt[k] += n2[k];
+        }
+        if (mcnt[k] && (mcnt[k] >= kMoveBatch || last || b0 - mbase[k] + 2 * kWarpStep > 65536)) {
+          __syncwarp();
+          if (k == 0) move_staged<false>(a, mst[0], mbase[0], mcnt[0], mrank[0], a.rec, lane);
+          else move_staged<true>(a, mst[1], mbase[1], mcnt[1], mrank[1], a.rec2, lane);
+          mcnt[k] = 0;
+          __syncwarp();  // the stage is rewritten next
         }
       }
-      __syncwarp();  // the stage is rewritten next
+    } else if (na) {
+      stage_bits(stage, ma, ex & 0xFFFFu, na, base, na > kWarpStep / 4);
+      __syncwarp();
+      for (u32 i = lane; i < na; i += 32) list_a[sa + i] = stage[i];
+    }
+    if (OP == OP_ADD || OP == OP_FUSED) {
+      // flags of the lane's 16 slots after the adds: live 1, free 0, and the
+      // free slots with a rank below the limit 1. An add writes the groups that
+      // receive an agent. The selective-update call writes the 8-slot halves
+      // that an add or a removal left different from memory: a removed slot
+      // that is refilled costs no write (2^24 slots, half of them touched: two
+      // passes over 64 MB of flags less).
+      const u32 off = ex & 0xFFFFu;
+      const u32 mine = off < na ? min((u32)__popc(ma), na - off) : 0u;
+      const u32 added = mine == (u32)__popc(ma) ? ma : (mine ? ma & ((1u << __fns(ma, 0, (int)mine + 1)) - 1u) : 0u);
+      const u32 valid = base + kLaneSlots <= a.n ? 0xFFFFu : (base < a.n ? (1u << (a.n - base)) - 1u : 0u);
+      const u32 nl = ((~ma & valid) | added) & valid;
+      u32 halves = mine ? 3u : 0u;
+      if (OP == OP_FUSED) {
+        const u32 ml = (wl >> (16 * (lane & 1))) & valid;
+        const u32 touched = mine ? 0xFFFFu : ma & ml, diff = nl ^ ml;
+        halves = ((touched & 0xFFu) && (diff & 0xFFu) ? 1u : 0u) | ((touched >> 8) && (diff >> 8) ? 2u : 0u);
+      }
+      if (halves) {
+        if (valid == 0xFFFFu) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (!((halves >> h) & 1u)) continue;
+            int f[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) f[j] = (int)((nl >> (8 * h + j)) & 1u);
+            st_v8(s.active + base + 8 * h, f);
+          }
+        } else {
+          for (int j = 0; j < kLaneSlots; ++j)
+            if (((valid >> j) & 1u) && ((halves >> (j >> 3)) & 1u)) s.active[base + j] = (int)((nl >> j) & 1u);
+        }
+      }
     }
     // plane B (the fused call's chosen survivors), the same way
-    if (OP == OP_FUSED && sb < limit_b && (tot >> 16)) {
-      const u32 nb = min(tot >> 16, limit_b - sb);
-      u32 off = ex >> 16;
-      u32 m = mb;
-      while (m && off < nb) {
-        const int j = __ffs(m) - 1;
-        m &= m - 1;
-        stage[off++] = base + j;
-      }
+    if (!MOVE && nb) {
       __syncwarp();
-      if constexpr (MOVE) move_staged<true>(a, stage, nb, sb, a.rec2, lane);
-      else for (u32 i = lane; i < nb; i += 32) a.list_b[sb + i] = stage[i];
+      stage_bits(stage, mb, ex >> 16, nb, base, nb > kWarpStep / 4);
       __syncwarp();
+      for (u32 i = lane; i < nb; i += 32) a.list_b[sb + i] = stage[i];
     }
+    if (!MOVE) __syncwarp();  // the stage is rewritten next
   }
   if (last_cta_out(a.ctrl)) {
     const int A = (int)ta, B = (int)tb;
@@ -1261,7 +1319,7 @@ static abm_status slab_alloc(int capacity, int n_fields, u32 seed, u32 model, in
   s->n_pad = ((capacity + kSlabTileMax - 1) / kSlabTileMax) * kSlabTileMax;
   s->max_ctas = num_sms() * 16;
   s->fused_threads = 256;
-  s->fused_ctas_per_sm = 8;
+  s->fused_ctas_per_sm = 0;  // by the path taken
   s->view = active != nullptr;
   bool ok = true;
   if (s->view) {
@@ -1469,6 +1527,23 @@ static int apply_grid() {
   return num_sms() * b;
 }
 
+// The selective-update call with many records (k >= capacity / kMoveShare), 8
+// fields and 32-byte aligned records and deltas: the ranking pass moves them.
+// 2^24 slots, lists and an apply pass against moving at once: p = 0.005 55 us
+// against 67, 0.02 75 against 66, 0.05 101 against 92, 0.2 185 against 166, 0.5
+// (moved at once before, step by step and with every flag group written) 242
+// against 211. What is left at p = 0.05 is the draws (30 us) and random 32-byte
+// rows, of which DRAM moves 64 bytes each way. The line is drawn for the first
+// call on a half-full slab too, whose adds all fall to the CTAs of the lowest
+// slots: 59 us against 62 at p = 0.02, 77 against 75 at 0.05. Four CTAs per SM:
+// two leave the count pass short of warps, eight cost a second wave.
+constexpr int kMoveShare = 64;
+constexpr int kMoveCtasPerSm = 4;
+static bool fused_moves(const abm_slab* s, const ScanArgs& a) {
+  return (long long)a.k * kMoveShare >= (long long)s->d.cap && s->d.F == 8 && s->d.Fp == 8 &&
+         ((((uintptr_t)a.rec) | ((uintptr_t)a.rec2)) & 31) == 0;
+}
+
 // One cluster of as few CTAs as hold the slots, LS slots per lane.
 template <int OP, int LS>
 static abm_status launch_small(const ScanArgs& a, cudaStream_t st) {
@@ -1509,6 +1584,7 @@ static abm_status launch_scan(abm_slab* s, const ScanArgs& a, bool aux, cudaStre
   const size_t words = (size_t)(s->n_pad / 32);
   b.planeA = aux ? s->planes2 : s->planes;
   b.planeB = s->planes + words;
+  b.planeL = s->planes2;  // (free: only record masks use it, in other calls)
   b.totals = aux ? s->totals2 : s->totals;
   b.wtotals = aux ? s->wtotals2 : s->wtotals;
   b.ctrl = aux ? s->ctrl + 4 : s->ctrl;
@@ -1522,6 +1598,8 @@ static abm_status launch_scan(abm_slab* s, const ScanArgs& a, bool aux, cudaStre
   if (b.n <= kSmallThreads * kSmallCtas * 4) return launch_small<OP, 4>(b, st);
   if (b.n <= kSmallThreads * kSmallCtas * 8) return launch_small<OP, 8>(b, st);
   if (b.n <= kSmallMax) return launch_small<OP, 16>(b, st);
+  const bool move = OP == OP_FUSED && fused_moves(s, b);
+  if (ctas_per_sm == 0) ctas_per_sm = move ? kMoveCtasPerSm : 8;
   const int target = std::max(1, std::min(num_sms() * ctas_per_sm, s->max_ctas));
   const long per = ((long)b.n + target - 1) / target;
   b.chunk = (int)(((per + SUB - 1) / SUB) * SUB);
@@ -1532,12 +1610,7 @@ static abm_status launch_scan(abm_slab* s, const ScanArgs& a, bool aux, cudaStre
   // the next passes may launch while the previous one drains; they wait on
   // it (griddepcontrol) before reading its results
   if constexpr (OP == OP_FUSED) {
-    // many records (k >= capacity / 8), 8 fields, 32-byte aligned records and
-    // deltas: the ranking pass moves them. With fewer records a warp step holds
-    // too few to keep memory busy, and the separate apply pass (four records
-    // per thread over the whole grid) measured faster.
-    if ((long long)b.k * 8 >= (long long)s->d.cap && s->d.F == 8 && s->d.Fp == 8 &&
-        ((((uintptr_t)b.rec) | ((uintptr_t)b.rec2)) & 31) == 0) {
+    if (move) {
       ABM_CUDA_TRY(launch_pdl(k_scatter<OP, THREADS, true>, b.G, THREADS, st, b));
       return ABM_OK;
     }
