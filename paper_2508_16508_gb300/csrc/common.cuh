@@ -117,6 +117,29 @@ __device__ __forceinline__ int uniform_below(u32 u, int n) {
 }
 
 // ----------------------------------------------------------------------------
+// Thread-block clusters: the cluster's barrier in two halves (every thread of
+// every CTA takes part), and reads of another CTA's shared memory
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// the word at this CTA's shared address p, in the cluster's CTA `rank`
+__device__ __forceinline__ u64 ld_cluster(const u64* p, u32 rank) {
+  u32 at;
+  u64 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(at) : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_cluster_f32(const float* p, u32 rank) {
+  u32 at;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+  return v;
+}
+
+// ----------------------------------------------------------------------------
 // relaxed GPU-scope 64-bit accesses for the tile states
 __device__ __forceinline__ u64 ld_relaxed(const u64* p) {
   u64 v;

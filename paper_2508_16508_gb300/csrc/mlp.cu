@@ -209,16 +209,18 @@ constexpr int kMaxLin = 9;       // linear maps: up to 8 hidden layers + the out
 constexpr int kFusedWidth = 128; // widest layer of the fused path
 constexpr int kFusedOut = 8;     // most outputs
 constexpr int kRowThreads = 512;
-constexpr int kRedLd = 132;      // row stride of the partial sums: 4 words past 128, so that the (row, unit) reads
-                                 // of the reduction fall into different banks
+constexpr int kTrainRows = 8;    // rows of a training slab
+constexpr int kLd = 132;         // row stride of weights, gradients and partial sums: 4 words past 128, so that rows
+                                 // that are read side by side fall into different banks
 
 struct FusedNet {
   int nlin;
   int din[kMaxLin], dout[kMaxLin];
   int offW[kMaxLin], offb[kMaxLin];      // in the flat parameters
-  int sW[kMaxLin], sB[kMaxLin], ld[kMaxLin];  // shared memory: weights [din][ld] (columns past dout zero), biases
-  int sA[kMaxLin + 1];                   // shared memory: activations [width][R]
-  int sRed;                              // shared memory: partial sums [splits][R][kRedLd]
+  int sW[kMaxLin], sB[kMaxLin];          // shared memory: weights [din][kLd] (columns past dout zero; the output
+                                         // layer's [din][kFusedOut]), biases
+  int sA[kMaxLin];                       // shared memory: activations, (x, x) pairs [width][R]
+  int sD, sRed;                          // shared memory: gradients [R][kLd], partial sums [splits][R][kLd]
   long long offA[kMaxLin + 1];           // global row-slab blocks
   int nparams;
 };
@@ -237,44 +239,63 @@ struct RowArgs {
   long long grows, ga, gc, gm0;  // row permutation (grows = 0: none)
 };
 
+// two FP32 FMAs in one instruction (each rounded as fmaf)
+typedef unsigned long long f32x2;
+__device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float2 split2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+
 // One CTA takes R rows at a time through the net, weights resident in shared
-// memory. A layer's [R x 128] output is tiled 4 columns x 4 rows per thread
-// (two 16-byte shared loads for 16 FMAs); the threads left over split the sum
-// over the inputs, and the partial sums meet in shared memory (fixed order:
-// the result does not depend on the launch). Weight rows are padded to 4 words
-// past the layer's width, so that the backward pass, whose lanes walk the
-// rows, reads 16 bytes per lane without bank conflicts.
-// R: 8 rows give every SM work at the usual batch of 1024; 16 (training) and 32
-// (inference) rows load the weights for fewer slabs once there are more than
-// 16 rows per SM.
+// memory. Bound by instruction issue (a step at 1024 rows is 8 rows per CTA),
+// so the inner loops are packed FMAs on operands that need no shuffling:
+// forward, a thread's tile is 4 columns x 4 rows, two columns to a packed FMA,
+// and activations are kept twice over ((x, x) pairs); backward, it is 4 inputs x
+// 4 rows, even and odd outputs in the two halves, from gradients kept row by
+// row. The threads left over split the sum over the inputs (outputs), and the
+// partial sums meet in shared memory (fixed order: the result does not depend
+// on the launch). Weight rows are 132 words apart whatever the layer's width
+// (constant offsets; the backward pass, whose lanes walk the rows, reads 16 bytes
+// per lane without bank conflicts).
+// R: 8 rows give every SM work at the usual batch of 1024; inference takes 16 once
+// there are more than 16 rows per SM. One step at 1024 rows of the 12-128-128-128-2
+// net: scalar FMAs and strides by width 16.5 us, this 15.0.
 template <int R, bool TRAIN>
 __global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__ RowArgs a) {
   extern __shared__ __align__(16) float sm[];
   __shared__ long long s_row[R];
   __shared__ float s_loss[R * kFusedOut];
+  __shared__ float s_dout[kFusedOut * R];       // d loss / d yhat, [output][R]
+  constexpr int NT = kRowThreads;
   constexpr int RG = R / 4;                     // row groups of a tile row
-  constexpr int KS = kRowThreads / (32 * RG);   // splits of a sum
+  constexpr int KS = NT / (32 * RG);            // splits of a sum
   const FusedNet& net = a.net;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int L = net.nlin, n_in = net.din[0], n_out = net.dout[L - 1];
   griddep_wait();  // the parameters (and, on a reused handle, the blocks) belong to the previous launch until here
   for (int l = 0; l < L; ++l) {
-    const int din = net.din[l], dout = net.dout[l], ld = net.ld[l];
+    const int din = net.din[l], dout = net.dout[l];
     const float* W = a.p + net.offW[l];
     float* s = sm + net.sW[l];
-    if ((dout & 3) == 0 && (net.offW[l] & 3) == 0) {
-      const int q = dout >> 2;
-      for (int i = tid; i < din * q; i += kRowThreads) cp_async16(s + (i / q) * ld + 4 * (i % q), W + 4 * i);
+    if (l == L - 1) {  // [din][kFusedOut]
+      for (int i = tid; i < din * dout; i += NT) s[(i / dout) * kFusedOut + i % dout] = W[i];
+    } else if ((dout & 3) == 0 && (net.offW[l] & 3) == 0) {  // a warp per row
+      if (4 * lane < dout)
+        for (int k = warp; k < din; k += NT / 32) cp_async16(s + k * kLd + 4 * lane, W + k * dout + 4 * lane);
     } else {
-      const int wd = (dout + 3) & ~3;
-      for (int i = tid; i < din * wd; i += kRowThreads) {
-        const int k = i / wd, c = i % wd;
-        s[k * ld + c] = c < dout ? W[k * dout + c] : 0.f;
-      }
+      for (int k = warp; k < din; k += NT / 32)
+        for (int c = lane; c < ((dout + 3) & ~3); c += 32) s[k * kLd + c] = c < dout ? W[k * dout + c] : 0.f;
     }
-    for (int i = tid; i < dout; i += kRowThreads) sm[net.sB[l] + i] = a.p[net.offb[l] + i];
+    for (int i = tid; i < dout; i += NT) sm[net.sB[l] + i] = a.p[net.offb[l] + i];
   }
   cp_async_commit();
+  float* const red = sm + net.sRed;
+  float* const drow = sm + net.sD;  // gradients of the current layer's outputs, [R][kLd]
+  const int rg = warp % RG, ks = warp / RG;
   const int nslab = (a.B + R - 1) / R;
   float loss = 0.f;
   for (int slab = blockIdx.x; slab < nslab; slab += gridDim.x) {
@@ -287,65 +308,68 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__
     }
     __syncthreads();
     {
-      float* s = sm + net.sA[0];
-      for (int i = tid; i < n_in * R; i += kRowThreads) {
+      float2* s = reinterpret_cast<float2*>(sm + net.sA[0]);
+      float* out = TRAIN ? a.act + net.offA[0] + (long long)slab * n_in * R : nullptr;
+      for (int i = tid; i < n_in * R; i += NT) {
         const int r = i % R, k = i / R;
         const float v = r < nr ? a.x[(size_t)s_row[r] * n_in + k] : 0.f;
-        s[i] = v;
-        if (TRAIN) a.act[net.offA[0] + (long long)slab * n_in * R + i] = v;
+        s[i] = make_float2(v, v);
+        if (TRAIN) out[i] = v;
       }
     }
     cp_async_wait_0();
     __syncthreads();
     // forward through the hidden layers
-    float* red = sm + net.sRed;
-    const int rg = warp % RG, ks = warp / RG;
     for (int l = 0; l + 1 < L; ++l) {
-      const int din = net.din[l], dout = net.dout[l], ld = net.ld[l];
-      const float* W = sm + net.sW[l];
-      const float* X = sm + net.sA[l];
-      const int c0 = 4 * lane;
-      if (c0 < dout) {
-        const int per = (din + KS - 1) / KS, k0 = ks * per, k1 = min(din, k0 + per);
-        float acc[4][4] = {};
-#pragma unroll 8
-        for (int k = k0; k < k1; ++k) {
-          const float4 wv = *reinterpret_cast<const float4*>(W + k * ld + c0);
-          const float4 xv = *reinterpret_cast<const float4*>(X + k * R + 4 * rg);
-          const float w4[4] = {wv.x, wv.y, wv.z, wv.w}, x4[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-          for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(x4[r], w4[c], acc[r][c]);
+      const int din = net.din[l], dout = net.dout[l];
+      if (4 * lane < dout) {
+        const int per = (din + KS - 1) / KS, k0 = ks * per, n = min(din - k0, per);
+        const float* W = sm + net.sW[l] + k0 * kLd + 4 * lane;
+        const float* X = sm + net.sA[l] + 2 * (k0 * R + 4 * rg);
+        f32x2 acc[4][2] = {};
+#pragma unroll 4
+        for (int k = 0; k < n; ++k) {
+          const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(W + k * kLd);
+          const ulonglong2 xa = *reinterpret_cast<const ulonglong2*>(X + k * (2 * R));
+          const ulonglong2 xb = *reinterpret_cast<const ulonglong2*>(X + k * (2 * R) + 4);
+          fma2(acc[0][0], xa.x, w.x);
+          fma2(acc[0][1], xa.x, w.y);
+          fma2(acc[1][0], xa.y, w.x);
+          fma2(acc[1][1], xa.y, w.y);
+          fma2(acc[2][0], xb.x, w.x);
+          fma2(acc[2][1], xb.x, w.y);
+          fma2(acc[3][0], xb.y, w.x);
+          fma2(acc[3][1], xb.y, w.y);
         }
+        float* o = red + (ks * R + 4 * rg) * kLd + 4 * lane;
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
-          *reinterpret_cast<float4*>(red + (ks * R + 4 * rg + r) * kRedLd + c0) =
-              make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+        for (int r = 0; r < 4; ++r) *reinterpret_cast<ulonglong2*>(o + r * kLd) = make_ulonglong2(acc[r][0], acc[r][1]);
       }
       __syncthreads();
-      float* Y = sm + net.sA[l + 1];
-      for (int i = tid; i < dout * R; i += kRowThreads) {
+      float2* Y = reinterpret_cast<float2*>(sm + net.sA[l + 1]);
+      float* out = TRAIN ? a.act + net.offA[l + 1] + (long long)slab * dout * R : nullptr;
+      const float* bias = sm + net.sB[l];
+      for (int i = tid; i < dout * R; i += NT) {
         const int r = i % R, c = i / R;
+        const float* p = red + r * kLd + c;
         float v = 0.f;
 #pragma unroll
-        for (int z = 0; z < KS; ++z) v += red[(z * R + r) * kRedLd + c];
-        v = r < nr ? fmaxf(v + sm[net.sB[l] + c], 0.f) : 0.f;
-        Y[i] = v;
-        if (TRAIN) a.act[net.offA[l + 1] + (long long)slab * dout * R + i] = v;
+        for (int z = 0; z < KS; ++z) v += p[z * R * kLd];
+        v = r < nr ? fmaxf(v + bias[c], 0.f) : 0.f;
+        Y[i] = make_float2(v, v);
+        if (TRAIN) out[i] = v;
       }
       __syncthreads();
     }
     // output layer: one warp per (row, output), lanes over the inputs
     {
-      const int l = L - 1, din = net.din[l], ld = net.ld[l];
+      const int l = L - 1, din = net.din[l];
       const float* W = sm + net.sW[l];
       const float* X = sm + net.sA[l];
-      float* D = sm + net.sA[L];
-      for (int e = warp; e < R * n_out; e += kRowThreads / 32) {
+      for (int e = warp; e < R * n_out; e += NT / 32) {
         const int r = e % R, o = e / R;
         float v = 0.f;
-        for (int k = lane; k < din; k += 32) v = fmaf(X[k * R + r], W[k * ld + o], v);
+        for (int k = lane; k < din; k += 32) v = fmaf(X[2 * (k * R + r)], W[k * kFusedOut + o], v);
 #pragma unroll
         for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, m);
         if (lane == 0) {
@@ -361,7 +385,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__
               d = (er > 0.f ? -a.tau : 1.f - a.tau) * a.scale;
             }
             s_loss[e] = le;
-            D[e] = d;
+            s_dout[e] = d;
             a.dact[net.offA[L] + (long long)slab * n_out * R + e] = d;
           }
         }
@@ -376,66 +400,73 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__
       for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, m);
       loss += v;
     }
-    // backward: the gradient of layer l's input replaces that input in shared memory
+    // backward: the gradients of layer l's input, from those of its outputs (drow; s_dout for the output layer)
     for (int l = L - 1; l > 0; --l) {
-      const int din = net.din[l], dout = net.dout[l], ld = net.ld[l];
-      const float* W = sm + net.sW[l];
-      const float* D = sm + net.sA[l + 1];
-      float* X = sm + net.sA[l];
+      const int din = net.din[l], dout = net.dout[l];
+      const float2* X = reinterpret_cast<const float2*>(sm + net.sA[l]);
       float* dst = a.dact + net.offA[l] + (long long)slab * din * R;
       if (l == L - 1) {  // at most 8 outputs: one thread per (input, row)
-        for (int i = tid; i < din * R; i += kRowThreads) {
+        const float* W = sm + net.sW[l];
+        for (int i = tid; i < din * R; i += NT) {
           const int r = i % R, k = i / R;
           float v = 0.f;
-          for (int o = 0; o < dout; ++o) v = fmaf(D[o * R + r], W[k * ld + o], v);
-          v = X[i] > 0.f ? v : 0.f;
-          X[i] = v;
+          for (int o = 0; o < dout; ++o) v = fmaf(s_dout[o * R + r], W[k * kFusedOut + o], v);
+          v = X[i].x > 0.f ? v : 0.f;
+          drow[r * kLd + k] = v;
           dst[i] = v;
         }
+        // columns up to the next multiple of 4, which the next layer down reads against zero weights
+        if (tid < R)
+          for (int k = din; k < ((din + 3) & ~3); ++k) drow[tid * kLd + k] = 0.f;
         __syncthreads();
         continue;
       }
       // lanes take the inputs lane, lane + 32, ...; the outputs are taken four at a time and split over the warps
-      const int nq = (dout + 3) >> 2, per = (nq + KS - 1) / KS, q0 = ks * per, q1 = min(nq, q0 + per);
-      float acc[4][4] = {};  // [input][row]
+      {
+        const int nq = (dout + 3) >> 2, per = (nq + KS - 1) / KS, q0 = ks * per, n = min(nq - q0, per);
+        const float* W[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) W[i] = sm + net.sW[l] + min(lane + 32 * i, din - 1) * kLd + 4 * q0;
+        const float* D = drow + 4 * rg * kLd + 4 * q0;
+        f32x2 acc[4][4] = {};  // [input][row]: even | odd outputs
 #pragma unroll 2
-      for (int q = q0; q < q1; ++q) {
-        float dv[4][4], wv[4][4];
+        for (int q = 0; q < n; ++q) {
+          ulonglong2 d[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          // columns past the width are zero in W; their rows of D are not read
-          const float4 t = 4 * q + j < dout ? *reinterpret_cast<const float4*>(D + (4 * q + j) * R + 4 * rg)
-                                            : make_float4(0.f, 0.f, 0.f, 0.f);
-          dv[j][0] = t.x; dv[j][1] = t.y; dv[j][2] = t.z; dv[j][3] = t.w;
+          for (int r = 0; r < 4; ++r) d[r] = *reinterpret_cast<const ulonglong2*>(D + r * kLd + 4 * q);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(W[i] + 4 * q);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              fma2(acc[i][r], d[r].x, w.x);
+              fma2(acc[i][r], d[r].y, w.y);
+            }
+          }
         }
+        float* o = red + (ks * R + 4 * rg) * kLd + lane;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int k = min(lane + 32 * i, din - 1);
-          const float4 t = *reinterpret_cast<const float4*>(W + k * ld + 4 * q);
-          wv[i][0] = t.x; wv[i][1] = t.y; wv[i][2] = t.z; wv[i][3] = t.w;
-        }
+        for (int i = 0; i < 4; ++i)
+          if (lane + 32 * i < din)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) acc[i][r] = fmaf(dv[j][r], wv[i][j], acc[i][r]);
+            for (int r = 0; r < 4; ++r) {
+              const float2 v = split2(acc[i][r]);
+              o[r * kLd + 32 * i] = v.x + v.y;
+            }
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (lane + 32 * i < din)
-#pragma unroll
-          for (int r = 0; r < 4; ++r) red[(ks * R + 4 * rg + r) * kRedLd + lane + 32 * i] = acc[i][r];
       __syncthreads();
-      for (int i = tid; i < din * R; i += kRowThreads) {
+      for (int i = tid; i < din * R; i += NT) {
         const int r = i % R, k = i / R;
+        const float* p = red + r * kLd + k;
         float v = 0.f;
 #pragma unroll
-        for (int z = 0; z < KS; ++z) v += red[(z * R + r) * kRedLd + k];
-        v = X[i] > 0.f ? v : 0.f;
-        X[i] = v;
+        for (int z = 0; z < KS; ++z) v += p[z * R * kLd];
+        v = X[i].x > 0.f ? v : 0.f;
+        drow[r * kLd + k] = v;
         dst[i] = v;
       }
+      if (tid < R)
+        for (int k = din; k < ((din + 3) & ~3); ++k) drow[tid * kLd + k] = 0.f;
       __syncthreads();
     }
   }
@@ -446,8 +477,6 @@ struct WgradArgs {
   FusedNet net;
   const float* act;
   const float* dact;
-  float* part;      // [splits][nparams]
-  unsigned* done;   // [tiles], zero between launches
   float *g, *p, *m, *v;
   int nslab, slabs_per_split;
   const float* lossp;
@@ -461,24 +490,28 @@ struct WgradArgs {
 constexpr int kWT = 32;         // inputs and outputs of a weight-gradient tile
 constexpr int kWRows = 128;     // rows staged at a time
 constexpr int kWThreads = 256;
+constexpr int kMaxRuns = 8;     // runs of rows = CTAs of a cluster (the portable size), at most
 
 __host__ __device__ inline int wgrad_tiles(const FusedNet& net, int l) {
   return ((net.din[l] + kWT - 1) / kWT) * ((net.dout[l] + kWT - 1) / kWT);
 }
 
-// Weight gradients X^T dY of every layer in one launch: a CTA owns a 32 x 32
-// tile of one layer's gradient and a run of rows. 64 threads cover the tile
-// with 4 x 4 outputs each and four such groups take a quarter of the staged rows
-// each (128 rows a stage: 32 KB of shared memory). The tiles of the first
-// inputs also sum the bias gradients. The last CTA of a tile to finish adds the
-// runs' partial gradients in run order (so the sums do not depend on timing)
-// and applies Adam to the tile's parameters.
-template <int R>
+// Weight gradients X^T dY of every layer in one launch: a cluster owns a 32 x
+// 32 tile of one layer's gradient, its CTAs a run of rows each. 64 threads cover
+// the tile with 4 x 4 outputs each and four such groups take a quarter of the
+// staged rows each (128 rows a stage: 32 KB of shared memory). The tiles of the
+// first inputs also sum the bias gradients. The CTAs' tiles meet in distributed
+// shared memory: after one cluster barrier each CTA adds up its share of the
+// tile in run order (so the sums do not depend on timing) and applies Adam to
+// those parameters. (Partial tiles in global memory, added by the last CTA to
+// finish, took 15.9 us a step at 1024 rows; this 9.5.)
+constexpr int kTileEntries = kWT * kWT + kWT;  // the tile and, below it, the bias row
+
 __global__ void __launch_bounds__(kWThreads) k_wgrad(const __grid_constant__ WgradArgs a) {
   __shared__ __align__(16) float s_x[kWRows / 4][kWT][4];   // [row quad][unit][row]
   __shared__ __align__(16) float s_d[kWRows / 4][kWT][4];
   __shared__ float s_b[8][kWT];
-  __shared__ bool s_last;
+  __shared__ float s_sum[kTileEntries];
   const FusedNet& net = a.net;
   const int tid = threadIdx.x;
   int l = 0, tile = blockIdx.x;
@@ -488,6 +521,7 @@ __global__ void __launch_bounds__(kWThreads) k_wgrad(const __grid_constant__ Wgr
   const int k0 = (tile / tn) * kWT, n0 = (tile % tn) * kWT;
   const int nk = min(kWT, din - k0), nn = min(kWT, dout - n0);
   const int s0 = blockIdx.y * a.slabs_per_split, s1 = min(a.nslab, s0 + a.slabs_per_split);
+  constexpr int R = kTrainRows;
   constexpr int SS = kWRows / R;  // slabs per stage
   constexpr int RQ = R / 4;
   const int grp = tid >> 6, kg = (tid & 63) >> 3, ng = tid & 7;
@@ -497,6 +531,7 @@ __global__ void __launch_bounds__(kWThreads) k_wgrad(const __grid_constant__ Wgr
   const float* D = a.dact + net.offA[l + 1];
   for (int s = s0; s < s1; s += SS) {
     // [slab][unit][R] -> [row quad][unit][4]; missing units and slabs are zero
+#pragma unroll
     for (int i = tid; i < SS * kWT * RQ; i += kWThreads) {
       const int q = i % RQ, u = (i / RQ) % kWT, j = i / (RQ * kWT);
       float4 x = make_float4(0.f, 0.f, 0.f, 0.f), d = x;
@@ -526,6 +561,7 @@ __global__ void __launch_bounds__(kWThreads) k_wgrad(const __grid_constant__ Wgr
         }
     }
     if (k0 == 0) {  // bias: output tid % 32, every eighth quad
+#pragma unroll
       for (int q = tid >> 5; q < kWRows / 4; q += 8) {
         const float4 d = *reinterpret_cast<const float4*>(s_d[q][tid & 31]);
         bacc += (d.x + d.y) + (d.z + d.w);
@@ -541,37 +577,32 @@ __global__ void __launch_bounds__(kWThreads) k_wgrad(const __grid_constant__ Wgr
     for (int j = 0; j < 4; ++j) s_t[grp * kWT * kWT + (kg + 8 * i) * kWT + ng + 8 * j] = acc[i][j];
   s_b[tid >> 5][tid & 31] = bacc;
   __syncthreads();
-  float* part = a.part + (long long)blockIdx.y * net.nparams;
-  for (int i = tid; i < kWT * kWT; i += kWThreads) {
-    const int k = i / kWT, n = i % kWT;
-    if (k < nk && n < nn)
-      part[net.offW[l] + (k0 + k) * dout + n0 + n] =
-          (s_t[i] + s_t[i + kWT * kWT]) + (s_t[i + 2 * kWT * kWT] + s_t[i + 3 * kWT * kWT]);
-  }
-  if (k0 == 0 && tid < nn) {
+#pragma unroll
+  for (int i = tid; i < kWT * kWT; i += kWThreads)
+    s_sum[i] = (s_t[i] + s_t[i + kWT * kWT]) + (s_t[i + 2 * kWT * kWT] + s_t[i + 3 * kWT * kWT]);
+  if (tid < kWT) {
     float b = 0.f;
 #pragma unroll
     for (int z = 0; z < 8; ++z) b += s_b[z][tid];
-    part[net.offb[l] + n0 + tid] = b;
+    s_sum[kWT * kWT + tid] = b;
   }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    const unsigned n = atomicAdd(&a.done[blockIdx.x], 1u);
-    s_last = n == gridDim.y - 1;
-    if (s_last) a.done[blockIdx.x] = 0u;
-    __threadfence();
-  }
-  __syncthreads();
-  if (!s_last) return;
-  const int S = gridDim.y;
-  const int entries = kWT * kWT + (k0 == 0 ? kWT : 0);
-  for (int i = tid; i < entries; i += kWThreads) {
+  const int S = gridDim.y;  // = the cluster's CTAs
+  cluster_arrive();
+  cluster_wait();
+  // this CTA's share of the tile's entries
+  const int entries = k0 == 0 ? kTileEntries : kWT * kWT;
+  const int share = (entries + S - 1) / S;
+  const int e0 = blockIdx.y * share, e1 = min(entries, e0 + share);
+  for (int i = e0 + tid; i < e1; i += kWThreads) {
     const int k = i / kWT, n = i % kWT;  // k = 32: the bias row
     if (n >= nn || (k < kWT && k >= nk)) continue;
     const int e = k < kWT ? net.offW[l] + (k0 + k) * dout + n0 + n : net.offb[l] + n0 + n;
+    float v[kMaxRuns];
+#pragma unroll
+    for (int z = 0; z < kMaxRuns; ++z) v[z] = z < S ? ld_cluster_f32(&s_sum[i], (u32)z) : 0.f;
     float gi = 0.f;
-    for (int z = 0; z < S; ++z) gi += __ldcg(a.part + (long long)z * net.nparams + e);
+#pragma unroll
+    for (int z = 0; z < kMaxRuns; ++z) gi += v[z];
     a.g[e] = gi;
     if (a.adam) {  // Adam (Kingma & Ba, 2015) with bias correction
       const float mi = a.b1 * a.m[e] + (1.f - a.b1) * gi;
@@ -581,13 +612,15 @@ __global__ void __launch_bounds__(kWThreads) k_wgrad(const __grid_constant__ Wgr
       a.p[e] -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
     }
   }
-  if (blockIdx.x == 0 && a.loss_out && tid < 32) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && a.loss_out && tid < 32) {
     float v = 0.f;
     for (int i = tid; i < a.nloss; i += 32) v += a.lossp[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
     if (tid == 0) *a.loss_out = v * a.loss_scale;
   }
+  cluster_arrive();  // no CTA leaves while another reads its sums
+  cluster_wait();
 }
 
 // features of a model: log1p(side), log1p(n0 sheep), log1p(n0 wolves), the 8
@@ -642,8 +675,6 @@ struct abm_mlp {
   // fused path (fused = 0: a GEMM per product)
   int fused;
   FusedNet net;          // shared-memory offsets filled in per launch shape
-  float* wpart;          // [kSplits][nparams] partial weight gradients
-  unsigned* wdone;       // [tiles] arrivals per weight-gradient tile
 };
 
 static void mlp_free(abm_mlp* n) {
@@ -657,8 +688,6 @@ static void mlp_free(abm_mlp* n) {
   cudaFree(n->lossp);
   cudaFree(n->d_off);
   cudaFree(n->d_fan);
-  cudaFree(n->wpart);
-  cudaFree(n->wdone);
   delete n;
 }
 
@@ -670,38 +699,36 @@ constexpr size_t kMaxSmem = 227 * 1024 - 2048;  // dynamic shared memory of a CT
 // Returns the bytes.
 static size_t fused_layout(FusedNet& f, int R, bool train) {
   int at = 0;
+  const auto take = [&](int n) {
+    const int o = at;
+    at += (n + 3) & ~3;
+    return o;
+  };
   for (int l = 0; l < f.nlin; ++l) {
-    f.sW[l] = at;
-    at += f.din[l] * f.ld[l];
+    f.sW[l] = take(f.din[l] * (l == f.nlin - 1 ? kFusedOut : kLd));
+    f.sB[l] = take(f.dout[l]);
   }
-  for (int l = 0; l < f.nlin; ++l) {
-    f.sB[l] = at;
-    at += (f.dout[l] + 3) & ~3;
+  if (train) {
+    for (int l = 0; l < f.nlin; ++l) f.sA[l] = take(2 * f.din[l] * R);
+    f.sD = take(R * kLd);
+  } else {
+    int w[2] = {1, 1};  // widest of the layers that take turns
+    for (int l = 0; l < f.nlin; ++l) w[l & 1] = std::max(w[l & 1], f.din[l]);
+    const int o[2] = {take(2 * w[0] * R), take(2 * w[1] * R)};
+    for (int l = 0; l < f.nlin; ++l) f.sA[l] = o[l & 1];
+    f.sD = at;
   }
-  int w[2] = {f.din[0], f.dout[0]};  // widest even and odd layer
-  for (int l = 2; l <= f.nlin; ++l) w[l & 1] = std::max(w[l & 1], f.dout[l - 1]);
-  const int base = at;
-  for (int l = 0; l <= f.nlin; ++l) {
-    if (train) {
-      f.sA[l] = at;
-      at += (l == 0 ? f.din[0] : f.dout[l - 1]) * R;
-    } else {
-      f.sA[l] = base + (l & 1) * w[0] * R;
-    }
-  }
-  if (!train) at = base + (w[0] + w[1]) * R;
-  f.sRed = at;
-  at += (kRowThreads / (32 * (R / 4))) * R * kRedLd;
+  f.sRed = take((kRowThreads / (32 * (R / 4))) * R * kLd);  // KS splits of k_rows
   return (size_t)at * sizeof(float);
 }
 
 // nets whose widths the fused tiles cover and whose shared memory fits with
-// the largest slabs (16 rows in training, 32 in inference)
+// the largest slabs (8 rows in training, 16 in inference)
 static bool fused_fits(FusedNet f) {
   for (int l = 0; l < f.nlin; ++l)
     if (f.din[l] > kFusedWidth || f.dout[l] > kFusedWidth) return false;
-  return f.dout[f.nlin - 1] <= kFusedOut && fused_layout(f, 16, true) <= kMaxSmem &&
-         fused_layout(f, 32, false) <= kMaxSmem;
+  return f.dout[f.nlin - 1] <= kFusedOut && fused_layout(f, kTrainRows, true) <= kMaxSmem &&
+         fused_layout(f, 16, false) <= kMaxSmem;
 }
 
 extern "C" abm_status abm_mlp_destroy(abm_mlp* n) {
@@ -746,7 +773,6 @@ extern "C" abm_status abm_mlp_create(int32_t n_in, int32_t hidden, int32_t layer
     const int w = l == 0 ? n_in : n->dout[l - 1];
     aoff += rows_pad * w;
   }
-  int wtiles = 1;
   n->net.nlin = n->nlin;
   n->net.nparams = (int)n->nparams;
   for (int l = 0; l < n->nlin; ++l) {
@@ -754,9 +780,7 @@ extern "C" abm_status abm_mlp_create(int32_t n_in, int32_t hidden, int32_t layer
     n->net.dout[l] = n->dout[l];
     n->net.offW[l] = (int)n->offW[l];
     n->net.offb[l] = (int)n->offb[l];
-    n->net.ld[l] = ((n->dout[l] + 3) & ~3) + (l == n->nlin - 1 ? 0 : 4);
     n->net.offA[l] = n->offA[l];
-    wtiles += wgrad_tiles(n->net, l);
   }
   n->net.offA[n->nlin] = n->offA[n->nlin];
   n->fused = fused_fits(n->net);
@@ -767,9 +791,7 @@ extern "C" abm_status abm_mlp_create(int32_t n_in, int32_t hidden, int32_t layer
             cudaMalloc(&n->part, (size_t)kSplits * std::max(hidden, n_in) * std::max(hidden, n_out) * 4) == cudaSuccess &&
             cudaMalloc(&n->lossp, 1024 * 4) == cudaSuccess &&
             cudaMalloc(&n->d_off, offs.size() * sizeof(long long)) == cudaSuccess &&
-            cudaMalloc(&n->d_fan, fan.size() * sizeof(int)) == cudaSuccess &&
-            (!n->fused || (cudaMalloc(&n->wpart, (size_t)kSplits * P * 4) == cudaSuccess &&
-                           cudaMalloc(&n->wdone, (size_t)wtiles * 4) == cudaSuccess));
+            cudaMalloc(&n->d_fan, fan.size() * sizeof(int)) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     mlp_free(n);
@@ -778,8 +800,7 @@ extern "C" abm_status abm_mlp_create(int32_t n_in, int32_t hidden, int32_t layer
   cudaStream_t st = (cudaStream_t)stream;
   if (cudaMemcpyAsync(n->d_off, offs.data(), offs.size() * sizeof(long long), cudaMemcpyHostToDevice, st) != cudaSuccess ||
       cudaMemcpyAsync(n->d_fan, fan.data(), fan.size() * sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemsetAsync(n->m, 0, P * 4, st) != cudaSuccess || cudaMemsetAsync(n->v, 0, P * 4, st) != cudaSuccess ||
-      (n->fused && cudaMemsetAsync(n->wdone, 0, (size_t)wtiles * 4, st) != cudaSuccess)) {
+      cudaMemsetAsync(n->m, 0, P * 4, st) != cudaSuccess || cudaMemsetAsync(n->v, 0, P * 4, st) != cudaSuccess) {
     mlp_free(n);
     return ABM_ERR_CUDA;
   }
@@ -905,11 +926,6 @@ static Perm make_perm(int64_t rows, int64_t a, int64_t c, int64_t m0) {
 }
 
 // ---- fused path, host side
-static int slab_rows(int B, bool train) {
-  // more than 16 rows per SM: larger slabs, so that a CTA goes through the resident weights with fewer barriers
-  return B <= 16 * num_sms() ? 8 : (train ? 16 : 32);
-}
-
 template <int R, bool TRAIN>
 static abm_status rows_launch(abm_mlp* n, RowArgs& ra, cudaStream_t st, int& grid) {
   static std::atomic<unsigned long long> attr{0};
@@ -936,8 +952,8 @@ struct AdamStep {
   float lr, b1, b2, eps, c1, c2;
 };
 
-template <int R>
 static abm_status fused_train(abm_mlp* n, RowArgs& ra, const AdamStep& ad, float* loss_out, cudaStream_t st) {
+  constexpr int R = kTrainRows;
   int grid = 0;
   abm_status e = rows_launch<R, true>(n, ra, st, grid);
   if (e != ABM_OK) return e;
@@ -946,16 +962,14 @@ static abm_status fused_train(abm_mlp* n, RowArgs& ra, const AdamStep& ad, float
   wa.net = ra.net;
   wa.act = n->act;
   wa.dact = n->dact;
-  wa.part = n->wpart;
-  wa.done = n->wdone;
   wa.g = n->g;
   wa.p = n->p;
   wa.m = n->m;
   wa.v = n->v;
   wa.nslab = (ra.B + R - 1) / R;
-  // runs of whole stages: 128 rows each while that gives at most kSplits runs
+  // runs of whole stages (128 rows each up to 1024 rows), one CTA of the cluster each
   const int stages = (wa.nslab * R + kWRows - 1) / kWRows;
-  const int per = (stages + kSplits - 1) / kSplits;
+  const int per = (stages + kMaxRuns - 1) / kMaxRuns, runs = (stages + per - 1) / per;
   wa.slabs_per_split = per * (kWRows / R);
   wa.lossp = n->lossp;
   wa.nloss = grid;
@@ -971,15 +985,18 @@ static abm_status fused_train(abm_mlp* n, RowArgs& ra, const AdamStep& ad, float
   int tiles = 0;
   for (int l = 0; l < n->nlin; ++l) tiles += wgrad_tiles(n->net, l);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)tiles, (unsigned)((stages + per - 1) / per));
+  cfg.gridDim = dim3((unsigned)tiles, (unsigned)runs);
   cfg.blockDim = dim3(kWThreads);
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = at[1].val.clusterDim.z = 1;
+  at[1].val.clusterDim.y = (unsigned)runs;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
-  ABM_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_wgrad<R>, wa));
+  cfg.numAttrs = 2;
+  ABM_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_wgrad, wa));
   return ABM_OK;
 }
 
@@ -1000,8 +1017,7 @@ static abm_status fused_gradients(abm_mlp* n, const float* x, const float* y, in
   ra.ga = pm.a;
   ra.gc = pm.c;
   ra.gm0 = pm.m0;
-  return slab_rows(B, true) == 8 ? fused_train<8>(n, ra, ad, loss_out, st)
-                                 : fused_train<16>(n, ra, ad, loss_out, st);
+  return fused_train(n, ra, ad, loss_out, st);
 }
 
 static abm_status fused_forward(abm_mlp* n, const float* x, int B, float* y, cudaStream_t st) {
@@ -1012,7 +1028,7 @@ static abm_status fused_forward(abm_mlp* n, const float* x, int B, float* y, cud
   ra.out = y;
   ra.B = B;
   int grid;
-  return slab_rows(B, false) == 8 ? rows_launch<8, false>(n, ra, st, grid) : rows_launch<32, false>(n, ra, st, grid);
+  return B <= 16 * num_sms() ? rows_launch<8, false>(n, ra, st, grid) : rows_launch<16, false>(n, ra, st, grid);
 }
 
 extern "C" abm_status abm_mlp_forward(abm_mlp* n, const float* x, int32_t B, float* y, void* stream) {

@@ -863,19 +863,6 @@ constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int kSmallCtas = 16;  // cluster size, at most (above 8: opt-in)
 constexpr int kSmallMax = kSmallCtas * kSmallThreads * 16;
 
-__device__ __forceinline__ void cluster_arrive() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// the 64-bit word at this CTA's shared address p, in the cluster's CTA `rank`
-__device__ __forceinline__ u64 ld_cluster(const u64* p, u32 rank) {
-  u32 at;
-  u64 v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(p)), "r"(rank));
-  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(at) : "memory");
-  return v;
-}
-
 // Records r0 .. r0 + n - 1 of a warp's staged slots (offsets from slot0): whole
 // rows, neighbouring lanes on neighbouring words of a record.
 // ADD: added to the row (wrapping); id_field >= 0: that field is id0 + r instead.

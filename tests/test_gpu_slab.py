@@ -545,3 +545,41 @@ def test_one_launch_sizes(eng, n, F):
         for f in range(F):
             np.testing.assert_array_equal(np_of(s.read(f)), o.fields[f])
     s.check()
+
+
+@pytest.mark.parametrize("n,p", [(262_145, 0.015), (300_001, 0.017), (300_001, 0.05), (300_001, 0.5),
+                                 (2_000_003, 0.02), (2_000_003, 0.3)])
+def test_selective_update_paths(eng, n, p):
+    """Whole numbers, so exact: the two sides of the record-moving line, from a half-full set on, with flags other
+    than 0 and 1: those are rewritten as 1 exactly in the 16-slot groups that receive an agent and the 8-slot groups
+    that lose one."""
+    from paper_2508_16508_gb300 import abm
+    T, k = workloads.threshold(p), workloads.k_for(p, n)
+    s, o = eng.Slab(n, 8, seed=2, init=abm.INIT_HALF_LIVE), oracle.Slab(n, 8)
+    o.c1_init(seed=2)
+    odd = np.where(o.active & (np.arange(n) % 37 == 0), 5, o.active).astype(np.int32)
+    s.write(-1, torch.from_numpy(odd).cuda())
+    for step in range(4):
+        rec = s.philox_records(step, abm.P_NEWREC0, abm.P_NEWREC1, k)
+        dl = s.philox_records(step, abm.P_DELTA0, abm.P_DELTA1, k)
+        before, ids = o.active.copy(), o.fields.copy()
+        s.selective_update(step, T, rec, dl)
+        o.c1_call(step, T, k, seed=2)
+        draws = np.zeros(-(-n // 16) * 16, bool)
+        new = draws.copy()
+        new[:n] = (o.fields != ids).any(0) & (o.active != 0)  # added or updated
+        got = np_of(s.read(-1))
+        np.testing.assert_array_equal(got != 0, o.active != 0)
+        for f in range(8):
+            np.testing.assert_array_equal(np_of(s.read(f)), o.fields[f])
+        # a flag that keeps an odd value was live, stays live, and lies in no group that was written
+        np.testing.assert_array_equal(got[got > 1], odd[got > 1])
+        freed = np.zeros_like(new)
+        freed[:n] = (before != 0) & (o.active == 0)  # certainly removed
+        wrote = np.repeat(freed.reshape(-1, 8).any(1), 8)[:n]
+        filled = np.zeros_like(new)
+        filled[:n] = (before == 0) & (o.active != 0)  # certainly added
+        wrote |= np.repeat(filled.reshape(-1, 16).any(1), 16)[:n]
+        assert got[wrote].max(initial=0) <= 1
+        odd = got
+    s.check()
