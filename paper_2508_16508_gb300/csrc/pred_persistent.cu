@@ -2,12 +2,12 @@
 // all phases of many steps in one cooperative launch, separated by a bounded
 // grid barrier instead of kernel boundaries.
 //
-// Per step, five barrier-separated phases (each species: move + claims;
-// eat / select / die with flags into bit-planes and per-unit counts; ranks ->
-// parent list and the first P free slots (P = parents); births), with the
-// wolves' ranks and births shifted by one step and run by two warps of each
-// CTA while the other fourteen move and feed the sheep (the schedule is
-// spelled out in k_persistent).
+// Per step, four barrier-separated phases (each species: move + claims;
+// eat / select / die with flags into bit-planes and per-unit counts; ranks and
+// births), with the wolves' ranks and births shifted by one step and run by two
+// warps of each CTA while the other fourteen move and feed the sheep, and the
+// sheep's ranks and births run by half of each CTA while the other half moves
+// the wolves (the schedule is spelled out in k_persistent).
 // Move and count phases deal 128-slot units to warps round-robin over the
 // CTAs (the live agents crowd the low slots) and list the live agents of a
 // CTA's units in shared memory for all its threads; the rank phases give CTA
@@ -24,7 +24,7 @@ namespace abm {
 constexpr int kPT = 512;                  // threads per CTA
 constexpr int kPWarps = kPT / 32;
 constexpr int kBarSpin = 1 << 24;         // bounded barrier wait (polls; a few seconds)
-constexpr int kPhases = 5;                // grid barriers per step (plus one closing a launch)
+constexpr int kPhases = 4;                // grid barriers per step (plus one closing a launch)
 
 // Grid barrier (all CTAs co-resident: cooperative launch) over a monotonic
 // arrival counter: the k-th barrier of a launch is passed once the counter
@@ -93,18 +93,24 @@ __device__ __forceinline__ bool grid_sync(u32* bar, int* err, u32& target, u32 e
 // beside the sheep work instead of before it; in the other phases all warps
 // form one team (the CTA barrier). NW = warps of the team (it starts at warp 0
 // for the sheep team and the whole CTA).
+// In phase 3 the first kMoveWarps warps move the wolves (named barrier 3) while
+// the others rank the sheep and place their births (named barrier 4).
 constexpr int kWolfWarps = 2;
 constexpr int kSheepWarps = kPWarps - kWolfWarps;
+constexpr int kMoveWarps = kPWarps / 2;
+constexpr int kBirthWarps = kPWarps - kMoveWarps;
+
+template <int ID, int NW>
+__device__ __forceinline__ void bar_team() {
+  asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(NW * 32) : "memory");
+}
 
 template <int NW>
 __device__ __forceinline__ void tsync() {
-  if (NW == kPWarps) {
-    __syncthreads();
-  } else if (NW == kSheepWarps) {
-    asm volatile("bar.sync 1, %0;" ::"n"(kSheepWarps * 32) : "memory");
-  } else {
-    asm volatile("bar.sync 2, %0;" ::"n"(kWolfWarps * 32) : "memory");
-  }
+  if (NW == kPWarps) __syncthreads();
+  else if (NW == kSheepWarps) bar_team<1, kSheepWarps>();
+  else if (NW == kMoveWarps) bar_team<3, kMoveWarps>();
+  else bar_team<2, kWolfWarps>();
 }
 
 // Work compaction over a CTA: in one round every warp loads the live flags of
@@ -209,7 +215,9 @@ __device__ __forceinline__ int4 move_one(const WorldDev& w, int t, int slot, int
 // phase 1/4: move every live agent; claims for the cell's grass (sheep) or
 // the cell's victim (wolves)
 // A world whose units fit in one round leaves the round's list, live words and
-// moved records in shared memory; `carried` = the list's length (-1 if not).
+// moved records in shared memory; `carried` = the list's length (-1 if not). A
+// place v < kQ * NW means unit b + G v in round 0 whatever the team, so a count
+// phase of more warps can take the list of a smaller team's move.
 // live masks of this thread's slots in round `round` of the unit dealing
 template <int S, int NW>
 __device__ __forceinline__ void round_flags(const WorldDev& w, int ext, int round, u32 (&m)[kQ]) {
@@ -268,7 +276,7 @@ __device__ __forceinline__ void p_move(const WorldDev& w, int t, int ext, const 
         cl.energy[e + NT] = mb.y;
       }
     }
-    carried = tot;
+    carried = round == 0 ? tot : -1;
     tsync<NW>();  // the list is rewritten by the next round
   }
 }
@@ -372,7 +380,7 @@ __device__ __forceinline__ void p_count(const WorldDev& w, int t, int ext, int k
   int starved = 0, won = 0;
   // one round and the move phase's list still in shared memory: neither the
   // live flags nor the agent records need reading again
-  const bool reuse = carried >= 0 && unit_at<NW>(0, 1) >= nblk;
+  const bool reuse = carried >= 0;
   for (int round = 0; unit_at<NW>(0, round) < nblk; ++round) {
     u32 m[kQ], fr[kQ];
 #pragma unroll
@@ -742,10 +750,224 @@ __device__ __forceinline__ void rank_team(const WorldDev& w, int ext, int kseg, 
   }
 }
 
-// births on a team of NT threads (tid = the thread's place in it)
-template <int S, int NT>
-__device__ __forceinline__ void p_births(const WorldDev& w, int t, int r, int F, int ext, int id0, int tid) {
-  const SpeciesDev& sp = w.sp[S];
+// The sheep's ranks and births in one phase, on the team of the last kBirthWarps
+// warps. CTA b owns units [b*kseg, (b+1)*kseg) and gives birth for the parents
+// there: their ranks follow from the segment sums, and the free slots of the
+// same ranks are looked up -- segment by segment sums, unit by unit counts, slot
+// by the plane words -- instead of being published in a list by the CTA that owns
+// them and awaited at a grid barrier. Two dependent reads more than the list,
+// one grid barrier less.
+constexpr int kMaxGrid = 512;     // CTAs, at most (two segments per thread of the births team)
+constexpr int kBirthLocal = 256;  // births of a CTA whose lists stay in shared memory
+struct BirthScratch {
+  u32 segF[kMaxGrid + 1];  // free slots before each segment
+  u32 par[kBirthLocal], slot[kBirthLocal];  // the CTA's parents and their free slots, by rank
+  u64 unit[kBirthWarps * 32];  // units to look up: free slots before << 32 | unit
+  u64 scan[kBirthWarps];
+  u32 scan2[kBirthWarps];
+  u32 pre[kBirthWarps * 32];   // parents before each own unit
+  u32 preP, j0, j1, nunit;
+};
+constexpr int kBirthStage = 64;  // own units whose parent words are staged ahead
+
+// exclusive scan of a u64 and a u32 over the births team, with the totals
+__device__ __forceinline__ void birth_scan(BirthScratch& sc, int tw, int lane, u64 a, u32 b, u64& ex_a, u32& ex_b,
+                                           u64& tot_a, u32& tot_b) {
+  u64 ia = a;
+  u32 ib = b;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const u64 x = __shfl_up_sync(0xFFFFFFFFu, ia, o);
+    const u32 y = __shfl_up_sync(0xFFFFFFFFu, ib, o);
+    if (lane >= o) {
+      ia += x;
+      ib += y;
+    }
+  }
+  if (lane == 31) {
+    sc.scan[tw] = ia;
+    sc.scan2[tw] = ib;
+  }
+  bar_team<4, kBirthWarps>();
+  u64 pa = 0, ta = 0;
+  u32 pb = 0, tb = 0;
+#pragma unroll
+  for (int k = 0; k < kBirthWarps; ++k) {
+    const u64 x = sc.scan[k];
+    const u32 y = sc.scan2[k];
+    if (k < tw) {
+      pa += x;
+      pb += y;
+    }
+    ta += x;
+    tb += y;
+  }
+  ex_a = pa + ia - a;
+  ex_b = pb + ib - b;
+  tot_a = ta;
+  tot_b = tb;
+  bar_team<4, kBirthWarps>();  // the arrays are reused
+}
+
+// the slots of unit u with a set bit in its plane words, in slot order: f(rank, slot), ranks from r0 on
+template <typename Fn>
+__device__ __forceinline__ void unit_bits(u32 word, int base, int ext, u32 r0, int lane, Fn f) {
+  u32 m = base < ext ? (word >> (4 * (lane & 7))) & 0xFu : 0u;
+  const u32 n = (u32)__popc(m);
+  u32 inc = n;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const u32 x = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+    if (lane >= o) inc += x;
+  }
+  u32 r = r0 + inc - n;
+  while (m) {
+    f(r++, base + __ffs(m) - 1);
+    m &= m - 1;
+  }
+}
+
+// Returns F and P (free slots below the extent, parents) in every thread of the team.
+__device__ __forceinline__ void rank_births(const WorldDev& w, int t, int ext, int kseg, int id0, u32& F, u32& P,
+                                            BirthScratch& sc, u32* s_pw /* [kBirthStage][4], 16-byte aligned */) {
+  constexpr int NT = kBirthWarps * 32;
+  const PersistDev& ps = w.ps;
+  const SpeciesDev& sp = w.sp[0];
+  const int tt = (int)threadIdx.x - kMoveWarps * 32, tw = tt >> 5, lane = tt & 31;
+  const int G = (int)gridDim.x;
+  const int nblk = (ext + 127) >> 7;
+  const int j0 = (int)blockIdx.x * kseg, n = max(0, min(nblk, j0 + kseg) - j0);
+  // everything that depends on no other read is requested up front
+  if (tt < min(n, kBirthStage)) cp_async16(s_pw + 4 * tt, ps.plane[0][1] + 4 * (j0 + tt));
+  cp_async_commit();
+  const int ja = 2 * tt;  // this thread's two segments (G <= kMaxGrid)
+  const u64 s0 = ja < G ? ps.seg[0][ja] : 0ull, s1 = ja + 1 < G ? ps.seg[0][ja + 1] : 0ull;
+  const u32 b0 = tt < n ? (u32)ps.blk[0][j0 + tt] : 0u;
+  u64 ex, tot;
+  u32 exp_, totp;
+  birth_scan(sc, tw, lane, s0 + s1, b0, ex, exp_, tot, totp);
+  F = (u32)(tot >> 32);
+  P = (u32)tot;
+  const u32 fa = (u32)(ex >> 32), fb = fa + (u32)(s0 >> 32), fc = fb + (u32)(s1 >> 32);
+  if (ja <= G) sc.segF[ja] = fa;
+  if (ja + 1 <= G) sc.segF[ja + 1] = fb;
+  if (ja == (int)blockIdx.x) sc.preP = (u32)ex;
+  if (ja + 1 == (int)blockIdx.x) sc.preP = (u32)(ex + s0);
+  sc.pre[tt] = exp_;
+  cp_async_wait_0();
+  bar_team<4, kBirthWarps>();
+  // this CTA's births: the ranks [preP, preP + nb) below r
+  const u32 preP = sc.preP;
+  const u32 r = (u32)min((long long)P, (long long)F + (sp.cap - ext));
+  const u64 own = (int)blockIdx.x == ja ? s0 : s1;  // (only the thread that holds the segment uses it)
+  if (ja == (int)blockIdx.x || ja + 1 == (int)blockIdx.x) sc.nunit = (u32)own;
+  const u32 f0 = preP;
+  // segments that hold the free slots of ranks f0 and min(preP + nb, F) - 1 (nb as below, from the owner's count)
+  bar_team<4, kBirthWarps>();
+  const u32 nb = r > preP ? min(r - preP, sc.nunit) : 0u;
+  const u32 f1 = min(preP + nb, F);
+  if (nb == 0) {
+    bar_team<4, kBirthWarps>();  // every thread has read the scratch before it is written again
+    return;
+  }
+  const bool local = nb <= (u32)kBirthLocal;  // else the lists go through global memory
+  if (f0 < f1) {
+    if (fa <= f0 && f0 < fb) sc.j0 = (u32)ja;
+    if (fb <= f0 && f0 < fc) sc.j0 = (u32)ja + 1;
+    if (fa <= f1 - 1 && f1 - 1 < fb) sc.j1 = (u32)ja;
+    if (fb <= f1 - 1 && f1 - 1 < fc) sc.j1 = (u32)ja + 1;
+  }
+  // the parents, by rank
+  {
+    u32 carry = 0;
+    for (int c0 = 0; c0 < n; c0 += NT) {
+      if (c0 > 0) {
+        const u32 v = c0 + tt < n ? (u32)ps.blk[0][j0 + c0 + tt] : 0u;
+        u64 e2, t2;
+        birth_scan(sc, tw, lane, 0ull, v, e2, exp_, t2, totp);
+        sc.pre[tt] = exp_;
+        bar_team<4, kBirthWarps>();
+      }
+      const int cn = min(NT, n - c0);
+      for (int q = tw; q < cn; q += kBirthWarps) {
+        const u32 r0 = carry + sc.pre[q];
+        if (r0 >= nb) continue;
+        const int base = ((j0 + c0 + q) << 7) + 4 * lane;
+        u32 word = 0;
+        if (base < ext) word = c0 + q < kBirthStage ? s_pw[4 * (c0 + q) + (lane >> 3)] : ps.plane[0][1][base >> 5];
+        unit_bits(word, base, ext, r0, lane, [&](u32 k, int slot) {
+          if (k >= nb) return;
+          if (local) sc.par[k] = (u32)slot;
+          else if (in_range(preP + k, sp.cap, w.err)) sp.parents[preP + k] = slot;
+        });
+      }
+      carry += totp;
+      bar_team<4, kBirthWarps>();  // sc.pre is rewritten by the next pass; the lists are complete after the last
+    }
+  }
+  // the first parent of each thread, in flight while the free slots are looked up
+  int p0 = -1;
+  int4 pa0 = make_int4(0, 0, 0, 0);
+  if ((u32)tt < nb) {
+    p0 = local ? (int)sc.par[tt] : sp.parents[preP + tt];
+    if (in_range(p0, sp.cap, w.err)) pa0 = sp.agent[p0];
+  }
+  if (f0 < f1) {
+    const int u1 = min(nblk, ((int)sc.j1 + 1) * kseg);
+    u32 carry = sc.segF[sc.j0];
+    for (int c0 = (int)sc.j0 * kseg; c0 < u1 && carry < f1; c0 += NT) {
+      if (tt == 0) sc.nunit = 0u;
+      const int u = c0 + tt;
+      const u32 v = u < u1 ? (u32)(ps.blk[0][u] >> 32) : 0u;
+      u64 e2, t2;
+      u32 pf, tot2;
+      birth_scan(sc, tw, lane, 0ull, v, e2, pf, t2, tot2);
+      pf += carry;
+      if (v && pf < f1 && pf + v > f0) sc.unit[atomicAdd(&sc.nunit, 1u)] = ((u64)pf << 32) | (u32)u;
+      bar_team<4, kBirthWarps>();
+      const int nu = (int)sc.nunit;
+      for (int e = tw; e < nu; e += kBirthWarps) {
+        const u64 x = sc.unit[e];
+        const int base = ((int)(u32)x << 7) + 4 * lane;
+        const u32 word = base < ext ? ps.plane[0][0][base >> 5] : 0u;
+        unit_bits(word, base, ext, (u32)(x >> 32), lane, [&](u32 k, int slot) {
+          if (k < f0 || k >= f1) return;
+          if (local) sc.slot[k - f0] = (u32)slot;
+          else if (in_range(k, sp.cap, w.err)) sp.freel[k] = slot;
+        });
+      }
+      carry += tot2;
+      bar_team<4, kBirthWarps>();
+    }
+  }
+  // births: the child of rank i fills the free slot of rank i, or the slots past the extent once those are used up
+  for (u32 k = (u32)tt; k < nb; k += NT) {
+    const u32 i = preP + k;
+    int p = p0;
+    int4 pa = pa0;
+    if (k != (u32)tt) {
+      p = local ? (int)sc.par[k] : sp.parents[i];
+      if (!in_range(p, sp.cap, w.err)) continue;
+      pa = sp.agent[p];
+    }
+    const int slot = i < F ? (local ? (int)sc.slot[k] : sp.freel[i]) : ext + (int)(i - F);
+    if (!in_range(p, sp.cap, w.err) || !in_range(slot, sp.cap, w.err)) continue;
+    const int half = pa.y >> 1;
+    sp.agent[p].y = pa.y - half;
+    sp.agent[slot] = make_int4(pa.x, half, (int)((u32)id0 + i), 0);
+    sp.active[slot] = 1;
+    const u64 key = claim_key(draw(w.seed, w.model, (u32)t, (u32)slot, ABM_P_VICTIM, 0u), slot);
+    if (w.variant & ABM_VARIANT_MANY_WOLVES)
+      list_push(w.victim, w.snext, w.skey, pa.x, slot, t, key);
+    else
+      atomicMin(&w.victim[pa.x], key);
+  }
+}
+
+// wolf births from the parent and free lists, on a team of NT threads (tid = the thread's place in it)
+template <int NT>
+__device__ __forceinline__ void p_births(const WorldDev& w, int r, int F, int ext, int id0, int tid) {
+  const SpeciesDev& sp = w.sp[1];
   // birth i -> CTA i mod G: the births spread over all SMs
   for (int i = blockIdx.x + gridDim.x * tid; i < r; i += gridDim.x * NT) {
     const int p = sp.parents[i];
@@ -756,13 +978,6 @@ __device__ __forceinline__ void p_births(const WorldDev& w, int t, int r, int F,
     sp.agent[p].y = pa.y - half;
     sp.agent[slot] = make_int4(pa.x, half, (int)((u32)id0 + (u32)i), 0);
     sp.active[slot] = 1;
-    if (S == 0) {
-      const u64 key = claim_key(draw(w.seed, w.model, (u32)t, (u32)slot, ABM_P_VICTIM, 0u), slot);
-      if (w.variant & ABM_VARIANT_MANY_WOLVES)
-        list_push(w.victim, w.snext, w.skey, pa.x, slot, t, key);
-      else
-        atomicMin(&w.victim[pa.x], key);
-    }
   }
 }
 
@@ -818,8 +1033,14 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
   __shared__ int s_acc[2 * kPWarps];
   __shared__ u32 s_live[kRoundUnits * 4];
   __shared__ __align__(16) int s_cell[kRoundUnits * 128];
-  __shared__ int s_energy[kRoundUnits * 128];
+  __shared__ __align__(16) int s_energy[kRoundUnits * 128];
   __shared__ int s_wolf[4];  // the wolf team's F, P, starved and eaten, for the whole CTA
+  __shared__ int s_sheep[3]; // the births team's F and P and the wolf movers' list length, for the whole CTA
+  // in phase 3 the wolf movers' lists fill half of the arrays; the births team takes the other halves
+  constexpr int kMoveEntries = kQ * kMoveWarps * 128;
+  static_assert(sizeof(BirthScratch) <= sizeof(s_cell) - kMoveEntries * sizeof(int), "births scratch");
+  static_assert(kBirthStage * 16 <= sizeof(s_energy) - kMoveEntries * sizeof(int), "births plane words");
+  BirthScratch& scratch = *reinterpret_cast<BirthScratch*>(s_cell + kMoveEntries);
   __shared__ StepBook s_book;
   const CtaList cl{s_clist, s_wcnt, s_live, s_cell, s_energy};
   const bool wolf_team = (int)threadIdx.x >= kSheepWarps * 32;
@@ -845,21 +1066,18 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
   clk.start();
   // Wolf ranks of step t-1 run beside the sheep moves of step t, and the wolf
   // moves of step t beside the sheep ranks: neither needs the other's
-  // results, so a step takes five barrier-separated phases:
+  // results, so a step takes four barrier-separated phases:
   //   P1  wolf team: wolf ranks (t-1) | sheep team: sheep move (t)
   //   P2  wolf counters and statistics (t-1) in every thread, then
   //       wolf team: wolf births (t-1) | sheep team: sheep eat / select / die (t)
-  //   P3  sheep ranks (t) | wolves move + victim claims (t) (a wolf only
-  //       needs a live sheep on its cell: the survivors registered in P2)
-  //   P4  sheep births (t) (lambs register as victims before wolves eat)
-  //   P5  wolves eat / kill / select / die (t)
-  // and the last step's wolf ranks and births close the launch. In P1 and P2
-  // the two teams meet only at the grid barriers; P3 to P5 use every warp.
-  // The barrier between P3 and P4 is split: a CTA counts itself in once its
-  // ranks are written and waits only after its wolf moves, so the wait
-  // overlaps the wolf moves (births touch no wolf, and a lamb lands on its
-  // parent's cell, which already holds a victim key, so no claim condition of
-  // the wolf move changes under it).
+  //   P3  eight warps: wolves move + victim claims (t) (a wolf only needs a
+  //       live sheep on its cell: the survivors registered in P2) | eight
+  //       warps: sheep ranks and births (t) (births touch no wolf, and a lamb
+  //       lands on its parent's cell, which already holds a victim key, so no
+  //       claim condition of the wolf move changes under it)
+  //   P4  wolves eat / kill / select / die (t)
+  // and the last step's wolf ranks and births close the launch. In P1 to P3
+  // the two teams meet only at the grid barriers.
   // wolf team: the ranks of step tw's wolves and that step's counters, left in s_wolf
   auto wolf_ranks = [&](int tw) {
     const int* accw = ps.acc + 4 * (tw & 1);
@@ -942,7 +1160,7 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
     const int kseg0 = (((ext[0] + 127) >> 7) + (int)gridDim.x - 1) / (int)gridDim.x;
     if (wolf_team) {
       if (it > 0)
-        p_births<1, kWolfWarps * 32>(w, t - 1, wb.r, wb.F, wb.ext, wb.id0, (int)threadIdx.x - kSheepWarps * 32);
+        p_births<kWolfWarps * 32>(w, wb.r, wb.F, wb.ext, wb.id0, (int)threadIdx.x - kSheepWarps * 32);
     } else {
       if (blockIdx.x == 0)  // wolf segment sums: last read in P1
         for (int j = threadIdx.x; j < (int)gridDim.x; j += kSheepWarps * 32) ps.seg[1][j] = 0ull;
@@ -950,45 +1168,44 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
     }
     grid_sync(ps.bar, w.err, bar_target);
     clk.lap(1);
-    // ---- P3: sheep ranks and lists | wolves move + claims
-    u32 mf[kQ];
-    round_flags<1, kPWarps>(w, ext[1], 0, mf);  // issued before the sheep ranks, used by the wolf move
-    u32 F0, P0;
-    // (s_cell is free between the count phase and the wolf move: plane staging)
-    rank_phase<0>(w, ext[0], kseg0, F0, P0, s_red, s_pre, reinterpret_cast<u32*>(s_cell));
-    const int avail0 = (int)F0 + (w.sp[0].cap - ext[0]);
-    const int r0 = min((int)P0, avail0);
-    const Births sb = {r0, (int)F0, ext[0], nid[0]};
-    // the ranks' half of the barrier; the wolf move needs none of them
-    grid_arrive(ps.bar, bar_target);
-    p_move<1, kPWarps>(w, t, ext[1], cl, carried, mf);
-    grid_wait(ps.bar, w.err, bar_target);
-    clk.lap(2);
-    // ---- P4: sheep births (every CTA's lists are complete: the split barrier's wait); sheep counters
-    int starved0 = 0, grass = 0;
-    if (book_thread()) {  // written in P2: loaded ahead of the births' own loads
-      starved0 = acc[0];
-      grass = acc[3];
+    // ---- P3: sheep ranks and births | wolves move + claims
+    if ((int)threadIdx.x < kMoveWarps * 32) {
+      u32 mf[kQ];
+      round_flags<1, kMoveWarps>(w, ext[1], 0, mf);
+      p_move<1, kMoveWarps>(w, t, ext[1], cl, carried, mf);
+      if (threadIdx.x == 0) s_sheep[2] = carried;
+    } else {
+      u32 F0, P0;
+      rank_births(w, t, ext[0], kseg0, nid[0], F0, P0, scratch, reinterpret_cast<u32*>(s_energy) + kMoveEntries);
+      if ((int)threadIdx.x == kMoveWarps * 32) {
+        s_sheep[0] = (int)F0;
+        s_sheep[1] = (int)P0;
+      }
     }
-    p_births<0, kPT>(w, t, sb.r, sb.F, sb.ext, sb.id0, threadIdx.x);
-    if (blockIdx.x == 0)  // sheep segment sums: last read by the rank phases
-      for (int j = threadIdx.x; j < (int)gridDim.x; j += kPT) ps.seg[0][j] = 0ull;
+    grid_sync(ps.bar, w.err, bar_target);
+    clk.lap(2);
+    // ---- sheep counters (every thread)
+    const int F0 = s_sheep[0], P0 = s_sheep[1];
+    carried = s_sheep[2];
+    const int avail0 = F0 + (w.sp[0].cap - ext[0]);
+    const int r0 = min(P0, avail0);
     nid[0] += r0;
-    if (r0 > (int)F0) ext[0] += r0 - (int)F0;
+    if (r0 > F0) ext[0] += r0 - F0;
+    if (blockIdx.x == 0)  // sheep segment sums: last read in P3
+      for (int j = threadIdx.x; j < (int)gridDim.x; j += kPT) ps.seg[0][j] = 0ull;
     if (book_thread()) {
       StepBook& b = s_book;
+      const int starved0 = acc[0];
       const int n_after = b.nstart0 + r0;
       if (n_after > b.hw[0]) b.hw[0] = n_after;
       b.nact[0] = n_after - starved0;
-      if ((int)P0 > avail0) b.ovf[0] = 1;
+      if (P0 > avail0) b.ovf[0] = 1;
       b.r0p = r0;
-      b.P0p = (int)P0;
+      b.P0p = P0;
       b.starved0p = starved0;
-      b.grassp = grass;
+      b.grassp = acc[3];
     }
-    grid_sync(ps.bar, w.err, bar_target);
-    clk.lap(3);
-    // ---- P5: wolves eat / kill / select / die / flags
+    // ---- P4: wolves eat / kill / select / die / flags
     const int kseg1 = (((ext[1] + 127) >> 7) + (int)gridDim.x - 1) / (int)gridDim.x;
     p_count<1, kPWarps>(w, t, ext[1], kseg1, acc, cl, carried, s_upar, s_acc);
     if (book_thread()) s_book.stp = stats ? stats + it : nullptr;
@@ -1013,7 +1230,7 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
     const Births wb = wolf_counters(t - 1);
     grid_sync(ps.bar, w.err, bar_target);
     clk.lap(5);
-    p_births<1, kPT>(w, t - 1, wb.r, wb.F, wb.ext, wb.id0, threadIdx.x);
+    p_births<kPT>(w, wb.r, wb.F, wb.ext, wb.id0, threadIdx.x);
     if (blockIdx.x == 0)  // wolf segment sums, for the next launch
       for (int j = threadIdx.x; j < (int)gridDim.x; j += kPT) ps.seg[1][j] = 0ull;
   }
@@ -1042,7 +1259,7 @@ __global__ void k_barrier_timeout(u32* bar, int* err, int limit) {
 int persistent_max_ctas() {
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_persistent<2>, kPT, 0) != cudaSuccess) return 0;
-  return nb * num_sms();
+  return std::min(nb * num_sms(), kMaxGrid);
 }
 
 int persistent_warps() { return kPWarps; }
