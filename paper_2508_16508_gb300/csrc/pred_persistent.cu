@@ -829,7 +829,8 @@ __device__ __forceinline__ void unit_bits(u32 word, int base, int ext, u32 r0, i
 
 // Returns F and P (free slots below the extent, parents) in every thread of the team.
 __device__ __forceinline__ void rank_births(const WorldDev& w, int t, int ext, int kseg, int id0, u32& F, u32& P,
-                                            BirthScratch& sc, u32* s_pw /* [kBirthStage][4], 16-byte aligned */) {
+                                            BirthScratch& sc, u32* s_pw /* [kBirthStage][4], 16-byte aligned */,
+                                            uint4* s_uw /* [kBirthWarps * 32] */) {
   constexpr int NT = kBirthWarps * 32;
   const PersistDev& ps = w.ps;
   const SpeciesDev& sp = w.sp[0];
@@ -917,20 +918,26 @@ __device__ __forceinline__ void rank_births(const WorldDev& w, int t, int ext, i
     u32 carry = sc.segF[sc.j0];
     for (int c0 = (int)sc.j0 * kseg; c0 < u1 && carry < f1; c0 += NT) {
       if (tt == 0) sc.nunit = 0u;
+      // counts and plane words of the pass's units in one round trip; the words of those that are needed go to
+      // shared memory, where the warps take them unit by unit
       const int u = c0 + tt;
       const u32 v = u < u1 ? (u32)(ps.blk[0][u] >> 32) : 0u;
+      const uint4 words = u < u1 ? reinterpret_cast<const uint4*>(ps.plane[0][0])[u] : make_uint4(0, 0, 0, 0);
       u64 e2, t2;
       u32 pf, tot2;
       birth_scan(sc, tw, lane, 0ull, v, e2, pf, t2, tot2);
       pf += carry;
-      if (v && pf < f1 && pf + v > f0) sc.unit[atomicAdd(&sc.nunit, 1u)] = ((u64)pf << 32) | (u32)u;
+      if (v && pf < f1 && pf + v > f0) {
+        const u32 e = atomicAdd(&sc.nunit, 1u);
+        sc.unit[e] = ((u64)pf << 32) | (u32)u;
+        s_uw[e] = words;
+      }
       bar_team<4, kBirthWarps>();
       const int nu = (int)sc.nunit;
       for (int e = tw; e < nu; e += kBirthWarps) {
         const u64 x = sc.unit[e];
         const int base = ((int)(u32)x << 7) + 4 * lane;
-        const u32 word = base < ext ? ps.plane[0][0][base >> 5] : 0u;
-        unit_bits(word, base, ext, (u32)(x >> 32), lane, [&](u32 k, int slot) {
+        unit_bits(reinterpret_cast<const u32*>(s_uw + e)[lane >> 3], base, ext, (u32)(x >> 32), lane, [&](u32 k, int slot) {
           if (k < f0 || k >= f1) return;
           if (local) sc.slot[k - f0] = (u32)slot;
           else if (in_range(k, sp.cap, w.err)) sp.freel[k] = slot;
@@ -1039,7 +1046,8 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
   // in phase 3 the wolf movers' lists fill half of the arrays; the births team takes the other halves
   constexpr int kMoveEntries = kQ * kMoveWarps * 128;
   static_assert(sizeof(BirthScratch) <= sizeof(s_cell) - kMoveEntries * sizeof(int), "births scratch");
-  static_assert(kBirthStage * 16 <= sizeof(s_energy) - kMoveEntries * sizeof(int), "births plane words");
+  static_assert((kBirthStage + kBirthWarps * 32) * 16 <= sizeof(s_energy) - kMoveEntries * sizeof(int), "births plane words");
+  u32* const birth_words = reinterpret_cast<u32*>(s_energy + kMoveEntries);
   BirthScratch& scratch = *reinterpret_cast<BirthScratch*>(s_cell + kMoveEntries);
   __shared__ StepBook s_book;
   const CtaList cl{s_clist, s_wcnt, s_live, s_cell, s_energy};
@@ -1176,7 +1184,8 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
       if (threadIdx.x == 0) s_sheep[2] = carried;
     } else {
       u32 F0, P0;
-      rank_births(w, t, ext[0], kseg0, nid[0], F0, P0, scratch, reinterpret_cast<u32*>(s_energy) + kMoveEntries);
+      rank_births(w, t, ext[0], kseg0, nid[0], F0, P0, scratch, birth_words,
+                  reinterpret_cast<uint4*>(birth_words + 4 * kBirthStage));
       if ((int)threadIdx.x == kMoveWarps * 32) {
         s_sheep[0] = (int)F0;
         s_sheep[1] = (int)P0;
