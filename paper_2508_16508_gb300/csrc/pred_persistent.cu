@@ -809,21 +809,52 @@ __device__ __forceinline__ void birth_scan(BirthScratch& sc, int tw, int lane, u
   bar_team<4, kBirthWarps>();  // the arrays are reused
 }
 
-// the slots of unit u with a set bit in its plane words, in slot order: f(rank, slot), ranks from r0 on
-template <typename Fn>
-__device__ __forceinline__ void unit_bits(u32 word, int base, int ext, u32 r0, int lane, Fn f) {
-  u32 m = base < ext ? (word >> (4 * (lane & 7))) & 0xFu : 0u;
+// The slots of a unit with a set bit in its plane words, in slot order: f(rank,
+// slot) for the ranks in [lo, hi), the first bit having rank r0. LANES lanes per
+// unit (32 or 8), 4 or 16 slots each.
+template <int LANES, typename Fn>
+__device__ __forceinline__ void unit_bits(const u32* words, bool on, int u, int ext, u32 r0, u32 lo, u32 hi,
+                                          int lane, Fn f) {
+  constexpr int S = 128 / LANES;
+  const int l = lane & (LANES - 1);
+  const int at = S * l, base = (u << 7) + at;
+  u32 m = on && base < ext ? (words[at >> 5] >> (at & 31)) & ((1u << S) - 1u) : 0u;
   const u32 n = (u32)__popc(m);
   u32 inc = n;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const u32 x = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-    if (lane >= o) inc += x;
+  for (int o = 1; o < LANES; o <<= 1) {
+    const u32 x = __shfl_up_sync(0xFFFFFFFFu, inc, o, LANES);
+    if (l >= o) inc += x;
   }
   u32 r = r0 + inc - n;
-  while (m) {
-    f(r++, base + __ffs(m) - 1);
-    m &= m - 1;
+  if (r + n <= lo) return;
+  for (; r < lo; ++r) m &= m - 1;
+  for (; m && r < hi; m &= m - 1) f(r++, base + __ffs(m) - 1);
+}
+
+// n units on the births team: a warp each where that takes one turn, else four to
+// a warp -- where the crowded low slots are nearly full, a CTA's births look up a
+// hundred units of one or two free slots. (A warp each throughout: 25.7 us a step
+// at 2048 x 2048 after 100 steps against 23.6; four to a warp throughout: 301 x 301
+// 14.8 against 14.3; one thread per unit 33 and 16.1.) unit(e) gives the e-th unit's plane
+// words, number and first rank.
+template <typename Un, typename Fn>
+__device__ __forceinline__ void units_bits(int n, int ext, u32 lo, u32 hi, int tt, Un unit, Fn f) {
+  const int lane = tt & 31;
+  const u32* words = nullptr;
+  int u = 0;
+  u32 r0 = 0;
+  if (n <= kBirthWarps) {
+    const int e = tt >> 5;
+    if (e >= n) return;
+    unit(e, words, u, r0);
+    unit_bits<32>(words, true, u, ext, r0, lo, hi, lane, f);
+    return;
+  }
+  for (int e0 = 0; e0 < n; e0 += 4 * kBirthWarps) {
+    const int e = e0 + (tt >> 3);
+    if (e < n) unit(e, words, u, r0);
+    unit_bits<8>(words, e < n, u, ext, r0, lo, hi, lane, f);
   }
 }
 
@@ -890,18 +921,17 @@ __device__ __forceinline__ void rank_births(const WorldDev& w, int t, int ext, i
         bar_team<4, kBirthWarps>();
       }
       const int cn = min(NT, n - c0);
-      for (int q = tw; q < cn; q += kBirthWarps) {
-        const u32 r0 = carry + sc.pre[q];
-        if (r0 >= nb) continue;
-        const int base = ((j0 + c0 + q) << 7) + 4 * lane;
-        u32 word = 0;
-        if (base < ext) word = c0 + q < kBirthStage ? s_pw[4 * (c0 + q) + (lane >> 3)] : ps.plane[0][1][base >> 5];
-        unit_bits(word, base, ext, r0, lane, [&](u32 k, int slot) {
-          if (k >= nb) return;
-          if (local) sc.par[k] = (u32)slot;
-          else if (in_range(preP + k, sp.cap, w.err)) sp.parents[preP + k] = slot;
-        });
-      }
+      units_bits(
+          cn, ext, 0u, nb, tt,
+          [&](int q, const u32*& words, int& u, u32& r0) {
+            u = j0 + c0 + q;
+            r0 = carry + sc.pre[q];
+            words = c0 + q < kBirthStage ? s_pw + 4 * (c0 + q) : ps.plane[0][1] + 4 * (size_t)u;
+          },
+          [&](u32 k, int slot) {
+            if (local) sc.par[k] = (u32)slot;
+            else if (in_range(preP + k, sp.cap, w.err)) sp.parents[preP + k] = slot;
+          });
       carry += totp;
       bar_team<4, kBirthWarps>();  // sc.pre is rewritten by the next pass; the lists are complete after the last
     }
@@ -934,15 +964,17 @@ __device__ __forceinline__ void rank_births(const WorldDev& w, int t, int ext, i
       }
       bar_team<4, kBirthWarps>();
       const int nu = (int)sc.nunit;
-      for (int e = tw; e < nu; e += kBirthWarps) {
-        const u64 x = sc.unit[e];
-        const int base = ((int)(u32)x << 7) + 4 * lane;
-        unit_bits(reinterpret_cast<const u32*>(s_uw + e)[lane >> 3], base, ext, (u32)(x >> 32), lane, [&](u32 k, int slot) {
-          if (k < f0 || k >= f1) return;
-          if (local) sc.slot[k - f0] = (u32)slot;
-          else if (in_range(k, sp.cap, w.err)) sp.freel[k] = slot;
-        });
-      }
+      units_bits(
+          nu, ext, f0, f1, tt,
+          [&](int e, const u32*& words, int& u, u32& r0) {
+            u = (int)(u32)sc.unit[e];
+            r0 = (u32)(sc.unit[e] >> 32);
+            words = reinterpret_cast<const u32*>(s_uw + e);
+          },
+          [&](u32 k, int slot) {
+            if (local) sc.slot[k - f0] = (u32)slot;
+            else if (in_range(k, sp.cap, w.err)) sp.freel[k] = slot;
+          });
       carry += tot2;
       bar_team<4, kBirthWarps>();
     }
