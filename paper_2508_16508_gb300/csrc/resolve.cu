@@ -5,9 +5,10 @@
 // key is order-independent, so the result is deterministic.
 //
 // Skewed (Zipf) claim distributions put a large share of the claims on a few
-// resources; each CTA therefore first folds its chunk of claims into a
-// shared-memory hash table (open addressing, smem 64-bit atomicMin) and then
-// issues one global atomicMin per distinct resource it saw.
+// resources, whose table entries would then serialise the atomics. Each CTA
+// therefore keeps the best claim of up to kHash resources in shared memory and
+// issues one global atomicMin for each of them at its end; claims on resources
+// that found their place taken go to the global table at once.
 #include <algorithm>
 #include <mutex>
 
@@ -15,84 +16,91 @@
 
 namespace abm {
 
-constexpr int kResThreads = 512;
-constexpr int kResPerThread = 8;
+constexpr int kResThreads = 1024;
+constexpr int kResPerThread = 4;
 constexpr int kResChunk = kResThreads * kResPerThread;
 constexpr int kHashBits = 13;
 constexpr int kHash = 1 << kHashBits;  // 8192 entries x 12 B = 96 KiB of shared memory
-constexpr int kMaxProbe = 64;
 
 __global__ void k_table_fill(u64* table, int R) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < R; i += gridDim.x * blockDim.x) table[i] = kNoKey;
 }
 
-__global__ void __launch_bounds__(kResThreads) k_claims(const int32_t* __restrict__ res,
-                                                        const u32* __restrict__ prio, int M, int R,
-                                                        u64* table) {
-  extern __shared__ unsigned char smem[];
-  u64* s_best = reinterpret_cast<u64*>(smem);
-  int* s_tag = reinterpret_cast<int*>(s_best + kHash);
-  __shared__ int s_used;  // distinct resources in the table
+// A place of the shared table belongs to the first resource that takes it. A
+// chunk of claims goes through three rounds with a barrier after each: take
+// places; lower the priorities (32-bit shared atomics, only by claims below the
+// priority of the chunks before: an equal one loses to the earlier index);
+// lower the index among the claims that hold a new priority. 4 M Zipf(1.1) claims
+// on 262144 resources: 33 us, bound by the scattered global atomics that are
+// left (about two million; reading an entry first to spare its atomic costs as
+// much as the atomic: 43 us; one CTA per SM with twice the places: 38 us). (Open
+// addressing with contended 64-bit shared atomics on packed keys: 39 us, and 147
+// instead of 62 us for the whole call where all resources are equally popular. A
+// shared filter of seen priorities with every unbeaten claim going to global memory:
+// 70 us, the hot entries' first claims serialise in L2.)
+__global__ void __launch_bounds__(kResThreads, 2) k_claims(const int32_t* __restrict__ res,
+                                                           const u32* __restrict__ prio, int M, int R, u64* table) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  volatile int* s_res = reinterpret_cast<int*>(smem);       // the resource of a place, -1: free
+  u32* s_prio = reinterpret_cast<u32*>(smem) + kHash;       // its smallest priority
+  u32* s_idx = reinterpret_cast<u32*>(smem) + 2 * kHash;    // and the smallest claim index with it
   for (int h = threadIdx.x; h < kHash; h += kResThreads) {
-    s_tag[h] = -1;
-    s_best[h] = kNoKey;
+    s_res[h] = -1;
+    s_prio[h] = 0xFFFFFFFFu;
+    s_idx[h] = 0xFFFFFFFFu;
   }
-  if (threadIdx.x == 0) s_used = 0;
-  __syncthreads();
   // a contiguous run of claims per CTA, in chunks of kResChunk (the last one ragged)
   const long long run = ((long long)M + gridDim.x - 1) / gridDim.x;
   const int lo = (int)min((long long)M, run * blockIdx.x), hi = (int)min((long long)M, run * (blockIdx.x + 1));
-  for (int m0 = lo; m0 < hi; m0 += kResChunk) {
-    int rr[kResPerThread];
-    u32 pp[kResPerThread];
+  __syncthreads();
+  for (long long m0 = lo; m0 < hi; m0 += kResChunk) {
+    int r[kResPerThread];
+    u32 p[kResPerThread];
 #pragma unroll
     for (int j = 0; j < kResPerThread; ++j) {
-      const int m = m0 + j * kResThreads + threadIdx.x;  // coalesced, all in flight
-      rr[j] = m < hi ? res[m] : -1;
-      pp[j] = m < hi ? prio[m] : 0u;
+      const long long m = m0 + j * kResThreads + threadIdx.x;  // coalesced, all in flight
+      r[j] = m < hi ? res[m] : -1;
+      p[j] = m < hi ? prio[m] : 0u;
+      if (r[j] >= R) r[j] = -1;
     }
 #pragma unroll
     for (int j = 0; j < kResPerThread; ++j) {
-      const int m = m0 + j * kResThreads + threadIdx.x;
-      const int r = rr[j];
-      if (r < 0 || r >= R) continue;
-      const u64 key = ((u64)pp[j] << 32) | (u32)m;
-      u32 h = ((u32)r * 2654435761u) >> (32 - kHashBits);
-      bool done = false;
-      for (int p = 0; p < kMaxProbe; ++p) {
-        int t = *reinterpret_cast<volatile int*>(&s_tag[h]);
-        if (t == -1) {
-          t = atomicCAS(&s_tag[h], -1, r);
-          if (t == -1) atomicAdd(&s_used, 1);
-        }
-        if (t == -1 || t == r) {
-          // most claims on a popular resource lose to one already seen: a plain
-          // read (keys only fall) spares them the contended 64-bit atomic
-          if (key < *reinterpret_cast<volatile u64*>(&s_best[h])) atomicMin(&s_best[h], key);
-          done = true;
-          break;
-        }
-        h = (h + 1) & (kHash - 1);
-      }
-      if (!done) atomicMin(&table[r], key);  // table full around h: go straight to global
+      const u32 h = ((u32)r[j] * 2654435761u) >> (32 - kHashBits);
+      if (r[j] >= 0 && s_res[h] == -1) s_res[h] = r[j];
     }
     __syncthreads();
-    // The table is folded into global memory only when it is half full or the
-    // CTA has no claims left: skewed claims (a few hot resources) then cost
-    // one global atomic per distinct resource per CTA, not per chunk.
-    if (s_used > kHash / 2 || m0 + kResChunk >= hi) {
-      for (int h = threadIdx.x; h < kHash; h += kResThreads) {
-        const int t = s_tag[h];
-        if (t >= 0) {
-          atomicMin(&table[t], s_best[h]);
-          s_tag[h] = -1;
-          s_best[h] = kNoKey;
-        }
+#pragma unroll
+    for (int j = 0; j < kResPerThread; ++j) {
+      if (r[j] < 0) continue;
+      const u32 h = ((u32)r[j] * 2654435761u) >> (32 - kHashBits);
+      const u32 m = (u32)m0 + j * kResThreads + threadIdx.x;
+      if (s_res[h] != r[j]) {
+        atomicMin(&table[r[j]], ((u64)p[j] << 32) | m);
+        r[j] = -1;
+      } else if (p[j] < *(volatile u32*)&s_prio[h] || *(volatile u32*)&s_idx[h] == 0xFFFFFFFFu) {
+        // below every earlier chunk's claim (or none came before, or this chunk is lowering the entry already). The
+        // index of the priority that no longer counts goes first, so that whoever sees a priority of this chunk sees
+        // that too and stays in
+        *(volatile u32*)&s_idx[h] = 0xFFFFFFFFu;
+        __threadfence_block();
+        atomicMin(&s_prio[h], p[j]);
+      } else {
+        r[j] = -1;
       }
-      __syncthreads();
-      if (threadIdx.x == 0) s_used = 0;
     }
     __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kResPerThread; ++j) {
+      if (r[j] < 0) continue;
+      const u32 h = ((u32)r[j] * 2654435761u) >> (32 - kHashBits);
+      if (p[j] == *(volatile u32*)&s_prio[h]) atomicMin(&s_idx[h], (u32)m0 + j * kResThreads + threadIdx.x);
+    }
+    __syncthreads();
+  }
+#pragma unroll 4
+  for (int h = threadIdx.x; h < kHash; h += kResThreads) {
+    const int r = s_res[h];
+    if (r >= 0) atomicMin(&table[r], ((u64)s_prio[h] << 32) | s_idx[h]);
   }
 }
 
@@ -141,7 +149,7 @@ static std::atomic<unsigned long long> g_res_attr{0};  // devices whose k_claims
 
 abm_status resolve_launch(const int32_t* claim_res, const uint32_t* claim_prio, int32_t M, int32_t R,
                           uint64_t* table, int32_t* out_winner, uint8_t* out_is_winner, cudaStream_t st) {
-  const size_t smem = (size_t)kHash * (sizeof(u64) + sizeof(int));
+  const size_t smem = (size_t)kHash * 3 * sizeof(u32);
   ABM_CUDA_TRY(smem_attr_once(k_claims, (int)smem, g_res_attr));
   const int sms = num_sms();
   if (M > 0) {

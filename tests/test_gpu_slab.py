@@ -583,3 +583,26 @@ def test_selective_update_paths(eng, n, p):
         assert got[wrote].max(initial=0) <= 1
         odd = got
     s.check()
+
+
+@pytest.mark.parametrize("M,R,levels", [(4095, 3, 1), (4097, 70_000, 2), (700_003, 5, 1), (700_003, 50_000, 3),
+                                        (1_500_000, 1, 2**32), (1_300_001, 1_000_000, 2**32)])
+def test_resolve_ties_and_hot_resources(eng, M, R, levels):
+    """Whole numbers, so exact: few priority levels (ties go to the smaller index, across chunks and CTAs) and
+    resources claimed by a large share of all, at the sizes around the kernel's chunks; top priorities and resources."""
+    rng = np.random.default_rng(M + R)
+    res = np.where(rng.random(M) < 0.3, R - 1, rng.integers(0, R, M)).astype(np.int32)
+    prio = rng.integers(0, levels, M).astype(np.uint32)
+    prio[rng.random(M) < 0.1] = 0xFFFFFFFF
+    order = np.lexsort((np.arange(M), prio, res))
+    first = order[np.r_[True, res[order][1:] != res[order][:-1]]]
+    want = np.full(R, -1, np.int64)
+    want[res[first]] = first
+    won = np.zeros(M, np.uint8)
+    won[first] = 1
+    r = eng.Resolver(R)
+    isw = torch.empty(M, dtype=torch.uint8, device="cuda")
+    w = r(torch.from_numpy(res).cuda(), torch.from_numpy(prio.view(np.int32)).cuda(), isw)
+    np.testing.assert_array_equal(np_of(w), want)
+    np.testing.assert_array_equal(np_of(isw), won)
+    assert torch.all(r.table == -1)
