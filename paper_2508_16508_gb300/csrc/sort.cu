@@ -38,7 +38,9 @@ struct SortScratch {
   u32* val[2];
   u32* hist;        // [kBins][G]: a pass's digit counts per chunk, then its positions
   u32* counts;      // [G] live slots per chunk
-  u32* digits;      // [kPasses][kBins] digit counts over all pairs, then [1] the nonbinary flag
+  u32* info;        // [0] pairs, [1] or of the keys, [2] or of their complements, [3] set when a live flag is
+                    // neither 0 nor 1 (the gather then copies the flags)
+  u32* digits;      // = info + 4: [kPasses][kBins] digit counts over all pairs
   int32_t* fields;  // [n_pad * Fp]: the next fields array
   int32_t* active;  // [n_pad]: the next live-flag array
 };
@@ -51,7 +53,7 @@ void sort_scratch_free(SortScratch* p) {
   }
   cudaFree(p->hist);
   cudaFree(p->counts);
-  cudaFree(p->digits);
+  cudaFree(p->info);
   cudaFree(p->fields);
   cudaFree(p->active);
   delete p;
@@ -74,8 +76,7 @@ __device__ __forceinline__ u32 block_total(u32 v, u32* s) {
   return t;
 }
 
-// live slots per chunk; also empties the digit counts and notes flags other
-// than 0 and 1 (the gather then copies the flags)
+// live slots per chunk; also notes flags other than 0 and 1
 __global__ void __launch_bounds__(kSortThreads) k_sort_count(SlabDev s, SortScratch p) {
   __shared__ u32 s_red[kSortWarps];
   const int chunk = chunk_of(s.cap, gridDim.x);
@@ -91,7 +92,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_count(SlabDev s, SortScra
   }
   const u32 t = block_total(n, s_red);
   if (threadIdx.x == 0) p.counts[blockIdx.x] = t;
-  if (other) p.digits[kPasses * kBins] = 1u;  // (emptied by the memset before this launch)
+  if (other) p.info[3] = 1u;  // (emptied by the memset before this launch)
 }
 
 // live slots before this chunk, and in all, in every thread
@@ -111,16 +112,18 @@ __device__ __forceinline__ void live_prefix(const SortScratch& p, u32& before, u
 // tile are strided loads of one sector each, 16 in flight per thread.
 __global__ void __launch_bounds__(kSortThreads, kSortCtasPerSm) k_sort_pack(SlabDev s, SortScratch p, int field) {
   __shared__ u32 s_red[kSortWarps];
-  __shared__ u32 s_hist[kPasses][kBins];
   __shared__ u32 s_wcnt[kSortWarps];
+  __shared__ u32 s_bits[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int b = 0; b < kPasses; ++b) s_hist[b][threadIdx.x] = 0u;
+  if (threadIdx.x < 2) s_bits[threadIdx.x] = 0u;
   griddep_wait();
   u32 before, total;
   live_prefix(p, before, total, s_red);
+  if (blockIdx.x == 0 && threadIdx.x == 0) p.info[0] = total;
   const int chunk = chunk_of(s.cap, gridDim.x);
   const long long lo = (long long)blockIdx.x * chunk;
   const u32 lt = (1u << lane) - 1u;
+  u32 ones = 0, zeros = 0;
   for (long long t0 = lo; t0 < lo + chunk && t0 < s.cap; t0 += kSortTile) {
     const int w0 = (int)t0 + warp * kWarpItems;
     u32 live[kSortItems], key[kSortItems];
@@ -132,7 +135,12 @@ __global__ void __launch_bounds__(kSortThreads, kSortCtasPerSm) k_sort_pack(Slab
 #pragma unroll
     for (int j = 0; j < kSortItems; ++j) {
       const int i = w0 + 32 * j + lane;
-      key[j] = live[j] ? (u32)s.fields[(size_t)i * s.Fp + field] ^ 0x80000000u : 0u;
+      key[j] = 0u;
+      if (live[j]) {
+        key[j] = (u32)s.fields[(size_t)i * s.Fp + field] ^ 0x80000000u;
+        ones |= key[j];
+        zeros |= ~key[j];
+      }
     }
     u32 n = 0;
 #pragma unroll
@@ -153,38 +161,28 @@ __global__ void __launch_bounds__(kSortThreads, kSortCtasPerSm) k_sort_pack(Slab
     for (int j = 0; j < kSortItems; ++j) {
       const int i = w0 + 32 * j + lane;
       const u32 r = rank + __popc(live[j] & lt);
-      const bool on = (live[j] >> lane) & 1u;
-      if (on) {
+      if ((live[j] >> lane) & 1u) {
         p.key[0][r] = key[j];
         p.val[0][r] = (u32)i;
       } else if (i < s.cap) {
         p.val[0][s.cap - 1 - (i - (int)r)] = (u32)i;
       }
       rank += __popc(live[j]);
-      // digit counts; a byte that is the same in the whole warp costs one atomic
-      if (live[j]) {
-        const int first = __ffs(live[j]) - 1;
-#pragma unroll
-        for (int b = 0; b < kPasses; ++b) {
-          const u32 d = (key[j] >> (8 * b)) & 0xFFu;
-          const u32 d0 = __shfl_sync(0xFFFFFFFFu, d, first);
-          if (__all_sync(0xFFFFFFFFu, !on || d == d0)) {
-            if (lane == first) atomicAdd(&s_hist[b][d0], (u32)__popc(live[j]));
-          } else if (on) {
-            atomicAdd(&s_hist[b][d], 1u);
-          }
-        }
-      }
     }
   }
+  ones = __reduce_or_sync(0xFFFFFFFFu, ones);
+  zeros = __reduce_or_sync(0xFFFFFFFFu, zeros);
+  if (lane == 0) {
+    atomicOr(&s_bits[0], ones);
+    atomicOr(&s_bits[1], zeros);
+  }
   __syncthreads();
-  for (int b = 0; b < kPasses; ++b)
-    if (s_hist[b][threadIdx.x]) atomicAdd(&p.digits[b * kBins + threadIdx.x], s_hist[b][threadIdx.x]);
+  if (threadIdx.x < 2) atomicOr(&p.info[1 + threadIdx.x], s_bits[threadIdx.x]);
 }
 
-// What a pass has to know, from the digit counts (every thread of a block of
-// kSortThreads): the number of pairs, whether the pass's byte varies, which of
-// the two buffers holds the pairs before it, and whether a later byte varies.
+// What a pass has to know: the number of pairs, whether the pass's byte varies,
+// which of the two buffers holds the pairs before it, and whether a later byte
+// varies.
 struct PassInfo {
   int n;
   bool run, last;
@@ -193,29 +191,37 @@ struct PassInfo {
   __device__ __forceinline__ u32* out(u32* const (&b)[2]) const { return odd ? b[0] : b[1]; }
 };
 
-__device__ __forceinline__ PassInfo pass_info(const SortScratch& p, int pass, u32* s_red) {
-  u32 c[kPasses];
-#pragma unroll
-  for (int b = 0; b < kPasses; ++b) c[b] = p.digits[b * kBins + threadIdx.x];
-  PassInfo f;
-  f.n = (int)block_total(c[0], s_red);
+__device__ __forceinline__ PassInfo pass_info(const SortScratch& p, int pass) {
+  const u32 diff = p.info[1] & p.info[2];
   u32 varies = 0;
 #pragma unroll
-  for (int b = 0; b < kPasses; ++b)
-    if (!__syncthreads_or(c[b] == (u32)f.n)) varies |= 1u << b;  // (also true of no pairs at all: nothing runs)
+  for (int b = 0; b < kPasses; ++b) varies |= ((diff >> (8 * b)) & 0xFFu) ? 1u << b : 0u;
+  PassInfo f;
+  f.n = (int)p.info[0];
   f.odd = __popc(varies & ((1u << pass) - 1u)) & 1;
   f.run = (varies >> pass) & 1u;
   f.last = (varies >> pass) == 1u;
   return f;
 }
 
+// lanes of the warp with the same digit d < 256 (ok lanes only): eight ballots, a
+// third of what a warp match of the digits takes
+__device__ __forceinline__ u32 digit_peers(u32 d, bool ok) {
+  u32 peers = __ballot_sync(0xFFFFFFFFu, ok);
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const u32 set = __ballot_sync(0xFFFFFFFFu, (d >> b) & 1u);
+    peers &= (d >> b) & 1u ? set : ~set;
+  }
+  return peers;
+}
+
 // a pass's digit counts per chunk
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(SortScratch p, int pass) {
   __shared__ u32 s_cnt[kBins];
-  __shared__ u32 s_red[kSortWarps];
   s_cnt[threadIdx.x] = 0u;
   griddep_wait();
-  const PassInfo f = pass_info(p, pass, s_red);
+  const PassInfo f = pass_info(p, pass);
   if (!f.run) return;
   const int chunk = chunk_of(f.n, gridDim.x);
   const long long lo = (long long)blockIdx.x * chunk;
@@ -235,18 +241,19 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_hist(SortScratch p, int p
     }
   }
   __syncthreads();
-  p.hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = s_cnt[threadIdx.x];
+  const u32 c = s_cnt[threadIdx.x];
+  p.hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = c;
+  if (c) atomicAdd(&p.digits[pass * kBins + threadIdx.x], c);
 }
 
 // digit counts per chunk -> positions: a digit's first position (a scan of the
 // digit counts, in every CTA) plus the counts of the chunks before; one warp
 // per digit
 __global__ void __launch_bounds__(kSortThreads) k_sort_scan(SortScratch p, int pass, int G) {
-  __shared__ u32 s_red[kSortWarps];
   __shared__ u64 s_warp[kSortWarps + 1];
   __shared__ u32 s_first[kBins];
   griddep_wait();
-  const PassInfo f = pass_info(p, pass, s_red);
+  const PassInfo f = pass_info(p, pass);
   if (!f.run) return;
   u32 ex, ex2, tot, tot2;
   block_scan2<kSortThreads>(p.digits[pass * kBins + threadIdx.x], 0u, ex, ex2, tot, tot2, s_warp);
@@ -281,8 +288,8 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scan(SortScratch p, int p
 }
 
 // Stable scatter of one pass, tile by tile of the CTA's chunk. Each warp ranks
-// its 512 consecutive pairs on its own (warp match; its digit counts in shared
-// memory), without block barriers; the warps' counts then give every pair its
+// its 512 consecutive pairs on its own (ballots of the digit's bits; its digit
+// counts in shared memory), without block barriers; the warps' counts then give every pair its
 // place in the tile's (digit, rank) order. The pairs are placed there in shared
 // memory and written out in that order, so that consecutive threads write
 // consecutive addresses of one digit's run.
@@ -291,10 +298,9 @@ __global__ void __launch_bounds__(kSortThreads, kSortCtasPerSm) k_sort_scatter(S
   __shared__ u32 s_wc[kSortWarps][kBins];  // per warp: pairs of each digit, then its first place in the tile order
   __shared__ u32 s_off[kBins];             // global position of a digit's place 0 of the tile order
   __shared__ u64 s_warp[kSortWarps + 1];
-  __shared__ u32 s_red[kSortWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   griddep_wait();
-  const PassInfo f = pass_info(p, pass, s_red);
+  const PassInfo f = pass_info(p, pass);
   if (!f.run) return;
   const u32 *key = f.in(p.key), *val = f.in(p.val);
   u32 *key_out = f.out(p.key), *val_out = f.out(p.val);
@@ -317,8 +323,8 @@ __global__ void __launch_bounds__(kSortThreads, kSortCtasPerSm) k_sort_scatter(S
 #pragma unroll
     for (int j = 0; j < kSortItems; ++j) {
       const bool ok = warp * kWarpItems + 32 * j + lane < n_tile;
-      const u32 d = ok ? (k[j] >> (8 * pass)) & 0xFFu : (u32)kBins;  // kBins: no pair
-      const u32 peers = __match_any_sync(0xFFFFFFFFu, d);
+      const u32 d = (k[j] >> (8 * pass)) & 0xFFu;
+      const u32 peers = digit_peers(d, ok);
       const u32 below = (u32)__popc(peers & lt);
       const u32 c = ok ? wc[d] : 0u;
       __syncwarp();
@@ -368,16 +374,139 @@ __global__ void __launch_bounds__(kSortThreads, kSortCtasPerSm) k_sort_scatter(S
   }
 }
 
+// Small sets: pack and sort in one CTA, pairs in shared memory, every pass with
+// the pairs in registers in between. Leaves the values in val[0] (as k_sort_pack
+// does) with no pass left to run, for the gather. (Seventeen launches of the
+// passes above take 78 us for 3000 slots.)
+constexpr int kOneThreads = 1024;
+constexpr int kOneWarps = kOneThreads / 32;
+constexpr int kOneMax = kOneThreads * kSortItems;
+constexpr size_t kOneSmem = (size_t)kOneMax * 8 + (size_t)kOneWarps * kBins * 4;
+
+__global__ void __launch_bounds__(kOneThreads, 1) k_sort_one(SlabDev s, SortScratch p, int field) {
+  extern __shared__ __align__(16) u32 s_one[];
+  u32 *s_key = s_one, *s_val = s_one + kOneMax, *s_wc = s_one + 2 * kOneMax;
+  __shared__ u64 s_warp[kOneWarps + 1];
+  __shared__ u32 s_bits[3];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const u32 lt = (1u << lane) - 1u;
+  const int w0 = warp * kWarpItems;
+  u32 k[kSortItems], v[kSortItems], rank[kSortItems / 2];
+  if (threadIdx.x < 3) s_bits[threadIdx.x] = 0u;
+  griddep_wait();
+  u32 ones = 0, zeros = 0, other = 0, mine = 0;
+#pragma unroll
+  for (int j = 0; j < kSortItems; ++j) {
+    const int i = w0 + 32 * j + lane;
+    v[j] = i < s.cap ? (u32)s.active[i] : 0u;
+  }
+#pragma unroll
+  for (int j = 0; j < kSortItems; ++j) {
+    const int i = w0 + 32 * j + lane;
+    k[j] = 0u;
+    if (v[j]) {
+      k[j] = (u32)s.fields[(size_t)i * s.Fp + field] ^ 0x80000000u;
+      ones |= k[j];
+      zeros |= ~k[j];
+    }
+    other |= v[j] & ~1u;
+    v[j] = __ballot_sync(0xFFFFFFFFu, v[j] != 0u);
+    mine += __popc(v[j]);
+  }
+  u32 at, at2, total, total2;
+  block_scan2<kOneThreads>(lane == 0 ? mine : 0u, 0u, at, at2, total, total2, s_warp);
+  at = __shfl_sync(0xFFFFFFFFu, at, 0);
+#pragma unroll
+  for (int j = 0; j < kSortItems; ++j) {
+    const int i = w0 + 32 * j + lane;
+    const u32 r = at + __popc(v[j] & lt);
+    if ((v[j] >> lane) & 1u) {
+      s_key[r] = k[j];
+      s_val[r] = (u32)i;
+    } else if (i < s.cap) {
+      p.val[0][s.cap - 1 - (i - (int)r)] = (u32)i;
+    }
+    at += __popc(v[j]);
+  }
+  ones = __reduce_or_sync(0xFFFFFFFFu, ones);
+  zeros = __reduce_or_sync(0xFFFFFFFFu, zeros);
+  other = __reduce_or_sync(0xFFFFFFFFu, other);
+  if (lane == 0) {
+    atomicOr(&s_bits[0], ones);
+    atomicOr(&s_bits[1], zeros);
+    atomicOr(&s_bits[2], other);
+  }
+  __syncthreads();
+  const u32 diff = s_bits[0] & s_bits[1];
+  const int n = (int)total;
+  u32* wc = s_wc + warp * kBins;
+  for (int sh = 0; sh < 32; sh += 8) {
+    if (!((diff >> sh) & 0xFFu)) continue;
+    for (int d = lane; d < kBins; d += 32) wc[d] = 0u;
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+      const int i = w0 + 32 * j + lane;
+      k[j] = i < n ? s_key[i] : 0u;
+      v[j] = i < n ? s_val[i] : 0u;
+    }
+    __syncwarp();
+    if (w0 < n) {
+#pragma unroll
+      for (int j = 0; j < kSortItems; ++j) {
+        const bool ok = w0 + 32 * j + lane < n;
+        const u32 d = (k[j] >> sh) & 0xFFu;
+        const u32 peers = digit_peers(d, ok);
+        const u32 below = (u32)__popc(peers & lt);
+        const u32 c = ok ? wc[d] : 0u;
+        __syncwarp();
+        if (ok && below == 0) wc[d] = c + (u32)__popc(peers);
+        __syncwarp();
+        if (j & 1) rank[j >> 1] |= (c + below) << 16;
+        else rank[j >> 1] = c + below;
+      }
+    }
+    __syncthreads();
+    // a digit's counts over the warps (four threads each, eight warps of counts a thread) -> first places
+    {
+      const int d = threadIdx.x >> 2, g = threadIdx.x & 3;
+      u32 c[kOneWarps / 4], sum = 0;
+#pragma unroll
+      for (int w = 0; w < kOneWarps / 4; ++w) {
+        c[w] = s_wc[(g * (kOneWarps / 4) + w) * kBins + d];
+        sum += c[w];
+      }
+      u32 ex, ex2, tot, tot2;
+      block_scan2<kOneThreads>(sum, 0u, ex, ex2, tot, tot2, s_warp);  // digit-major, warps ascending
+#pragma unroll
+      for (int w = 0; w < kOneWarps / 4; ++w) {
+        s_wc[(g * (kOneWarps / 4) + w) * kBins + d] = ex;
+        ex += c[w];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+      if (w0 + 32 * j + lane < n) {
+        const u32 to = wc[(k[j] >> sh) & 0xFFu] + ((rank[j >> 1] >> (16 * (j & 1))) & 0xFFFFu);
+        s_key[to] = k[j];
+        s_val[to] = v[j];
+      }
+    }
+    __syncthreads();
+  }
+  for (int i = threadIdx.x; i < n; i += kOneThreads) p.val[0][i] = s_val[i];
+  if (threadIdx.x < 4) p.info[threadIdx.x] = threadIdx.x == 0 ? total : (threadIdx.x == 3 ? s_bits[2] : 0u);
+}
+
 // Row i of the sorted slab <- its old row. A thread moves 16-byte quads of
 // rows, four in flight; the quads of one row go to neighbouring threads. Bound
 // by the random rows' DRAM bursts.
 __global__ void __launch_bounds__(kSortThreads) k_sort_gather(SlabDev s, SortScratch p, int32_t* perm_out) {
-  __shared__ u32 s_red[kSortWarps];
   griddep_wait();
   // after the last pass: the buffer that holds the pairs, and their number
-  const PassInfo f = pass_info(p, kPasses, s_red);
+  const PassInfo f = pass_info(p, kPasses);
   const u32* val = f.in(p.val);
-  const bool exact = p.digits[kPasses * kBins] != 0u;
+  const bool exact = p.info[3] != 0u;
   constexpr int U = 4;
   const u32 q = (u32)s.Fp >> 2, sh = q == 4 ? 2 : q - 1;  // 1 to 4 quads a row
   const u32 n = (u32)s.cap * q, T = gridDim.x * kSortThreads;
@@ -430,7 +559,8 @@ static abm_status sort_scratch(abm_slab* s, SortScratch** out) {
          cudaMalloc(&p->val[b], sizeof(u32) * (size_t)p->cap) == cudaSuccess;
   ok = ok && cudaMalloc(&p->hist, sizeof(u32) * (size_t)kBins * p->G) == cudaSuccess;
   ok = ok && cudaMalloc(&p->counts, sizeof(u32) * (size_t)p->G) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->digits, sizeof(u32) * (kPasses * kBins + 1)) == cudaSuccess;
+  ok = ok && cudaMalloc(&p->info, sizeof(u32) * (4 + kPasses * kBins)) == cudaSuccess;
+  p->digits = p->info + 4;
   ok = ok && cudaMalloc(&p->fields, sizeof(int32_t) * (size_t)p->n_pad * p->Fp) == cudaSuccess;
   ok = ok && cudaMalloc(&p->active, sizeof(int32_t) * (size_t)p->n_pad) == cudaSuccess;
   // rows past the capacity are never gathered: keep them as the slab keeps its own
@@ -460,14 +590,20 @@ extern "C" abm_status abm_sort(abm_slab* s, int32_t field, int32_t* out_perm, vo
   if (e != ABM_OK) return e;
   cudaStream_t st = (cudaStream_t)stream;
   const int G = p->G;
-  ABM_CUDA_TRY(cudaMemsetAsync(p->digits, 0, sizeof(u32) * (kPasses * kBins + 1), st));
-  k_sort_count<<<G, kSortThreads, 0, st>>>(s->d, *p);
-  ABM_LAUNCH_CHECK();
-  ABM_CUDA_TRY(launch_pdl(k_sort_pack, G, kSortThreads, st, s->d, *p, (int)field));
-  for (int pass = 0; pass < kPasses; ++pass) {
-    ABM_CUDA_TRY(launch_pdl(k_sort_hist, G, kSortThreads, st, *p, pass));
-    ABM_CUDA_TRY(launch_pdl(k_sort_scan, kBins / kSortWarps, kSortThreads, st, *p, pass, G));
-    ABM_CUDA_TRY(launch_pdl(k_sort_scatter, G, kSortThreads, st, *p, pass));
+  if (s->d.cap <= kOneMax) {
+    static std::atomic<unsigned long long> attr{0};
+    ABM_CUDA_TRY(smem_attr_once(k_sort_one, (int)kOneSmem, attr));
+    ABM_CUDA_TRY(launch_pdl_smem(k_sort_one, 1, kOneThreads, kOneSmem, st, s->d, *p, (int)field));
+  } else {
+    ABM_CUDA_TRY(cudaMemsetAsync(p->info, 0, sizeof(u32) * (4 + kPasses * kBins), st));
+    k_sort_count<<<G, kSortThreads, 0, st>>>(s->d, *p);
+    ABM_LAUNCH_CHECK();
+    ABM_CUDA_TRY(launch_pdl(k_sort_pack, G, kSortThreads, st, s->d, *p, (int)field));
+    for (int pass = 0; pass < kPasses; ++pass) {
+      ABM_CUDA_TRY(launch_pdl(k_sort_hist, G, kSortThreads, st, *p, pass));
+      ABM_CUDA_TRY(launch_pdl(k_sort_scan, kBins / kSortWarps, kSortThreads, st, *p, pass, G));
+      ABM_CUDA_TRY(launch_pdl(k_sort_scatter, G, kSortThreads, st, *p, pass));
+    }
   }
   const long long quads = (long long)s->d.cap * (s->d.Fp >> 2);
   const int grid = (int)std::min<long long>((quads + kSortThreads - 1) / kSortThreads, (long long)num_sms() * 8);

@@ -448,7 +448,7 @@ def test_argument_errors(eng):
     assert L.abm_select(s.h, C.byref(p), None, None, None) == abm.ERR_ARG
 
 
-@pytest.mark.parametrize("n,F", [(1, 1), (4095, 4), (4096, 9), (4097, 16), (8193, 5), (700_001, 2)])
+@pytest.mark.parametrize("n,F", [(1, 1), (33, 3), (4097, 16), (16_384, 4), (16_385, 9), (20_481, 5), (700_001, 2)])
 @pytest.mark.parametrize("keys", ["equal", "byte2", "signed", "all_bits", "none_live", "all_live"])
 def test_sort_agents_key_ranges(eng, n, F, keys):
     """Whole numbers, so exact: keys whose bytes are all alike (their passes are left out), in every position,
