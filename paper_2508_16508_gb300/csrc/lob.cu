@@ -48,7 +48,8 @@ constexpr int kWarpLevels = 256;        // level path: prices in [lowest ask, hi
 constexpr int kWarpMarginal = 64;       // level path: orders on one marginal level, at most
 constexpr u32 kShareBits = 21;          // level words: shares in the low 21 bits, orders above
 constexpr u32 kShareMask = (1u << kShareBits) - 1u;
-constexpr u32 kLive = 1u << 31, kAsk = 1u << 30;  // packed slot word: live | ask | qty
+constexpr int32_t kNoPrice = 0;         // level path: a dead slot's price in registers (prices start at 1): as a bid, far
+                                        // below every level
 
 
 // order-preserving map of int32 onto u32
@@ -220,16 +221,17 @@ __device__ __forceinline__ void grp_sync() {
   else __syncthreads();
 }
 
-// Three sums, a min, a max and an or over the G warps (every thread gets
-// them). One barrier; the exchange buffer alternates between calls.
-struct Agg6 {
-  u32 s0, s1, s2, mn, mx, orr;
+// Two sums, a signed min, a signed max and an or over the G warps (every thread
+// gets them). One barrier; the exchange buffer alternates between calls.
+struct Agg5 {
+  u32 s0, s1;
+  int32_t mn, mx;
+  u32 orr;
 };
 template <int G>
-__device__ __forceinline__ Agg6 grp_agg6(Agg6 a, u32 (*x)[G][8], int& par) {
+__device__ __forceinline__ Agg5 grp_agg5(Agg5 a, u32 (*x)[G][8], int& par) {
   a.s0 = __reduce_add_sync(0xFFFFFFFFu, a.s0);
   a.s1 = __reduce_add_sync(0xFFFFFFFFu, a.s1);
-  a.s2 = __reduce_add_sync(0xFFFFFFFFu, a.s2);
   a.mn = __reduce_min_sync(0xFFFFFFFFu, a.mn);
   a.mx = __reduce_max_sync(0xFFFFFFFFu, a.mx);
   a.orr = __reduce_or_sync(0xFFFFFFFFu, a.orr);
@@ -238,22 +240,20 @@ __device__ __forceinline__ Agg6 grp_agg6(Agg6 a, u32 (*x)[G][8], int& par) {
     u32* d = x[par][threadIdx.x >> 5];
     d[0] = a.s0;
     d[1] = a.s1;
-    d[2] = a.s2;
-    d[3] = a.mn;
-    d[4] = a.mx;
-    d[5] = a.orr;
+    d[2] = (u32)a.mn;
+    d[3] = (u32)a.mx;
+    d[4] = a.orr;
   }
   __syncthreads();
-  Agg6 r{0u, 0u, 0u, 0xFFFFFFFFu, 0u, 0u};
+  Agg5 r{0u, 0u, INT32_MAX, INT32_MIN, 0u};
 #pragma unroll
   for (int w = 0; w < G; ++w) {
     const u32* d = x[par][w];
     r.s0 += d[0];
     r.s1 += d[1];
-    r.s2 += d[2];
-    r.mn = min(r.mn, d[3]);
-    r.mx = max(r.mx, d[4]);
-    r.orr |= d[5];
+    r.mn = min(r.mn, (int32_t)d[2]);
+    r.mx = max(r.mx, (int32_t)d[3]);
+    r.orr |= d[4];
   }
   par ^= 1;
   return r;
@@ -347,10 +347,13 @@ __global__ void __launch_bounds__(G * 32)
     cp_async_wait_0();
     grp_sync<G>();
 
-    // this thread's slots into registers: price and live | ask | qty
+    // this thread's slots into registers: price (kNoPrice: dead) and qty | side
+    // in the sign bit. The loops over the slots are what a book costs (the kernel
+    // is bound by instruction issue), so each keeps to what it needs.
     int32_t px[SPL];
     u32 w[SPL];
-    u32 cnt = 0, mn = 0xFFFFFFFFu, mx = 0u, sb = 0, sa = 0, flags = 0;
+    int32_t mn = INT32_MAX, mx = INT32_MIN;  // lowest ask, highest bid
+    u32 qor = 0, zero = 0;
 #pragma unroll
     for (int g = 0; g < SPL / 4; ++g) {
       const int v = g * T + t;
@@ -364,36 +367,47 @@ __global__ void __launch_bounds__(G * 32)
       for (int c = 0; c < 4; ++c) {
         const int k = 4 * g + c;
         const bool live = av[c] != 0, ask = sv[c] != 0;
-        const bool lbid = live && !ask, lask = live && ask;
-        const u32 q = (u32)qv[c], qm = q & kShareMask;
-        flags |= (live && q > kShareMask) ? 1u : 0u;  // too large (or negative) for the level words
-        flags |= (live && q == 0) ? 2u : 0u;
-        px[k] = pv[c];
-        w[k] = live ? (kLive | (ask ? kAsk : 0u) | qm) : 0u;
-        cnt += lask ? 0x10000u : (lbid ? 1u : 0u);
-        sa += lask ? qm : 0u;
-        sb += lbid ? qm : 0u;
-        mn = min(mn, lask ? ord32(pv[c]) : 0xFFFFFFFFu);
-        mx = max(mx, lbid ? ord32(pv[c]) : 0u);
+        const u32 q = live ? (u32)qv[c] : 0u;
+        px[k] = live ? pv[c] : kNoPrice;
+        qor |= q;
+        zero += live && q == 0 ? 1u : 0u;
+        if (live && ask) mn = min(mn, pv[c]);
+        if (live && !ask) mx = max(mx, pv[c]);
+        w[k] = live && ask ? q | 0x80000000u : q;
       }
     }
-    // share sums saturate per thread, so the sums cannot wrap; for G > 1 the
-    // barrier inside also frees the staging arrays
-    const Agg6 r1 = grp_agg6<G>(Agg6{cnt, min(sb, 1u << kShareBits), min(sa, 1u << kShareBits), mn, mx, flags}, s_x,
-                                par);
+    // for G > 1 the barrier inside also frees the staging arrays
+    const Agg5 r1 = grp_agg5<G>(Agg5{zero, 0u, mn, mx, qor}, s_x, par);
     if (G == 1) __syncwarp();
     if (b + (int)gridDim.x < n_books)
       grp_stage<T, kVec16>(s_act, n, b + gridDim.x, cap, active, side, price, qty);
-    const bool zq = r1.orr & 2u;
-    const bool cross = (r1.s0 & 0xFFFFu) != 0 && (r1.s0 >> 16) != 0 && r1.mx >= r1.mn;
-    const int32_t pmin = (int32_t)(r1.mn ^ 0x80000000u), pmax = (int32_t)(r1.mx ^ 0x80000000u);
+    const bool zq = r1.s0 != 0;
+    const int32_t pmin = r1.mn, pmax = r1.mx;
+    // (without asks or without bids the test can hold for one extreme price: no volume comes of it)
+    const bool cross = pmax >= pmin;
     const long long L = cross ? (long long)pmax - (long long)pmin + 1 : 0;
-    if (cross && ((r1.orr & 1u) || r1.s1 > kShareMask || r1.s2 > kShareMask || L > kWarpLevels)) {
-      if (t == 0) out_volume[b] = -1;  // the sort path takes it
-      continue;
+    if (cross) {
+      // a level word holds share sums below 2^kShareBits: certainly if every qty could be the or of them all, else by
+      // the sums themselves (saturating per thread, so that they cannot wrap)
+      bool wide = L > kWarpLevels || r1.orr > kShareMask;
+      if (!wide && (u64)r1.orr * (u32)cap > kShareMask) {
+        u32 sb = 0, sa = 0;
+#pragma unroll
+        for (int k = 0; k < SPL; ++k) {
+          const u32 q = w[k] & kShareMask;
+          if ((int32_t)w[k] < 0) sa += q;
+          else sb += q;
+        }
+        const Agg5 r2 = grp_agg5<G>(Agg5{min(sb, 1u << kShareBits), min(sa, 1u << kShareBits), 0, 0, 0u}, s_x, par);
+        wide = r2.s0 > kShareMask || r2.s1 > kShareMask;
+      }
+      if (wide) {
+        if (t == 0) out_volume[b] = -1;  // the sort path takes it
+        continue;
+      }
     }
     u32 V = 0;
-    int32_t pb = 0, pa = 0;
+    int lb = 0, la = 0;  // the marginal levels
     u32 Dn = 0, Sp = 0;
     if (cross) {
       for (int l = t; l < L; l += T) {
@@ -401,11 +415,12 @@ __global__ void __launch_bounds__(G * 32)
         lva[l] = 0u;
       }
       grp_sync<G>();
+      // live asks lie at or above pmin and live bids at or below pmax, so one
+      // unsigned comparison tells an order in the range from the others and the dead
 #pragma unroll
       for (int k = 0; k < SPL; ++k) {
-        const bool ask = w[k] & kAsk;
-        const bool in = (w[k] & kLive) && (ask ? px[k] <= pmax : px[k] >= pmin);
-        if (in) atomicAdd((ask ? lva : lvb) + (px[k] - pmin), (w[k] & kShareMask) | (1u << kShareBits));
+        const u32 l = (u32)px[k] - (u32)pmin;
+        if (l < (u32)L) atomicAdd(lvb + (kWarpLevels & (u32)((int32_t)w[k] >> 31)) + l, (w[k] & kShareMask) | (1u << kShareBits));
       }
       grp_sync<G>();
       // D(l) = bid shares at levels >= l, S(l) = ask shares at levels <= l;
@@ -440,7 +455,7 @@ __global__ void __launch_bounds__(G * 32)
           lva[l0 + j] = Sl[j] | (ha[j] & ~kShareMask);
         }
       }
-      V = grp_agg6<G>(Agg6{0u, 0u, 0u, 0xFFFFFFFFu, best, 0u}, s_x, par).mx;
+      V = (u32)grp_agg5<G>(Agg5{0u, 0u, 0, (int32_t)best, 0u}, s_x, par).mx;  // (below 2^kShareBits)
       if (V > 0) {
         // D falls and S rises with the level: count the levels at or above V
         u32 cb = 0, ca = 0;
@@ -449,15 +464,14 @@ __global__ void __launch_bounds__(G * 32)
           cb += (l0 + j < L) && Dl[j] >= V;
           ca += (l0 + j < L) && Sl[j] >= V;
         }
-        const Agg6 r3 = grp_agg6<G>(Agg6{cb, ca, 0u, 0xFFFFFFFFu, 0u, 0u}, s_x, par);
-        const int lb = (int)r3.s0 - 1, la = (int)L - (int)r3.s1;
+        const Agg5 r3 = grp_agg5<G>(Agg5{cb, ca, 0, 0, 0u}, s_x, par);
+        lb = (int)r3.s0 - 1;
+        la = (int)L - (int)r3.s1;
         grp_sync<G>();
         if ((lvb[lb] >> kShareBits) > kWarpMarginal || (lva[la] >> kShareBits) > kWarpMarginal) {
           if (t == 0) out_volume[b] = -1;  // a crowded marginal level: the sort path takes it
           continue;
         }
-        pb = pmin + lb;
-        pa = pmin + la;
         Dn = lb + 1 < L ? lvb[lb + 1] & kShareMask : 0u;  // bid shares priced above pb
         Sp = la > 0 ? lva[la - 1] & kShareMask : 0u;      // ask shares priced below pa
       }
@@ -473,19 +487,36 @@ __global__ void __launch_bounds__(G * 32)
     // in per-thread bit masks (bit k = this thread's slot k), listed below
     using Mask = typename std::conditional<(SPL > 32), u64, u32>::type;
     Mask mmb = 0, mma = 0;
+    if (V > 0) {
+      // d = levels past the marginal one minus 1: bids l - lb - 1, asks la - l - 1.
+      // Whole fills have d in [0, L), the marginal orders d = -1; the others and the
+      // dead (level -pmin as unsigned) are far outside.
+      const u32 cb = 0u - (u32)lb - 1u, ca = (u32)la;
 #pragma unroll
-    for (int k = 0; k < SPL; ++k) {
-      const int i = 4 * ((k >> 2) * T + t) + (k & 3);
-      const bool live = w[k] & kLive, ask = w[k] & kAsk;
-      const u32 q = w[k] & kShareMask;
-      const bool whole = live && (q == 0 || (V > 0 && (ask ? px[k] < pa : px[k] > pb)));
-      const bool marg = live && q > 0 && V > 0 && px[k] == (ask ? pa : pb);
-      if (whole) {
-        qty[o + i] = 0;
-        active[o + i] = 0;
+      for (int k = 0; k < SPL; ++k) {
+        const int i = 4 * ((k >> 2) * T + t) + (k & 3);
+        const u32 ask = (u32)((int32_t)w[k] >> 31);  // all ones
+        const u32 d = (((u32)px[k] - (u32)pmin) ^ ask) + (ask ? ca : cb);
+        if (d < (u32)L) {
+          qty[o + i] = 0;
+          active[o + i] = 0;
+        }
+        if (d == 0xFFFFFFFFu) {
+          if (ask) mma |= (Mask)1 << k;
+          else mmb |= (Mask)1 << k;
+        }
       }
-      mmb |= (Mask)(marg && !ask) << k;
-      mma |= (Mask)(marg && ask) << k;
+    }
+    if (zq) {  // live orders without shares leave the book, whatever their price
+#pragma unroll
+      for (int k = 0; k < SPL; ++k) {
+        const int i = 4 * ((k >> 2) * T + t) + (k & 3);
+        if (px[k] != kNoPrice && (w[k] & 0x7FFFFFFFu) == 0) {
+          active[o + i] = 0;
+          mmb &= ~((Mask)1 << k);
+          mma &= ~((Mask)1 << k);
+        }
+      }
     }
     if (V > 0) {
       // list positions: scan of the per-thread counts; qty and time of the
@@ -525,7 +556,7 @@ __global__ void __launch_bounds__(G * 32)
     }
     if (t == 0) {
       out_volume[b] = (long long)V;
-      out_price[b] = V > 0 ? pa : -1;
+      out_price[b] = V > 0 ? pmin + la : -1;
     }
   }
   cp_async_wait_0();
