@@ -181,7 +181,7 @@ abm_status abm_sort(abm_slab* s, int32_t field, int32_t* out_perm, void* stream)
 #define ABM_LOB_MAX_CAP 2048
 /* Launch shape of abm_lob_match's price-level path for the rest of the
  * process: warps matching one book (1, 2 or 4; 0 = the default: 1 for books of
- * up to 256 slots, else 2). Results
+ * up to 256 slots, 2 up to 1024, else 4). Results
  * never depend on it. ABM_ERR_ARG for other values. Host only. */
 abm_status abm_lob_tune(int32_t warps_per_book);
 abm_status abm_lob_match(int32_t n_books, int32_t cap, int32_t* active, const int32_t* side, const int32_t* price,

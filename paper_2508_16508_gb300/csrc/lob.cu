@@ -747,11 +747,11 @@ static abm_status lob_launch(bool vec16, int n_books, int cap, int32_t* active, 
                              cudaStream_t st) {
   abm_status e;
   int g = g_lob_warps_per_book.load(std::memory_order_relaxed);
-  // One warp matches a book of up to 256 slots (8 per lane) faster than two
-  // that meet at a barrier after every step: 40,000 books of 128 slots 61 us
-  // against 107, of 256 slots 89 against 107; above, a lane's 16 and more slots
-  // make its chain too long (768 slots: 422 against 255).
-  if (g == 0) g = cap <= 256 ? 1 : 2;
+  // One warp matches a book of up to 256 slots (8 per lane) faster than two that
+  // meet at a barrier after every step (20,000 books of 128 slots 25 us against 43,
+  // of 256 slots 31 against 41; 768 slots 114 against 90), and four share more than
+  // 1024 slots better than two (2048 slots 207 against 230; 1024 slots 106 against 105).
+  if (g == 0) g = cap <= 256 ? 1 : (cap <= 1024 ? 2 : 4);
   switch (g) {
     case 1:
       e = vec16 ? lob_launch_g<1, true>(n_books, cap, active, side, price, qty, time, vol, px, st)
