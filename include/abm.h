@@ -522,7 +522,10 @@ abm_status abm_batch_create(const abm_batch_model* models, int32_t n, void* stre
 abm_status abm_batch_destroy(abm_batch* b);
 /* Launch shape: CTA size (128..1024), CTAs per SM, and steps per launch
  * (a run of nsteps is split into ceil(nsteps / steps_per_launch) launches,
- * each replayable in a CUDA graph). Results never depend on it. */
+ * each replayable in a CUDA graph). Results never depend on it. Until this or
+ * one of the next two calls is made, the library chooses a shape by the number
+ * and size of the models; then what was not set is 256 threads, 4 CTAs per SM,
+ * one model per CTA and 16 slots per thread. */
 abm_status abm_batch_tune(abm_batch* b, int32_t threads, int32_t ctas_per_sm, int32_t steps_per_launch);
 /* Launch shape: models run at once by one CTA (1, 2 or 4), each on a group of
  * threads / models_per_cta threads with its own barrier, so that small models

@@ -12,6 +12,7 @@
 // up. A CTA never waits for another CTA.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstring>
 #include <new>
 #include <numeric>
@@ -603,7 +604,7 @@ __global__ void __launch_bounds__(256) k_batch_digest(BatchDev b, u64* out) {
     const int4* ag = b.agent[sp] + m.oa[sp];
     const int ext = k.extent[sp];
 #pragma unroll 2
-    for (int i = 4 * (int)threadIdx.x; i < ext; i += 4 * (int)blockDim.x) {
+    for (int i = 4 * (int)threadIdx.x; i < ext; i += 4 * 256) {
       const int4 f = *reinterpret_cast<const int4*>(act + i);
       const int fv[4] = {f.x, f.y, f.z, f.w};
       int4 a[4];
@@ -618,8 +619,8 @@ __global__ void __launch_bounds__(256) k_batch_digest(BatchDev b, u64* out) {
     }
   }
   const int32_t* grass = b.regrow + m.oc;
-#pragma unroll 4
-  for (int c = threadIdx.x; c < m.ncells; c += blockDim.x) h += digest_cell(c, grass[c], k.step);
+#pragma unroll 8
+  for (int c = threadIdx.x; c < m.ncells; c += 256) h += digest_cell(c, grass[c], k.step);
   for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xFFFFFFFFu, h, o);
   if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = h;
   __syncthreads();
@@ -641,6 +642,8 @@ struct abm_batch {
   std::vector<BModel> models;
   long long slots[2], cells;
   int threads, ctas_per_sm, steps_per_launch, models_per_cta, agents_per_thread;
+  bool shape_set;             // the caller chose a launch shape (else batch_default_shape does)
+  long long size_max[2], size_sum[2];  // by sweep: the largest model's size and their sum (batch_default_shape)
   // fixed-capacity rerun of the models whose slabs overflowed (abm_batch_rerun_overflowed)
   abm_batch* rerun;
   std::vector<int> rerun_of;  // per model: its index in `rerun`, or -1
@@ -719,6 +722,13 @@ extern "C" abm_status abm_batch_create(const abm_batch_model* models, int32_t n,
   b->slots[0] = oa[0];
   b->slots[1] = oa[1];
   b->cells = oc;
+  for (const BModel& m : b->models) {
+    const long long sz[2] = {((long long)m.cap[0] + m.cap[1] + 7) / 8, m.ncells};
+    for (int k = 0; k < 2; ++k) {
+      b->size_max[k] = std::max(b->size_max[k], sz[k]);
+      b->size_sum[k] += sz[k];
+    }
+  }
   BatchDev& d = b->d;
   d.nmodels = n;
   bool ok = true;
@@ -770,6 +780,7 @@ extern "C" abm_status abm_batch_create(const abm_batch_model* models, int32_t n,
   b->steps_per_launch = 1 << 30;
   b->models_per_cta = 1;
   b->agents_per_thread = 16;
+  b->shape_set = false;
   *out = b;
   return ABM_OK;
 }
@@ -778,6 +789,7 @@ extern "C" abm_status abm_batch_tune(abm_batch* b, int32_t threads, int32_t ctas
   if (!b || (threads != 128 && threads != 256 && threads != 512 && threads != 1024) || ctas_per_sm < 1 ||
       threads * ctas_per_sm > 2048 || steps_per_launch < 1)
     return ABM_ERR_ARG;
+  b->shape_set = true;
   b->threads = threads;
   b->ctas_per_sm = ctas_per_sm;
   b->steps_per_launch = steps_per_launch;
@@ -825,9 +837,10 @@ static abm_status batch_launch(const BatchDev& d, int grid, int nsteps, int ext,
 // thread (32 slots only up to 512 threads: a chunk's list must fit the CTA's
 // static shared memory)
 template <int A>
-static abm_status batch_shape(const abm_batch* b, int grid, int s, int ext, int live_words, cudaStream_t st) {
+static abm_status batch_shape(const abm_batch* b, int threads, int models_per_cta, int grid, int s, int ext, int live_words,
+                              cudaStream_t st) {
   if constexpr (A == 32) {
-    switch (b->threads * 10 + b->models_per_cta) {
+    switch (threads * 10 + models_per_cta) {
       case 1281: return batch_launch<128, 1, A>(b->d, grid, s, ext, live_words, st);
       case 2561: return batch_launch<256, 1, A>(b->d, grid, s, ext, live_words, st);
       case 2562: return batch_launch<256, 2, A>(b->d, grid, s, ext, live_words, st);
@@ -837,7 +850,7 @@ static abm_status batch_shape(const abm_batch* b, int grid, int s, int ext, int 
       default: return ABM_ERR_ARG;
     }
   } else {
-    switch (b->threads * 10 + b->models_per_cta) {
+    switch (threads * 10 + models_per_cta) {
       case 1281: return batch_launch<128, 1, A>(b->d, grid, s, ext, live_words, st);
       case 2561: return batch_launch<256, 1, A>(b->d, grid, s, ext, live_words, st);
       case 2562: return batch_launch<256, 2, A>(b->d, grid, s, ext, live_words, st);
@@ -851,9 +864,40 @@ static abm_status batch_shape(const abm_batch* b, int grid, int s, int ext, int 
   }
 }
 
+// The launch shape of a batch whose caller chose none. r = the batch's size in
+// largest models per SM: with few of them a step's time is the largest models'
+// chain, which more threads shorten; with many, small CTAs keep more models in
+// flight. Sizes are cells (extent sweeps) or an eighth of the slots (capacity
+// sweeps; equal at the usual 4 side^2 a species). A run's first 40 steps, with
+// agents on every cell, cost up to ten times its later ones and gain more from
+// large CTAs (4096 models of sides 16..256, us a step at steps 0..9 and after
+// 120: 256 threads x 4 CTAs per SM x 16 slots 5405 and 559, x 32 slots 7626 and
+// 638, 512 x 2 x 32 4304 and 546, 1024 x 1 x 16 3626 and 695), so the lines are
+// drawn for both. Steps 0..9 and after 120, against 256 x 4 x 16 throughout:
+//   capacity  600 of 16..256 (r 1.4) 644 and 104 (1785 and 188), 1500 of 16..256
+//   1610 and 198 (2592 and 272), 300 of 64..128 116 and 31 (303 and 36), 1500 of
+//   64..128 487 and 89 (583 and 92)
+//   extent    600 of 16..256 546 and 33 (1550 and 50), 4096 of 16..256 3699 and
+//   133 (4983 and 130), 300 of 64..128 148 and 14 (237 and 15; 1024 threads 87
+//   and 18)
+struct BatchShape {
+  int threads, ctas_per_sm, models_per_cta, agents_per_thread;
+};
+static BatchShape batch_default_shape(const abm_batch* b, int ext) {
+  const double big = (double)std::max<long long>(1, b->size_max[ext]);
+  const double r = (double)b->size_sum[ext] / (big * num_sms());
+  if (big <= 64 * 64) return r <= 1.5 ? BatchShape{512, 2, 1, 16} : BatchShape{256, 4, 1, 16};
+  const double x = std::sqrt(big / (128.0 * 128.0));  // side of the largest model / 128
+  if (r <= 1.4 * std::sqrt(x) && !(ext && x < 1.5)) return BatchShape{1024, 1, 1, 16};
+  if (r <= (ext ? 4.0 * std::pow(x, 1.6) : 12.0 * x))
+    return BatchShape{512, 2, 1, ext && (x < 1.5 || r > 4.0) ? 16 : 32};
+  return BatchShape{256, 4, 1, 16};
+}
+
 extern "C" abm_status abm_batch_agents_per_thread(abm_batch* b, int32_t agents_per_thread) {
   if (!b || (agents_per_thread != 8 && agents_per_thread != 16 && agents_per_thread != 32)) return ABM_ERR_ARG;
   if (agents_per_thread == 32 && b->threads > 512) return ABM_ERR_ARG;
+  b->shape_set = true;
   b->agents_per_thread = agents_per_thread;
   return ABM_OK;
 }
@@ -862,6 +906,7 @@ extern "C" abm_status abm_batch_models_per_cta(abm_batch* b, int32_t models_per_
   if (!b || (models_per_cta != 1 && models_per_cta != 2 && models_per_cta != 4)) return ABM_ERR_ARG;
   // groups of at least 128 threads (the launch shapes instantiated)
   if (b->threads / models_per_cta < 128) return ABM_ERR_ARG;
+  b->shape_set = true;
   b->models_per_cta = models_per_cta;
   return ABM_OK;
 }
@@ -869,20 +914,23 @@ extern "C" abm_status abm_batch_models_per_cta(abm_batch* b, int32_t models_per_
 extern "C" abm_status abm_batch_run(abm_batch* b, int32_t nsteps, int32_t sweep, void* stream) {
   if (!b || nsteps < 0 || (sweep != ABM_SWEEP_CAPACITY && sweep != ABM_SWEEP_EXTENT)) return ABM_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  const int grid = std::max(1, std::min(b->d.nmodels, num_sms() * b->ctas_per_sm));
   const int ext = sweep == ABM_SWEEP_EXTENT;
+  const BatchShape sh = b->shape_set ? BatchShape{b->threads, b->ctas_per_sm, b->models_per_cta, b->agents_per_thread}
+                                     : batch_default_shape(b, ext);
+  const int grid = std::max(1, std::min(b->d.nmodels, num_sms() * sh.ctas_per_sm));
   // the live-flag bitmask of the largest sweep of the batch, per model run at
   // once (at most 1Mi slots per CTA, and as much as the CTA's shared memory
   // allows; larger models read their flags twice)
-  const int G = b->models_per_cta;
+  const int G = sh.models_per_cta;
   int live_words = 0;
   for (const BModel& m : b->models) live_words = std::max(live_words, (std::max(m.cap[0], m.cap[1]) + 31) / 32);
   live_words = std::min(live_words, kBatchLiveWordsMax / G);
   for (int done = 0; done < nsteps;) {
     const int s = std::min(nsteps - done, b->steps_per_launch);
-    const abm_status e = b->agents_per_thread == 8    ? batch_shape<8>(b, grid, s, ext, live_words, st)
-                         : b->agents_per_thread == 32 ? batch_shape<32>(b, grid, s, ext, live_words, st)
-                                                      : batch_shape<16>(b, grid, s, ext, live_words, st);
+    const abm_status e =
+        sh.agents_per_thread == 8    ? batch_shape<8>(b, sh.threads, G, grid, s, ext, live_words, st)
+        : sh.agents_per_thread == 32 ? batch_shape<32>(b, sh.threads, G, grid, s, ext, live_words, st)
+                                     : batch_shape<16>(b, sh.threads, G, grid, s, ext, live_words, st);
     if (e != ABM_OK) return e;
     ABM_LAUNCH_CHECK();
     done += s;
@@ -1037,6 +1085,7 @@ extern "C" abm_status abm_batch_rerun_overflowed(abm_batch* b, const int32_t* ca
   abm_batch* r = nullptr;
   abm_status e = abm_batch_create(rm.data(), (int32_t)rm.size(), stream, &r);
   if (e != ABM_OK) return e;
+  r->shape_set = b->shape_set;
   r->threads = b->threads;
   r->ctas_per_sm = b->ctas_per_sm;
   r->steps_per_launch = b->steps_per_launch;

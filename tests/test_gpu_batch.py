@@ -176,3 +176,20 @@ def test_batch_run_replays_from_a_cuda_graph(eng):
     torch.cuda.synchronize()
     assert torch.equal(a.digest(), b.digest())
     assert [c["step"] for c in b.counters()] == [30] * len(models)
+
+
+@pytest.mark.parametrize("sweep,n,side", [(0, 20, 64), (0, 300, 40), (0, 20, 70), (0, 400, 66), (1, 20, 64), (1, 300, 40),
+                                          (1, 20, 70), (1, 400, 66), (1, 20, 200), (1, 310, 200)])
+def test_default_launch_shapes_agree(eng, sweep, n, side):
+    """A batch that was given no launch shape (the library's own, by the number
+    and size of the models) against one that was."""
+    models = [dict(side=side - (m % 3), seed=side, model=m, params=workloads.predation_params(),
+                   cap=(4 * side * side - 5 * m, 2 * side * side - m), n0=(side * 9, side * 2)) for m in range(n)]
+    a, b = eng.Batch(models), eng.Batch(models)
+    b.tune(256, 4)
+    for steps in (3, 9):
+        a.run(steps, sweep=sweep)
+        b.run(steps, sweep=sweep)
+    assert torch.equal(a.digest(), b.digest())
+    assert a.counters() == b.counters()
+    a.check()
