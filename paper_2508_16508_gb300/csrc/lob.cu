@@ -221,48 +221,53 @@ __device__ __forceinline__ void grp_sync() {
   else __syncthreads();
 }
 
-// Two sums, a signed min, a signed max and an or over the G warps (every thread
-// gets them). One barrier; the exchange buffer alternates between calls.
-struct Agg5 {
-  u32 s0, s1;
+// Signed min and max, or, and "any" over the G warps (every thread gets them).
+// One barrier; the exchange buffer alternates between calls.
+struct Agg {
   int32_t mn, mx;
   u32 orr;
+  bool any;
 };
 template <int G>
-__device__ __forceinline__ Agg5 grp_agg5(Agg5 a, u32 (*x)[G][8], int& par) {
-  a.s0 = __reduce_add_sync(0xFFFFFFFFu, a.s0);
-  a.s1 = __reduce_add_sync(0xFFFFFFFFu, a.s1);
+__device__ __forceinline__ Agg grp_agg(Agg a, u32 (*x)[G][4], int& par) {
   a.mn = __reduce_min_sync(0xFFFFFFFFu, a.mn);
   a.mx = __reduce_max_sync(0xFFFFFFFFu, a.mx);
   a.orr = __reduce_or_sync(0xFFFFFFFFu, a.orr);
+  a.any = __any_sync(0xFFFFFFFFu, a.any);
   if (G == 1) return a;
-  if ((threadIdx.x & 31) == 0) {
-    u32* d = x[par][threadIdx.x >> 5];
-    d[0] = a.s0;
-    d[1] = a.s1;
-    d[2] = (u32)a.mn;
-    d[3] = (u32)a.mx;
-    d[4] = a.orr;
-  }
+  if ((threadIdx.x & 31) == 0)
+    *reinterpret_cast<uint4*>(x[par][threadIdx.x >> 5]) = make_uint4((u32)a.mn, (u32)a.mx, a.orr, a.any ? 1u : 0u);
   __syncthreads();
-  Agg5 r{0u, 0u, INT32_MAX, INT32_MIN, 0u};
+  Agg r{INT32_MAX, INT32_MIN, 0u, false};
 #pragma unroll
   for (int w = 0; w < G; ++w) {
-    const u32* d = x[par][w];
-    r.s0 += d[0];
-    r.s1 += d[1];
-    r.mn = min(r.mn, (int32_t)d[2]);
-    r.mx = max(r.mx, (int32_t)d[3]);
-    r.orr |= d[4];
+    const uint4 d = *reinterpret_cast<const uint4*>(x[par][w]);
+    r.mn = min(r.mn, (int32_t)d.x);
+    r.mx = max(r.mx, (int32_t)d.y);
+    r.orr |= d.z;
+    r.any = r.any || d.w != 0u;
   }
   par ^= 1;
   return r;
 }
 
+// Max of a u32 over the G warps (every thread gets it). One barrier.
+template <int G>
+__device__ __forceinline__ u32 grp_max(u32 v, u32 (*x)[G][4], int& par) {
+  v = __reduce_max_sync(0xFFFFFFFFu, v);
+  if (G == 1) return v;
+  if ((threadIdx.x & 31) == 0) x[par][threadIdx.x >> 5][0] = v;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < G; ++w) v = max(v, x[par][w][0]);
+  par ^= 1;
+  return v;
+}
+
 // Exclusive scan of two u32 over the G warps' threads, with the totals.
 template <int G>
 __device__ __forceinline__ void grp_scan2(u32 a, u32 b, u32& ex_a, u32& ex_b, u32& tot_a, u32& tot_b,
-                                          u32 (*x)[G][8], int& par) {
+                                          u32 (*x)[G][4], int& par) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u32 ia = warp_incl_scan(a, lane), ib = warp_incl_scan(b, lane);
   if (G == 1) {
@@ -331,11 +336,12 @@ __global__ void __launch_bounds__(G * 32)
   constexpr int LPT = kWarpLevels / T;  // levels per thread in the scan
   constexpr int n = T * SPL;            // staged words per array
   extern __shared__ __align__(16) unsigned char lob_smem[];
-  __shared__ u32 s_x[2][G][8];
+  __shared__ __align__(16) u32 s_x[2][G][4];
+  __shared__ u32 s_mar[2][3];  // per side: the marginal level, the shares of the better ones, its orders
+  __shared__ u32 s_cnt;        // marginal orders listed: bids | asks << 16
   int32_t* s_act = reinterpret_cast<int32_t*>(lob_smem);  // then side, price, qty at +n, +2n, +3n
-  u32* lvb = reinterpret_cast<u32*>(s_act + 4 * n);        // bid level words, then D | orders << 21
-  u32* lva = lvb + kWarpLevels;                            // ask level words, then S | orders << 21
-  u32* m_qty = lva + kWarpLevels;                          // [2][kWarpMarginal]
+  u32* lv = reinterpret_cast<u32*>(s_act + 4 * n);        // level words: bids, then asks
+  u32* m_qty = lv + 2 * kWarpLevels;                      // [2][kWarpMarginal]: slots, then quantities
   u64* m_key = reinterpret_cast<u64*>(m_qty + 2 * kWarpMarginal);  // [2][kWarpMarginal]
   const int t = threadIdx.x;
   int par = 0;
@@ -347,13 +353,19 @@ __global__ void __launch_bounds__(G * 32)
     cp_async_wait_0();
     grp_sync<G>();
 
-    // this thread's slots into registers: price (kNoPrice: dead) and qty | side
-    // in the sign bit. The loops over the slots are what a book costs (the kernel
-    // is bound by instruction issue), so each keeps to what it needs.
+    // the level words are free since that barrier; the next one comes before they are used
+#pragma unroll
+    for (int l = t; l < 2 * kWarpLevels / 4; l += T) reinterpret_cast<uint4*>(lv)[l] = make_uint4(0u, 0u, 0u, 0u);
+    if (t == 0) s_cnt = 0u;
+
+    // this thread's slots into registers: price (kNoPrice: dead) and qty | ask in
+    // the sign bit, dead slots as bids of one share (far below every level). The
+    // loops over the slots are most of a book's instructions, so each keeps to what
+    // it needs.
     int32_t px[SPL];
     u32 w[SPL];
     int32_t mn = INT32_MAX, mx = INT32_MIN;  // lowest ask, highest bid
-    u32 qor = 0, zero = 0;
+    u32 qor = 0, qmin = 1;
 #pragma unroll
     for (int g = 0; g < SPL / 4; ++g) {
       const int v = g * T + t;
@@ -366,22 +378,22 @@ __global__ void __launch_bounds__(G * 32)
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const int k = 4 * g + c;
-        const bool live = av[c] != 0, ask = sv[c] != 0;
-        const u32 q = live ? (u32)qv[c] : 0u;
+        const bool live = av[c] != 0, ask = live && sv[c] != 0;
+        const u32 q = live ? (u32)qv[c] : 1u;
         px[k] = live ? pv[c] : kNoPrice;
         qor |= q;
-        zero += live && q == 0 ? 1u : 0u;
-        if (live && ask) mn = min(mn, pv[c]);
-        if (live && !ask) mx = max(mx, pv[c]);
-        w[k] = live && ask ? q | 0x80000000u : q;
+        qmin = min(qmin, q);
+        if (ask) mn = min(mn, px[k]);
+        else mx = max(mx, px[k]);
+        w[k] = ask ? q | 0x80000000u : q;
       }
     }
     // for G > 1 the barrier inside also frees the staging arrays
-    const Agg5 r1 = grp_agg5<G>(Agg5{zero, 0u, mn, mx, qor}, s_x, par);
+    const Agg r1 = grp_agg<G>(Agg{mn, mx, qor, qmin == 0}, s_x, par);
     if (G == 1) __syncwarp();
     if (b + (int)gridDim.x < n_books)
       grp_stage<T, kVec16>(s_act, n, b + gridDim.x, cap, active, side, price, qty);
-    const bool zq = r1.s0 != 0;
+    const bool zq = r1.any;
     const int32_t pmin = r1.mn, pmax = r1.mx;
     // (without asks or without bids the test can hold for one extreme price: no volume comes of it)
     const bool cross = pmax >= pmin;
@@ -396,10 +408,11 @@ __global__ void __launch_bounds__(G * 32)
         for (int k = 0; k < SPL; ++k) {
           const u32 q = w[k] & kShareMask;
           if ((int32_t)w[k] < 0) sa += q;
-          else sb += q;
+          else sb += px[k] != kNoPrice ? q : 0u;
         }
-        const Agg5 r2 = grp_agg5<G>(Agg5{min(sb, 1u << kShareBits), min(sa, 1u << kShareBits), 0, 0, 0u}, s_x, par);
-        wide = r2.s0 > kShareMask || r2.s1 > kShareMask;
+        u32 ex_b, ex_a, tb, ta;
+        grp_scan2<G>(min(sb, 1u << kShareBits), min(sa, 1u << kShareBits), ex_b, ex_a, tb, ta, s_x, par);
+        wide = tb > kShareMask || ta > kShareMask;
       }
       if (wide) {
         if (t == 0) out_volume[b] = -1;  // the sort path takes it
@@ -408,72 +421,78 @@ __global__ void __launch_bounds__(G * 32)
     }
     u32 V = 0;
     int lb = 0, la = 0;  // the marginal levels
-    u32 Dn = 0, Sp = 0;
+    u32 Dn = 0, Sp = 0;  // bid shares priced above pb, ask shares priced below pa
     if (cross) {
-      for (int l = t; l < L; l += T) {
-        lvb[l] = 0u;
-        lva[l] = 0u;
-      }
-      grp_sync<G>();
       // live asks lie at or above pmin and live bids at or below pmax, so one
-      // unsigned comparison tells an order in the range from the others and the dead
+      // unsigned comparison tells an order in the range from the others and the
+      // dead. (Quantities below 2^kShareBits: w >> 23 is 256 for asks, 0 for bids.)
+      static_assert(kWarpLevels == 256 && kShareBits <= 23, "level word of an order");
 #pragma unroll
       for (int k = 0; k < SPL; ++k) {
         const u32 l = (u32)px[k] - (u32)pmin;
-        if (l < (u32)L) atomicAdd(lvb + (kWarpLevels & (u32)((int32_t)w[k] >> 31)) + l, (w[k] & kShareMask) | (1u << kShareBits));
+        if (l < (u32)L) atomicAdd(lv + (l + (w[k] >> 23)), (w[k] & kShareMask) | (1u << kShareBits));
       }
       grp_sync<G>();
       // D(l) = bid shares at levels >= l, S(l) = ask shares at levels <= l;
-      // thread t owns levels [LPT * t, LPT * t + LPT)
+      // thread t owns levels [LPT * t, LPT * t + LPT). Levels from L on hold no
+      // order: D = 0 there.
       u32 hb[LPT], ha[LPT];
       u32 tb = 0, ta = 0;
       const int l0 = t * LPT;
 #pragma unroll
+      for (int j = 0; j < LPT; j += 2) {
+        const uint2 vb = *reinterpret_cast<const uint2*>(lv + l0 + j);
+        const uint2 va = *reinterpret_cast<const uint2*>(lv + kWarpLevels + l0 + j);
+        hb[j] = vb.x;
+        hb[j + 1] = vb.y;
+        ha[j] = va.x;
+        ha[j + 1] = va.y;
+      }
+#pragma unroll
       for (int j = 0; j < LPT; ++j) {
-        hb[j] = l0 + j < L ? lvb[l0 + j] : 0u;
-        ha[j] = l0 + j < L ? lva[l0 + j] : 0u;
         tb += hb[j] & kShareMask;
         ta += ha[j] & kShareMask;
       }
       u32 pre_b, pre_a, BT, AT;
       grp_scan2<G>(tb, ta, pre_b, pre_a, BT, AT, s_x, par);
-      u32 best = 0;
-      u32 Dl[LPT], Sl[LPT];
+      u32 best = 0, D = BT - pre_b, S = pre_a;
 #pragma unroll
       for (int j = 0; j < LPT; ++j) {
-        Dl[j] = BT - pre_b;
-        pre_b += hb[j] & kShareMask;
-        pre_a += ha[j] & kShareMask;
-        Sl[j] = pre_a;
-        if (l0 + j < L) best = max(best, min(Dl[j], Sl[j]));
+        S += ha[j] & kShareMask;
+        best = max(best, min(D, S));
+        D -= hb[j] & kShareMask;
       }
-      if (G == 1) __syncwarp();  // (G > 1: the scan's barrier came after every read)
-#pragma unroll
-      for (int j = 0; j < LPT; ++j) {
-        if (l0 + j < L) {
-          lvb[l0 + j] = Dl[j] | (hb[j] & ~kShareMask);
-          lva[l0 + j] = Sl[j] | (ha[j] & ~kShareMask);
-        }
-      }
-      V = (u32)grp_agg5<G>(Agg5{0u, 0u, 0, (int32_t)best, 0u}, s_x, par).mx;  // (below 2^kShareBits)
+      V = grp_max<G>(best, s_x, par);
       if (V > 0) {
-        // D falls and S rises with the level: count the levels at or above V
-        u32 cb = 0, ca = 0;
+        // D falls and S rises with the level: the one bid level with D >= V and less
+        // above it, the one ask level with S >= V and less below it
+        D = BT - pre_b;
+        S = pre_a;
 #pragma unroll
         for (int j = 0; j < LPT; ++j) {
-          cb += (l0 + j < L) && Dl[j] >= V;
-          ca += (l0 + j < L) && Sl[j] >= V;
+          const u32 Dnext = D - (hb[j] & kShareMask), Snext = S + (ha[j] & kShareMask);
+          if (D >= V && Dnext < V) {
+            s_mar[0][0] = (u32)(l0 + j);
+            s_mar[0][1] = Dnext;
+            s_mar[0][2] = hb[j] >> kShareBits;
+          }
+          if (Snext >= V && S < V) {
+            s_mar[1][0] = (u32)(l0 + j);
+            s_mar[1][1] = S;
+            s_mar[1][2] = ha[j] >> kShareBits;
+          }
+          D = Dnext;
+          S = Snext;
         }
-        const Agg5 r3 = grp_agg5<G>(Agg5{cb, ca, 0, 0, 0u}, s_x, par);
-        lb = (int)r3.s0 - 1;
-        la = (int)L - (int)r3.s1;
         grp_sync<G>();
-        if ((lvb[lb] >> kShareBits) > kWarpMarginal || (lva[la] >> kShareBits) > kWarpMarginal) {
+        lb = (int)s_mar[0][0];
+        la = (int)s_mar[1][0];
+        Dn = s_mar[0][1];
+        Sp = s_mar[1][1];
+        if (max(s_mar[0][2], s_mar[1][2]) > kWarpMarginal) {
           if (t == 0) out_volume[b] = -1;  // a crowded marginal level: the sort path takes it
           continue;
         }
-        Dn = lb + 1 < L ? lvb[lb + 1] & kShareMask : 0u;  // bid shares priced above pb
-        Sp = la > 0 ? lva[la - 1] & kShareMask : 0u;      // ask shares priced below pa
       }
     }
     if (V == 0 && !zq) {
@@ -488,15 +507,14 @@ __global__ void __launch_bounds__(G * 32)
     using Mask = typename std::conditional<(SPL > 32), u64, u32>::type;
     Mask mmb = 0, mma = 0;
     if (V > 0) {
-      // d = levels past the marginal one minus 1: bids l - lb - 1, asks la - l - 1.
-      // Whole fills have d in [0, L), the marginal orders d = -1; the others and the
-      // dead (level -pmin as unsigned) are far outside.
-      const u32 cb = 0u - (u32)lb - 1u, ca = (u32)la;
+      // d = levels past the marginal one minus 1. Whole fills have d in [0, L), the
+      // marginal orders d = -1; the others and the dead (price 0) are far outside.
+      const u32 cb = (u32)pmin + (u32)lb + 1u, ca = (u32)pmin + (u32)la - 1u;
 #pragma unroll
       for (int k = 0; k < SPL; ++k) {
         const int i = 4 * ((k >> 2) * T + t) + (k & 3);
-        const u32 ask = (u32)((int32_t)w[k] >> 31);  // all ones
-        const u32 d = (((u32)px[k] - (u32)pmin) ^ ask) + (ask ? ca : cb);
+        const bool ask = (int32_t)w[k] < 0;
+        const u32 d = ask ? ca - (u32)px[k] : (u32)px[k] - cb;
         if (d < (u32)L) {
           qty[o + i] = 0;
           active[o + i] = 0;
@@ -511,7 +529,7 @@ __global__ void __launch_bounds__(G * 32)
 #pragma unroll
       for (int k = 0; k < SPL; ++k) {
         const int i = 4 * ((k >> 2) * T + t) + (k & 3);
-        if (px[k] != kNoPrice && (w[k] & 0x7FFFFFFFu) == 0) {
+        if ((w[k] & 0x7FFFFFFFu) == 0) {
           active[o + i] = 0;
           mmb &= ~((Mask)1 << k);
           mma &= ~((Mask)1 << k);
@@ -519,27 +537,32 @@ __global__ void __launch_bounds__(G * 32)
       }
     }
     if (V > 0) {
-      // list positions: scan of the per-thread counts; qty and time of the
-      // marginal orders from global memory (neither written by this kernel)
-      const u32 cb = (u32)popc_mask(mmb), ca = (u32)popc_mask(mma);
-      u32 eb, ea, nm0, nm1;
-      grp_scan2<G>(cb, ca, eb, ea, nm0, nm1, s_x, par);
+      // the marginal orders' slots listed in any order, then their qty and time from
+      // global memory (neither written by this kernel) in one round trip
+      if (mmb | mma) {
+        const u32 at = atomicAdd(&s_cnt, (u32)popc_mask(mmb) | ((u32)popc_mask(mma) << 16));
 #pragma unroll
-      for (int s = 0; s < 2; ++s) {
-        Mask m = s ? mma : mmb;
-        u32 pos = s ? ea : eb;
-        while (m) {
-          const int k = ffs_mask(m) - 1;
-          m &= m - 1;
-          const u32 i = 4u * (u32)((k >> 2) * T + t) + (u32)(k & 3);
-          m_qty[s * kWarpMarginal + pos] = (u32)qty[o + i];
-          m_key[s * kWarpMarginal + pos] = ((u64)ord32(time[o + i]) << 32) | i;
-          ++pos;
+        for (int s = 0; s < 2; ++s) {
+          Mask m = s ? mma : mmb;
+          u32* list = m_qty + (s ? kWarpMarginal + (at >> 16) : (at & 0xFFFFu));
+          while (m) {
+            const int k = ffs_mask(m) - 1;
+            m &= m - 1;
+            *list++ = 4u * (u32)((k >> 2) * T + t) + (u32)(k & 3);
+          }
         }
       }
       grp_sync<G>();
-      for (int e = t; e < (int)(nm0 + nm1); e += T) {
-        const int s = e >= (int)nm0, f = e - (s ? (int)nm0 : 0), m = s ? (int)nm1 : (int)nm0;
+      const u32 nm0 = s_cnt & 0xFFFFu, nm1 = s_cnt >> 16;
+      for (u32 e = t; e < nm0 + nm1; e += T) {
+        const u32 f = e < nm0 ? e : e - nm0 + kWarpMarginal, i = m_qty[f];
+        const u32 q = (u32)qty[o + i];
+        m_key[f] = ((u64)ord32(time[o + i]) << 32) | i;
+        m_qty[f] = q;
+      }
+      grp_sync<G>();
+      for (u32 e = t; e < nm0 + nm1; e += T) {
+        const int s = e >= nm0, f = (int)e - (s ? (int)nm0 : 0), m = s ? (int)nm1 : (int)nm0;
         const u32* mq = m_qty + s * kWarpMarginal;
         const u64* mk = m_key + s * kWarpMarginal;
         const u64 mine = mk[f];
