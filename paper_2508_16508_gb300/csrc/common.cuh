@@ -314,6 +314,13 @@ __device__ __forceinline__ void warp_add(int* dst, int v) {
 // griddep_wait() before touching anything the predecessor writes.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Lets the next launch in the stream, if it is a dependent one, start its CTAs
+// once every CTA of this grid has come here: they wait in griddep_wait() for
+// this grid's end, so that a launch's latency passes beside its predecessor. A
+// kernel that calls it must also wait for its own predecessor in every CTA: the
+// dependent's wait covers this grid only.
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl_smem(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};

@@ -347,6 +347,10 @@ __global__ void __launch_bounds__(G * 32)
   int par = 0;
   for (int i = cap + t; i < n; i += T) s_act[i] = 0;  // padding slots: never copied, never live
   griddep_wait();
+  // the sort path's few CTAs may start (and the next call's beside those: 100 steps
+  // of 500 books 761 -> 748 us). Not from k_lob_add: its successor's CTAs then
+  // crowd the SMs that are free at that moment (968 us).
+  griddep_launch();
   if ((int)blockIdx.x < n_books) grp_stage<T, kVec16>(s_act, n, blockIdx.x, cap, active, side, price, qty);
   for (int b = blockIdx.x; b < n_books; b += gridDim.x) {
     const size_t o = (size_t)b * cap;
@@ -604,6 +608,7 @@ __global__ void __launch_bounds__(kLobThreads)
   __shared__ u64 s_scan[kLobWarps + 1];
   __shared__ unsigned long long s_v;
   griddep_wait();
+  griddep_launch();
   for (int c0 = blockIdx.x * kLobThreads; c0 < n_books; c0 += gridDim.x * kLobThreads) {
     if (threadIdx.x == 0) s_cnt = 0;
     __syncthreads();
@@ -771,10 +776,15 @@ static abm_status lob_launch(bool vec16, int n_books, int cap, int32_t* active, 
   abm_status e;
   int g = g_lob_warps_per_book.load(std::memory_order_relaxed);
   // One warp matches a book of up to 256 slots (8 per lane) faster than two that
-  // meet at a barrier after every step (20,000 books of 128 slots 25 us against 43,
-  // of 256 slots 31 against 41; 768 slots 114 against 90), and four share more than
-  // 1024 slots better than two (2048 slots 207 against 230; 1024 slots 106 against 105).
-  if (g == 0) g = cap <= 256 ? 1 : (cap <= 1024 ? 2 : 4);
+  // meet at a barrier after every step (20,000 books of 128 slots 22 us against 35,
+  // of 256 slots 27 against 33; 768 slots 90 against 77), and four share more than
+  // 1024 slots better than two (2048 slots 187 against 196; 1024 slots the same).
+  // With few books a book's own chain counts, which more warps shorten: 100 steps of
+  // orders and matching, 500 books of 256 slots 645 us with two warps against 685,
+  // of 1000 slots 761 with four against 798; 2000 of 1000 1301 against 1366, 3000 the
+  // same; 500 of 128 569 with two against 561, 1000 of 500 815 with four against 796.
+  const bool few = n_books <= 2048;
+  if (g == 0) g = cap <= (few ? 128 : 256) ? 1 : (cap <= (few ? 512 : 1024) ? 2 : 4);
   switch (g) {
     case 1:
       e = vec16 ? lob_launch_g<1, true>(n_books, cap, active, side, price, qty, time, vol, px, st)
