@@ -777,14 +777,15 @@ static abm_status lob_launch(bool vec16, int n_books, int cap, int32_t* active, 
   int g = g_lob_warps_per_book.load(std::memory_order_relaxed);
   // One warp matches a book of up to 256 slots (8 per lane) faster than two that
   // meet at a barrier after every step (20,000 books of 128 slots 22 us against 35,
-  // of 256 slots 27 against 33; 768 slots 90 against 77), and four share more than
-  // 1024 slots better than two (2048 slots 187 against 196; 1024 slots the same).
+  // 50,000 of 256 slots 73 against 89; 20,000 of 512 57 against 56, of 768 93 against
+  // 82), and four share more than 768 slots better than two (65536 books of 1024
+  // slots 299 against 313, 16384 of 2048 158 against 169; 768 slots the same).
   // With few books a book's own chain counts, which more warps shorten: 100 steps of
   // orders and matching, 500 books of 256 slots 645 us with two warps against 685,
   // of 1000 slots 761 with four against 798; 2000 of 1000 1301 against 1366, 3000 the
   // same; 500 of 128 569 with two against 561, 1000 of 500 815 with four against 796.
   const bool few = n_books <= 2048;
-  if (g == 0) g = cap <= (few ? 128 : 256) ? 1 : (cap <= (few ? 512 : 1024) ? 2 : 4);
+  if (g == 0) g = cap <= (few ? 128 : 256) ? 1 : (cap <= (few ? 512 : 768) ? 2 : 4);
   switch (g) {
     case 1:
       e = vec16 ? lob_launch_g<1, true>(n_books, cap, active, side, price, qty, time, vol, px, st)

@@ -264,8 +264,8 @@ def test_market_graph_replay_equals_eager(eng):
             assert torch.equal(replay.t[f], eager.t[f]), f
 
 
-@pytest.mark.parametrize("n_books,cap", [(2048, 129), (2049, 129), (2049, 257), (2048, 512), (2048, 513), (2049, 513),
-                                         (2049, 1025)])
+@pytest.mark.parametrize("n_books,cap", [(2048, 129), (2049, 129), (2049, 257), (2048, 512), (2048, 513), (2049, 768),
+                                         (2049, 769)])
 def test_match_default_shapes(eng, n_books, cap):
     """Each side of the lines between the default numbers of warps per book."""
     assert (check_match(eng, workloads.random_books(n_books, cap, 0.6, seed=cap)) > 0).any()
