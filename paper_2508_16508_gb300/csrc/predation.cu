@@ -746,10 +746,142 @@ extern "C" abm_status abm_image_capacity(abm_world* w, size_t* bytes) {
   return ABM_OK;
 }
 
+// n words between device memory and pinned host memory by the CTAs of one grid
+// row, 16 bytes of the host's at a time.
+template <bool LOAD>
+__device__ __forceinline__ void row_copy(u32* own, u32* host, size_t n) {
+  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+  const size_t head = min(n, (size_t)((0u - (u32)((uintptr_t)host >> 2)) & 3u));
+  const size_t q = (n - head) / 4, tail = head + 4 * q;
+  if (t < head) (LOAD ? own : host)[t] = (LOAD ? host : own)[t];
+  uint4* const h4 = reinterpret_cast<uint4*>(host + head);
+#pragma unroll 2
+  for (size_t i = t; i < q; i += step) {
+    u32* o = own + head + 4 * i;
+    if (LOAD) {
+      const uint4 v = h4[i];
+      o[0] = v.x;
+      o[1] = v.y;
+      o[2] = v.z;
+      o[3] = v.w;
+    } else {
+      h4[i] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+  }
+  if (tail + t < n) (LOAD ? own : host)[tail + t] = (LOAD ? host : own)[tail + t];
+}
+template <typename T>
+__device__ __forceinline__ void row_fill(T* dst, size_t n, T v) {
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) dst[i] = v;
+}
+
+// The parts of a checkpoint image, one to a grid row: row r < 5 moves part r
+// (flags and records of the two species, the grass) between the world and the
+// image `im` in pinned host memory; row 0 the counters too. As copies and memsets one
+// by one, about 3 us each however little they move, a 40 x 40 world took 45 us to
+// save and 68 to load in front of and behind a step's kernel, now about 15 each;
+// 301 x 301 (1 MB) 34 and 80, now 21 and 19; 2048 x 2048 (46 MB) 340 to load, now
+// 244. Writing 46 MB to the host takes the copy engine 272 us and the kernel 284
+// (11 MB: 91 and 77), so worlds whose largest image is above kKernelSaveMax keep to
+// the copies.
+constexpr size_t kKernelSaveMax = (size_t)128 << 20;
+constexpr int kImageParts = 5, kLoadRows = 8;
+template <bool LOAD>
+__device__ __forceinline__ void image_part(const WorldDev& w, const int (&extent)[2], u32* im, int r) {
+  size_t o = sizeof(WorldCtr) / 4;
+  for (int k = 0; k < kImageParts; ++k) {
+    u32* own;
+    size_t n;
+    if (k == 4) {
+      own = reinterpret_cast<u32*>(w.regrow);
+      n = (size_t)w.ncells;
+    } else {
+      const SpeciesDev& sp = w.sp[k >> 1];
+      own = (k & 1) ? reinterpret_cast<u32*>(sp.agent) : reinterpret_cast<u32*>(sp.active);
+      n = (size_t)extent[k >> 1] * ((k & 1) ? 4 : 1);
+    }
+    if (k == r) {
+      row_copy<LOAD>(own, im + o, n);
+      return;
+    }
+    o += n;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_image_save(WorldDev w, u32* im) {
+  const int extent[2] = {w.ctr->extent[0], w.ctr->extent[1]};
+  if (blockIdx.y == 0 && blockIdx.x == 0 && threadIdx.x < sizeof(WorldCtr) / 4)
+    im[threadIdx.x] = reinterpret_cast<const u32*>(w.ctr)[threadIdx.x];
+  image_part<false>(w, extent, im, (int)blockIdx.y);
+}
+
+// The state of a loaded world beside the image's own parts (rows 5 to 7: what
+// lies past the extents of the two species, and the scratch of the steps), and
+// those parts too unless they were copied before (im = nullptr: rows from 5 on).
+__global__ void __launch_bounds__(256) k_image_load(WorldDev w, const __grid_constant__ WorldCtr h, u32* im, int tiles0,
+                                                    int tiles1, int segs) {
+  const int r = (int)blockIdx.y + (im ? 0 : kImageParts);
+  const int extent[2] = {h.extent[0], h.extent[1]};
+  if (r < kImageParts) {
+    image_part<true>(w, extent, im, r);
+    return;
+  }
+  if (r < kImageParts + 2) {  // past the extent: empty slots, as in a world that never used them
+    const SpeciesDev& sp = w.sp[r - kImageParts];
+    const size_t n = (size_t)extent[r - kImageParts], rest = (size_t)sp.cap - n;
+    row_fill(sp.active + n, rest, 0);
+    row_fill(sp.agent + n, rest, make_int4(0, 0, 0, 0));
+    row_fill(sp.tiles, (size_t)(r == kImageParts ? tiles0 : tiles1), (u64)0);
+    return;
+  }
+  row_fill(w.gclaim, (size_t)w.ncells, kNoKey);
+  row_fill(w.victim, (size_t)w.ncells, kNoKey);
+  row_fill(w.wclaim, (size_t)w.ncells, kNoKey);
+  row_fill(w.ps.seg[0], (size_t)segs, (u64)0);
+  row_fill(w.ps.seg[1], (size_t)segs, (u64)0);
+  row_fill(w.ps.acc, 8, 0);
+  row_fill(w.ps.bar, 2, 0u);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *w.ctr = h;
+}
+
+// CTAs per grid row of the image kernels
+static int image_ctas(const abm_world* w) {
+  const long long most = std::max<long long>(std::max(w->d.sp[0].cap, w->d.sp[1].cap), w->d.ncells);
+  return (int)std::max<long long>(1, std::min<long long>((most + 511) / 512, 2 * num_sms()));
+}
+
+// The address kernels know a host buffer by, if it is pinned from its first to
+// its last byte (nullptr: copied by the copy engine, through the driver's own
+// staging where the buffer is pageable).
+static u32* pinned_image(const void* buf, size_t bytes) {
+  cudaPointerAttributes a, z;
+  if (((uintptr_t)buf & 3) || cudaPointerGetAttributes(&a, buf) != cudaSuccess ||
+      cudaPointerGetAttributes(&z, (const char*)buf + bytes - 1) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer ||
+      (const char*)z.devicePointer - (const char*)a.devicePointer != (ptrdiff_t)(bytes - 1))
+    return nullptr;
+  return reinterpret_cast<u32*>(a.devicePointer);
+}
+
 extern "C" abm_status abm_save(abm_world* w, void* buf, size_t* bytes, void* stream) {
   if (!w || !bytes) return ABM_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   WorldCtr h;
+  size_t most = 0;
+  if (buf && abm_image_capacity(w, &most) == ABM_OK && *bytes >= most && most <= kKernelSaveMax) {
+    // room for any image: one kernel writes it, and its size is read from it
+    if (u32* im = pinned_image(buf, most)) {
+      k_image_save<<<dim3((unsigned)image_ctas(w), kImageParts), 256, 0, st>>>(w->d, im);
+      ABM_LAUNCH_CHECK();
+      ABM_CUDA_TRY(cudaStreamSynchronize(st));
+      std::memcpy(&h, buf, sizeof(WorldCtr));
+      *bytes = image_bytes(w, h);
+      return ABM_OK;
+    }
+  }
   ABM_CUDA_TRY(cudaMemcpyAsync(&h, w->d.ctr, sizeof(WorldCtr), cudaMemcpyDeviceToHost, st));
   ABM_CUDA_TRY(cudaStreamSynchronize(st));
   const size_t need = image_bytes(w, h);
@@ -793,30 +925,23 @@ extern "C" abm_status abm_load(abm_world* w, const void* buf, size_t bytes, void
   for (int s = 0; s < 2; ++s)
     if (h.extent[s] < 0 || h.extent[s] > w->d.sp[s].cap) return ABM_ERR_ARG;
   if (bytes < image_bytes(w, h)) return ABM_ERR_ARG;
-  ABM_CUDA_TRY(cudaMemcpyAsync(w->d.ctr, p, sizeof(WorldCtr), cudaMemcpyHostToDevice, st));
-  p += sizeof(WorldCtr);
-  for (int s = 0; s < 2; ++s) {
-    const size_t n = (size_t)h.extent[s], cap = (size_t)w->d.sp[s].cap;
-    if (n) {
-      ABM_CUDA_TRY(cudaMemcpyAsync(w->d.sp[s].active, p, n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-      p += n * sizeof(int32_t);
-      ABM_CUDA_TRY(cudaMemcpyAsync(w->d.sp[s].agent, p, n * sizeof(int4), cudaMemcpyHostToDevice, st));
-      p += n * sizeof(int4);
+  u32* const im = pinned_image(buf, image_bytes(w, h));
+  if (!im) {
+    p += sizeof(WorldCtr);
+    for (int s = 0; s < 2; ++s) {
+      const size_t n = (size_t)h.extent[s];
+      if (n) {
+        ABM_CUDA_TRY(cudaMemcpyAsync(w->d.sp[s].active, p, n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+        p += n * sizeof(int32_t);
+        ABM_CUDA_TRY(cudaMemcpyAsync(w->d.sp[s].agent, p, n * sizeof(int4), cudaMemcpyHostToDevice, st));
+        p += n * sizeof(int4);
+      }
     }
-    if (n < cap) {  // past the extent: empty slots, as in a world that never used them
-      ABM_CUDA_TRY(cudaMemsetAsync(w->d.sp[s].active + n, 0, (cap - n) * sizeof(int32_t), st));
-      ABM_CUDA_TRY(cudaMemsetAsync(w->d.sp[s].agent + n, 0, (cap - n) * sizeof(int4), st));
-    }
-    const int ntiles = w->cap_pad[s] / kPredTile;
-    ABM_CUDA_TRY(cudaMemsetAsync(w->d.sp[s].tiles, 0, sizeof(u64) * (size_t)ntiles, st));
+    ABM_CUDA_TRY(cudaMemcpyAsync(w->d.regrow, p, (size_t)w->d.ncells * sizeof(int32_t), cudaMemcpyHostToDevice, st));
   }
-  ABM_CUDA_TRY(cudaMemcpyAsync(w->d.regrow, p, (size_t)w->d.ncells * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-  k_reset_tables<<<num_sms() * 4, 256, 0, st>>>(w->d);
+  k_image_load<<<dim3((unsigned)image_ctas(w), im ? kLoadRows : kLoadRows - kImageParts), 256, 0, st>>>(
+      w->d, h, im, w->cap_pad[0] / kPredTile, w->cap_pad[1] / kPredTile, std::max(1, w->pgrid_max));
   ABM_LAUNCH_CHECK();
-  ABM_CUDA_TRY(cudaMemsetAsync(w->d.ps.acc, 0, sizeof(int) * 8, st));
-  for (int s = 0; s < 2; ++s)
-    ABM_CUDA_TRY(cudaMemsetAsync(w->d.ps.seg[s], 0, sizeof(u64) * (size_t)std::max(1, w->pgrid_max), st));
-  ABM_CUDA_TRY(cudaMemsetAsync(w->d.ps.bar, 0, sizeof(u32) * 2, st));
   w->bar_next = 0;
   ABM_CUDA_TRY(cudaStreamSynchronize(st));
   *w->d.class_host = extent_class(w->d, h.extent[0], h.extent[1]);

@@ -383,3 +383,29 @@ def test_small_world_launches_agree(eng, side, cap, n0, kw):
     compare_state(gp, ow, "persistent")
     gw.check()
     gp.check()
+
+
+@pytest.mark.parametrize("side,cap,n0,steps", [(1, (1, 1), (0, 0), 0), (3, (5, 3), (5, 0), 1), (37, (3001, 1203), (700, 203), 4),
+                                               (128, (70001, 35002), (6000, 1501), 9)])
+def test_images_in_pinned_memory(eng, side, cap, n0, steps):
+    """Images that one kernel writes and reads (pinned buffers, by alignment) are those that copies move."""
+    p = workloads.predation_params()
+    w = eng.World(side, 11, 2, p, cap, n0)
+    w.step(steps)
+    n = w.image_bytes()
+    want = torch.zeros(n, dtype=torch.uint8)
+    assert w.save_into(want) == n
+    for shift in (0, 4, 12, 1):
+        room = torch.full((w.image_capacity() + 64,), 77, dtype=torch.uint8).pin_memory()
+        img = room[shift:shift + w.image_capacity()]
+        assert w.save_into(img) == n
+        assert torch.equal(img[:n], want) and bool((room[:shift] == 77).all()) and bool((room[shift + n:] == 77).all())
+        v = eng.World(side, 11, 2, p, cap, (cap[0], 0))
+        v.step(2)
+        v.load_from(img[:n])
+        assert v.save(None) == want.numpy().tobytes()
+        w2 = eng.World(side, 11, 2, p, cap, n0)
+        w2.step(steps + 3)
+        v.step(3)
+        assert v.save(None) == w2.save(None)
+        v.check()
