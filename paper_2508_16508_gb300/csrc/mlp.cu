@@ -298,24 +298,41 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__
   const int rg = warp % RG, ks = warp / RG;
   const int nslab = (a.B + R - 1) / R;
   float loss = 0.f;
+  // inference: the next slab's inputs are fetched beside this one's layers
+  constexpr int NX = TRAIN ? 1 : kFusedWidth * R / NT;
+  float xn[NX] = {};
+  const auto fetch = [&](int slab) {
+#pragma unroll
+    for (int j = 0; j < NX; ++j) {
+      const int i = tid + j * NT, r = i % R, k = i / R;
+      const long long row = (long long)slab * R + r;
+      xn[j] = k < n_in && row < a.B ? a.x[(size_t)row * n_in + k] : 0.f;
+    }
+  };
+  if (!TRAIN) fetch(blockIdx.x);
   for (int slab = blockIdx.x; slab < nslab; slab += gridDim.x) {
     const int r0 = slab * R;
     const int nr = min(R, a.B - r0);  // rows of this slab; the others stay zero in every block
-    if (tid < nr) {
-      long long row = r0 + tid;
-      if (a.grows) row = (a.ga * (a.gm0 + row) + a.gc) % a.grows;
-      s_row[tid] = row;
-    }
-    __syncthreads();
-    {
-      float2* s = reinterpret_cast<float2*>(sm + net.sA[0]);
-      float* out = TRAIN ? a.act + net.offA[0] + (long long)slab * n_in * R : nullptr;
+    float2* const s = reinterpret_cast<float2*>(sm + net.sA[0]);
+    if (TRAIN) {
+      if (tid < nr) {
+        long long row = r0 + tid;
+        if (a.grows) row = (a.ga * (a.gm0 + row) + a.gc) % a.grows;
+        s_row[tid] = row;
+      }
+      __syncthreads();
+      float* out = a.act + net.offA[0] + (long long)slab * n_in * R;
       for (int i = tid; i < n_in * R; i += NT) {
         const int r = i % R, k = i / R;
         const float v = r < nr ? a.x[(size_t)s_row[r] * n_in + k] : 0.f;
         s[i] = make_float2(v, v);
-        if (TRAIN) out[i] = v;
+        out[i] = v;
       }
+    } else {
+#pragma unroll
+      for (int j = 0; j < NX; ++j)
+        if (tid + j * NT < n_in * R) s[tid + j * NT] = make_float2(xn[j], xn[j]);
+      fetch(slab + gridDim.x);
     }
     cp_async_wait_0();
     __syncthreads();
@@ -361,37 +378,44 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__
       }
       __syncthreads();
     }
-    // output layer: one warp per (row, output), lanes over the inputs
+    // output layer: the inputs split over the warps, and over a warp's 32 / R lanes of a row; the partial sums of the
+    // warps meet in `red`. (A warp per row and output, lanes over the inputs, read the activations R banks apart.)
     {
-      const int l = L - 1, din = net.din[l];
+      const int l = L - 1, din = net.din[l], r = lane % R;
       const float* W = sm + net.sW[l];
       const float* X = sm + net.sA[l];
-      for (int e = warp; e < R * n_out; e += NT / 32) {
-        const int r = e % R, o = e / R;
+      const int per = (din + NT / 32 - 1) / (NT / 32), k0 = warp * per, k1 = min(din, k0 + per);
+      for (int o = 0; o < n_out; ++o) {
         float v = 0.f;
-        for (int k = lane; k < din; k += 32) v = fmaf(X[2 * (k * R + r)], W[k * kFusedOut + o], v);
+        for (int k = k0 + lane / R; k < k1; k += 32 / R) v = fmaf(X[2 * (k * R + r)], W[k * kFusedOut + o], v);
 #pragma unroll
-        for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, m);
-        if (lane == 0) {
-          v += sm[net.sB[l] + o];
-          if (!TRAIN) {
-            if (r < nr) a.out[(size_t)(r0 + r) * n_out + o] = v;
-          } else {
-            // pinball loss at quantile tau: e = y - yhat, max(tau e, (tau - 1) e), averaged over all entries
-            float d = 0.f, le = 0.f;
-            if (r < nr) {
-              const float er = a.y[(size_t)s_row[r] * n_out + o] - v;
-              le = er > 0.f ? a.tau * er : (a.tau - 1.f) * er;
-              d = (er > 0.f ? -a.tau : 1.f - a.tau) * a.scale;
-            }
-            s_loss[e] = le;
-            s_dout[e] = d;
-            a.dact[net.offA[L] + (long long)slab * n_out * R + e] = d;
-          }
-        }
+        for (int m = R; m < 32; m <<= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, m);
+        if (lane < R) red[(warp * kFusedOut + o) * R + r] = v;
       }
     }
-    if (!TRAIN) continue;  // (the next slab's first barrier keeps its row list apart)
+    __syncthreads();
+    if (tid < R * n_out) {
+      const int r = tid % R, o = tid / R;
+      float v = 0.f;
+#pragma unroll
+      for (int z = 0; z < NT / 32; ++z) v += red[(z * kFusedOut + o) * R + r];
+      v += sm[net.sB[L - 1] + o];
+      if (!TRAIN) {
+        if (r < nr) a.out[(size_t)(r0 + r) * n_out + o] = v;
+      } else {
+        // pinball loss at quantile tau: e = y - yhat, max(tau e, (tau - 1) e), averaged over all entries
+        float d = 0.f, le = 0.f;
+        if (r < nr) {
+          const float er = a.y[(size_t)s_row[r] * n_out + o] - v;
+          le = er > 0.f ? a.tau * er : (a.tau - 1.f) * er;
+          d = (er > 0.f ? -a.tau : 1.f - a.tau) * a.scale;
+        }
+        s_loss[tid] = le;
+        s_dout[tid] = d;
+        a.dact[net.offA[L] + (long long)slab * n_out * R + tid] = d;
+      }
+    }
+    if (!TRAIN) continue;  // (`red` is written again behind the next slab's first barrier)
     __syncthreads();
     if (warp == 0) {
       float v = 0.f;
