@@ -267,7 +267,6 @@ __device__ __forceinline__ float2 split2(f32x2 v) {
 template <int R, bool TRAIN>
 __global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__ RowArgs a) {
   extern __shared__ __align__(16) float sm[];
-  __shared__ long long s_row[R];
   __shared__ float s_loss[R * kFusedOut];
   __shared__ float s_dout[kFusedOut * R];       // d loss / d yhat, [output][R]
   constexpr int NT = kRowThreads;
@@ -282,15 +281,17 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__
     const float* W = a.p + net.offW[l];
     float* s = sm + net.sW[l];
     if (l == L - 1) {  // [din][kFusedOut]
-      for (int i = tid; i < din * dout; i += NT) s[(i / dout) * kFusedOut + i % dout] = W[i];
+      for (int i = tid; i < din * dout; i += NT) cp_async4(s + (i / dout) * kFusedOut + i % dout, W + i);
     } else if ((dout & 3) == 0 && (net.offW[l] & 3) == 0) {  // a warp per row
       if (4 * lane < dout)
         for (int k = warp; k < din; k += NT / 32) cp_async16(s + k * kLd + 4 * lane, W + k * dout + 4 * lane);
     } else {
       for (int k = warp; k < din; k += NT / 32)
-        for (int c = lane; c < ((dout + 3) & ~3); c += 32) s[k * kLd + c] = c < dout ? W[k * dout + c] : 0.f;
+        for (int c = lane; c < ((dout + 3) & ~3); c += 32)
+          if (c < dout) cp_async4(s + k * kLd + c, W + k * dout + c);
+          else s[k * kLd + c] = 0.f;
     }
-    for (int i = tid; i < dout; i += NT) sm[net.sB[l] + i] = a.p[net.offb[l] + i];
+    for (int i = tid; i < dout; i += NT) cp_async4(sm + net.sB[l] + i, a.p + net.offb[l] + i);
   }
   cp_async_commit();
   float* const red = sm + net.sRed;
@@ -314,17 +315,17 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__
     const int r0 = slab * R;
     const int nr = min(R, a.B - r0);  // rows of this slab; the others stay zero in every block
     float2* const s = reinterpret_cast<float2*>(sm + net.sA[0]);
+    float target = 0.f;  // training: y of the (row, output) whose loss this thread takes
     if (TRAIN) {
-      if (tid < nr) {
-        long long row = r0 + tid;
-        if (a.grows) row = (a.ga * (a.gm0 + row) + a.gc) % a.grows;
-        s_row[tid] = row;
-      }
-      __syncthreads();
+      const auto source = [&](int r) -> long long {  // the row of the data set that is row r of the slab
+        const long long row = r0 + r;
+        return a.grows ? (a.ga * (a.gm0 + row) + a.gc) % a.grows : row;
+      };
+      if (tid < R * n_out && tid % R < nr) target = a.y[(size_t)source(tid % R) * n_out + tid / R];
       float* out = a.act + net.offA[0] + (long long)slab * n_in * R;
       for (int i = tid; i < n_in * R; i += NT) {
         const int r = i % R, k = i / R;
-        const float v = r < nr ? a.x[(size_t)s_row[r] * n_in + k] : 0.f;
+        const float v = r < nr ? a.x[(size_t)source(r) * n_in + k] : 0.f;
         s[i] = make_float2(v, v);
         out[i] = v;
       }
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) k_rows(const __grid_constant__
         // pinball loss at quantile tau: e = y - yhat, max(tau e, (tau - 1) e), averaged over all entries
         float d = 0.f, le = 0.f;
         if (r < nr) {
-          const float er = a.y[(size_t)s_row[r] * n_out + o] - v;
+          const float er = target - v;
           le = er > 0.f ? a.tau * er : (a.tau - 1.f) * er;
           d = (er > 0.f ? -a.tau : 1.f - a.tau) * a.scale;
         }
