@@ -16,6 +16,7 @@
 // Every thread keeps the world counters in registers and updates them from
 // the same totals, so no counter needs a broadcast.
 #include <algorithm>
+#include <atomic>
 
 #include "pred_world.cuh"
 
@@ -24,6 +25,7 @@ namespace abm {
 constexpr int kPT = 512;                  // threads per CTA
 constexpr int kPWarps = kPT / 32;
 constexpr int kBarSpin = 1 << 24;         // bounded barrier wait (polls; a few seconds)
+constexpr int kClusterCtas = 16;           // CTAs of the one-cluster launch
 constexpr int kPhases = 4;                // grid barriers per step (plus one closing a launch)
 
 // Grid barrier (all CTAs co-resident: cooperative launch) over a monotonic
@@ -1060,8 +1062,9 @@ struct PhaseClock {
 };
 
 // MINB = resident CTAs per SM the register budget is cut for (1: up to 128
-// registers a thread, 2: 64).
-template <int MINB>
+// registers a thread, 2: 64). CLUSTER: the grid is one cluster, whose hardware
+// barrier takes the place of the grid barrier.
+template <int MINB, bool CLUSTER = false>
 __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps, abm_step_stats* stats,
                                                      unsigned long long* phase_ns) {
   __shared__ u64 s_red[2 * kPWarps];
@@ -1103,6 +1106,17 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
     s_book.nstart0 = s_book.r0p = s_book.P0p = s_book.starved0p = s_book.grassp = 0;
     s_book.stp = nullptr;
   }
+  const auto sync = [&]() -> bool {
+    if constexpr (CLUSTER) {
+      __syncwarp();
+      cluster_arrive();
+      cluster_wait();
+      return false;
+    } else {
+      return grid_sync(ps.bar, w.err, bar_target);
+    }
+  };
+  if (CLUSTER && ld_relaxed32(reinterpret_cast<const u32*>(w.err)) != 0u) return;  // (an earlier launch's: the same in every thread)
   clk.start();
   // Wolf ranks of step t-1 run beside the sheep moves of step t, and the wolf
   // moves of step t beside the sheep ranks: neither needs the other's
@@ -1182,7 +1196,7 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
       if (blockIdx.x == 0 && threadIdx.x == 0) acc[0] = acc[1] = acc[2] = acc[3] = 0;  // last read in P1 of step t-1
       p_move<0, kSheepWarps>(w, t, ext[0], cl, carried, mf);
     }
-    const bool bad = grid_sync(ps.bar, w.err, bar_target);
+    const bool bad = sync();
     clk.lap(0);
     if (bad) return;
     // ---- P2: wolf counters (t-1) | wolf births (t-1) beside sheep eat / select / die / flags
@@ -1206,7 +1220,7 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
         for (int j = threadIdx.x; j < (int)gridDim.x; j += kSheepWarps * 32) ps.seg[1][j] = 0ull;
       p_count<0, kSheepWarps>(w, t, ext[0], kseg0, acc, cl, carried, s_upar, s_acc);
     }
-    grid_sync(ps.bar, w.err, bar_target);
+    sync();
     clk.lap(1);
     // ---- P3: sheep ranks and births | wolves move + claims
     if ((int)threadIdx.x < kMoveWarps * 32) {
@@ -1223,7 +1237,7 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
         s_sheep[1] = (int)P0;
       }
     }
-    grid_sync(ps.bar, w.err, bar_target);
+    sync();
     clk.lap(2);
     // ---- sheep counters (every thread)
     const int F0 = s_sheep[0], P0 = s_sheep[1];
@@ -1251,7 +1265,7 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
     p_count<1, kPWarps>(w, t, ext[1], kseg1, acc, cl, carried, s_upar, s_acc);
     if (book_thread()) s_book.stp = stats ? stats + it : nullptr;
     ++t;
-    grid_sync(ps.bar, w.err, bar_target);
+    sync();
     clk.lap(4);
   }
   // the last step's wolf ranks and births (every warp is free: the whole CTA ranks)
@@ -1269,7 +1283,7 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
     }
     __syncthreads();
     const Births wb = wolf_counters(t - 1);
-    grid_sync(ps.bar, w.err, bar_target);
+    sync();
     clk.lap(5);
     p_births<kPT>(w, wb.r, wb.F, wb.ext, wb.id0, threadIdx.x);
     if (blockIdx.x == 0)  // wolf segment sums, for the next launch
@@ -1307,10 +1321,32 @@ int persistent_warps() { return kPWarps; }
 
 int persistent_round_units() { return kQ * kSheepWarps; }
 
-abm_status launch_persistent(const WorldDev& d, u32* bar_next, int grid, int nsteps, abm_step_stats* stats,
+abm_status launch_persistent(const WorldDev& d, u32* bar_next, int grid, bool cluster, int nsteps, abm_step_stats* stats,
                              cudaStream_t st, unsigned long long* phase_ns) {
   WorldDev dd = d;
   dd.bar_base = *bar_next;
+  if (cluster) {
+    static std::atomic<unsigned long long> wide{0};  // devices on which the kernel may use clusters above 8
+    int dev = 0;
+    ABM_CUDA_TRY(cudaGetDevice(&dev));
+    const unsigned long long bit = (dev >= 0 && dev < 64) ? 1ull << dev : 0ull;
+    if (!bit || !(wide.load(std::memory_order_acquire) & bit)) {
+      ABM_CUDA_TRY(cudaFuncSetAttribute(k_persistent<1, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      wide.fetch_or(bit, std::memory_order_release);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClusterCtas);
+    cfg.blockDim = dim3(kPT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kClusterCtas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    ABM_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_persistent<1, true>, dd, nsteps, stats, phase_ns));
+    return ABM_OK;
+  }
   void* args[] = {(void*)&dd, (void*)&nsteps, (void*)&stats, (void*)&phase_ns};
   // one CTA per SM: the variant with the larger register budget
   const void* fn = grid <= num_sms() ? (const void*)k_persistent<1> : (const void*)k_persistent<2>;

@@ -49,7 +49,7 @@ struct WorldDev {
   // size class of the extents, which chooses the launch of the next steps (never the results): pinned host word, set by
   // a launch that ends in another class than the one it was given (class_known), so that other launches write nothing
   int* class_host;
-  int class_known, class_small, class_round;
+  int class_known, class_small, class_cluster, class_round;
   int* err;
   int side, ncells;
   u32 seed, model;
@@ -66,9 +66,12 @@ struct WorldDev {
   u64* wnext;       // [cap wolves]
 };
 
-// 0: few enough slots for one CTA's shared memory to be faster; 1: the sheep units fit one round of one CTA per SM; 2: more
+// 0: few enough slots for one CTA's shared memory to be faster; 1: for one cluster to be; 2: the sheep units fit one round
+// of one CTA per SM; 3: more
 __host__ __device__ inline int extent_class(const WorldDev& w, int ext0, int ext1) {
-  return ext0 + ext1 <= w.class_small ? 0 : (ext0 <= w.class_round ? 1 : 2);
+  if (ext0 + ext1 <= w.class_small) return 0;
+  if (ext0 + ext1 <= w.class_cluster) return 1;
+  return ext0 <= w.class_round ? 2 : 3;
 }
 __device__ __forceinline__ void note_class(const WorldDev& w, int ext0, int ext1) {
   const int k = extent_class(w, ext0, ext1);
@@ -80,7 +83,7 @@ int persistent_max_ctas();
 int persistent_warps();
 // units (128 slots) of a species that one CTA takes in one round of the persistent kernel's sheep phases
 int persistent_round_units();
-abm_status launch_persistent(const WorldDev& d, u32* bar_next, int grid, int nsteps, abm_step_stats* stats,
+abm_status launch_persistent(const WorldDev& d, u32* bar_next, int grid, bool cluster, int nsteps, abm_step_stats* stats,
                              cudaStream_t st,
                              unsigned long long* phase_ns = nullptr);
 

@@ -352,6 +352,7 @@ __global__ void k_view_commit(WorldCtr* c, int sp, const int32_t* counters, cons
 // ============================================================================
 using namespace abm;
 
+constexpr int kClusterSlots = 20000, kClusterCells = 256 * 256;  // for one cluster (see launch_steps)
 constexpr int kResidentSlots = 3072;  // slots up to which one CTA is faster than the grid (see launch_steps)
 
 struct abm_world {
@@ -499,6 +500,7 @@ extern "C" abm_status abm_create(const abm_config* cfg, void* stream, abm_world*
   w->engine = ABM_ENGINE_PERSISTENT;
   w->pgrid = std::min(w->pgrid_max, num_sms() * 2);
   d.class_small = resident_fits(d) ? kResidentSlots : -1;
+  d.class_cluster = d.ncells <= kClusterCells ? kClusterSlots : -1;
   d.class_round = num_sms() * persistent_round_units() * 128;
   *d.class_host = extent_class(d, cfg->n0[0], cfg->n0[1]);
   k_world_init<<<num_sms() * 4, 256, 0, st>>>(d, cfg->n0[0], cfg->n0[1]);
@@ -518,19 +520,24 @@ extern "C" abm_status abm_create(const abm_config* cfg, void* stream, abm_world*
 // Class 0: one CTA with the state in its shared memory (launch_resident). A
 // step there costs 4 us for a few hundred agents and grows with the slots,
 // 12.8 us at 3441; the persistent kernel takes 14 us from 1 to 10,000.
-// Class 1: one persistent CTA per SM while that takes every sheep unit in one
+// Class 1: sixteen persistent CTAs in one cluster, whose hardware barrier is
+// 0.6 us shorter than the grid's, four times a step: 100 x 100 cells 12.2 -> 10.6
+// us a step, 150 x 150 13.4 -> 11.8, 220 x 220 (17,000 slots) 13.1 -> 12.1; at 301 x
+// 301 (32,000) sixteen SMs lose what it gains, 14.0 and 14.2. Only for lattices of
+// at most kClusterCells, whose agents cannot grow far past that line in one launch.
+// Class 2: one persistent CTA per SM while that takes every sheep unit in one
 // round (then the moved agents stay in shared memory for the meals). A barrier
 // of fewer CTAs and twice the registers per thread are worth 2 us a step: 301 x
 // 301 cells 18.1 -> 15.8 us, 1400 x 1400 (3811 sheep units) 21.1 -> 18.9.
-// Class 2: the tuned number of CTAs; at 2048 x 2048 (two rounds of one CTA per
+// Class 3: the tuned number of CTAs; at 2048 x 2048 (two rounds of one CTA per
 // SM) the second CTA per SM wins, 33.7 us against 38.7.
 static abm_status launch_steps(abm_world* w, int nsteps, abm_step_stats* stats, cudaStream_t st,
                                unsigned long long* phase_ns = nullptr) {
   WorldDev d = w->d;
   d.class_known = *reinterpret_cast<volatile int*>(d.class_host);
   if (d.class_known == 0 && !phase_ns) return launch_resident(d, nsteps, stats, st);
-  const int grid = d.class_known < 2 ? std::min(w->pgrid, num_sms()) : w->pgrid;
-  return launch_persistent(d, &w->bar_next, grid, nsteps, stats, st, phase_ns);
+  const int grid = d.class_known < 3 ? std::min(w->pgrid, num_sms()) : w->pgrid;
+  return launch_persistent(d, &w->bar_next, grid, d.class_known == 1 && !phase_ns, nsteps, stats, st, phase_ns);
 }
 
 // ev (nullable): 7 events recorded around the six kernels of the step

@@ -409,3 +409,23 @@ def test_images_in_pinned_memory(eng, side, cap, n0, steps):
         v.step(3)
         assert v.save(None) == w2.save(None)
         v.check()
+
+
+@pytest.mark.parametrize("side,cap,n0,variant,kw", [
+    (256, (60000, 9000), (15000, 4500), 0, dict(sheep_gain=30, regrowth=2)),             # grows past 20000 slots
+    (257, (60000, 9000), (9000, 900), 0, {}),                                            # too many cells
+    (150, (50001, 20003), (5400, 1301), 0, {}), (90, (20000, 9000), (2000, 700), 1, {}), (64, (40000, 40000), (1, 1), 3, {})])
+def test_cluster_launches_agree(eng, side, cap, n0, variant, kw):
+    """One cluster of CTAs and the persistent grid (which step_profiled always takes) in turn on one world, and the
+    grid alone on another."""
+    p = workloads.predation_params(**kw)
+    a, b = (eng.World(side, 6, 1, p, cap, n0, variant=variant) for _ in range(2))
+    sa, sb = a.new_stats(24), b.new_stats(24)
+    for k in range(0, 24, 8):
+        a.step(1, sa[k:k + 1])
+        a.step(5, sa[k + 1:k + 6])
+        a.step_profiled(2, sa[k + 6:k + 8])
+        b.step_profiled(8, sb[k:k + 8])
+    assert torch.equal(sa, sb)
+    assert a.save() == b.save()
+    a.check()
