@@ -327,15 +327,16 @@ def selective_update_leg(torch, engine, abm, autotune, hbm_peak, steps=8, warmup
         if it >= warmup:
             times.append(e0.elapsed_time(e1))
     s.check()
+    live = int(s.read(-1).sum())
     del s
     ms = statistics.median(times)
-    # per slot: key + value built (read flag + key field, write 8 B), five passes of
-    # (histogram read 4 B, scatter read 8 B + write 8 B), the row gather (value read 4 B,
-    # row read + write 4 F B each, live flag and permutation written 4 B each)
-    b = n * (8 + 8 + 5 * 20 + 4 + 2 * 4 * F + 8)
+    # per slot: flag counted, flag and key field packed, a pair or a listed placeholder written; per live slot four
+    # passes (the keys vary in every byte) of histogram read 4 B, scatter read 8 B + write 8 B; per slot the row gather
+    # (value read 4 B, row read + write 4 F B each, live flag and permutation written 4 B each)
+    b = n * (4 + 8 + 4 + 4 + 2 * 4 * F + 8) + live * (4 + 4 * 20)
     out["sort_agents"] = {"ms": ms, "algorithmic_bytes": b, "gbs": b / (ms * 1e-3) / 1e9,
                           "frac": b / (ms * 1e-3) / 1e9 / hbm_peak,
-                          "method": "LSD radix sort, 4 key-byte passes + 1 live-flag pass, then the row gather"}
+                          "method": "LSD radix sort of the live slots' keys, one pass per byte that varies, then the row gather"}
     # conflict pass: M = N/4 claims over R = N/64 resources, Zipf(1.1)
     M, R = n // 4, n // 64
     res = torch.from_numpy(workloads.zipf_claims(M, R, s=c["zipf_s"], seed=c["zipf_seed"])).cuda()
@@ -357,7 +358,7 @@ def selective_update_leg(torch, engine, abm, autotune, hbm_peak, steps=8, warmup
     ms = statistics.median(times)
     b = 17 * M + 20 * R
     out["resolve"] = {"M": M, "R": R, "ms": ms, "algorithmic_bytes": b, "gbs": b / (ms * 1e-3) / 1e9,
-                      "frac": b / (ms * 1e-3) / 1e9 / hbm_peak, "bound": "L2 atomics (2 MiB table)"}
+                      "frac": b / (ms * 1e-3) / 1e9 / hbm_peak, "bound": "scattered L2 atomics (2 MiB table)"}
     del flush
     return out
 
@@ -863,9 +864,9 @@ def run_ours(args, rank, world, local):
         pw.tune(tw["engine"], tw["ctas_per_sm"])
         pw.step(W)
         phase = pw.step_profiled(K)
-        line["phases_us_per_step"] = {n: 1e3 * phase[i] / max(K, 1) for i, n in enumerate(
-            ("P1_prev_wolf_ranks_sheep_move", "P2_prev_wolf_births_sheep_eat_select", "P3_sheep_ranks_wolf_move",
-             "P4_sheep_births", "P5_wolf_eat_select", "closing_wolf_ranks"))}
+        line["phases_us_per_step"] = {n: 1e3 * phase[i] / max(K, 1) for i, n in (
+            (0, "P1_prev_wolf_ranks_sheep_move"), (1, "P2_prev_wolf_births_sheep_eat_select"),
+            (2, "P3_sheep_ranks_births_wolf_move"), (4, "P4_wolf_eat_select"), (5, "closing_wolf_ranks"))}
         line["phases_us_per_step"]["same_trajectory"] = pw.counters() == gw.counters()
         del pw
         # end to end through the public API: the state loaded from host memory,

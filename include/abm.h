@@ -181,8 +181,8 @@ abm_status abm_sort(abm_slab* s, int32_t field, int32_t* out_perm, void* stream)
 #define ABM_LOB_MAX_CAP 2048
 /* Launch shape of abm_lob_match's price-level path for the rest of the
  * process: warps matching one book (1, 2 or 4; 0 = the default: 1 for books of
- * up to 256 slots, 2 up to 1024, else 4). Results
- * never depend on it. ABM_ERR_ARG for other values. Host only. */
+ * up to 256 slots, 2 up to 768, else 4, and with at most 2048 books 1 up to 128,
+ * 2 up to 512, else 4). Results never depend on it. ABM_ERR_ARG for other values. Host only. */
 abm_status abm_lob_tune(int32_t warps_per_book);
 abm_status abm_lob_match(int32_t n_books, int32_t cap, int32_t* active, const int32_t* side, const int32_t* price,
                          int32_t* qty, const int32_t* time, int64_t* out_volume, int32_t* out_price, void* stream);
@@ -396,16 +396,17 @@ abm_status abm_step_graph(abm_world* w, int32_t nsteps, int32_t reps, abm_step_s
  * [2] sheep births, [3] wolf move, [4] wolf eat/select/compact, [5] wolf
  * births. Persistent engine: block 0's global-timer laps between the grid
  * barriers, [0] previous step's wolf ranks + sheep move, [1] previous step's
- * wolf births + sheep eat/select/flags, [2] sheep ranks + wolf move, [3]
- * sheep births, [4] wolf eat/select/flags, [5] the last step's wolf ranks
+ * wolf births + sheep eat/select/flags, [2] sheep ranks and births + wolf
+ * move, [3] = 0, [4] wolf eat/select/flags, [5] the last step's wolf ranks
  * (once per call). Both: [7] whole call by events, [6] = 0.
  * Synchronises `stream`. */
 abm_status abm_step_profiled(abm_world* w, int32_t nsteps, abm_step_stats* stats, float* phase_ms,
                              void* stream);
 /* Execution engine of abm_step: ABM_ENGINE_PERSISTENT (default) runs all
- * requested steps in one cooperative launch of at most `ctas_per_sm` CTAs per
- * SM (one while the sheep extent is small enough for that to be faster)
- * with bounded grid barriers between the phases; ABM_ENGINE_KERNELS runs six
+ * requested steps in one launch: a cooperative one of at most `ctas_per_sm` CTAs
+ * per SM with bounded grid barriers between the phases, or, while the extents
+ * are small enough for that to be faster, of one CTA per SM, of one cluster, or
+ * of one CTA that holds the world in shared memory; ABM_ENGINE_KERNELS runs six
  * kernels per step (and is what abm_step_profiled, energy statistics and
  * abm_step_graph use). Results are identical. */
 #define ABM_ENGINE_PERSISTENT 0

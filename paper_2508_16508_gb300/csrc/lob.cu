@@ -327,6 +327,14 @@ __device__ __forceinline__ void grp_stage(int32_t* s_act, int n, int b, int cap,
 // 4 * (g * T + t) + c. The book's words move from the staging arrays into
 // registers, and the next book is staged at once. Deferred books get
 // out_volume = -1 and are left untouched.
+//
+// Bound by the chain of a book's dependent steps at the occupancy that the staged
+// words allow (11 CTAs per SM): 65536 books of 1024 slots take 299 us with four
+// warps per book and move 1.5 GB (232 us at the copy rate); issue slots are half
+// full. Levels written back and counted, marginal orders listed and fetched one by
+// one: 326 us with two warps, and 454 before the loops over the slots were cut to
+// what each needs. Loads straight into registers with the next book prefetched
+// into L2 are no faster (297 to 315 us).
 template <int G, int SPL, bool kVec16>
 __global__ void __launch_bounds__(G * 32)
     k_lob_match_levels(int n_books, int cap, int32_t* active, const int32_t* __restrict__ side,
