@@ -706,7 +706,7 @@ def lob_leg(torch, engine, hbm_peak, reps=10, n_books=None, warps=None):
                      "graph_us_per_step": 1e3 * statistics.median(gts) / M["steps"],
                      "graph_same_result": same_graph,
                      "traded_shares": eager[0], "orders_placed": eager[1],
-                     "launches": 3 * M["steps"],
+                     "launches": 2 * M["steps"],
                      "paper_ms_100_steps_500_books": 2212.47,
                      "note": "paper figure: Table 4 (JAX, its own hardware): context, not a target"}
     return out

@@ -28,12 +28,12 @@
 // below pa fill whole, those beyond fill nothing, and only the orders on the
 // two marginal levels are ranked by (time, slot), by counting.
 //
-// Sort path (k_lob_deferred): a book whose range is wider than kWarpLevels
+// Sort path (lob_sort_book): a book whose range is wider than kWarpLevels
 // prices, whose marginal level holds more than kWarpMarginal orders, or whose
-// bid or ask shares reach 2^21 is left untouched by the level path (its
-// volume set to -1) and matched by a second kernel, one CTA per book: bitonic
-// sort of the whole book in shared memory, cumulative sums, a binary search
-// per bid.
+// bid or ask shares reach 2^21 is left untouched by the level path and matched
+// by a bitonic sort of the whole book in shared memory, cumulative sums and a
+// binary search per bid: by the same CTA where every book has one, else (its
+// volume set to -1) by a second kernel, k_lob_deferred.
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
@@ -43,7 +43,6 @@
 namespace abm {
 
 constexpr int kLobThreads = 256;        // sort path: threads per book
-constexpr int kLobWarps = kLobThreads / 32;
 constexpr int kWarpLevels = 256;        // level path: prices in [lowest ask, highest bid], at most
 constexpr int kWarpMarginal = 64;       // level path: orders on one marginal level, at most
 constexpr u32 kShareBits = 21;          // level words: shares in the low 21 bits, orders above
@@ -56,8 +55,9 @@ constexpr int32_t kNoPrice = 0;         // level path: a dead slot's price in re
 __device__ __forceinline__ u32 ord32(int32_t p) { return (u32)p ^ 0x80000000u; }
 
 // Block-wide exclusive scan of a u64 (every thread gets its prefix and the
-// total). Three barriers; the buffer is free again when it returns.
-__device__ __forceinline__ u64 block_sum_scan_u64(u64 v, u64& total, u64* s_warp /* [kLobWarps + 1] */) {
+// total). T threads. Three barriers; the buffer is free again when it returns.
+template <int T>
+__device__ __forceinline__ u64 block_sum_scan_u64(u64 v, u64& total, u64* s_warp /* [T / 32 + 1] */) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   u64 incl = v;
 #pragma unroll
@@ -68,19 +68,19 @@ __device__ __forceinline__ u64 block_sum_scan_u64(u64 v, u64& total, u64* s_warp
   if (lane == 31) s_warp[warp] = incl;
   __syncthreads();
   if (warp == 0) {
-    const u64 w = lane < kLobWarps ? s_warp[lane] : 0ull;
+    const u64 w = lane < (T / 32) ? s_warp[lane] : 0ull;
     u64 wi = w;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const u64 t = __shfl_up_sync(0xFFFFFFFFu, wi, o);
       if (lane >= o) wi += t;
     }
-    if (lane < kLobWarps) s_warp[lane] = wi - w;
-    if (lane == kLobWarps - 1) s_warp[kLobWarps] = wi;
+    if (lane < (T / 32)) s_warp[lane] = wi - w;
+    if (lane == (T / 32) - 1) s_warp[(T / 32)] = wi;
   }
   __syncthreads();
   const u64 ex = s_warp[warp] + incl - v;
-  total = s_warp[kLobWarps];
+  total = s_warp[(T / 32)];
   __syncthreads();
   return ex;
 }
@@ -94,9 +94,10 @@ struct LobBook {
   int32_t* qt;
 };
 
-// The sort path for one book (see the file comment). n = R * kLobThreads
-// padded slots; key/cum share one u64 array and ord a u32 array, both [n], in
+// The sort path for one book (see the file comment) by T threads. n padded slots
+// (a power of two, a multiple of T); key/cum share one u64 array and ord a u32 array, both [n], in
 // the work area. nbid/nask: live orders per side.
+template <int T>
 __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nbid, int nask, int32_t* active,
                                  int32_t* qty, const int32_t* __restrict__ time, long long* out_volume,
                                  int32_t* out_price, u64* key, u32* ord, u64* s_scan, unsigned long long* s_v) {
@@ -105,7 +106,7 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
   if (threadIdx.x == 0) *s_v = 0ull;
   // key: side | price (bids descending; prices positive) | time (signed
   // order); ties by slot, empty slots (slot + n) last
-  for (int i = threadIdx.x; i < n; i += kLobThreads) {
+  for (int i = threadIdx.x; i < n; i += T) {
     u64 k = kNoKey;
     u32 r = (u32)(i + n);
     if (d.act[i]) {
@@ -120,7 +121,7 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
   __syncthreads();
   for (int kk = 2; kk <= n; kk <<= 1) {
     for (int j = kk >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < n; i += kLobThreads) {
+      for (int i = threadIdx.x; i < n; i += T) {
         const int l = i ^ j;
         if (l > i) {
           const bool up = (i & kk) == 0;
@@ -141,12 +142,12 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
   // sorted: bids [0, nbid), asks [nbid, nbid + nask), empty slots after. The
   // keys are dead now: cum[e] (same array) = shares of entries [0, e].
   u64* cum = key;
-  const int nl = nbid + nask, per = n / kLobThreads;
+  const int nl = nbid + nask, per = n / T;
   u64 local = 0;
   for (int e = threadIdx.x * per; e < (threadIdx.x + 1) * per; ++e)
     local += e < nl ? (u64)(u32)d.qt[ord[e]] : 0ull;
   u64 tot;
-  u64 run = block_sum_scan_u64(local, tot, s_scan);
+  u64 run = block_sum_scan_u64<T>(local, tot, s_scan);
   for (int e = threadIdx.x * per; e < (threadIdx.x + 1) * per; ++e) {
     run += e < nl ? (u64)(u32)d.qt[ord[e]] : 0ull;
     cum[e] = run;
@@ -156,7 +157,7 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
   // V: bid i may trade the shares in (QB_{i-1}, min(QB_i, QA(J_i))], J_i = the
   // asks priced at or below it
   u64 vbest = 0;
-  for (int i = threadIdx.x; i < nbid; i += kLobThreads) {
+  for (int i = threadIdx.x; i < nbid; i += T) {
     const int32_t p = d.px[ord[i]];
     int lo = 0, hi = nask;
     while (lo < hi) {
@@ -176,7 +177,7 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
     out_volume[b] = (long long)V;
     if (V == 0) out_price[b] = -1;
   }
-  for (int e = threadIdx.x; e < nl; e += kLobThreads) {
+  for (int e = threadIdx.x; e < nl; e += T) {
     const bool is_bid = e < nbid;
     const u64 start = is_bid ? (e > 0 ? cum[e - 1] : 0ull) : (e > nbid ? cum[e - 1] - bid_total : 0ull);
     const u64 end = is_bid ? cum[e] : cum[e] - bid_total;
@@ -192,11 +193,46 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
   }
 }
 
+// Loads a book and matches it by the sort path; `work`: 28 bytes per padded slot.
+template <int T>
+__device__ __noinline__ void lob_sort_book(int n, int b, int cap, int32_t* active, const int32_t* __restrict__ side,
+                                           const int32_t* __restrict__ price, int32_t* qty,
+                                           const int32_t* __restrict__ time, long long* out_volume, int32_t* out_price,
+                                           unsigned char* work) {
+  __shared__ u64 s_scan[T / 32 + 1];
+  __shared__ unsigned long long s_v;
+  int32_t* w = reinterpret_cast<int32_t*>(work);
+  const LobBook d{w, w + n, w + 2 * n, w + 3 * n};
+  u64* key = reinterpret_cast<u64*>(w + 4 * n);
+  const size_t o = (size_t)b * cap;
+  int nbid = 0, nask = 0;
+  for (int i = threadIdx.x; i < n; i += T) {
+    const bool in = i < cap;
+    const int32_t a = in ? active[o + i] : 0;
+    const int32_t s = in ? side[o + i] : 0;
+    d.act[i] = a;
+    d.sid[i] = s;
+    d.px[i] = in ? price[o + i] : 0;
+    d.qt[i] = in ? qty[o + i] : 0;
+    nbid += __syncthreads_count(a != 0 && s == 0);
+    nask += __syncthreads_count(a != 0 && s != 0);
+  }
+  lob_match_sorted<T>(d, n, b, cap, nbid, nask, active, qty, time, out_volume, out_price, key,
+                      reinterpret_cast<u32*>(key + n), s_scan, &s_v);
+  __syncthreads();  // the work area is used again
+}
+
 // Shared memory of one CTA of the level path (one book at a time): the staged
 // book (4 arrays of n words; slots >= cap hold active = 0), the level words of
 // both sides, and the marginal lists (qty, key = time | slot) of both sides.
 __host__ __device__ constexpr size_t grp_smem_bytes(int n) {
   return 16 * (size_t)n + 2 * kWarpLevels * sizeof(u32) + 2 * kWarpMarginal * (sizeof(u32) + sizeof(u64));
+}
+
+// Padded slots of the sort path for a book of up to n (a power of two) slots, and its work area
+__host__ __device__ constexpr int sort_pad(int n) { return n < kLobThreads ? kLobThreads : n; }
+__host__ __device__ constexpr size_t sort_smem_bytes(int pad) {
+  return (size_t)pad * (4 * sizeof(int32_t) + sizeof(u64) + sizeof(u32));
 }
 
 __device__ __forceinline__ int popc_mask(u32 m) { return __popc(m); }
@@ -325,8 +361,9 @@ __device__ __forceinline__ void grp_stage(int32_t* s_act, int n, int b, int cap,
 // Level path: a CTA of G warps (T = 32 G threads) matches one book at a time;
 // SPL = slots per thread (cap <= T * SPL), thread t holding slots
 // 4 * (g * T + t) + c. The book's words move from the staging arrays into
-// registers, and the next book is staged at once. Deferred books get
-// out_volume = -1 and are left untouched.
+// registers, and the next book is staged at once. Books for the sort path are left
+// untouched and get out_volume = -1, or with FOLD (every CTA has one book) are
+// handed to it at the end.
 //
 // Bound by the chain of a book's dependent steps at the occupancy that the staged
 // words allow (11 CTAs per SM): 65536 books of 1024 slots take 299 us with four
@@ -335,7 +372,7 @@ __device__ __forceinline__ void grp_stage(int32_t* s_act, int n, int b, int cap,
 // one: 326 us with two warps, and 454 before the loops over the slots were cut to
 // what each needs. Loads straight into registers with the next book prefetched
 // into L2 are no faster (297 to 315 us).
-template <int G, int SPL, bool kVec16>
+template <int G, int SPL, bool kVec16, bool FOLD>
 __global__ void __launch_bounds__(G * 32)
     k_lob_match_levels(int n_books, int cap, int32_t* active, const int32_t* __restrict__ side,
                        const int32_t* __restrict__ price, int32_t* qty, const int32_t* __restrict__ time,
@@ -353,11 +390,12 @@ __global__ void __launch_bounds__(G * 32)
   u64* m_key = reinterpret_cast<u64*>(m_qty + 2 * kWarpMarginal);  // [2][kWarpMarginal]
   const int t = threadIdx.x;
   int par = 0;
+  int defer = -1;  // FOLD: this CTA's book, if the sort path has to take it
   for (int i = cap + t; i < n; i += T) s_act[i] = 0;  // padding slots: never copied, never live
   griddep_wait();
   // the sort path's few CTAs may start (and the next call's beside those: 100 steps
-  // of 500 books 761 -> 748 us). Not from k_lob_add: its successor's CTAs then
-  // crowd the SMs that are free at that moment (968 us).
+  // of 500 books in two launches a round 761 -> 748 us). Not from k_lob_add: its
+  // successor's CTAs then crowd the SMs that are free at that moment (968 us).
   griddep_launch();
   if ((int)blockIdx.x < n_books) grp_stage<T, kVec16>(s_act, n, blockIdx.x, cap, active, side, price, qty);
   for (int b = blockIdx.x; b < n_books; b += gridDim.x) {
@@ -427,7 +465,8 @@ __global__ void __launch_bounds__(G * 32)
         wide = tb > kShareMask || ta > kShareMask;
       }
       if (wide) {
-        if (t == 0) out_volume[b] = -1;  // the sort path takes it
+        if (FOLD) defer = b;  // the sort path takes it
+        else if (t == 0) out_volume[b] = -1;
         continue;
       }
     }
@@ -502,7 +541,8 @@ __global__ void __launch_bounds__(G * 32)
         Dn = s_mar[0][1];
         Sp = s_mar[1][1];
         if (max(s_mar[0][2], s_mar[1][2]) > kWarpMarginal) {
-          if (t == 0) out_volume[b] = -1;  // a crowded marginal level: the sort path takes it
+          if (FOLD) defer = b;  // a crowded marginal level: the sort path takes it
+          else if (t == 0) out_volume[b] = -1;
           continue;
         }
       }
@@ -595,6 +635,12 @@ __global__ void __launch_bounds__(G * 32)
     }
   }
   cp_async_wait_0();
+  if constexpr (FOLD) {
+    if (defer >= 0) {
+      grp_sync<G>();  // the level path's shared memory becomes the work area
+      lob_sort_book<T>(sort_pad(T * SPL), defer, cap, active, side, price, qty, time, out_volume, out_price, lob_smem);
+    }
+  }
 }
 
 // Sort path for the books the level path deferred (out_volume < 0), one CTA
@@ -605,16 +651,9 @@ __global__ void __launch_bounds__(kLobThreads)
     k_lob_deferred(int n_books, int cap, int32_t* active, const int32_t* __restrict__ side,
                    const int32_t* __restrict__ price, int32_t* qty, const int32_t* __restrict__ time,
                    long long* out_volume, int32_t* out_price) {
-  constexpr int n = R * kLobThreads;
   extern __shared__ __align__(16) unsigned char lob_smem[];
-  int32_t* w = reinterpret_cast<int32_t*>(lob_smem);
-  const LobBook d{w, w + n, w + 2 * n, w + 3 * n};
-  u64* key = reinterpret_cast<u64*>(w + 4 * n);
-  u32* ord = reinterpret_cast<u32*>(key + n);
   __shared__ int s_list[kLobThreads];
   __shared__ int s_cnt;
-  __shared__ u64 s_scan[kLobWarps + 1];
-  __shared__ unsigned long long s_v;
   griddep_wait();
   griddep_launch();
   for (int c0 = blockIdx.x * kLobThreads; c0 < n_books; c0 += gridDim.x * kLobThreads) {
@@ -624,24 +663,10 @@ __global__ void __launch_bounds__(kLobThreads)
     if (bq < n_books && out_volume[bq] < 0) s_list[atomicAdd(&s_cnt, 1)] = bq;
     __syncthreads();
     const int m = s_cnt;
-    for (int j = 0; j < m; ++j) {
-      const int b = s_list[j];
-      const size_t o = (size_t)b * cap;
-      int nbid = 0, nask = 0;
-      for (int i = threadIdx.x; i < n; i += kLobThreads) {
-        const bool in = i < cap;
-        const int32_t a = in ? active[o + i] : 0;
-        const int32_t s = in ? side[o + i] : 0;
-        d.act[i] = a;
-        d.sid[i] = s;
-        d.px[i] = in ? price[o + i] : 0;
-        d.qt[i] = in ? qty[o + i] : 0;
-        nbid += __syncthreads_count(a != 0 && s == 0);
-        nask += __syncthreads_count(a != 0 && s != 0);
-      }
-      lob_match_sorted(d, n, b, cap, nbid, nask, active, qty, time, out_volume, out_price, key, ord, s_scan, &s_v);
-      __syncthreads();  // shared arrays are reused by the next book
-    }
+    for (int j = 0; j < m; ++j)
+      lob_sort_book<kLobThreads>(R * kLobThreads, s_list[j], cap, active, side, price, qty, time, out_volume, out_price,
+                                 lob_smem);
+    __syncthreads();
   }
 }
 
@@ -724,43 +749,64 @@ static int lob_pad(int cap) {
 
 static std::atomic<int> g_lob_warps_per_book{0};  // level path: warps per book (1, 2 or 4; 0: by the capacity)
 
-template <int G, int SPL, bool kVec16>
-static abm_status lob_launch_levels(int n_books, int cap, int32_t* active, const int32_t* side, const int32_t* price,
-                                    int32_t* qty, const int32_t* time, long long* vol, int32_t* px, cudaStream_t st) {
+// FOLD: every book has a CTA of its own at once, which also takes it by the sort
+// path where that is called for. grid = 0: as many CTAs as the device holds.
+template <int G, int SPL, bool kVec16, bool FOLD>
+static abm_status lob_levels(int& grid, int n_books, int cap, int32_t* active, const int32_t* side,
+                             const int32_t* price, int32_t* qty, const int32_t* time, long long* vol, int32_t* px,
+                             cudaStream_t st) {
   // the shared-memory limit and the occupancy are per device: looked up once for each
   static std::atomic<unsigned long long> attr{0};
   static std::atomic<int> occ_dev[64];
-  const size_t smem = grp_smem_bytes(G * 32 * SPL);
-  ABM_CUDA_TRY(smem_attr_once(k_lob_match_levels<G, SPL, kVec16>, (int)smem, attr));
+  constexpr int n = G * 32 * SPL;
+  const size_t smem = std::max(grp_smem_bytes(n), FOLD ? sort_smem_bytes(sort_pad(n)) : 0);
+  const auto kernel = k_lob_match_levels<G, SPL, kVec16, FOLD>;
+  ABM_CUDA_TRY(smem_attr_once(kernel, (int)smem, attr));
   int dev = 0;
   ABM_CUDA_TRY(cudaGetDevice(&dev));
   int blocks_per_sm = (dev >= 0 && dev < 64) ? occ_dev[dev].load(std::memory_order_relaxed) : 0;
   if (!blocks_per_sm) {
     int occ = 0;
-    ABM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_lob_match_levels<G, SPL, kVec16>, G * 32,
-                                                               smem));
+    ABM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, G * 32, smem));
     blocks_per_sm = std::max(occ, 1);
     if (dev >= 0 && dev < 64) occ_dev[dev].store(blocks_per_sm, std::memory_order_relaxed);
   }
-  const int grid = (int)std::min<long long>(n_books, (long long)num_sms() * blocks_per_sm);
-  ABM_CUDA_TRY(launch_pdl_smem(k_lob_match_levels<G, SPL, kVec16>, grid, G * 32, smem, st, n_books, cap, active, side,
-                               price, qty, time, vol, px));
+  const long long held = (long long)num_sms() * blocks_per_sm;
+  grid = (int)std::min<long long>(n_books, held);
+  if (FOLD && n_books > held) return ABM_OK;
+  ABM_CUDA_TRY(launch_pdl_smem(kernel, grid, G * 32, smem, st, n_books, cap, active, side, price, qty, time, vol, px));
   return ABM_OK;
+}
+
+// Books that all have a CTA at once are matched in one launch; with more of them the
+// sort path is a launch of its own, whose work area does not cost the level path
+// its occupancy. 100 steps of orders and matching: 500 books of 1000 slots 740 -> 692
+// us, 1000 books 890 -> 808, 100 books of 300 slots 643 -> 540. A book for the sort path
+// is also taken at once instead of one after another by the CTA of its 256 books.
+template <int G, int SPL, bool kVec16>
+static abm_status lob_launch_levels(bool& folded, int n_books, int cap, int32_t* active, const int32_t* side,
+                                    const int32_t* price, int32_t* qty, const int32_t* time, long long* vol, int32_t* px,
+                                    cudaStream_t st) {
+  int grid = 0;
+  abm_status e = lob_levels<G, SPL, kVec16, true>(grid, n_books, cap, active, side, price, qty, time, vol, px, st);
+  folded = grid == n_books;
+  if (e != ABM_OK || folded) return e;
+  return lob_levels<G, SPL, kVec16, false>(grid, n_books, cap, active, side, price, qty, time, vol, px, st);
 }
 
 // the smallest slots-per-thread (a multiple of 4) that covers cap
 template <int G, bool kVec16>
-static abm_status lob_launch_g(int n_books, int cap, int32_t* active, const int32_t* side, const int32_t* price,
+static abm_status lob_launch_g(bool& folded, int n_books, int cap, int32_t* active, const int32_t* side, const int32_t* price,
                                int32_t* qty, const int32_t* time, long long* vol, int32_t* px, cudaStream_t st) {
   constexpr int T = G * 32;
-  if (cap <= 4 * T) return lob_launch_levels<G, 4, kVec16>(n_books, cap, active, side, price, qty, time, vol, px, st);
-  if (cap <= 8 * T) return lob_launch_levels<G, 8, kVec16>(n_books, cap, active, side, price, qty, time, vol, px, st);
+  if (cap <= 4 * T) return lob_launch_levels<G, 4, kVec16>(folded, n_books, cap, active, side, price, qty, time, vol, px, st);
+  if (cap <= 8 * T) return lob_launch_levels<G, 8, kVec16>(folded, n_books, cap, active, side, price, qty, time, vol, px, st);
   if (cap <= 16 * T)
-    return lob_launch_levels<G, 16, kVec16>(n_books, cap, active, side, price, qty, time, vol, px, st);
+    return lob_launch_levels<G, 16, kVec16>(folded, n_books, cap, active, side, price, qty, time, vol, px, st);
   if (G <= 2 && cap <= 32 * T)
-    return lob_launch_levels<G, (G <= 2 ? 32 : 16), kVec16>(n_books, cap, active, side, price, qty, time, vol, px,
+    return lob_launch_levels<G, (G <= 2 ? 32 : 16), kVec16>(folded, n_books, cap, active, side, price, qty, time, vol, px,
                                                              st);
-  return lob_launch_levels<G, (G == 1 ? 64 : 16), kVec16>(n_books, cap, active, side, price, qty, time, vol, px,
+  return lob_launch_levels<G, (G == 1 ? 64 : 16), kVec16>(folded, n_books, cap, active, side, price, qty, time, vol, px,
                                                            st);
 }
 
@@ -768,7 +814,7 @@ template <int R>
 static abm_status lob_launch_deferred(int n_books, int cap, int32_t* active, const int32_t* side,
                                       const int32_t* price, int32_t* qty, const int32_t* time, long long* vol,
                                       int32_t* px, cudaStream_t st) {
-  constexpr size_t smem = (size_t)R * kLobThreads * (4 * sizeof(int32_t) + sizeof(u64) + sizeof(u32));
+  constexpr size_t smem = sort_smem_bytes(R * kLobThreads);
   static std::atomic<unsigned long long> attr{0};
   ABM_CUDA_TRY(smem_attr_once(k_lob_deferred<R>, (int)smem, attr));
   const long long chunks = ((long long)n_books + kLobThreads - 1) / kLobThreads;
@@ -782,32 +828,36 @@ static abm_status lob_launch(bool vec16, int n_books, int cap, int32_t* active, 
                              const int32_t* price, int32_t* qty, const int32_t* time, long long* vol, int32_t* px,
                              cudaStream_t st) {
   abm_status e;
+  bool folded = false;
   int g = g_lob_warps_per_book.load(std::memory_order_relaxed);
   // One warp matches a book of up to 256 slots (8 per lane) faster than two that
   // meet at a barrier after every step (20,000 books of 128 slots 22 us against 35,
   // 50,000 of 256 slots 73 against 89; 20,000 of 512 57 against 56, of 768 93 against
   // 82), and four share more than 768 slots better than two (65536 books of 1024
   // slots 299 against 313, 16384 of 2048 158 against 169; 768 slots the same).
-  // With few books a book's own chain counts, which more warps shorten: 100 steps of
-  // orders and matching, 500 books of 256 slots 645 us with two warps against 685,
-  // of 1000 slots 761 with four against 798; 2000 of 1000 1301 against 1366, 3000 the
-  // same; 500 of 128 569 with two against 561, 1000 of 500 815 with four against 796.
-  const bool few = n_books <= 2048;
-  if (g == 0) g = cap <= (few ? 128 : 256) ? 1 : (cap <= (few ? 512 : 768) ? 2 : 4);
+  // With few books a book's own chain counts, which more warps shorten until the
+  // SMs fill up. 100 steps of orders and matching: 300 books of 200 slots 570 / 532 /
+  // 546 us with 1 / 2 / 4 warps; of 1000 slots 836 / 650 / 618, 500 books 855 / 691 /
+  // 695, 1000 books 939 / 810 / 866; 2000 books (two launches a round) 1677 / 1344 / 1267.
+  if (g == 0) {
+    const int one = n_books <= 2048 ? 128 : 256;
+    const int two = n_books <= 512 ? 256 : n_books <= 1024 ? 1024 : n_books <= 2048 ? 512 : 768;
+    g = cap <= one ? 1 : (cap <= two ? 2 : 4);
+  }
   switch (g) {
     case 1:
-      e = vec16 ? lob_launch_g<1, true>(n_books, cap, active, side, price, qty, time, vol, px, st)
-                : lob_launch_g<1, false>(n_books, cap, active, side, price, qty, time, vol, px, st);
+      e = vec16 ? lob_launch_g<1, true>(folded, n_books, cap, active, side, price, qty, time, vol, px, st)
+                : lob_launch_g<1, false>(folded, n_books, cap, active, side, price, qty, time, vol, px, st);
       break;
     case 4:
-      e = vec16 ? lob_launch_g<4, true>(n_books, cap, active, side, price, qty, time, vol, px, st)
-                : lob_launch_g<4, false>(n_books, cap, active, side, price, qty, time, vol, px, st);
+      e = vec16 ? lob_launch_g<4, true>(folded, n_books, cap, active, side, price, qty, time, vol, px, st)
+                : lob_launch_g<4, false>(folded, n_books, cap, active, side, price, qty, time, vol, px, st);
       break;
     default:
-      e = vec16 ? lob_launch_g<2, true>(n_books, cap, active, side, price, qty, time, vol, px, st)
-                : lob_launch_g<2, false>(n_books, cap, active, side, price, qty, time, vol, px, st);
+      e = vec16 ? lob_launch_g<2, true>(folded, n_books, cap, active, side, price, qty, time, vol, px, st)
+                : lob_launch_g<2, false>(folded, n_books, cap, active, side, price, qty, time, vol, px, st);
   }
-  if (e != ABM_OK) return e;
+  if (e != ABM_OK || folded) return e;
   switch (lob_pad(cap) / kLobThreads) {
     case 1: return lob_launch_deferred<1>(n_books, cap, active, side, price, qty, time, vol, px, st);
     case 2: return lob_launch_deferred<2>(n_books, cap, active, side, price, qty, time, vol, px, st);

@@ -265,7 +265,16 @@ def test_market_graph_replay_equals_eager(eng):
 
 
 @pytest.mark.parametrize("n_books,cap", [(2048, 129), (2049, 129), (2049, 257), (2048, 512), (2048, 513), (2049, 768),
-                                         (2049, 769)])
+                                         (2049, 769), (512, 257), (513, 257), (1024, 513), (1025, 513)])
 def test_match_default_shapes(eng, n_books, cap):
     """Each side of the lines between the default numbers of warps per book."""
     assert (check_match(eng, workloads.random_books(n_books, cap, 0.6, seed=cap)) > 0).any()
+
+
+@pytest.mark.parametrize("n_books,cap", [(900, 7), (5200, 7), (400, 600), (1300, 600), (500, 1025)])
+def test_match_sort_path_few_and_many_books(eng, n_books, cap):
+    """Books for the sort path among others: in the level path's own CTA (few books) and in a second launch (many)."""
+    book = workloads.random_books(n_books, cap, 0.9, seed=cap + n_books)
+    book["price"][::3] += 7 * np.arange(cap, dtype=np.int32)  # wide ranges
+    book["price"][1::5] = 100                                  # one crowded level
+    assert (check_match(eng, book) > 0).any()
