@@ -126,26 +126,6 @@ struct ScanArgs {
   const int32_t* list_base;  // OP_SELECT: device offset added to every rank (nullable)
 };
 
-// copy or add one record into a slot's fields
-__device__ __forceinline__ void apply_record(int32_t* dst, const int32_t* src, int F, bool add) {
-  if ((F & 3) == 0 && ((((uintptr_t)src) & 15) == 0)) {
-    for (int f = 0; f < F; f += 4) {
-      int4 r = *reinterpret_cast<const int4*>(src + f);
-      int4* d = reinterpret_cast<int4*>(dst + f);
-      if (add) {
-        int4 o = *d;
-        r.x = (int)((u32)o.x + (u32)r.x);
-        r.y = (int)((u32)o.y + (u32)r.y);
-        r.z = (int)((u32)o.z + (u32)r.z);
-        r.w = (int)((u32)o.w + (u32)r.w);
-      }
-      *d = r;
-    }
-  } else {
-    for (int f = 0; f < F; ++f) dst[f] = add ? (int)((u32)dst[f] + (u32)src[f]) : src[f];
-  }
-}
-
 template <int THREADS>
 __device__ __forceinline__ void block_sum2(u32& a, u32& b, u64* s_red) {
   u64 v = ((u64)a << 32) | b;
@@ -740,22 +720,126 @@ __device__ __forceinline__ void move_rows_v8(const ScanArgs& a, const int32_t* r
   }
 }
 
-// Pass 3: record j goes to (or is added to) the slot at rank j, four records
-// per thread in flight, all loads issued before the stores; coalesced record
-// reads, one field run written per slot (one 32-byte store for 8 fields).
-// Two CTAs of 256 threads per SM (96 registers) measured faster than three
-// with two rows in flight where rows are read.
+__device__ __forceinline__ int wrap_add(int a, int b) { return (int)((u32)a + (u32)b); }
+__device__ __forceinline__ int4 wrap_add(int4 a, int4 b) {
+  return make_int4(wrap_add(a.x, b.x), wrap_add(a.y, b.y), wrap_add(a.z, b.z), wrap_add(a.w, b.w));
+}
+__device__ __forceinline__ void set_word(int& v, int, int x) { v = x; }
+__device__ __forceinline__ void set_word(int4& v, int c, int x) {
+  if (c == 0) v.x = x;
+  else if (c == 1) v.y = x;
+  else if (c == 2) v.z = x;
+  else v.w = x;
+}
+
+// Rows of any other shape: records [0, n) of `rec` (or their rec_idx entries) in
+// units V (int4 where the fields are a multiple of four and the records 16-byte
+// aligned, else words), a warp taking 32 records and neighbouring lanes
+// neighbouring units: a record's words are read and written together, U of a
+// lane's in flight. (A record per thread, field by field: the loads of one warp 32
+// records apart, each waited for before its store. 199,000 records of 11 fields
+// added to a set of 931,561 slots 89 -> 9 us;
+// the fused call's 1.4 M moves of 12 fields on 4 M slots 76 -> 64.)
+template <typename V, bool ADDROW, bool STAMP, bool IDX>
+__device__ __forceinline__ void move_rows(const ScanArgs& a, const int32_t* rec, const int32_t* list, int n, int id_field,
+                                          int id0) {
+  constexpr int W = sizeof(V) / 4, U = 16 / (2 * W) > 4 ? 8 : 4;
+  const SlabDev& s = a.s;
+  const V* const src = reinterpret_cast<const V*>(rec);
+  V* const dst = reinterpret_cast<V*>(s.fields);
+  const int F = s.F / W, Fp = s.Fp / W, lane = threadIdx.x & 31;
+  if (F == 1) {  // a unit a row: U records per thread in flight
+    const int stride = gridDim.x * blockDim.x;
+    for (int j0 = blockIdx.x * blockDim.x + threadIdx.x; j0 < n; j0 += U * stride) {
+      V v[U], o[U];
+      int slot[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + u * stride;
+        slot[u] = j < n ? list[j] : -1;
+        if (j < n && !in_range(slot[u], s.cap, s.err)) slot[u] = -1;
+        if (slot[u] >= 0) v[u] = __ldg(src + (IDX ? s.rec_idx[j] : j));
+        if (STAMP && slot[u] >= 0) set_word(v[u], id_field, (int)((u32)id0 + (u32)j));
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (ADDROW && slot[u] >= 0) o[u] = dst[(size_t)slot[u] * Fp];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (slot[u] >= 0) dst[(size_t)slot[u] * Fp] = ADDROW ? wrap_add(o[u], v[u]) : v[u];
+    }
+    return;
+  }
+  const int rq = 32 / F, rm = 32 % F, r0 = lane / F, f0 = lane % F;
+  const int warps = gridDim.x * (blockDim.x >> 5);
+  for (int j0 = 32 * (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); j0 < n; j0 += 32 * warps) {
+    const int m = min(32, n - j0);
+    int slot = -1, from = j0 + lane;
+    if (lane < m) {
+      slot = list[j0 + lane];
+      if (!in_range(slot, s.cap, s.err)) slot = -1;
+      if (IDX) from = s.rec_idx[j0 + lane];
+    }
+    int r = r0, f = f0;
+    for (int e0 = 0; e0 < m * F; e0 += 32 * U) {
+      V v[U], o[U];
+      size_t at[U];
+      bool ok[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int sl = __shfl_sync(0xFFFFFFFFu, slot, r & 31), sr = __shfl_sync(0xFFFFFFFFu, from, r & 31);
+        ok[u] = e0 + 32 * u + lane < m * F && sl >= 0;
+        at[u] = (size_t)(ok[u] ? sl : 0) * Fp + f;
+        if (ok[u]) v[u] = __ldg(src + (size_t)sr * F + f);
+        if (ADDROW && ok[u]) o[u] = dst[at[u]];
+        if (STAMP && ok[u] && f == id_field / W) set_word(v[u], id_field % W, (int)((u32)id0 + (u32)(j0 + r)));
+        r += rq;
+        f += rm;
+        if (f >= F) {
+          f -= F;
+          ++r;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (ok[u]) dst[at[u]] = ADDROW ? wrap_add(o[u], v[u]) : v[u];
+    }
+  }
+}
+
+template <int OP, typename V>
+__device__ __forceinline__ void apply_rows(const ScanArgs& a, int ra, int rb, int id0) {
+  if (OP == OP_UPDATE) {
+    const bool idx = a.use_rec_idx != 0;
+    if (a.op_kind == ABM_OP_ADD) {
+      if (idx) move_rows<V, true, false, true>(a, a.rec, a.list_a, ra, -1, 0);
+      else move_rows<V, true, false, false>(a, a.rec, a.list_a, ra, -1, 0);
+    } else {
+      if (idx) move_rows<V, false, false, true>(a, a.rec, a.list_a, ra, -1, 0);
+      else move_rows<V, false, false, false>(a, a.rec, a.list_a, ra, -1, 0);
+    }
+  } else if (OP == OP_ADD && a.id_field >= 0) {
+    move_rows<V, false, true, false>(a, a.rec, a.list_a, ra, a.id_field, id0);
+  } else {
+    move_rows<V, false, false, false>(a, a.rec, a.list_a, ra, -1, 0);
+  }
+  if (OP == OP_FUSED) move_rows<V, true, false, false>(a, a.rec2, a.list_b, rb, -1, 0);
+}
+
+// Pass 3: record j goes to (or is added to) the slot at rank j, several in flight
+// per thread, all loads issued before the stores; coalesced record reads, one
+// field run written per slot (one 32-byte store for 8 fields). Two CTAs of 256
+// threads per SM (96 registers) measured faster than three with two rows in flight
+// where rows are read.
 template <int OP>
 __global__ void __launch_bounds__(256, 2) k_apply(ScanArgs a) {
   griddep_wait();
   const SlabDev& s = a.s;
   const int ra = s.meta[0], rb = s.meta[1];
   const int id0 = s.meta[2];
-  const int total = ra + rb;
-  const int stride = gridDim.x * blockDim.x;
-  const bool f8 = s.F == 8 && s.Fp == 8 && ((((uintptr_t)a.rec) | ((uintptr_t)a.rec2)) & 15) == 0;
+  const uintptr_t al = (uintptr_t)a.rec | (uintptr_t)a.rec2;
   // 8 fields, records 32-byte aligned (the rows always are): whole rows per instruction
-  if (f8 && ((((uintptr_t)a.rec) | ((uintptr_t)a.rec2) | ((uintptr_t)s.fields)) & 31) == 0) {
+  if (s.F == 8 && s.Fp == 8 && ((al | (uintptr_t)s.fields) & 31) == 0) {
     if (OP == OP_UPDATE) {
       const bool idx = a.use_rec_idx != 0;
       if (a.op_kind == ABM_OP_ADD) {
@@ -771,79 +855,10 @@ __global__ void __launch_bounds__(256, 2) k_apply(ScanArgs a) {
       move_rows_v8<4, false, false, false>(a, a.rec, a.list_a, ra, -1, 0);
     }
     if (OP == OP_FUSED) move_rows_v8<4, true, false, false>(a, a.rec2, a.list_b, rb, -1, 0);
-    return;
-  }
-  for (int j0 = blockIdx.x * blockDim.x + threadIdx.x; j0 < total; j0 += 4 * stride) {
-    if (f8) {
-      int slot[4];
-      int4 r0[4], r1[4];
-      bool add[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int j = j0 + u * stride;
-        slot[u] = -1;
-        add[u] = false;
-        if (j < total) {
-          const int32_t* src;
-          if (j < ra) {
-            slot[u] = a.list_a[j];
-            const int rj = (OP == OP_UPDATE && a.use_rec_idx) ? s.rec_idx[j] : j;
-            src = a.rec + (size_t)rj * 8;
-            add[u] = OP == OP_UPDATE && a.op_kind == ABM_OP_ADD;
-          } else {
-            slot[u] = a.list_b[j - ra];
-            src = a.rec2 + (size_t)(j - ra) * 8;
-            add[u] = true;
-          }
-          r0[u] = __ldg(reinterpret_cast<const int4*>(src));
-          r1[u] = __ldg(reinterpret_cast<const int4*>(src) + 1);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (slot[u] < 0) continue;
-        int4* d = reinterpret_cast<int4*>(s.fields + (size_t)slot[u] * 8);
-        if (OP == OP_ADD && a.id_field >= 0) {  // stamp the id into the record before storing it
-          const int j = j0 + u * stride;
-          const int id = (int)((u32)id0 + (u32)j);
-          int4& r = a.id_field < 4 ? r0[u] : r1[u];
-          switch (a.id_field & 3) {
-            case 0: r.x = id; break;
-            case 1: r.y = id; break;
-            case 2: r.z = id; break;
-            default: r.w = id; break;
-          }
-        }
-        if (add[u]) {
-          const int4 o0 = d[0], o1 = d[1];
-          r0[u] = make_int4((int)((u32)o0.x + (u32)r0[u].x), (int)((u32)o0.y + (u32)r0[u].y),
-                            (int)((u32)o0.z + (u32)r0[u].z), (int)((u32)o0.w + (u32)r0[u].w));
-          r1[u] = make_int4((int)((u32)o1.x + (u32)r1[u].x), (int)((u32)o1.y + (u32)r1[u].y),
-                            (int)((u32)o1.z + (u32)r1[u].z), (int)((u32)o1.w + (u32)r1[u].w));
-        }
-        d[0] = r0[u];
-        d[1] = r1[u];
-      }
-      continue;
-    }
-    for (int u = 0; u < 4; ++u) {
-      const int j = j0 + u * stride;
-      if (j >= total) break;
-      if (j < ra) {
-        const int slot = a.list_a[j];
-        int32_t* dst = s.fields + (size_t)slot * s.Fp;
-        if (OP == OP_UPDATE) {
-          const int rj = a.use_rec_idx ? s.rec_idx[j] : j;
-          apply_record(dst, a.rec + (size_t)rj * s.F, s.F, a.op_kind == ABM_OP_ADD);
-        } else {
-          apply_record(dst, a.rec + (size_t)j * s.F, s.F, false);
-          if (OP == OP_ADD && a.id_field >= 0) dst[a.id_field] = (int)((u32)id0 + (u32)j);
-        }
-      } else {
-        const int i = j - ra;
-        apply_record(s.fields + (size_t)a.list_b[i] * s.Fp, a.rec2 + (size_t)i * s.F, s.F, true);
-      }
-    }
+  } else if ((s.F & 3) == 0 && (al & 15) == 0) {
+    apply_rows<OP, int4>(a, ra, rb, id0);
+  } else {
+    apply_rows<OP, int>(a, ra, rb, id0);
   }
 }
 
@@ -1603,7 +1618,7 @@ static abm_status launch_scan(abm_slab* s, const ScanArgs& a, bool aux, cudaStre
     }
   }
   if (OP != OP_REMOVE) ABM_CUDA_TRY(launch_pdl(k_scatter<OP, THREADS>, b.G, THREADS, st, b));
-  if (OP == OP_ADD || OP == OP_UPDATE || OP == OP_FUSED)
+  if constexpr (OP == OP_ADD || OP == OP_UPDATE || OP == OP_FUSED)
     ABM_CUDA_TRY(launch_pdl(k_apply<OP>, apply_grid<OP>(), 256, st, b));
   return ABM_OK;
 }

@@ -606,3 +606,59 @@ def test_resolve_ties_and_hot_resources(eng, M, R, levels):
     np.testing.assert_array_equal(np_of(w), want)
     np.testing.assert_array_equal(np_of(isw), won)
     assert torch.all(r.table == -1)
+
+
+@pytest.mark.parametrize("F,shift", [(1, 0), (2, 1), (4, 0), (5, 0), (8, 1), (8, 4), (11, 3), (12, 0), (12, 2), (13, 0),
+                                     (16, 4), (16, 1)])
+def test_row_shapes(eng, F, shift):
+    """Whole numbers, so exact: rows of every width and records at every alignment above the one-launch sizes."""
+    from paper_2508_16508_gb300 import abm
+    n, k = 262_150, 40_003
+    rng = np.random.default_rng(F * 8 + shift)
+    s = eng.Slab(n, F, seed=9)
+    act = (rng.random(n) < 0.5).astype(np.int32)
+    fld = rng.integers(-50, 50, (F, n)).astype(np.int32)
+    s.write(-1, torch.from_numpy(act).cuda())
+    for f in range(F):
+        s.write(f, torch.from_numpy(fld[f]).cuda())
+    rec = rng.integers(-2**31, 2**31, (k, F)).astype(np.int32)
+    rmask = (rng.random(k) < 0.5).astype(np.int32)
+    dev = torch.zeros(k * F + shift, dtype=torch.int32, device="cuda")[shift:].view(k, F)
+    dev.copy_(torch.from_numpy(rec))
+    for mask, op in ((None, abm.OP_ADD), (None, abm.OP_SET), (rmask, abm.OP_ADD), (rmask, abm.OP_SET)):
+        sel = np.flatnonzero((act != 0) & (fld[0] >= -10))
+        rows = rec if mask is None else rec[mask != 0]
+        r = min(len(sel), len(rows))
+        s.update_distinct(abm.pred(abm.PRED_FIELD, field=0, cmp=abm.CMP_GE, value=-10), dev,
+                          None if mask is None else torch.from_numpy(mask).cuda(), op=op)
+        for f in range(F):
+            fld[f][sel[:r]] = rows[:r, f] + (fld[f][sel[:r]] if op == abm.OP_ADD else 0)
+    for id_field in (-1, 0, F - 1):
+        free = np.flatnonzero(act == 0)[:k]
+        first = s.counters()["next_id"]
+        s.add(dev, id_field=id_field)
+        for f in range(F):
+            fld[f][free] = rec[:len(free), f] if f != id_field else first + np.arange(len(free))
+        act[free] = 1
+    for f in range(F):
+        np.testing.assert_array_equal(np_of(s.read(f)), fld[f], err_msg=str(f))
+    np.testing.assert_array_equal(np_of(s.read(-1)) != 0, act != 0)
+    s.check()
+
+
+@pytest.mark.parametrize("F", [1, 4, 5, 7])
+def test_selective_update_row_shapes(eng, F):
+    """The same for the one call of the three operations, against the oracle."""
+    from paper_2508_16508_gb300 import abm
+    n, p = 270_001, 0.2
+    T, k = workloads.threshold(p), workloads.k_for(p, n)
+    s, o = eng.Slab(n, F, seed=4, init=abm.INIT_HALF_LIVE), oracle.Slab(n, F)
+    o.c1_init(seed=4)
+    for step in range(3):
+        s.selective_update(step, T, s.philox_records(step, abm.P_NEWREC0, abm.P_NEWREC1, k),
+                           s.philox_records(step, abm.P_DELTA0, abm.P_DELTA1, k))
+        o.c1_call(step, T, k, seed=4)
+    np.testing.assert_array_equal(np_of(s.read(-1)) != 0, o.active != 0)
+    for f in range(F):
+        np.testing.assert_array_equal(np_of(s.read(f)), o.fields[f])
+    s.check()
