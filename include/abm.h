@@ -23,6 +23,7 @@
  *  - Spin-waits inside kernels are bounded. A wait that runs out sets a
  *    device error word and the kernel returns; abm_*_check() reports
  *    ABM_ERR_DEVICE_TIMEOUT and the handle's results are then undefined.
+ *    (Hardware barriers of a CTA or a cluster wait for no flag.)
  *  - Check build (libabm_check.so, the same sources compiled with -DABM_CHECK,
  *    slower): every data-dependent index (a slot from a list, a cell from an
  *    agent record, a parent, a victim) is tested before use; a violation is

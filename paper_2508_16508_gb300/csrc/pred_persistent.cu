@@ -1116,7 +1116,15 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
       return grid_sync(ps.bar, w.err, bar_target);
     }
   };
-  if (CLUSTER && ld_relaxed32(reinterpret_cast<const u32*>(w.err)) != 0u) return;  // (an earlier launch's: the same in every thread)
+  if constexpr (CLUSTER) {
+    // An error of an earlier launch ends this one, as the grid barrier does. All CTAs read the word before any of them
+    // can record an error of this launch (the barrier), and one thread reads it for its CTA: every thread of the cluster
+    // decides alike, or those that stay would wait at the teams' barriers for those that left.
+    __shared__ u32 s_err;
+    if (threadIdx.x == 0) s_err = ld_relaxed32(reinterpret_cast<const u32*>(w.err));
+    sync();
+    if (s_err != 0u) return;
+  }
   clk.start();
   // Wolf ranks of step t-1 run beside the sheep moves of step t, and the wolf
   // moves of step t beside the sheep ranks: neither needs the other's

@@ -88,3 +88,40 @@ print(json.dumps(out))
     assert r["clean"] == abm.OK
     assert r["damaged"] == abm.ERR_CHECK
     assert (r["index_in"], r["index_out"], r["index_neg"]) == (abm.OK, abm.ERR_CHECK, abm.ERR_CHECK)
+
+
+def run_child(code: str) -> dict:
+    env = dict(os.environ)
+    env["ABM_LIBRARY"] = "check"
+    head = "import json, sys, torch\nsys.path.insert(0, %r)\nimport workloads\nfrom paper_2508_16508_gb300 import abm, engine\n"
+    p = subprocess.run([sys.executable, "-c", head % os.path.dirname(HERE) + code], env=env, capture_output=True, text=True,
+                       timeout=300)
+    assert p.returncode == 0, p.stderr[-3000:]
+    return json.loads(p.stdout.strip().splitlines()[-1])
+
+
+BAD_CELLS = r'''
+L, st = abm.lib(), abm.stream_handle()
+side = 100
+# 4500 slots: the launch of one cluster
+w = engine.World(side, 3, 0, workloads.predation_params(sheep_repro=%r, wolf_repro=0), (20000, 9000), (4000, 500))
+v = w.slab(0)
+cells = v.read(0)
+cells[:4000:7] = side * side + 5
+v.write(0, cells)
+w.slab_commit(0)
+out = {}
+for k in range(2):
+    w.step(3)
+    out[f"status{k}"] = int(L.abm_world_check(w.h, st))
+    out[f"step{k}"] = w.counters()["step"]
+print(json.dumps(out))
+'''
+
+
+def test_cluster_launch_decides_on_errors_as_one():
+    """Check build: cells outside the lattice are recorded in the first phase of the first step, while later CTAs of
+    the cluster may still be starting. The launch runs to its end; the next one, which finds the error, ends at once."""
+    from paper_2508_16508_gb300 import abm
+    r = run_child(BAD_CELLS % 0)
+    assert r == dict(status0=abm.ERR_CHECK, status1=abm.ERR_CHECK, step0=3, step1=3)
