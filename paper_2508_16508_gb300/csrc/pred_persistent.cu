@@ -997,6 +997,7 @@ __device__ __forceinline__ void rank_births(const WorldDev& w, int t, int ext, i
     sp.agent[p].y = pa.y - half;
     sp.agent[slot] = make_int4(pa.x, half, (int)((u32)id0 + i), 0);
     sp.active[slot] = 1;
+    if (!in_range(pa.x, w.ncells, w.err)) continue;  // check builds: the parent's cell (the meal phase took it for cell 0)
     const u64 key = claim_key(draw(w.seed, w.model, (u32)t, (u32)slot, ABM_P_VICTIM, 0u), slot);
     if (w.variant & ABM_VARIANT_MANY_WOLVES)
       list_push(w.victim, w.snext, w.skey, pa.x, slot, t, key);

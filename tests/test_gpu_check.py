@@ -125,3 +125,11 @@ def test_cluster_launch_decides_on_errors_as_one():
     from paper_2508_16508_gb300 import abm
     r = run_child(BAD_CELLS % 0)
     assert r == dict(status0=abm.ERR_CHECK, status1=abm.ERR_CHECK, step0=3, step1=3)
+
+
+def test_births_on_bad_cells_stay_inside():
+    """Check build: a parent whose cell lies outside the lattice gives birth without touching that cell's entry; the
+    violation is recorded and the canaries of both species stay whole."""
+    from paper_2508_16508_gb300 import abm
+    r = run_child(BAD_CELLS % 0.9)
+    assert (r["status0"], r["status1"], r["step0"]) == (abm.ERR_CHECK, abm.ERR_CHECK, 3)
