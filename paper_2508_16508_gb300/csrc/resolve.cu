@@ -27,9 +27,9 @@ __global__ void k_table_fill(u64* table, int R) {
 }
 
 // A place of the shared table belongs to the first resource that takes it. A
-// chunk of claims goes through three rounds with a barrier after each: take
-// places; lower the priorities (32-bit shared atomics, only by claims below the
-// priority of the chunks before: an equal one loses to the earlier index);
+// chunk of claims goes through two rounds with a barrier after each: take
+// places and lower the priorities (32-bit shared atomics, only by claims below the
+// priority of the chunks before: an equal one loses to the earlier index); then
 // lower the index among the claims that hold a new priority. 4 M Zipf(1.1) claims
 // on 262144 resources: 33 us, bound by the scattered global atomics that are
 // left (about two million; reading an entry first to spare its atomic costs as
@@ -38,6 +38,26 @@ __global__ void k_table_fill(u64* table, int R) {
 // instead of 62 us for the whole call where all resources are equally popular. A
 // shared filter of seen priorities with every unbeaten claim going to global memory:
 // 70 us, the hot entries' first claims serialise in L2.)
+//
+// A resource that finds its place taken has a second one: with one place, two hot
+// resources that share it cost one global atomic per claim on the loser, all on one
+// address (4 M claims on two such resources 713 us, now 18). Only a chunk's first
+// kResThreads claims take second places, which is enough for a resource that is
+// hot: cold ones cost more in the table than as an atomic (all claims taking them:
+// 4 M claims on resources of equal popularity 42.9 us against 41.8; one place 41.1).
+// A resource's two places; the complement moves resource 0, which every multiplier leaves at 0.
+__device__ __forceinline__ int first_place(int r) { return (int)(((u32)r * 2654435761u) >> (32 - kHashBits)); }
+__device__ __forceinline__ int second_place(int r) {
+  const int h = (int)((~(u32)r * 2246822519u) >> (32 - kHashBits));
+  return h == first_place(r) ? h ^ (kHash / 2) : h;
+}
+// place h, if it is resource r's (it was, or it was free and now is), else -1
+__device__ __forceinline__ int take_place(volatile int* s_res, int r, int h) {
+  int v = s_res[h];
+  if (v == -1) v = atomicCAS(const_cast<int*>(s_res) + h, -1, r);
+  return v == r || v == -1 ? h : -1;
+}
+
 __global__ void __launch_bounds__(kResThreads, 2) k_claims(const int32_t* __restrict__ res,
                                                            const u32* __restrict__ prio, int M, int R, u64* table) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -63,37 +83,33 @@ __global__ void __launch_bounds__(kResThreads, 2) k_claims(const int32_t* __rest
       p[j] = m < hi ? prio[m] : 0u;
       if (r[j] >= R) r[j] = -1;
     }
+    int h[kResPerThread];  // the place of the claim's resource, -1: no claim, none, or already beaten
 #pragma unroll
     for (int j = 0; j < kResPerThread; ++j) {
-      const u32 h = ((u32)r[j] * 2654435761u) >> (32 - kHashBits);
-      if (r[j] >= 0 && s_res[h] == -1) s_res[h] = r[j];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < kResPerThread; ++j) {
+      h[j] = -1;
       if (r[j] < 0) continue;
-      const u32 h = ((u32)r[j] * 2654435761u) >> (32 - kHashBits);
-      const u32 m = (u32)m0 + j * kResThreads + threadIdx.x;
-      if (s_res[h] != r[j]) {
-        atomicMin(&table[r[j]], ((u64)p[j] << 32) | m);
-        r[j] = -1;
-      } else if (p[j] < *(volatile u32*)&s_prio[h] || *(volatile u32*)&s_idx[h] == 0xFFFFFFFFu) {
+      int at = take_place(s_res, r[j], first_place(r[j]));
+      if (at < 0) {
+        const int h2 = second_place(r[j]);
+        at = j == 0 ? take_place(s_res, r[j], h2) : (s_res[h2] == r[j] ? h2 : -1);
+      }
+      if (at < 0) {
+        atomicMin(&table[r[j]], ((u64)p[j] << 32) | ((u32)m0 + j * kResThreads + threadIdx.x));
+      } else if (p[j] < *(volatile u32*)&s_prio[at] || *(volatile u32*)&s_idx[at] == 0xFFFFFFFFu) {
         // below every earlier chunk's claim (or none came before, or this chunk is lowering the entry already). The
         // index of the priority that no longer counts goes first, so that whoever sees a priority of this chunk sees
         // that too and stays in
-        *(volatile u32*)&s_idx[h] = 0xFFFFFFFFu;
+        *(volatile u32*)&s_idx[at] = 0xFFFFFFFFu;
         __threadfence_block();
-        atomicMin(&s_prio[h], p[j]);
-      } else {
-        r[j] = -1;
+        atomicMin(&s_prio[at], p[j]);
+        h[j] = at;
       }
     }
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < kResPerThread; ++j) {
-      if (r[j] < 0) continue;
-      const u32 h = ((u32)r[j] * 2654435761u) >> (32 - kHashBits);
-      if (p[j] == *(volatile u32*)&s_prio[h]) atomicMin(&s_idx[h], (u32)m0 + j * kResThreads + threadIdx.x);
+      if (h[j] < 0) continue;
+      if (p[j] == *(volatile u32*)&s_prio[h[j]]) atomicMin(&s_idx[h[j]], (u32)m0 + j * kResThreads + threadIdx.x);
     }
     __syncthreads();
   }

@@ -608,6 +608,32 @@ def test_resolve_ties_and_hot_resources(eng, M, R, levels):
     assert torch.all(r.table == -1)
 
 
+def same_place(first, count, R):
+    """Resources of one place of k_claims' shared table, `first` among them: 13 bits of a product."""
+    place = ((np.arange(R, dtype=np.uint64) * 2654435761) & 0xFFFFFFFF) >> 19
+    return np.nonzero(place == place[first])[0][:count].astype(np.int32)
+
+
+@pytest.mark.parametrize("M", [1, 1023, 1025, 4097, 50_000, 2_000_003])
+@pytest.mark.parametrize("first,count,crowd", [(0, 2, 0.0), (0, 5, 0.3), (5, 3, 0.9), (777, 31, 0.0)])
+def test_resolve_resources_that_share_a_place(eng, M, first, count, crowd):
+    """Whole numbers, so exact: hot resources that all have the same first place of the shared table, alone and among
+    claims on all others, with ties and claims outside the range."""
+    R = 1 << 18
+    rng = np.random.default_rng(M + count)
+    hot = same_place(first, count, R)
+    assert len(hot) == count
+    res = np.where(rng.random(M) < crowd, rng.integers(-2, R + 2, M), hot[rng.integers(0, count, M)]).astype(np.int32)
+    prio = rng.integers(0, 1000, M).astype(np.uint32)
+    r = eng.Resolver(R)
+    isw = torch.empty(M, dtype=torch.uint8, device="cuda")
+    w = r(torch.from_numpy(res).cuda(), torch.from_numpy(prio.view(np.int32)).cuda(), isw)
+    ow, oisw = oracle.resolve(res, prio, R)
+    np.testing.assert_array_equal(np_of(w), ow)
+    np.testing.assert_array_equal(np_of(isw), oisw)
+    assert torch.all(r.table == -1)
+
+
 @pytest.mark.parametrize("F,shift", [(1, 0), (2, 1), (4, 0), (5, 0), (8, 1), (8, 4), (11, 3), (12, 0), (12, 2), (13, 0),
                                      (16, 4), (16, 1)])
 def test_row_shapes(eng, F, shift):
