@@ -106,6 +106,7 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
   if (threadIdx.x == 0) *s_v = 0ull;
   // key: side | price (bids descending; prices positive) | time (signed
   // order); ties by slot, empty slots (slot + n) last
+#pragma unroll 4
   for (int i = threadIdx.x; i < n; i += T) {
     u64 k = kNoKey;
     u32 r = (u32)(i + n);
@@ -119,20 +120,33 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
     ord[i] = r;
   }
   __syncthreads();
+  // bitonic sort, a thread's pairs four at a time: all their loads before the first exchange
   for (int kk = 2; kk <= n; kk <<= 1) {
     for (int j = kk >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < n; i += T) {
-        const int l = i ^ j;
-        if (l > i) {
+      for (int p0 = threadIdx.x; p0 < n / 2; p0 += 4 * T) {
+        u64 ka[4], kb[4];
+        u32 oa[4], ob[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int p = p0 + u * T;
+          if (p >= n / 2) continue;
+          const int i = 2 * p - (p & (j - 1));  // the pair's lower entry: p with a zero bit put in at j
+          ka[u] = key[i];
+          kb[u] = key[i + j];
+          oa[u] = ord[i];
+          ob[u] = ord[i + j];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int p = p0 + u * T;
+          if (p >= n / 2) continue;
+          const int i = 2 * p - (p & (j - 1));
           const bool up = (i & kk) == 0;
-          const bool gt = key[i] > key[l] || (key[i] == key[l] && ord[i] > ord[l]);
-          if (gt == up) {
-            const u64 tk = key[i];
-            key[i] = key[l];
-            key[l] = tk;
-            const u32 to = ord[i];
-            ord[i] = ord[l];
-            ord[l] = to;
+          if ((ka[u] > kb[u] || (ka[u] == kb[u] && oa[u] > ob[u])) == up) {
+            key[i] = kb[u];
+            key[i + j] = ka[u];
+            ord[i] = ob[u];
+            ord[i + j] = oa[u];
           }
         }
       }
@@ -152,17 +166,20 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
     run += e < nl ? (u64)(u32)d.qt[ord[e]] : 0ull;
     cum[e] = run;
   }
+  int32_t* const spx = d.sid;  // prices in sorted order (the sides are in the order now)
+#pragma unroll 4
+  for (int e = threadIdx.x; e < nl; e += T) spx[e] = d.px[ord[e]];
   __syncthreads();
   const u64 bid_total = nbid > 0 ? cum[nbid - 1] : 0ull;
   // V: bid i may trade the shares in (QB_{i-1}, min(QB_i, QA(J_i))], J_i = the
   // asks priced at or below it
   u64 vbest = 0;
   for (int i = threadIdx.x; i < nbid; i += T) {
-    const int32_t p = d.px[ord[i]];
+    const int32_t p = spx[i];
     int lo = 0, hi = nask;
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if (d.px[ord[nbid + mid]] <= p) lo = mid + 1;
+      if (spx[nbid + mid] <= p) lo = mid + 1;
       else hi = mid;
     }
     const u64 qa = lo > 0 ? cum[nbid + lo - 1] - bid_total : 0ull;
@@ -183,7 +200,7 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
     const u64 end = is_bid ? cum[e] : cum[e] - bid_total;
     const u64 q = end - start;
     const u64 fill = V > start ? (V - start < q ? V - start : q) : 0ull;
-    if (!is_bid && V > start && V <= end) out_price[b] = d.px[ord[e]];
+    if (!is_bid && V > start && V <= end) out_price[b] = spx[e];
     if (fill || q == 0) {
       const u32 s = ord[e];
       const int32_t left = (int32_t)(q - fill);
@@ -194,6 +211,10 @@ __device__ void lob_match_sorted(const LobBook& d, int n, int b, int cap, int nb
 }
 
 // Loads a book and matches it by the sort path; `work`: 28 bytes per padded slot.
+// A CTA of the level path has 32 to 128 threads for it, so each of them keeps several
+// accesses in flight: one pair after another, one wide book of 1000 slots took 73 us
+// (500 books) and 137 (1000 books), of 60 slots 42; now 34, 60 and 13 (by 256 threads in a
+// launch of their own before: 56, 58 and 17).
 template <int T>
 __device__ __noinline__ void lob_sort_book(int n, int b, int cap, int32_t* active, const int32_t* __restrict__ side,
                                            const int32_t* __restrict__ price, int32_t* qty,
@@ -205,7 +226,8 @@ __device__ __noinline__ void lob_sort_book(int n, int b, int cap, int32_t* activ
   const LobBook d{w, w + n, w + 2 * n, w + 3 * n};
   u64* key = reinterpret_cast<u64*>(w + 4 * n);
   const size_t o = (size_t)b * cap;
-  int nbid = 0, nask = 0;
+  u64 cnt = 0;  // live bids | asks << 32
+#pragma unroll 4
   for (int i = threadIdx.x; i < n; i += T) {
     const bool in = i < cap;
     const int32_t a = in ? active[o + i] : 0;
@@ -214,9 +236,10 @@ __device__ __noinline__ void lob_sort_book(int n, int b, int cap, int32_t* activ
     d.sid[i] = s;
     d.px[i] = in ? price[o + i] : 0;
     d.qt[i] = in ? qty[o + i] : 0;
-    nbid += __syncthreads_count(a != 0 && s == 0);
-    nask += __syncthreads_count(a != 0 && s != 0);
+    if (a != 0) cnt += s == 0 ? 1ull : 1ull << 32;
   }
+  block_sum_scan_u64<T>(cnt, cnt, s_scan);
+  const int nbid = (int)(u32)cnt, nask = (int)(cnt >> 32);
   lob_match_sorted<T>(d, n, b, cap, nbid, nask, active, qty, time, out_volume, out_price, key,
                       reinterpret_cast<u32*>(key + n), s_scan, &s_v);
   __syncthreads();  // the work area is used again
@@ -229,8 +252,7 @@ __host__ __device__ constexpr size_t grp_smem_bytes(int n) {
   return 16 * (size_t)n + 2 * kWarpLevels * sizeof(u32) + 2 * kWarpMarginal * (sizeof(u32) + sizeof(u64));
 }
 
-// Padded slots of the sort path for a book of up to n (a power of two) slots, and its work area
-__host__ __device__ constexpr int sort_pad(int n) { return n < kLobThreads ? kLobThreads : n; }
+// The sort path's work area for n padded slots
 __host__ __device__ constexpr size_t sort_smem_bytes(int pad) {
   return (size_t)pad * (4 * sizeof(int32_t) + sizeof(u64) + sizeof(u32));
 }
@@ -366,8 +388,8 @@ __device__ __forceinline__ void grp_stage(int32_t* s_act, int n, int b, int cap,
 // handed to it at the end.
 //
 // Bound by the chain of a book's dependent steps at the occupancy that the staged
-// words allow (11 CTAs per SM): 65536 books of 1024 slots take 299 us with four
-// warps per book and move 1.5 GB (232 us at the copy rate); issue slots are half
+// words allow (10 CTAs per SM): 65536 books of 1024 slots take 299 us with four
+// warps per book and move 1.66 GB (249 us at the copy rate); issue slots are half
 // full. Levels written back and counted, marginal orders listed and fetched one by
 // one: 326 us with two warps, and 454 before the loops over the slots were cut to
 // what each needs. Loads straight into registers with the next book prefetched
@@ -638,7 +660,7 @@ __global__ void __launch_bounds__(G * 32)
   if constexpr (FOLD) {
     if (defer >= 0) {
       grp_sync<G>();  // the level path's shared memory becomes the work area
-      lob_sort_book<T>(sort_pad(T * SPL), defer, cap, active, side, price, qty, time, out_volume, out_price, lob_smem);
+      lob_sort_book<T>(n, defer, cap, active, side, price, qty, time, out_volume, out_price, lob_smem);
     }
   }
 }
@@ -759,7 +781,7 @@ static abm_status lob_levels(int& grid, int n_books, int cap, int32_t* active, c
   static std::atomic<unsigned long long> attr{0};
   static std::atomic<int> occ_dev[64];
   constexpr int n = G * 32 * SPL;
-  const size_t smem = std::max(grp_smem_bytes(n), FOLD ? sort_smem_bytes(sort_pad(n)) : 0);
+  const size_t smem = std::max(grp_smem_bytes(n), FOLD ? sort_smem_bytes(n) : 0);
   const auto kernel = k_lob_match_levels<G, SPL, kVec16, FOLD>;
   ABM_CUDA_TRY(smem_attr_once(kernel, (int)smem, attr));
   int dev = 0;

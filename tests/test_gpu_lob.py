@@ -278,3 +278,22 @@ def test_match_sort_path_few_and_many_books(eng, n_books, cap):
     book["price"][::3] += 7 * np.arange(cap, dtype=np.int32)  # wide ranges
     book["price"][1::5] = 100                                  # one crowded level
     assert (check_match(eng, book) > 0).any()
+
+
+@pytest.mark.parametrize("warps", [0, 1, 2, 4])
+@pytest.mark.parametrize("n_books,cap", [(40, 1), (40, 3), (40, 128), (40, 129), (40, 512), (40, 1024), (40, 1025), (40, 2048),
+                                         (9000, 128), (4000, 1024)])
+def test_match_sort_path_sizes(eng, warps, n_books, cap):
+    """Wide books only, at the padded sizes of the sort path: full and nearly full, many equal prices and times (so
+    that slots decide), quantities up to the largest int32."""
+    rng = np.random.default_rng(cap + n_books + warps)
+    book = workloads.random_books(n_books, cap, 0.97, seed=cap + n_books)
+    book["price"] = rng.choice([1, 5, 300, 301, 7000, 2**31 - 1], (n_books, cap)).astype(np.int32)
+    book["time"] = rng.choice([-(2**31), -1, 0, 2**31 - 1], (n_books, cap)).astype(np.int32)
+    book["qty"][::2] = rng.choice([1, 2**31 - 1], book["qty"][::2].shape).astype(np.int32)
+    eng.OrderBooks.tune(warps)
+    try:
+        vol = check_match(eng, book)
+    finally:
+        eng.OrderBooks.tune(0)
+    assert cap == 1 or (vol > 0).any()
