@@ -169,7 +169,8 @@ abm_status abm_sort(abm_slab* s, int32_t field, int32_t* out_perm, void* stream)
  * it, 0, qty); filled orders become inactive, the others keep the rest of
  * their qty. out_volume (device int64[n_books]) = V; out_price (device
  * int32[n_books]) = the price of the ask holding share V, -1 if V = 0.
- * One CTA per book, sorted in shared memory.
+ * One to four warps per book: share sums per price where the prices that can
+ * trade span at most 256 ticks, else a sort in shared memory.
  *
  * abm_lob_add -- new orders into each book's vacant slots (the add of
  * Section 4 per book; the stock-exchange case of Section 4's example): order
@@ -182,7 +183,7 @@ abm_status abm_sort(abm_slab* s, int32_t field, int32_t* out_perm, void* stream)
 #define ABM_LOB_MAX_CAP 2048
 /* Launch shape of abm_lob_match's price-level path for the rest of the
  * process: warps matching one book (1, 2 or 4; 0 = the default: by the slots of
- * a book and the number of books, more for larger and for fewer books).
+ * a book and the books per SM, more for larger and for fewer books).
  * Results never depend on it. ABM_ERR_ARG for other values. Host only. */
 abm_status abm_lob_tune(int32_t warps_per_book);
 abm_status abm_lob_match(int32_t n_books, int32_t cap, int32_t* active, const int32_t* side, const int32_t* price,

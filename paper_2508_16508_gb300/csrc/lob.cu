@@ -857,13 +857,18 @@ static abm_status lob_launch(bool vec16, int n_books, int cap, int32_t* active, 
   // 50,000 of 256 slots 73 against 89; 20,000 of 512 57 against 56, of 768 93 against
   // 82), and four share more than 768 slots better than two (65536 books of 1024
   // slots 299 against 313, 16384 of 2048 158 against 169; 768 slots the same).
-  // With few books a book's own chain counts, which more warps shorten until the
-  // SMs fill up. 100 steps of orders and matching: 300 books of 200 slots 570 / 532 /
-  // 546 us with 1 / 2 / 4 warps; of 1000 slots 836 / 650 / 618, 500 books 855 / 691 /
-  // 695, 1000 books 939 / 810 / 866; 2000 books (two launches a round) 1677 / 1344 / 1267.
+  // With few books a book's own chain counts, which more warps shorten until the SMs
+  // fill up; so the lines lie at books per SM. A placement and a matching round, us with
+  // 1 / 2 / 4 warps: 300 books of 200 slots 5.7 / 5.3 / 5.5, of 400 6.6 / 5.7 / 5.6, of 1000
+  // 8.2 / 6.3 / 6.0; 500 books of 400 6.7 / 5.8 / 5.9, of 1000 8.3 / 6.8 / 6.8; 1000 books of 200
+  // 6.0 / 5.9 / 6.5, of 1000 9.5 / 8.2 / 8.8; 1700 books of 200 6.4 / 6.6 / 9.0, of 400 7.7 / 7.4 /
+  // 9.1, of 768 14.7 / 11.9 / 11.3. Books of 513 to 1024 slots take two warps between the first
+  // lines (four of them no longer find room on the SMs) and four again above seven books
+  // per SM, where the books do not all have a CTA at once and a round is two launches.
   if (g == 0) {
-    const int one = n_books <= 2048 ? 128 : 256;
-    const int two = n_books <= 512 ? 256 : n_books <= 1024 ? 1024 : n_books <= 2048 ? 512 : 768;
+    const int sms = num_sms();
+    const int one = n_books <= 8 * sms ? 128 : 256;
+    const int two = 2 * n_books <= 7 * sms ? 256 : n_books <= 7 * sms ? 1024 : 2 * n_books <= 27 * sms ? 512 : 768;
     g = cap <= one ? 1 : (cap <= two ? 2 : 4);
   }
   switch (g) {

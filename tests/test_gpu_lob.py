@@ -271,6 +271,16 @@ def test_match_default_shapes(eng, n_books, cap):
     assert (check_match(eng, workloads.random_books(n_books, cap, 0.6, seed=cap)) > 0).any()
 
 
+@pytest.mark.parametrize("eighths,caps", [(28, (256, 257, 1024)), (56, (256, 513, 1024)), (64, (128, 129, 256)),
+                                          (108, (256, 257, 512, 513, 768, 769))])
+def test_match_default_shapes_by_sms(eng, eighths, caps):
+    """Each side of the lines between the default numbers of warps per book, which lie at books per SM."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for n_books in (eighths * sms // 8, eighths * sms // 8 + 1):
+        for cap in caps:
+            assert (check_match(eng, workloads.random_books(n_books, cap, 0.6, seed=cap)) > 0).any()
+
+
 @pytest.mark.parametrize("n_books,cap", [(900, 7), (5200, 7), (400, 600), (1300, 600), (500, 1025)])
 def test_match_sort_path_few_and_many_books(eng, n_books, cap):
     """Books for the sort path among others: in the level path's own CTA (few books) and in a second launch (many)."""
