@@ -124,6 +124,7 @@ struct ScanArgs {
   int32_t* out_count;      // device outputs (nullable)
   int negate;              // OP_SELECT: select where the predicate is false
   const int32_t* list_base;  // OP_SELECT: device offset added to every rank (nullable)
+  u32 div1, div4;            // one launch: 65536 / units of a row, rounded up, in words and in 16 bytes
 };
 
 template <int THREADS>
@@ -869,64 +870,120 @@ __global__ void __launch_bounds__(256, 2) k_apply(ScanArgs a) {
 // distributed shared memory between two cluster barriers. Three launches that
 // each touch 0.4 MB cost their launches and round trips, not their bytes. GPU
 // time of a select / update / remove / add back to back, three launches against
-// one: 1000 slots 9.2 / 11.0 / 9.2 / 8.2 -> 2.2 / 2.8 / 2.1 / 1.8 us; 100,003
+// one, few records: 1000 slots 9.2 / 11.0 / 9.2 / 8.2 -> 2.2 / 2.8 / 2.1 / 1.8 us; 100,003
 // slots 10.2 / 14.3 / 10.3 / 8.2 -> 5.5 / 7.0 / 5.0 / 3.2; at 262,144 slots,
 // where 16 SMs do what 64 CTAs do above it, 8.4 / 11.0 / 7.7 / 4.2 (three
-// launches at 300,000: 8.2 / 12.3 / 8.2 / 8.2).
+// launches at 300,000: 8.2 / 12.3 / 8.2 / 8.2). For many records see small_moves.
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int kSmallCtas = 16;  // cluster size, at most (above 8: opt-in)
 constexpr int kSmallMax = kSmallCtas * kSmallThreads * 16;
 
-// Records r0 .. r0 + n - 1 of a warp's staged slots (offsets from slot0): whole
-// rows, neighbouring lanes on neighbouring words of a record.
+// word c of v, if it has one
+__device__ __forceinline__ void stamp_word(int& v, int c, int x) { v = c == 0 ? x : v; }
+__device__ __forceinline__ void stamp_word(int4& v, int c, int x) {
+  v = make_int4(c == 0 ? x : v.x, c == 1 ? x : v.y, c == 2 ? x : v.z, c == 3 ? x : v.w);
+}
+
+// Records r0 .. r0 + n - 1, their slots staged by the warp (offsets from slot0) or, with
+// LIST, in a list that the cluster wrote (list[r0] on), in units V (int4 where the fields are a multiple of four and the records 16-byte aligned, else
+// words), neighbouring lanes on neighbouring units of a record, U of a lane's in flight.
 // ADD: added to the row (wrapping); id_field >= 0: that field is id0 + r instead.
-__device__ __forceinline__ void move_small(const SlabDev& s, const unsigned short* stage, int slot0, u32 n, u32 r0,
-                                           const int32_t* rec, const int32_t* rec_idx, bool add, int id_field, int id0,
-                                           int lane) {
-  const u32 F = (u32)s.F;
-  if ((F & 3u) == 0u && ((uintptr_t)rec & 15) == 0) {
-    const u32 q = F >> 2;
-    for (u32 e = lane; e < n * q; e += 32) {
-      const u32 i = q == 1 ? e : (q == 2 ? e >> 1 : e / q), c = e - i * q;
-      const int slot = slot0 + stage[i];
-      if (!in_range(slot, s.cap, s.err)) continue;
-      const u32 j = rec_idx ? (u32)rec_idx[r0 + i] : r0 + i;
-      int4 r = __ldg(reinterpret_cast<const int4*>(rec) + (size_t)j * q + c);
-      int4* d = reinterpret_cast<int4*>(s.fields + (size_t)slot * s.Fp) + c;
-      if (add) {
-        const int4 o = *d;
-        r = make_int4((int)((u32)o.x + (u32)r.x), (int)((u32)o.y + (u32)r.y), (int)((u32)o.z + (u32)r.z),
-                      (int)((u32)o.w + (u32)r.w));
+template <typename V, int U, bool ADD, bool LIST>
+__device__ __forceinline__ void move_small_units(const SlabDev& s, const unsigned short* stage, const int32_t* list,
+                                                 int slot0, u32 n, u32 r0, const int32_t* rec, const int32_t* rec_idx,
+                                                 int id_field, int id0, int lane, u32 div1, u32 div4) {
+  constexpr int W = sizeof(V) / 4;
+  const V* const src = reinterpret_cast<const V*>(rec);
+  V* const dst = reinterpret_cast<V*>(s.fields);
+  const u32 F = (u32)s.F / W, Fp = (u32)s.Fp / W;
+  const u32 inv = W == 4 ? div4 : div1;  // x / F = x * inv >> 16 for x <= 32
+  const u32 rq = (32u * inv) >> 16, rm = 32u - rq * F;
+  u32 i = ((u32)lane * inv) >> 16, f = (u32)lane - i * F;
+  for (u32 e0 = lane; e0 < n * F; e0 += 32 * U) {
+    V v[U], o[U];
+    u32 at[U];
+    bool ok[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      ok[u] = e0 + 32 * u < n * F;
+      if (ok[u]) {
+        const int slot = LIST ? __ldcg(list + r0 + i) : slot0 + stage[i];
+        ok[u] = in_range(slot, s.cap, s.err);
+        at[u] = (u32)slot * Fp + f;
+        const u32 j = rec_idx ? (u32)rec_idx[r0 + i] : r0 + i;
+        v[u] = __ldg(src + (size_t)j * F + f);
+        if (ADD && ok[u]) o[u] = dst[at[u]];
+        if (!ADD) stamp_word(v[u], id_field - W * (int)f, (int)((u32)id0 + r0 + i));
       }
-      const int id = (int)((u32)id0 + r0 + i), f = id_field - 4 * (int)c;
-      if (f == 0) r.x = id;
-      if (f == 1) r.y = id;
-      if (f == 2) r.z = id;
-      if (f == 3) r.w = id;
-      *d = r;
+      i += rq;
+      f += rm;
+      if (f >= F) {
+        f -= F;
+        ++i;
+      }
     }
-  } else {
-    for (u32 e = lane; e < n * F; e += 32) {
-      const u32 i = e / F, f = e - i * F;
-      const int slot = slot0 + stage[i];
-      if (!in_range(slot, s.cap, s.err)) continue;
-      const u32 j = rec_idx ? (u32)rec_idx[r0 + i] : r0 + i;
-      int v = rec[(size_t)j * F + f];
-      int32_t* d = s.fields + (size_t)slot * s.Fp + f;
-      if (add) v = (int)((u32)*d + (u32)v);
-      if ((int)f == id_field) v = (int)((u32)id0 + r0 + i);
-      *d = v;
-    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (ok[u]) dst[at[u]] = ADD ? wrap_add(o[u], v[u]) : v[u];
+  }
+}
+
+// U: four words, or two int4 where rows are read; one int4 where they are only written (the next store does not wait for
+// the one before, and a CTA that runs once pays for every instruction it fetches).
+template <bool ADD, bool LIST>
+__device__ __forceinline__ void move_small(const SlabDev& s, const unsigned short* stage, const int32_t* list, int slot0,
+                                           u32 n, u32 r0, const int32_t* rec, const int32_t* rec_idx, int id_field, int id0,
+                                           int lane, u32 div1, u32 div4) {
+  if ((s.F & 3) == 0 && ((uintptr_t)rec & 15) == 0)
+    move_small_units<int4, ADD ? 2 : 1, ADD, LIST>(s, stage, list, slot0, n, r0, rec, rec_idx, id_field, id0, lane, div1,
+                                                   div4);
+  else
+    move_small_units<int, 4, ADD, LIST>(s, stage, list, slot0, n, r0, rec, rec_idx, id_field, id0, lane, div1, div4);
+}
+
+// Adds fall to the lowest free slots, updates to the first that satisfy a predicate, so
+// on a set that is not in its steady state one CTA can own most of a call's records. The
+// cluster then lists the slots and splits the records evenly, at a cluster barrier and a
+// round trip more (3.5 us), where the CTA with most records has this much more to do than
+// the average: in ns, a record costs a CTA 0.72 + 0.04 F, and a warp, which may own half its
+// slots, 2 to 4 a unit. Without and with: adds of 7864 records to 262,144 half-live slots
+// 11.9 and 10.0 us (4 fields), 13.6 and 10.0 (8), 23.1 and 11.0 (11); of 3932 records to
+// 131,072 slots 7.3 and 7.6 (4), 8.3 and 7.6 (8); updates of 262 of those 10.0 and 6.3 (11).
+__device__ __forceinline__ bool small_crowded(u32 most, u32 all, int F, u32 units, u32 half_warp) {
+  const u32 more = most - all / gridDim.x;
+  return more * (18u + (u32)F) / 25u > 3500u || min(more, half_warp) * units > 1000u;
+}
+
+// This warp's run of the na records of the first list and the nb of the second. (Out of
+// line: the kernel's usual way is as short as without it.)
+template <int OP>
+__device__ __noinline__ void move_even(const ScanArgs& a, u32 na, u32 nb, int id0) {
+  const int lane = threadIdx.x & 31;
+  const u32 warps = gridDim.x * kSmallWarps, w = blockIdx.x * kSmallWarps + (threadIdx.x >> 5);
+  u32 per = (na + warps - 1) / warps, r0 = min(na, per * w);
+  u32 n = min(per, na - r0);
+  if (OP == OP_UPDATE && a.op_kind == ABM_OP_ADD)
+    move_small<true, true>(a.s, nullptr, a.list_a, 0, n, r0, a.rec, a.use_rec_idx ? a.s.rec_idx : nullptr, -1, 0, lane, a.div1, a.div4);
+  else
+    move_small<false, true>(a.s, nullptr, a.list_a, 0, n, r0, a.rec, OP == OP_UPDATE && a.use_rec_idx ? a.s.rec_idx : nullptr,
+                            OP == OP_ADD ? a.id_field : -1, id0, lane, a.div1, a.div4);
+  if (OP == OP_FUSED) {
+    per = (nb + warps - 1) / warps;
+    r0 = min(nb, per * w);
+    n = min(per, nb - r0);
+    move_small<true, true>(a.s, nullptr, a.list_b, 0, n, r0, a.rec2, nullptr, -1, 0, lane, a.div1, a.div4);
   }
 }
 
 template <int OP, int LS>
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constant__ ScanArgs a) {
   constexpr int STEP = 32 * LS;  // slots of a warp
+  constexpr bool MOVES = OP == OP_ADD || OP == OP_UPDATE || OP == OP_FUSED;
   __shared__ u64 s_w[kSmallWarps];
   __shared__ u64 s_tot;     // this CTA's counts: A << 32 | B
   __shared__ u64 s_pre[2];  // the CTAs before, all
+  __shared__ int s_even;    // the cluster splits the records evenly
   __shared__ unsigned short s_stage[kSmallWarps * STEP];
   const SlabDev& s = a.s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -991,28 +1048,40 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
     wv += __shfl_xor_sync(0xFFFFFFFFu, wv, o);
     wpre += __shfl_xor_sync(0xFFFFFFFFu, wpre, o);
   }
+  const u32 limit = (u32)(OP == OP_UPDATE ? nrec : (OP == OP_SELECT || OP == OP_ARRAY ? 0x7FFFFFFF : a.k));
   u64 pre = 0, all = wv;
+  bool even = false;
   if (gridDim.x > 1) {
     if (threadIdx.x == 0) s_tot = wv;
     cluster_arrive();
     cluster_wait();
     if (warp == 0) {
-      u64 t = lane < (int)gridDim.x ? ld_cluster(&s_tot, (u32)lane) : 0ull;
-      u64 p = lane < (int)blockIdx.x ? t : 0ull;
+      const u64 t = lane < (int)gridDim.x ? ld_cluster(&s_tot, (u32)lane) : 0ull;
+      u64 p = t;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
-        p += __shfl_xor_sync(0xFFFFFFFFu, p, o);
+      for (int o = 1; o < kSmallCtas; o <<= 1) {
+        const u64 x = __shfl_up_sync(0xFFFFFFFFu, p, o);
+        if (lane >= o) p += x;
       }
-      if (lane == 0) {
-        s_pre[0] = p;
-        s_pre[1] = t;
+      if (lane == (int)gridDim.x - 1) s_pre[1] = p;
+      p -= t;
+      if (lane == (int)blockIdx.x) s_pre[0] = p;
+      if (MOVES) {  // the records of each list that a CTA has to move, by its slots' ranks
+        const u32 before = (u32)(p >> 32), mine = before < limit ? min((u32)(t >> 32), limit - before) : 0u;
+        const u32 before2 = (u32)p, mine2 = before2 < (u32)a.k ? min((u32)t, (u32)a.k - before2) : 0u;
+        const u32 most = __reduce_max_sync(0xFFFFFFFFu, mine), sum = __reduce_add_sync(0xFFFFFFFFu, mine);
+        const u32 most2 = __reduce_max_sync(0xFFFFFFFFu, mine2), sum2 = __reduce_add_sync(0xFFFFFFFFu, mine2);
+        const u32 units = (s.F & 3) == 0 && (((uintptr_t)a.rec | (uintptr_t)a.rec2) & 15) == 0 ? s.F >> 2 : s.F;
+        const bool crowded = small_crowded(most, sum, s.F, units, STEP / 2);
+        const bool crowded2 = OP == OP_FUSED && small_crowded(most2, sum2, s.F, units, STEP / 2);
+        if (lane == 0) s_even = crowded || crowded2;
       }
     }
     __syncthreads();
     cluster_arrive();  // the others' counts are read; waited for before leaving
     pre = s_pre[0];
     all = s_pre[1];
+    if (MOVES) even = s_even != 0;
   } else {
     __syncthreads();  // every thread has read the counters that are changed below
   }
@@ -1038,7 +1107,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
       }
     }
   }
-  const u32 limit = (u32)(OP == OP_UPDATE ? nrec : (OP == OP_SELECT || OP == OP_ARRAY ? 0x7FFFFFFF : a.k));
   u32 na = 0;
   if (OP != OP_REMOVE && sa < limit) na = min(tot & 0xFFFFu, limit - sa);
   if (OP == OP_ADD || OP == OP_FUSED) {
@@ -1078,6 +1146,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
   }
   // the selected slots in rank order, then lists and records
   unsigned short* stage = s_stage + warp * STEP;
+  const int32_t* const idx = OP == OP_UPDATE && a.use_rec_idx ? s.rec_idx : nullptr;
+  const bool add = OP == OP_UPDATE && a.op_kind == ABM_OP_ADD;
+  const int idf = OP == OP_ADD ? a.id_field : -1;
   if (OP != OP_REMOVE && na) {
     u32 pos = ex & 0xFFFFu;
 #pragma unroll
@@ -1085,13 +1156,12 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
       if ((ma >> j) & 1u) stage[pos++] = (unsigned short)(LS * lane + j);
     __syncwarp();
     int32_t* const list = a.list_a + (OP == OP_SELECT && a.list_base ? *a.list_base : 0);
-    if (OP != OP_FUSED)  // (the selective-update call hands no list out)
+    if (OP != OP_FUSED || even)  // (the selective-update call hands no list out)
       for (u32 i = lane; i < na; i += 32) list[sa + i] = slot0 + stage[i];
-    if (OP == OP_ADD || OP == OP_FUSED)
-      move_small(s, stage, slot0, na, sa, a.rec, nullptr, false, OP == OP_ADD ? a.id_field : -1, id0, lane);
-    if (OP == OP_UPDATE)
-      move_small(s, stage, slot0, na, sa, a.rec, a.use_rec_idx ? s.rec_idx : nullptr, a.op_kind == ABM_OP_ADD, -1, 0,
-                 lane);
+    if (MOVES && !even) {
+      if (add) move_small<true, false>(s, stage, nullptr, slot0, na, sa, a.rec, idx, -1, 0, lane, a.div1, a.div4);
+      else move_small<false, false>(s, stage, nullptr, slot0, na, sa, a.rec, idx, idf, id0, lane, a.div1, a.div4);
+    }
     __syncwarp();
   }
   if (OP == OP_FUSED && sb < (u32)a.k && (tot >> 16)) {
@@ -1101,7 +1171,18 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
     for (int j = 0; j < LS; ++j)
       if ((mb >> j) & 1u) stage[pos++] = (unsigned short)(LS * lane + j);
     __syncwarp();
-    move_small(s, stage, slot0, nb, sb, a.rec2, nullptr, true, -1, 0, lane);
+    if (even)
+      for (u32 i = lane; i < nb; i += 32) a.list_b[sb + i] = slot0 + stage[i];
+    else
+      move_small<true, false>(s, stage, nullptr, slot0, nb, sb, a.rec2, nullptr, -1, 0, lane, a.div1, a.div4);
+  }
+  if (MOVES && even) {
+    __syncwarp();
+    cluster_wait();
+    cluster_arrive();  // the lists are complete
+    cluster_wait();
+    move_even<OP>(a, min((u32)A, limit), OP == OP_FUSED ? min((u32)B, (u32)a.k) : 0u, id0);
+    cluster_arrive();  // (the wait at the end)
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     if (OP == OP_SELECT || OP == OP_ARRAY) {
@@ -1546,6 +1627,26 @@ static bool fused_moves(const abm_slab* s, const ScanArgs& a) {
          ((((uintptr_t)a.rec) | ((uintptr_t)a.rec2)) & 31) == 0;
 }
 
+// Whether one cluster is faster than the passes for a call on n <= kSmallMax slots that
+// moves up to k records of F fields (16-byte units where `quads`): its SMs are at most
+// sixteen, and the slots of a lane leave that much less time for records. What a CTA
+// moves at most, in ns, against lines drawn from 1 to 16 fields and k from 0.002 to 0.5 n
+// (adds to half-live and nearly full sets, updates of the first slots and of slots spread
+// over the set). 131,072 slots, us of the passes and of the cluster: adds of 0.1 n to a
+// half-live set, 5 fields 10.5 and 8.3, 11 fields 11.9 and 9.3, of 0.5 n 8 fields 10.9 and
+// 9.0, 16 fields 12.4 and 11.4 (its updates 10.7 and 13.1), 11 fields 12.9 and 14.1; 262,144
+// slots: adds of 0.03 n 10.7 and 10.3 (1 field), 10.0 and 10.3 (8), 12.2 and 11.0 (11), of
+// 0.1 n 10.7 and 12.1 (8; to a nearly full set 10.7 and 8.3), 11.9 and 13.2 (11); the
+// selective-update call at p = 0.01 12.4 and 11.7 (8), at 0.03 11.6 and 13.8. Up to 65,536 slots
+// the cluster is always faster (11 fields, 0.5 n: 12.6 and 9.0).
+static bool small_moves(int n, long long k, int F, bool quads, bool fused) {
+  if (n <= kSmallMax / 4) return true;
+  const int lanes = n <= kSmallMax / 2 ? 8 : 16;  // slots of a lane
+  const long long ctas = (n + kSmallThreads * lanes - 1) / (kSmallThreads * lanes);
+  const long long ns = std::min<long long>(k, n / 2) / ctas * (18 + (quads ? F : 2 * F)) / 25;
+  return ns <= (lanes == 8 ? (fused ? 3700 : 4700) : (fused ? 300 : 1750));
+}
+
 // One cluster of as few CTAs as hold the slots, LS slots per lane.
 template <int OP, int LS>
 static abm_status launch_small(const ScanArgs& a, cudaStream_t st) {
@@ -1560,6 +1661,9 @@ static abm_status launch_small(const ScanArgs& a, cudaStream_t st) {
       wide.fetch_or(bit, std::memory_order_release);
     }
   }
+  ScanArgs b = a;
+  b.div1 = (65536u + (u32)a.s.F - 1u) / (u32)a.s.F;
+  b.div4 = a.s.F >= 4 ? (65536u + (u32)(a.s.F / 4) - 1u) / (u32)(a.s.F / 4) : 0u;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)ctas);
   cfg.blockDim = dim3(kSmallThreads);
@@ -1572,7 +1676,7 @@ static abm_status launch_small(const ScanArgs& a, cudaStream_t st) {
   at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  ABM_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_small<OP, LS>, a));
+  ABM_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_small<OP, LS>, b));
   return ABM_OK;
 }
 
@@ -1597,9 +1701,13 @@ static abm_status launch_scan(abm_slab* s, const ScanArgs& a, bool aux, cudaStre
     return ABM_OK;
   }
   // small sets: one launch (see k_small); few slots per lane while one cluster has the lanes
-  if (b.n <= kSmallThreads * kSmallCtas * 4) return launch_small<OP, 4>(b, st);
-  if (b.n <= kSmallThreads * kSmallCtas * 8) return launch_small<OP, 8>(b, st);
-  if (b.n <= kSmallMax) return launch_small<OP, 16>(b, st);
+  constexpr bool MOVES = OP == OP_ADD || OP == OP_UPDATE || OP == OP_FUSED;
+  const bool quads = (s->d.F & 3) == 0 && (((uintptr_t)b.rec | (uintptr_t)b.rec2) & 15) == 0;
+  if (b.n <= kSmallMax && (!MOVES || small_moves(b.n, b.k, s->d.F, quads, OP == OP_FUSED))) {
+    if (b.n <= kSmallMax / 4) return launch_small<OP, 4>(b, st);
+    if (b.n <= kSmallMax / 2) return launch_small<OP, 8>(b, st);
+    return launch_small<OP, 16>(b, st);
+  }
   const bool move = OP == OP_FUSED && fused_moves(s, b);
   if (ctas_per_sm == 0) ctas_per_sm = move ? kMoveCtasPerSm : 8;
   const int target = std::max(1, std::min(num_sms() * ctas_per_sm, s->max_ctas));

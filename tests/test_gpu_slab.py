@@ -688,3 +688,72 @@ def test_selective_update_row_shapes(eng, F):
     for f in range(F):
         np.testing.assert_array_equal(np_of(s.read(f)), o.fields[f])
     s.check()
+
+
+@pytest.mark.parametrize("n,F,k,shift", [(262_144, 4, 31_000, 0), (262_144, 4, 33_000, 0), (131_072, 11, 46_000, 0),
+                                         (131_072, 11, 48_000, 0), (262_144, 8, 4500, 0), (262_144, 8, 4800, 1),
+                                         (262_144, 16, 300, 1), (200_001, 1, 28_000, 0), (200_001, 5, 10_000, 0),
+                                         (131_073, 8, 200_000, 0), (131_000, 8, 131_000, 0), (100_003, 13, 90_000, 3),
+                                         (100_003, 3, 9_000, 0), (65_536, 15, 70_000, 0), (60_000, 15, 3000, 0),
+                                         (1025, 7, 1025, 0), (5, 12, 9, 2)])
+def test_record_moves_of_small_sets(eng, n, F, k, shift):
+    """Whole numbers, so exact: sets of up to 262,144 slots on both sides of the number of records above which the calls
+    take the passes, and of that above which a cluster splits crowded records evenly; records at every alignment, every
+    id field, some flags odd."""
+    from paper_2508_16508_gb300 import abm
+    rng = np.random.default_rng(n + F + k)
+    s = eng.Slab(n, F, seed=9)
+    act = np.where(rng.random(n) < 0.5, rng.choice([1, 1, 1, 7], n), 0).astype(np.int32)
+    fld = rng.integers(-50, 50, (F, n)).astype(np.int32)
+    s.write(-1, torch.from_numpy(act).cuda())
+    for f in range(F):
+        s.write(f, torch.from_numpy(fld[f]).cuda())
+    rec = rng.integers(-2**31, 2**31, (k, F)).astype(np.int32)
+    dev = torch.zeros(k * F + shift, dtype=torch.int32, device="cuda")[shift:].view(k, F)
+    dev.copy_(torch.from_numpy(rec))
+    rmask = (rng.random(min(k, n)) < 0.5).astype(np.int32)
+
+    def check(where):
+        for f in range(F):
+            np.testing.assert_array_equal(np_of(s.read(f)), fld[f], err_msg=f"{where}, field {f}")
+        np.testing.assert_array_equal(np_of(s.read(-1)) != 0, act != 0, err_msg=where)
+
+    for masked, op in ((False, abm.OP_ADD), (False, abm.OP_SET), (True, abm.OP_ADD), (True, abm.OP_SET)):
+        sel = np.flatnonzero((act != 0) & (fld[0] >= -30))
+        rows = rec[:len(rmask)][rmask != 0] if masked else rec
+        r = min(len(sel), len(rows))
+        slots, cnt = s.update_distinct(abm.pred(abm.PRED_FIELD, field=0, cmp=abm.CMP_GE, value=-30),
+                                       dev[:len(rmask)] if masked else dev,
+                                       torch.from_numpy(rmask).cuda() if masked else None, op=op)
+        assert int(cnt) == r
+        np.testing.assert_array_equal(np_of(slots)[:r], sel[:r])
+        for f in range(F):
+            fld[f][sel[:r]] = rows[:r, f] + (fld[f][sel[:r]] if op == abm.OP_ADD else 0)
+        check(f"update {masked} {op}")
+    for id_field in [-1] + list(range(F)):
+        gone = rng.random(n) < 0.4
+        s.remove(abm.pred(abm.PRED_MASK, mask=torch.from_numpy(gone.astype(np.int32)).cuda()))
+        act[gone] = 0
+        free = np.flatnonzero(act == 0)
+        r = min(k, len(free))
+        first = s.counters()["next_id"]
+        slots, cnt = s.add(dev, id_field=id_field)
+        assert int(cnt) == r
+        np.testing.assert_array_equal(np_of(slots)[:r], free[:r])
+        act[free[:r]] = 1
+        for f in range(F):
+            fld[f][free[:r]] = first + np.arange(r) if f == id_field else rec[:r, f]
+        check(f"add {id_field}")
+    if F <= 8:
+        o = oracle.Slab(n, F)
+        o.active[:] = np_of(s.read(-1))
+        for f in range(F):
+            o.fields[f][:] = fld[f]
+        for step in range(2):
+            s.selective_update(step, workloads.threshold(0.3), s.philox_records(step, abm.P_NEWREC0, abm.P_NEWREC1, k),
+                               s.philox_records(step, abm.P_DELTA0, abm.P_DELTA1, k))
+            o.c1_call(step, workloads.threshold(0.3), k, seed=9)
+        np.testing.assert_array_equal(np_of(s.read(-1)) != 0, o.active != 0)
+        for f in range(F):
+            np.testing.assert_array_equal(np_of(s.read(f)), o.fields[f])
+    s.check()
