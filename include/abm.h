@@ -427,6 +427,14 @@ abm_status abm_diag_barrier_timeout(int32_t spin_limit, void* stream);
  * range, else ABM_OK. Other builds: ABM_OK (nothing is tested). Synchronises
  * `stream`. */
 abm_status abm_diag_check_index(int64_t i, int64_t n, void* stream);
+/* Diagnostics, host only: the launches that calls take, with the largest cluster
+ * that the device has room for as an argument. abm_diag_small_lanes: a set
+ * operation on n slots that moves up to k records (quads != 0: of 16-byte units;
+ * fused != 0: abm_selective_update): 4, 8 or 16 slots per lane of one cluster, or
+ * 0 for the passes over the set. abm_diag_steps_way: abm_step on a world of
+ * size class 0..3: 0 one CTA, 1 one cluster, 2 one CTA per SM, 3 the tuned grid. */
+int32_t abm_diag_small_lanes(int32_t n, int32_t k, int32_t n_fields, int32_t quads, int32_t fused, int32_t most_ctas);
+int32_t abm_diag_steps_way(int32_t size_class, int32_t profiled, int32_t cluster_fits);
 /* Synchronises `stream`; reports a recorded device error (e.g. a timed-out wait). */
 abm_status abm_world_check(abm_world* w, void* stream);
 

@@ -166,6 +166,8 @@ def _sig(L):
         "abm_world_slab": ([vp, i32, pp, vp], st),
         "abm_world_slab_commit": ([vp, i32, vp], st),
         "abm_diag_check_index": ([i64, i64, vp], st),
+        "abm_diag_small_lanes": ([i32, i32, i32, i32, i32, i32], i32),
+        "abm_diag_steps_way": ([i32, i32, i32], i32),
         "abm_capacity_features": ([vp, i32, vp, vp, vp], st),
         "abm_capacity_from_prediction": ([vp, i32, C.c_float, i32, vp, vp, vp, vp], st),
         "abm_lob_match": ([i32, i32, vp, vp, vp, vp, vp, vp, vp, vp], st),

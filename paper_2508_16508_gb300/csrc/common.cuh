@@ -376,4 +376,36 @@ inline cudaError_t smem_attr_once(K* kernel, int bytes, std::atomic<unsigned lon
   if (e == cudaSuccess && bit) done.fetch_or(bit, std::memory_order_release);
   return e;
 }
+
+// CTAs of the largest cluster of a kernel (16, 8, 4, 2 or 1) that the device and the
+// context have room for: fewer than 16 where no GPC has 16 SMs free to them (a
+// partitioned device, a context limited to some SMs). Asked once per device; launches
+// take another way, or fewer CTAs, where the answer is too small.
+template <typename... KArgs>
+inline int cluster_limit(void (*kernel)(KArgs...), int threads, std::atomic<int> (&known)[64]) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  if (dev >= 0 && dev < 64) {
+    const int n = known[dev].load(std::memory_order_acquire);
+    if (n > 0) return n;
+  }
+  int limit = 1;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
+  for (int c = 16; c > 1 && limit == 1; c >>= 1) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)c);
+    cfg.blockDim = dim3((unsigned)threads);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)c;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) cudaGetLastError();
+    else if (n > 0) limit = c;
+  }
+  if (dev >= 0 && dev < 64) known[dev].store(limit, std::memory_order_release);
+  return limit;
+}
 }

@@ -996,7 +996,9 @@ static abm_status fused_train(abm_mlp* n, RowArgs& ra, const AdamStep& ad, float
   wa.nslab = (ra.B + R - 1) / R;
   // runs of whole stages (128 rows each up to 1024 rows), one CTA of the cluster each
   const int stages = (wa.nslab * R + kWRows - 1) / kWRows;
-  const int per = (stages + kMaxRuns - 1) / kMaxRuns, runs = (stages + per - 1) / per;
+  static std::atomic<int> known[64];
+  const int most = std::min(kMaxRuns, cluster_limit(k_wgrad, kWThreads, known));
+  const int per = (stages + most - 1) / most, runs = (stages + per - 1) / per;
   wa.slabs_per_split = per * (kWRows / R);
   wa.lossp = n->lossp;
   wa.nloss = grid;

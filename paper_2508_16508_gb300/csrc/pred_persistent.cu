@@ -1328,6 +1328,11 @@ int persistent_max_ctas() {
 
 int persistent_warps() { return kPWarps; }
 
+bool persistent_cluster_fits() {
+  static std::atomic<int> known[64];
+  return cluster_limit(k_persistent<1, true>, kPT, known) >= kClusterCtas;
+}
+
 int persistent_round_units() { return kQ * kSheepWarps; }
 
 abm_status launch_persistent(const WorldDev& d, u32* bar_next, int grid, bool cluster, int nsteps, abm_step_stats* stats,
@@ -1335,14 +1340,6 @@ abm_status launch_persistent(const WorldDev& d, u32* bar_next, int grid, bool cl
   WorldDev dd = d;
   dd.bar_base = *bar_next;
   if (cluster) {
-    static std::atomic<unsigned long long> wide{0};  // devices on which the kernel may use clusters above 8
-    int dev = 0;
-    ABM_CUDA_TRY(cudaGetDevice(&dev));
-    const unsigned long long bit = (dev >= 0 && dev < 64) ? 1ull << dev : 0ull;
-    if (!bit || !(wide.load(std::memory_order_acquire) & bit)) {
-      ABM_CUDA_TRY(cudaFuncSetAttribute(k_persistent<1, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-      wide.fetch_or(bit, std::memory_order_release);
-    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kClusterCtas);
     cfg.blockDim = dim3(kPT);

@@ -81,6 +81,8 @@ __device__ __forceinline__ void note_class(const WorldDev& w, int ext0, int ext1
 // persistent step kernel (pred_persistent.cu)
 int persistent_max_ctas();
 int persistent_warps();
+// whether the one-cluster launch can be placed on the current device
+bool persistent_cluster_fits();
 // units (128 slots) of a species that one CTA takes in one round of the persistent kernel's sheep phases
 int persistent_round_units();
 abm_status launch_persistent(const WorldDev& d, u32* bar_next, int grid, bool cluster, int nsteps, abm_step_stats* stats,

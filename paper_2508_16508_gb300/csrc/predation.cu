@@ -531,13 +531,24 @@ extern "C" abm_status abm_create(const abm_config* cfg, void* stream, abm_world*
 // 301 cells 18.1 -> 15.8 us, 1400 x 1400 (3811 sheep units) 21.1 -> 18.9.
 // Class 3: the tuned number of CTAs; at 2048 x 2048 (two rounds of one CTA per
 // SM) the second CTA per SM wins, 33.7 us against 38.7.
+// The cluster only where one can be placed; a profiled call runs on the grid.
+static int steps_way(int size_class, bool profiled, bool cluster) {
+  if (profiled) return size_class < 3 ? 2 : 3;
+  return size_class == 1 && !cluster ? 2 : size_class;
+}
+
+extern "C" int32_t abm_diag_steps_way(int32_t size_class, int32_t profiled, int32_t cluster_fits) {
+  return steps_way(size_class, profiled != 0, cluster_fits != 0);
+}
+
 static abm_status launch_steps(abm_world* w, int nsteps, abm_step_stats* stats, cudaStream_t st,
                                unsigned long long* phase_ns = nullptr) {
   WorldDev d = w->d;
   d.class_known = *reinterpret_cast<volatile int*>(d.class_host);
-  if (d.class_known == 0 && !phase_ns) return launch_resident(d, nsteps, stats, st);
-  const int grid = d.class_known < 3 ? std::min(w->pgrid, num_sms()) : w->pgrid;
-  return launch_persistent(d, &w->bar_next, grid, d.class_known == 1 && !phase_ns, nsteps, stats, st, phase_ns);
+  const int way = steps_way(d.class_known, phase_ns != nullptr, d.class_known == 1 && persistent_cluster_fits());
+  if (way == 0) return launch_resident(d, nsteps, stats, st);
+  return launch_persistent(d, &w->bar_next, way == 3 ? w->pgrid : std::min(w->pgrid, num_sms()), way == 1, nsteps, stats, st,
+                           phase_ns);
 }
 
 // ev (nullable): 7 events recorded around the six kernels of the step

@@ -1627,9 +1627,8 @@ static bool fused_moves(const abm_slab* s, const ScanArgs& a) {
          ((((uintptr_t)a.rec) | ((uintptr_t)a.rec2)) & 31) == 0;
 }
 
-// Whether one cluster is faster than the passes for a call on n <= kSmallMax slots that
-// moves up to k records of F fields (16-byte units where `quads`): its SMs are at most
-// sixteen, and the slots of a lane leave that much less time for records. What a CTA
+// Where one cluster is faster than the passes, for a call on n slots that moves up to k
+// records of F fields (16-byte units where `quads`): its SMs are at most sixteen, and the slots of a lane leave that much less time for records. What a CTA
 // moves at most, in ns, against lines drawn from 1 to 16 fields and k from 0.002 to 0.5 n
 // (adds to half-live and nearly full sets, updates of the first slots and of slots spread
 // over the set). 131,072 slots, us of the passes and of the cluster: adds of 0.1 n to a
@@ -1639,12 +1638,15 @@ static bool fused_moves(const abm_slab* s, const ScanArgs& a) {
 // 0.1 n 10.7 and 12.1 (8; to a nearly full set 10.7 and 8.3), 11.9 and 13.2 (11); the
 // selective-update call at p = 0.01 12.4 and 11.7 (8), at 0.03 11.6 and 13.8. Up to 65,536 slots
 // the cluster is always faster (11 fields, 0.5 n: 12.6 and 9.0).
-static bool small_moves(int n, long long k, int F, bool quads, bool fused) {
-  if (n <= kSmallMax / 4) return true;
-  const int lanes = n <= kSmallMax / 2 ? 8 : 16;  // slots of a lane
+// The slots of a lane (4, 8 or 16) of one cluster of at most `most` CTAs, or 0: the passes.
+static int small_lanes(int n, long long k, int F, bool quads, bool fused, int most) {
+  int lanes = 4;
+  while (lanes <= 16 && (long long)n > (long long)most * kSmallThreads * lanes) lanes *= 2;
+  if (lanes > 16) return 0;
+  if (lanes == 4) return lanes;
   const long long ctas = (n + kSmallThreads * lanes - 1) / (kSmallThreads * lanes);
   const long long ns = std::min<long long>(k, n / 2) / ctas * (18 + (quads ? F : 2 * F)) / 25;
-  return ns <= (lanes == 8 ? (fused ? 3700 : 4700) : (fused ? 300 : 1750));
+  return ns <= (lanes == 8 ? (fused ? 3700 : 4700) : (fused ? 300 : 1750)) ? lanes : 0;
 }
 
 // One cluster of as few CTAs as hold the slots, LS slots per lane.
@@ -1703,10 +1705,14 @@ static abm_status launch_scan(abm_slab* s, const ScanArgs& a, bool aux, cudaStre
   // small sets: one launch (see k_small); few slots per lane while one cluster has the lanes
   constexpr bool MOVES = OP == OP_ADD || OP == OP_UPDATE || OP == OP_FUSED;
   const bool quads = (s->d.F & 3) == 0 && (((uintptr_t)b.rec | (uintptr_t)b.rec2) & 15) == 0;
-  if (b.n <= kSmallMax && (!MOVES || small_moves(b.n, b.k, s->d.F, quads, OP == OP_FUSED))) {
-    if (b.n <= kSmallMax / 4) return launch_small<OP, 4>(b, st);
-    if (b.n <= kSmallMax / 2) return launch_small<OP, 8>(b, st);
-    return launch_small<OP, 16>(b, st);
+  if (b.n <= kSmallMax) {
+    static std::atomic<int> most[64];
+    switch (small_lanes(b.n, MOVES ? b.k : 0, s->d.F, quads, OP == OP_FUSED,
+                        std::min(kSmallCtas, cluster_limit(k_small<OP, 16>, kSmallThreads, most)))) {
+      case 4: return launch_small<OP, 4>(b, st);
+      case 8: return launch_small<OP, 8>(b, st);
+      case 16: return launch_small<OP, 16>(b, st);
+    }
   }
   const bool move = OP == OP_FUSED && fused_moves(s, b);
   if (ctas_per_sm == 0) ctas_per_sm = move ? kMoveCtasPerSm : 8;
@@ -1843,6 +1849,11 @@ extern "C" abm_status abm_selective_update(abm_slab* s, uint32_t step, uint32_t 
   a.list_a = s->lista;
   a.list_b = s->listb;
   return launch_fused(s, a, (cudaStream_t)stream);
+}
+
+extern "C" int32_t abm_diag_small_lanes(int32_t n, int32_t k, int32_t n_fields, int32_t quads, int32_t fused,
+                                        int32_t most_ctas) {
+  return small_lanes(n, k, n_fields, quads != 0, fused != 0, std::min(kSmallCtas, most_ctas));
 }
 
 extern "C" abm_status abm_slab_tune(abm_slab* s, int32_t threads, int32_t ctas_per_sm, void* stream) {

@@ -75,3 +75,19 @@ def test_check_build_exports_the_same_functions():
     L.abm_strerror.restype = C.c_char_p
     L.abm_strerror.argtypes = [C.c_int32]
     assert b"check build" in L.abm_strerror(8)
+
+
+def test_launches_without_room_for_a_cluster(lib_path):
+    """The launches chosen where the device has no room for a cluster of 16 CTAs, or for any (the answer is passed in):
+    more slots per lane while they fit, then the passes; worlds of the cluster's class run on the grid."""
+    from paper_2508_16508_gb300 import abm
+    lanes = abm.lib().abm_diag_small_lanes
+    for most, last in ((16, 262_144), (8, 131_072), (4, 65_536), (2, 32_768), (1, 16_384)):
+        got = [lanes(n, 0, 8, 1, 0, most) for n in (1, last // 4, last // 4 + 1, last // 2, last // 2 + 1, last, last + 1)]
+        assert got == [4, 4, 8, 8, 16, 16, 0]
+    assert lanes(262_144, 1 << 30, 8, 1, 0, 16) == 0 and lanes(65_536, 1 << 30, 15, 0, 1, 16) == 4  # many records
+    assert lanes((1 << 28) - 1, 0, 1, 0, 0, 16) == 0
+    way = abm.lib().abm_diag_steps_way
+    assert [way(c, 0, 1) for c in range(4)] == [0, 1, 2, 3]
+    assert [way(c, 0, 0) for c in range(4)] == [0, 2, 2, 3]
+    assert [way(c, 1, 1) for c in range(4)] == [2, 2, 2, 3]
