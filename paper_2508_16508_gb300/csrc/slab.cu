@@ -318,11 +318,12 @@ __device__ __forceinline__ uint4 mask_pair_draw(u32 j, const u32 (&mk)[5], const
 // the lane's eight draws are independent and all in flight together. The pass
 // is bound by the Philox draws (one per pair of slots): fewer draws in flight
 // at a higher occupancy measured slower.
-// The flags are not written here: most removed slots are refilled by the same
+// Flags of removed slots (whole 8-slot groups, as 0/1): with few records they are
+// written here. LATE (see kLateShare): most removed slots are refilled by the same
 // call, so the ranking pass, which knows every final flag, writes the groups
-// that end up different. It compares with plane L. Flags other than 0 and 1
-// are put right at once (whole 8-slot groups, as 0/1).
-template <int THREADS>
+// that end up different. It compares with plane L; flags other than 0 and 1
+// are put right here.
+template <int THREADS, bool LATE>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count_fused(ScanArgs a) {
   constexpr int WARPS = THREADS / 32;
   __shared__ u64 s_red[WARPS];
@@ -370,9 +371,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count_fused(ScanArg
     const u32 al = ml & ~dr;        // still live
     const u32 ma = valid & ~al;     // free after the removals
     const u32 mb = al & dc;         // chosen among the live
-    u32 fl = ml;  // flags that are 1 in memory
-    if (odd & ~1) {
-      const u32 nl = ml & ~mr;
+    const u32 nl = ml & ~mr;
+    u32 fl = ml;  // LATE: flags that are 1 in memory
+    if (LATE && (odd & ~1)) {
       fl = 0;
       for (int j = 0; j < kLaneSlots; ++j) {
         if (base + j >= a.n) break;
@@ -384,15 +385,31 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count_fused(ScanArg
         }
       }
     }
+    if (!LATE) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (!((mr >> (8 * h)) & 0xFFu)) continue;
+        const int b = base + 8 * h;
+        if (b + 8 <= a.n) {
+          int f[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) f[j] = (int)((nl >> (8 * h + j)) & 1u);
+          st_v8(s.active + b, f);
+        } else {
+          for (int j = 0; j < 8; ++j)
+            if (b + j < a.n) s.active[b + j] = (int)((nl >> (8 * h + j)) & 1u);
+        }
+      }
+    }
     ca += __popc(ma);
     cb += __popc(mb);
     const u32 na = __shfl_down_sync(0xFFFFFFFFu, ma, 1);
     const u32 nb = __shfl_down_sync(0xFFFFFFFFu, mb, 1);
-    const u32 nf = __shfl_down_sync(0xFFFFFFFFu, fl, 1);
+    const u32 nf = LATE ? __shfl_down_sync(0xFFFFFFFFu, fl, 1) : 0u;
     if (!(lane & 1) && base < a.n) {
       a.planeA[base >> 5] = ma | (na << 16);
       a.planeB[base >> 5] = mb | (nb << 16);
-      a.planeL[base >> 5] = fl | (nf << 16);
+      if (LATE) a.planeL[base >> 5] = fl | (nf << 16);
     }
   }
   u64 v = ((u64)ca << 32) | cb;
@@ -478,7 +495,7 @@ __device__ __forceinline__ void stage_bits(S* stage, u32 m, u32 pos, u32 end, in
 // MOVE (selective-update call, 8 fields, 32-byte aligned records): the pass
 // moves the records itself instead of writing the rank-ordered slot lists, and
 // no apply pass follows.
-template <int OP, int THREADS, bool MOVE = false>
+template <int OP, int THREADS, bool MOVE = false, bool LATE = false>
 __global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(ScanArgs a) {
   constexpr int WARPS = THREADS / 32;
   __shared__ u64 s_red[WARPS];
@@ -499,7 +516,7 @@ __global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(S
     if (wlo < whi && base < a.n) {
       wa_next = a.planeA[base >> 5];
       if (OP == OP_FUSED) wb_next = a.planeB[base >> 5];
-      if (OP == OP_FUSED) wl_next = a.planeL[base >> 5];
+      if (LATE) wl_next = a.planeL[base >> 5];
     }
   }
   u32 pa = 0, pb = 0, ta = 0, tb = 0;
@@ -546,7 +563,7 @@ __global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(S
       if (b0 + kWarpStep < whi && nbase < a.n) {
         wa_next = a.planeA[nbase >> 5];
         if (OP == OP_FUSED) wb_next = a.planeB[nbase >> 5];
-        if (OP == OP_FUSED) wl_next = a.planeL[nbase >> 5];
+        if (LATE) wl_next = a.planeL[nbase >> 5];
       }
     }
     u32 ma = 0, mb = 0;
@@ -598,24 +615,23 @@ __global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(S
     }
     if (OP == OP_ADD || OP == OP_FUSED) {
       // flags of the lane's 16 slots after the adds: live 1, free 0, and the
-      // free slots with a rank below the limit 1. An add writes the groups that
-      // receive an agent. The selective-update call writes the 8-slot halves
-      // that an add or a removal left different from memory: a removed slot
-      // that is refilled costs no write (2^24 slots, half of them touched: two
-      // passes over 64 MB of flags less).
+      // free slots with a rank below the limit 1. Written are the groups that
+      // receive an agent, or LATE the 8-slot halves that an add or a removal left
+      // different from memory: a removed slot that is refilled costs no write
+      // (2^24 slots, half of them touched: two passes over 64 MB of flags less).
       const u32 off = ex & 0xFFFFu;
       const u32 mine = off < na ? min((u32)__popc(ma), na - off) : 0u;
-      const u32 added = mine == (u32)__popc(ma) ? ma : (mine ? ma & ((1u << __fns(ma, 0, (int)mine + 1)) - 1u) : 0u);
-      const u32 valid = base + kLaneSlots <= a.n ? 0xFFFFu : (base < a.n ? (1u << (a.n - base)) - 1u : 0u);
-      const u32 nl = ((~ma & valid) | added) & valid;
-      u32 halves = mine ? 3u : 0u;
-      if (OP == OP_FUSED) {
-        const u32 ml = (wl >> (16 * (lane & 1))) & valid;
-        const u32 touched = mine ? 0xFFFFu : ma & ml, diff = nl ^ ml;
-        halves = ((touched & 0xFFu) && (diff & 0xFFu) ? 1u : 0u) | ((touched >> 8) && (diff >> 8) ? 2u : 0u);
-      }
-      if (halves) {
-        if (valid == 0xFFFFu) {
+      if (LATE || mine) {
+        const u32 added = mine == (u32)__popc(ma) ? ma : (mine ? ma & ((1u << __fns(ma, 0, (int)mine + 1)) - 1u) : 0u);
+        const u32 valid = base + kLaneSlots <= a.n ? 0xFFFFu : (base < a.n ? (1u << (a.n - base)) - 1u : 0u);
+        const u32 nl = ((~ma & valid) | added) & valid;
+        u32 halves = 3u;
+        if (LATE) {
+          const u32 ml = (wl >> (16 * (lane & 1))) & valid;
+          const u32 touched = mine ? 0xFFFFu : ma & ml, diff = nl ^ ml;
+          halves = ((touched & 0xFFu) && (diff & 0xFFu) ? 1u : 0u) | ((touched >> 8) && (diff >> 8) ? 2u : 0u);
+        }
+        if (halves && valid == 0xFFFFu) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             if (!((halves >> h) & 1u)) continue;
@@ -624,7 +640,7 @@ __global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(S
             for (int j = 0; j < 8; ++j) f[j] = (int)((nl >> (8 * h + j)) & 1u);
             st_v8(s.active + base + 8 * h, f);
           }
-        } else {
+        } else if (halves) {
           for (int j = 0; j < kLaneSlots; ++j)
             if (((valid >> j) & 1u) && ((halves >> (j >> 3)) & 1u)) s.active[base + j] = (int)((nl >> j) & 1u);
         }
@@ -1610,6 +1626,12 @@ static int apply_grid() {
   return num_sms() * b;
 }
 
+// The selective-update call with at least capacity / kLateShare records writes the flags
+// of removed slots late. A call pays 1 to 2 us for plane L and saves the writes of the removed
+// slots that it refills, all of them once the set is full (after some 3 / p calls). 2^24
+// slots, early and late, first calls and full set: p = 0.001 45.5 and 47.5 us, 47.5 and 47.5;
+// 0.003 47.5 and 49.1, 52.1 and 50.6; 0.005 49.1 and 50.1, 55.2 and 52.6; 0.01 52.7 and 53.7,
+// 61.3 and 57.8.
 // The selective-update call with many records (k >= capacity / kMoveShare), 8
 // fields and 32-byte aligned records and deltas: the ranking pass moves them.
 // 2^24 slots, lists and an apply pass against moving at once: p = 0.005 55 us
@@ -1621,6 +1643,7 @@ static int apply_grid() {
 // slots: 59 us against 62 at p = 0.02, 77 against 75 at 0.05. Four CTAs per SM:
 // two leave the count pass short of warps, eight cost a second wave.
 constexpr int kMoveShare = 64;
+constexpr int kLateShare = 256;
 constexpr int kMoveCtasPerSm = 4;
 static bool fused_moves(const abm_slab* s, const ScanArgs& a) {
   return (long long)a.k * kMoveShare >= (long long)s->d.cap && s->d.F == 8 && s->d.Fp == 8 &&
@@ -1720,19 +1743,26 @@ static abm_status launch_scan(abm_slab* s, const ScanArgs& a, bool aux, cudaStre
   const long per = ((long)b.n + target - 1) / target;
   b.chunk = (int)(((per + SUB - 1) / SUB) * SUB);
   b.G = (int)(((long)b.n + b.chunk - 1) / b.chunk);
-  if constexpr (OP == OP_FUSED) k_count_fused<THREADS><<<b.G, THREADS, 0, st>>>(b);
-  else k_count<OP, THREADS><<<b.G, THREADS, 0, st>>>(b);
-  ABM_LAUNCH_CHECK();
   // the next passes may launch while the previous one drains; they wait on
   // it (griddepcontrol) before reading its results
   if constexpr (OP == OP_FUSED) {
+    const bool late = move || (long long)b.k * kLateShare >= (long long)s->d.cap;
+    if (late) k_count_fused<THREADS, true><<<b.G, THREADS, 0, st>>>(b);
+    else k_count_fused<THREADS, false><<<b.G, THREADS, 0, st>>>(b);
+    ABM_LAUNCH_CHECK();
     if (move) {
-      ABM_CUDA_TRY(launch_pdl(k_scatter<OP, THREADS, true>, b.G, THREADS, st, b));
+      ABM_CUDA_TRY(launch_pdl(k_scatter<OP, THREADS, true, true>, b.G, THREADS, st, b));
       return ABM_OK;
     }
+    if (late) ABM_CUDA_TRY(launch_pdl(k_scatter<OP, THREADS, false, true>, b.G, THREADS, st, b));
+    else ABM_CUDA_TRY(launch_pdl(k_scatter<OP, THREADS>, b.G, THREADS, st, b));
+    ABM_CUDA_TRY(launch_pdl(k_apply<OP>, apply_grid<OP>(), 256, st, b));
+    return ABM_OK;
   }
+  k_count<OP, THREADS><<<b.G, THREADS, 0, st>>>(b);
+  ABM_LAUNCH_CHECK();
   if (OP != OP_REMOVE) ABM_CUDA_TRY(launch_pdl(k_scatter<OP, THREADS>, b.G, THREADS, st, b));
-  if constexpr (OP == OP_ADD || OP == OP_UPDATE || OP == OP_FUSED)
+  if constexpr (OP == OP_ADD || OP == OP_UPDATE)
     ABM_CUDA_TRY(launch_pdl(k_apply<OP>, apply_grid<OP>(), 256, st, b));
   return ABM_OK;
 }

@@ -585,6 +585,32 @@ def test_selective_update_paths(eng, n, p):
     s.check()
 
 
+@pytest.mark.parametrize("n,p", [(2_000_003, 0.0038), (2_000_003, 0.0041), (300_001, 0.001), (300_001, 0.01)])
+def test_selective_update_early_and_late_flags(eng, n, p):
+    """The same on both sides of the number of records from which removed slots' flags are written late."""
+    test_selective_update_paths(eng, n, p)
+
+
+@pytest.mark.parametrize("threads,ctas", [(128, 16), (256, 2), (512, 4)])
+@pytest.mark.parametrize("F,p", [(8, 0.002), (8, 0.008), (8, 0.1), (5, 0.002), (5, 0.008), (5, 0.1)])
+def test_selective_update_shapes(eng, threads, ctas, F, p):
+    """Every launch shape of the passes takes each of their ways (whole numbers, so exact)."""
+    n = 700_001
+    T, k = workloads.threshold(p), workloads.k_for(p, n)
+    s, o = eng.Slab(n, F, seed=3, init=1), oracle.Slab(n, F)
+    s.tune(threads, ctas)
+    o.c1_init(seed=3)
+    from paper_2508_16508_gb300 import abm
+    for step in range(6):
+        s.selective_update(step, T, s.philox_records(step, abm.P_NEWREC0, abm.P_NEWREC1, k),
+                           s.philox_records(step, abm.P_DELTA0, abm.P_DELTA1, k))
+        o.c1_call(step, T, k, seed=3)
+    np.testing.assert_array_equal(np_of(s.read(-1)), o.active)
+    for f in range(F):
+        np.testing.assert_array_equal(np_of(s.read(f)), o.fields[f])
+    s.check()
+
+
 @pytest.mark.parametrize("M,R,levels", [(4095, 3, 1), (4097, 70_000, 2), (700_003, 5, 1), (700_003, 50_000, 3),
                                         (1_500_000, 1, 2**32), (1_300_001, 1_000_000, 2**32)])
 def test_resolve_ties_and_hot_resources(eng, M, R, levels):
