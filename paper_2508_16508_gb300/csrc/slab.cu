@@ -124,6 +124,8 @@ struct ScanArgs {
   int32_t* out_count;      // device outputs (nullable)
   int negate;              // OP_SELECT: select where the predicate is false
   const int32_t* list_base;  // OP_SELECT: device offset added to every rank (nullable)
+  int* crowded;              // OP_FUSED: the slab's word (nullable)
+  int crowded_known;         // its value at the launch
   u32 div1, div4;            // one launch: 65536 / units of a row, rounded up, in words and in 16 bytes
 };
 
@@ -686,6 +688,8 @@ __global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(S
         a.out_count[1] = added;
         a.out_count[2] = min(a.k, B);
       }
+      const int crowded = 2 * (u64)(u32)A > 5 * (u64)(u32)added;
+      if (a.crowded && crowded != a.crowded_known) *reinterpret_cast<volatile int*>(a.crowded) = crowded;
     }
     __threadfence();
   }
@@ -1388,6 +1392,7 @@ static void slab_free(abm_slab* s) {
   cudaFree(s->listb);
   cudaFree(s->d.meta);
   cudaFree(s->ctrl);
+  if (s->crowded) cudaFreeHost(s->crowded);  // (the frees above waited for every launch)
   sort_scratch_free(s->sort);
   delete s;
 }
@@ -1441,6 +1446,10 @@ static abm_status slab_alloc(int capacity, int n_fields, u32 seed, u32 model, in
             cudaMalloc(&s->listb, sizeof(int32_t) * (size_t)capacity) == cudaSuccess &&
             cudaMalloc(&s->d.meta, sizeof(int32_t) * 4) == cudaSuccess &&
             cudaMalloc(&s->ctrl, sizeof(u32) * 8) == cudaSuccess;
+  if (ok && n_fields == 8 && capacity > kSmallMax) {
+    ok = cudaHostAlloc(&s->crowded, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess;
+    if (ok) *s->crowded = 1;
+  }
   if (!ok) {
     cudaGetLastError();
     slab_free(s);
@@ -1632,22 +1641,25 @@ static int apply_grid() {
 // slots, early and late, first calls and full set: p = 0.001 45.5 and 47.5 us, 47.5 and 47.5;
 // 0.003 47.5 and 49.1, 52.1 and 50.6; 0.005 49.1 and 50.1, 55.2 and 52.6; 0.01 52.7 and 53.7,
 // 61.3 and 57.8.
-// The selective-update call with many records (k >= capacity / kMoveShare), 8
-// fields and 32-byte aligned records and deltas: the ranking pass moves them.
-// 2^24 slots, lists and an apply pass against moving at once: p = 0.005 55 us
-// against 67, 0.02 75 against 66, 0.05 101 against 92, 0.2 185 against 166, 0.5
-// (moved at once before, step by step and with every flag group written) 242
-// against 211. What is left at p = 0.05 is the draws (30 us) and random 32-byte
-// rows, of which DRAM moves 64 bytes each way. The line is drawn for the first
-// call on a half-full slab too, whose adds all fall to the CTAs of the lowest
-// slots: 59 us against 62 at p = 0.02, 77 against 75 at 0.05. Four CTAs per SM:
-// two leave the count pass short of warps, eight cost a second wave.
+// The selective-update call with many records, 8 fields and 32-byte aligned records and
+// deltas: the ranking pass moves them (four CTAs per SM: two leave the count pass short of
+// warps, eight cost a second wave). Lists and an apply pass against moving at once on full
+// sets of 2^24 slots: p = 0.01 57.8 us against 67, 0.0157 62 and 62, 0.02 68 and 66, 0.03 79 and
+// 76, 0.05 101 and 93, 0.1 145 and 126, 0.3 246 and 192. What is left at p = 0.05 is the draws
+// (30 us) and random 32-byte rows, of which DRAM moves 64 bytes each way. While a set fills
+// up, the adds that refill no removed slot go to the lowest free ones, to a few CTAs that
+// run on alone, where an apply pass spreads them: p = 0.02 after 20 and 60 calls 62 and 64 us
+// against 73 and 81, 0.03 71 and 77 against 85 and 89, 0.05 94 and 100 against 101 and 103, 0.1
+// 141 and 145 against 132 and 126. So from kMoveShare on records are moved at once when the
+// last call left at most 1.5 times its adds free, from kMoveAlways on always.
 constexpr int kMoveShare = 64;
+constexpr int kMoveAlways = 12;
 constexpr int kLateShare = 256;
 constexpr int kMoveCtasPerSm = 4;
 static bool fused_moves(const abm_slab* s, const ScanArgs& a) {
-  return (long long)a.k * kMoveShare >= (long long)s->d.cap && s->d.F == 8 && s->d.Fp == 8 &&
-         ((((uintptr_t)a.rec) | ((uintptr_t)a.rec2)) & 31) == 0;
+  if (s->d.F != 8 || s->d.Fp != 8 || ((((uintptr_t)a.rec) | ((uintptr_t)a.rec2)) & 31) != 0) return false;
+  if ((long long)a.k * kMoveAlways >= (long long)s->d.cap) return true;
+  return (long long)a.k * kMoveShare >= (long long)s->d.cap && a.crowded && !a.crowded_known;
 }
 
 // Where one cluster is faster than the passes, for a call on n slots that moves up to k
@@ -1736,6 +1748,10 @@ static abm_status launch_scan(abm_slab* s, const ScanArgs& a, bool aux, cudaStre
       case 8: return launch_small<OP, 8>(b, st);
       case 16: return launch_small<OP, 16>(b, st);
     }
+  }
+  if (OP == OP_FUSED && s->crowded) {
+    b.crowded = s->crowded;
+    b.crowded_known = *reinterpret_cast<volatile int*>(s->crowded);
   }
   const bool move = OP == OP_FUSED && fused_moves(s, b);
   if (ctas_per_sm == 0) ctas_per_sm = move ? kMoveCtasPerSm : 8;

@@ -591,6 +591,31 @@ def test_selective_update_early_and_late_flags(eng, n, p):
     test_selective_update_paths(eng, n, p)
 
 
+@pytest.mark.parametrize("n,p", [(300_001, 0.02), (270_003, 0.06)])
+def test_selective_update_while_the_set_fills(eng, n, p):
+    """From a half-full set to a full one and, emptied, on again: the launches change on the way (whole numbers, so
+    exact). With and without waiting for a call before the next is made."""
+    from paper_2508_16508_gb300 import abm
+    T, k = workloads.threshold(p), workloads.k_for(p, n)
+    s, o = eng.Slab(n, 8, seed=6, init=abm.INIT_HALF_LIVE), oracle.Slab(n, 8)
+    o.c1_init(seed=6)
+    for step in range(int(8 / p)):
+        if step == int(5 / p):
+            keep = (np.arange(n) % 3 == 0).astype(np.int32)
+            s.remove(abm.pred(abm.PRED_MASK, mask=torch.from_numpy(1 - keep).cuda()))
+            o.active[:] = o.active * keep
+        c = s.selective_update(step, T, s.philox_records(step, abm.P_NEWREC0, abm.P_NEWREC1, k),
+                               s.philox_records(step, abm.P_DELTA0, abm.P_DELTA1, k))
+        d = o.c1_call(step, T, k, seed=6)
+        if step % 3 == 0:
+            assert np_of(c).tolist() == [d["removed"], d["added"], d["updated"]]
+    np.testing.assert_array_equal(np_of(s.read(-1)), o.active)
+    for f in range(8):
+        np.testing.assert_array_equal(np_of(s.read(f)), o.fields[f])
+    assert s.counters()["n_active"] == int(o.active.sum())
+    s.check()
+
+
 @pytest.mark.parametrize("threads,ctas", [(128, 16), (256, 2), (512, 4)])
 @pytest.mark.parametrize("F,p", [(8, 0.002), (8, 0.008), (8, 0.1), (5, 0.002), (5, 0.008), (5, 0.1)])
 def test_selective_update_shapes(eng, threads, ctas, F, p):
