@@ -1064,8 +1064,9 @@ struct PhaseClock {
 
 // MINB = resident CTAs per SM the register budget is cut for (1: up to 128
 // registers a thread, 2: 64). CLUSTER: the grid is one cluster, whose hardware
-// barrier takes the place of the grid barrier.
-template <int MINB, bool CLUSTER = false>
+// barrier takes the place of the grid barrier. TWO: one of a call's two launches
+// (WorldDev::stop_at, follow).
+template <int MINB, bool CLUSTER = false, bool TWO = false>
 __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps, abm_step_stats* stats,
                                                      unsigned long long* phase_ns) {
   __shared__ u64 s_red[2 * kPWarps];
@@ -1092,6 +1093,23 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
   if (threadIdx.x < kRoundUnits * 4) s_upar[threadIdx.x] = 0u;
   PhaseClock clk{phase_ns, s_book};
   u32 bar_target = w.bar_base;  // arrival count that completes the next barrier
+  // TWO: the steps of this launch, the call's steps before it (in shared memory: in registers they cost 2% of a step)
+  __shared__ int s_steps[2];
+  if constexpr (TWO) {
+    griddep_wait();
+    const int left = w.follow ? *w.left : nsteps;
+    if (threadIdx.x == 0) {
+      s_steps[0] = left;
+      s_steps[1] = nsteps - left;
+    }
+    if (left <= 0) {  // none left: the arrivals that the host has counted
+      if (!CLUSTER && blockIdx.x == 0 && threadIdx.x == 0)
+        red_release_add(w.ps.bar, gridDim.x * ((u32)kPhases * (u32)nsteps + 1u));
+      return;
+    }
+    __syncthreads();
+  }
+  const volatile int* const steps = s_steps;
   WorldCtr* c = w.ctr;
   const PersistDev& ps = w.ps;
   // counters the phases read: one copy per thread, all updated identically
@@ -1124,7 +1142,10 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
     __shared__ u32 s_err;
     if (threadIdx.x == 0) s_err = ld_relaxed32(reinterpret_cast<const u32*>(w.err));
     sync();
-    if (s_err != 0u) return;
+    if (s_err != 0u) {
+      if (TWO && blockIdx.x == 0 && threadIdx.x == 0 && !w.follow) *w.left = 0;  // the call ends here
+      return;
+    }
   }
   clk.start();
   // Wolf ranks of step t-1 run beside the sheep moves of step t, and the wolf
@@ -1194,7 +1215,7 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
     }
     return wb;
   };
-  for (int it = 0; it < nsteps; ++it) {
+  for (int it = 0; it < (TWO ? steps[0] : nsteps); ++it) {
     int* acc = ps.acc + 4 * (t & 1);
     // ---- P1: wolf ranks of the previous step | sheep move
     if (wolf_team) {
@@ -1213,7 +1234,7 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
     if (book_thread()) {
       s_book.nstart0 = s_book.nact[0];
       if (stats) {
-        abm_step_stats* st = stats + it;
+        abm_step_stats* st = stats + it + (TWO ? steps[1] : 0);
         st->n_start[0] = s_book.nact[0];
         st->n_start[1] = s_book.nact[1];
         st->extent[0] = ext[0];
@@ -1272,7 +1293,8 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
     // ---- P4: wolves eat / kill / select / die / flags
     const int kseg1 = (((ext[1] + 127) >> 7) + (int)gridDim.x - 1) / (int)gridDim.x;
     p_count<1, kPWarps>(w, t, ext[1], kseg1, acc, cl, carried, s_upar, s_acc);
-    if (book_thread()) s_book.stp = stats ? stats + it : nullptr;
+    if (book_thread()) s_book.stp = stats ? stats + it + (TWO ? steps[1] : 0) : nullptr;
+    if (TWO && CLUSTER && threadIdx.x == 0 && ext[0] + ext[1] > w.stop_at) s_steps[0] = it + 1;
     ++t;
     sync();
     clk.lap(4);
@@ -1299,6 +1321,9 @@ __global__ void __launch_bounds__(kPT, MINB) k_persistent(WorldDev w, int nsteps
       for (int j = threadIdx.x; j < (int)gridDim.x; j += kPT) ps.seg[1][j] = 0ull;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
+    // the arrivals of the steps that were not left (every CTA has passed the last barrier's count)
+    if (TWO && !CLUSTER) red_release_add(ps.bar, gridDim.x * (u32)kPhases * (u32)steps[1]);
+    if (TWO && !w.follow) *w.left = nsteps - steps[0];
     c->step = t;
     for (int s = 0; s < 2; ++s) {
       c->extent[s] = ext[s];
@@ -1329,8 +1354,9 @@ int persistent_max_ctas() {
 int persistent_warps() { return kPWarps; }
 
 bool persistent_cluster_fits() {
-  static std::atomic<int> known[64];
-  return cluster_limit(k_persistent<1, true>, kPT, known) >= kClusterCtas;
+  static std::atomic<int> known[64], known_two[64];
+  return cluster_limit(k_persistent<1, true>, kPT, known) >= kClusterCtas &&
+         cluster_limit(k_persistent<1, true, true>, kPT, known_two) >= kClusterCtas;
 }
 
 int persistent_round_units() { return kQ * kSheepWarps; }
@@ -1344,18 +1370,22 @@ abm_status launch_persistent(const WorldDev& d, u32* bar_next, int grid, bool cl
     cfg.gridDim = dim3(kClusterCtas);
     cfg.blockDim = dim3(kPT);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = kClusterCtas;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
-    ABM_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_persistent<1, true>, dd, nsteps, stats, phase_ns));
+    cfg.numAttrs = d.follow ? 2 : 1;
+    const bool two = d.follow || d.stop_at != kNoStop;
+    ABM_CUDA_TRY(cudaLaunchKernelEx(&cfg, two ? k_persistent<1, true, true> : k_persistent<1, true>, dd, nsteps, stats, phase_ns));
     return ABM_OK;
   }
   void* args[] = {(void*)&dd, (void*)&nsteps, (void*)&stats, (void*)&phase_ns};
   // one CTA per SM: the variant with the larger register budget
-  const void* fn = grid <= num_sms() ? (const void*)k_persistent<1> : (const void*)k_persistent<2>;
+  const void* fn = d.follow ? (const void*)k_persistent<1, false, true>
+                   : grid <= num_sms() ? (const void*)k_persistent<1> : (const void*)k_persistent<2>;
   ABM_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(kPT), args, 0, st));
   // arrivals this launch adds to the counter
   if (nsteps > 0) *bar_next += ((u32)kPhases * (u32)nsteps + 1u) * (u32)grid;

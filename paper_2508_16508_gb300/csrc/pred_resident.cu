@@ -62,6 +62,8 @@ struct ResidentBook {
   int nstart0, r0p, P0p, starved0p, grassp;  // of the previous step's sheep
 };
 
+// TWO: the first of a call's two launches (WorldDev::stop_at).
+template <bool TWO>
 __global__ void __launch_bounds__(kRT, 1) k_resident(WorldDev w, ResidentLayout lay, int nsteps,
                                                      abm_step_stats* stats) {
   extern __shared__ __align__(16) unsigned char sm[];
@@ -287,7 +289,12 @@ __global__ void __launch_bounds__(kRT, 1) k_resident(WorldDev w, ResidentLayout 
     }
   };
 
+  int done = TWO ? 0 : nsteps;
   for (int it = 0; it < nsteps; ++it, ++t) {
+    if (TWO) {
+      if (ext[0] + ext[1] > w.stop_at) break;
+      done = it + 1;
+    }
     // P1: sheep move | wolf ranks of the previous step
     if (!last_warp) move(0, warp, kRTeam);
     else if (it > 0) ranks(1);
@@ -335,11 +342,11 @@ __global__ void __launch_bounds__(kRT, 1) k_resident(WorldDev w, ResidentLayout 
     count(1, warp, kRWarps);
     __syncthreads();
   }
-  if (nsteps > 0) {  // the last step's wolf ranks and births
+  if (done > 0) {  // the last step's wolf ranks and births
     if (warp == 0) ranks(1);
     __syncthreads();
     int r1, F1, ext1, id1;
-    wolf_counters(t - 1, stats ? stats + nsteps - 1 : nullptr, r1, F1, ext1, id1);
+    wolf_counters(t - 1, stats ? stats + done - 1 : nullptr, r1, F1, ext1, id1);
     births(1, t - 1, r1, F1, ext1, id1, warp, kRWarps);
     __syncthreads();
   }
@@ -358,6 +365,7 @@ __global__ void __launch_bounds__(kRT, 1) k_resident(WorldDev w, ResidentLayout 
       else if (words(lay.born, s)[i >> 5] & bit) w.sp[s].active[i] = 1;
     }
   if (tid == 0) {
+    if (TWO) *w.left = nsteps - done;
     c->step = t;
     for (int s = 0; s < 2; ++s) {
       c->extent[s] = ext[s];
@@ -380,11 +388,13 @@ bool resident_fits(const WorldDev& d) {
 }
 
 abm_status launch_resident(const WorldDev& d, int nsteps, abm_step_stats* stats, cudaStream_t st) {
-  static std::atomic<unsigned long long> attr{0};
+  static std::atomic<unsigned long long> attr[2];
   const int cap[2] = {d.sp[0].cap, d.sp[1].cap};
   const ResidentLayout lay = resident_layout(d.ncells, cap);
-  ABM_CUDA_TRY(smem_attr_once(k_resident, kResidentMaxSmem, attr));
-  k_resident<<<1, kRT, (size_t)lay.bytes, st>>>(d, lay, nsteps, stats);
+  const bool two = d.stop_at != kNoStop;
+  const auto kernel = two ? k_resident<true> : k_resident<false>;
+  ABM_CUDA_TRY(smem_attr_once(kernel, kResidentMaxSmem, attr[two]));
+  kernel<<<1, kRT, (size_t)lay.bytes, st>>>(d, lay, nsteps, stats);
   ABM_LAUNCH_CHECK();
   return ABM_OK;
 }

@@ -64,6 +64,10 @@ struct WorldDev {
   u64* snext;       // [cap sheep]
   u64* wkey;        // [cap wolves]
   u64* wnext;       // [cap wolves]
+  // a call of two launches: the first stops once the extents exceed stop_at slots and leaves the rest of its steps in
+  // *left (device), which the second one (follow) runs
+  int* left;
+  int stop_at, follow;
 };
 
 // 0: few enough slots for one CTA's shared memory to be faster; 1: for one cluster to be; 2: the sheep units fit one round
@@ -73,6 +77,7 @@ __host__ __device__ inline int extent_class(const WorldDev& w, int ext0, int ext
   if (ext0 + ext1 <= w.class_cluster) return 1;
   return ext0 <= w.class_round ? 2 : 3;
 }
+constexpr int kNoStop = 0x7FFFFFFF;
 __device__ __forceinline__ void note_class(const WorldDev& w, int ext0, int ext1) {
   const int k = extent_class(w, ext0, ext1);
   if (k != w.class_known) *reinterpret_cast<volatile int*>(w.class_host) = k;

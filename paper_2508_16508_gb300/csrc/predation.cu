@@ -353,7 +353,9 @@ __global__ void k_view_commit(WorldCtr* c, int sp, const int32_t* counters, cons
 using namespace abm;
 
 constexpr int kClusterSlots = 20000, kClusterCells = 256 * 256;  // for one cluster (see launch_steps)
-constexpr int kResidentSlots = 3072;  // slots up to which one CTA is faster than the grid (see launch_steps)
+constexpr int kResidentSlots = 3072;  // slots up to which one CTA is faster (see launch_steps)
+constexpr int kResidentStop = 4096, kClusterStop = 32768;  // slots at which a launch hands over,
+constexpr int kStopSteps = 128, kStopMost = 1 << 20;        // in calls of this many steps (see launch_steps)
 
 struct abm_world {
   WorldDev d;
@@ -398,6 +400,7 @@ static void world_free(abm_world* w) {
   cudaFree(w->d.snext);
   cudaFree(w->d.wkey);
   cudaFree(w->d.wnext);
+  cudaFree(w->d.left);
   if (w->d.class_host) cudaFreeHost(w->d.class_host);  // (the frees above waited for every launch)
   if (w->gexec) cudaGraphExecDestroy(w->gexec);
   slab_free_view(w->view[0]);
@@ -456,6 +459,7 @@ extern "C" abm_status abm_create(const abm_config* cfg, void* stream, abm_world*
   ok = ok && cudaMalloc(&d.wclaim, sizeof(u64) * (size_t)d.ncells) == cudaSuccess;
   ok = ok && cudaMalloc(&d.ctr, sizeof(WorldCtr)) == cudaSuccess;
   ok = ok && cudaMalloc(&d.err, sizeof(int)) == cudaSuccess;
+  ok = ok && cudaMalloc(&d.left, sizeof(int)) == cudaSuccess;
   ok = ok && cudaHostAlloc(&d.class_host, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess;
   w->pgrid_max = persistent_max_ctas();
   if (w->pgrid_max < 1) ok = false;
@@ -518,19 +522,31 @@ extern "C" abm_status abm_create(const abm_config* cfg, void* stream, abm_world*
 // The launch of the next steps, by the size class of the extents that the last
 // finished launch left (a later one only costs speed, never results).
 // Class 0: one CTA with the state in its shared memory (launch_resident). A
-// step there costs 4 us for a few hundred agents and grows with the slots,
-// 12.8 us at 3441; the persistent kernel takes 14 us from 1 to 10,000.
+// step there costs 3 us for a few hundred agents and grows with the slots that are
+// live. Us a step against one cluster's, right after the start with every slot live,
+// after 40 steps and after 60: 1000 slots 7.7 / 3.9 / 2.6 against 12.8 / 9.2 / 7.0, 2000 slots
+// 11.6 / 7.0 / 3.9 against 12.8 / 8.2 / 7.0, 3000 slots 14.1 / 10.0 / 5.0 against 12.8 / 8.6 / 7.4, 4000
+// slots 17.4 / 13.2 / 6.2, 6000 slots 23.9 / 19.6 / 8.4 against 13.2 / 8.7 / 7.5: the line is
+// drawn between the crowded start and the long run.
 // Class 1: sixteen persistent CTAs in one cluster, whose hardware barrier is
 // 0.6 us shorter than the grid's, four times a step: 100 x 100 cells 12.2 -> 10.6
 // us a step, 150 x 150 13.4 -> 11.8, 220 x 220 (17,000 slots) 13.1 -> 12.1; at 301 x
 // 301 (32,000) sixteen SMs lose what it gains, 14.0 and 14.2. Only for lattices of
-// at most kClusterCells, whose agents cannot grow far past that line in one launch.
+// at most kClusterCells: larger ones outgrow it.
 // Class 2: one persistent CTA per SM while that takes every sheep unit in one
 // round (then the moved agents stay in shared memory for the meals). A barrier
 // of fewer CTAs and twice the registers per thread are worth 2 us a step: 301 x
 // 301 cells 18.1 -> 15.8 us, 1400 x 1400 (3811 sheep units) 21.1 -> 18.9.
 // Class 3: the tuned number of CTAs; at 2048 x 2048 (two rounds of one CTA per
 // SM) the second CTA per SM wins, 33.7 us against 38.7.
+//
+// Extents are bounded by the capacities only, and a launch keeps its way to its end. A
+// call of kStopSteps or more steps whose capacities lie past kResidentStop (kClusterStop)
+// slots is therefore two launches: the first stops where the extents pass that
+// line, and the second, the cluster (the grid), runs the steps that are left, mostly
+// none: 1 to 4 us a call. Worlds that outgrow their launch, 400 steps in a call: 24 x 24
+// cells with 8000 sheep 13.1 us a step (29.8 to the end in one CTA), 256 x 256 with
+// 130,000 15.5 (48.7 in one cluster).
 // The cluster only where one can be placed; a profiled call runs on the grid.
 static int steps_way(int size_class, bool profiled, bool cluster) {
   if (profiled) return size_class < 3 ? 2 : 3;
@@ -545,10 +561,20 @@ static abm_status launch_steps(abm_world* w, int nsteps, abm_step_stats* stats, 
                                unsigned long long* phase_ns = nullptr) {
   WorldDev d = w->d;
   d.class_known = *reinterpret_cast<volatile int*>(d.class_host);
-  const int way = steps_way(d.class_known, phase_ns != nullptr, d.class_known == 1 && persistent_cluster_fits());
-  if (way == 0) return launch_resident(d, nsteps, stats, st);
-  return launch_persistent(d, &w->bar_next, way == 3 ? w->pgrid : std::min(w->pgrid, num_sms()), way == 1, nsteps, stats, st,
-                           phase_ns);
+  const bool fits = d.class_known <= 1 && persistent_cluster_fits();
+  const int way = steps_way(d.class_known, phase_ns != nullptr, fits), grid = std::min(w->pgrid, num_sms());
+  // may the extents outgrow the launch on the way?
+  const long long caps = (long long)d.sp[0].cap + d.sp[1].cap, stop = way == 0 ? kResidentStop : kClusterStop;
+  const bool two = way <= 1 && nsteps >= kStopSteps && nsteps <= kStopMost && caps > stop;
+  d.stop_at = two ? (int)stop : kNoStop;
+  d.follow = 0;
+  abm_status e;
+  if (way == 0) e = launch_resident(d, nsteps, stats, st);
+  else e = launch_persistent(d, &w->bar_next, way == 3 ? w->pgrid : grid, way == 1, nsteps, stats, st, phase_ns);
+  if (e != ABM_OK || !two) return e;
+  d.stop_at = kNoStop;
+  d.follow = 1;
+  return launch_persistent(d, &w->bar_next, grid, way == 0 && fits, nsteps, stats, st);
 }
 
 // ev (nullable): 7 events recorded around the six kernels of the step

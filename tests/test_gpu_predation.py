@@ -429,3 +429,35 @@ def test_cluster_launches_agree(eng, side, cap, n0, variant, kw):
     assert torch.equal(sa, sb)
     assert a.save() == b.save()
     a.check()
+
+
+@pytest.mark.parametrize("side,cap,n0,variant,kw", [
+    (24, (8000, 3000), (300, 50), 0, dict(sheep_gain=60, regrowth=1, sheep_repro=0.6, wolf_gain=1)),   # one CTA, then the cluster
+    (40, (5000, 900), (900, 100), 2, dict(sheep_repro=0.3)),
+    (45, (3000, 1097), (1500, 300), 0, dict(sheep_gain=40, regrowth=1, wolf_gain=1)),                  # just past the line
+    (200, (60000, 9000), (9000, 900), 0, dict(sheep_gain=60, regrowth=1, sheep_repro=0.5, wolf_gain=1)),  # cluster, then grid
+    (150, (50000, 20000), (5400, 1301), 1, dict(sheep_gain=30, regrowth=1, sheep_repro=0.4)),
+    (60, (40000, 40000), (1000, 200), 0, {})])                                                          # stays small
+def test_calls_that_outgrow_their_launch(eng, side, cap, n0, variant, kw):
+    """Calls long enough that a launch hands the rest of its steps to the next one, where the population outgrows it
+    and where it does not, against the grid (which step_profiled always takes): statistics, state and later calls."""
+    p = workloads.predation_params(**kw)
+    a, b = (eng.World(side, 8, 1, p, cap, n0, variant=variant) for _ in range(2))
+    steps = (128, 3, 150, 127, 1, 130)
+    sa, sb = a.new_stats(sum(steps)), b.new_stats(sum(steps))
+    at = 0
+    for n in steps:
+        a.step(n, sa[at:at + n])
+        b.step_profiled(n, sb[at:at + n])
+        at += n
+        if n == 3:
+            a.step_profiled(5)
+            b.step(5)
+    assert torch.equal(sa, sb)
+    assert a.save() == b.save()
+    a.check()
+    # several calls in flight, without statistics
+    for _ in range(3):
+        a.step(128)
+    b.step_profiled(384)
+    assert a.save() == b.save()
