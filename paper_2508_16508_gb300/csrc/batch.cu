@@ -880,6 +880,12 @@ static abm_status batch_shape(const abm_batch* b, int threads, int models_per_ct
 //   extent    600 of 16..256 546 and 33 (1550 and 50), 4096 of 16..256 3699 and
 //   133 (4983 and 130), 300 of 64..128 148 and 14 (237 and 15; 1024 threads 87
 //   and 18)
+// Over 19 batches (40 to 4096 models, sides 16 to 256, capacities of 1, 2 and 4 side^2,
+// both sweeps) steps 0..40 take 0.35 to 1.01 of what they take with 256 x 4 x 16, steps
+// 100..500 0.47 to 1.13: above 1.03 only extent sweeps of 1000 models of 64..128 and 300 of
+// 16..64, which save more in their first 40 steps (0.63 and 0.70) than in the next 460 is
+// lost. (256 x 4 x 16 from step 100 on for more models than four per SM: 1.13 -> 1.02 there,
+// but 0.70 -> 0.98 for 700 of 100..180.)
 struct BatchShape {
   int threads, ctas_per_sm, models_per_cta, agents_per_thread;
 };
