@@ -228,8 +228,12 @@ def ptr(t) -> C.c_void_p:
 def stream_handle(stream=None) -> C.c_void_p:
     if stream is None:
         import torch
-        # the current stream's handle without a Stream object around it (3.1 -> 0.6 us a call)
-        return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        # the current stream's handle without a Stream object around it (3.1 -> 0.6 us a call), where this torch has the
+        # call (a private one)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return C.c_void_p(raw(torch.cuda.current_device()))
+        stream = torch.cuda.current_stream()
     return C.c_void_p(stream.cuda_stream)
 
 

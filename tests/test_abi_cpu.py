@@ -91,3 +91,16 @@ def test_launches_without_room_for_a_cluster(lib_path):
     assert [way(c, 0, 1) for c in range(4)] == [0, 1, 2, 3]
     assert [way(c, 0, 0) for c in range(4)] == [0, 2, 2, 3]
     assert [way(c, 1, 1) for c in range(4)] == [2, 2, 2, 3]
+
+
+def test_stream_handle_without_the_private_call(monkeypatch):
+    """The current stream's handle comes from torch's public call where the private one is missing."""
+    torch = pytest.importorskip("torch")
+    from paper_2508_16508_gb300 import abm
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 41 + device, raising=False)
+    assert abm.stream_handle().value == 41
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: type("Stream", (), {"cuda_stream": 77})())
+    assert abm.stream_handle().value == 77
+    assert abm.stream_handle(type("Stream", (), {"cuda_stream": 5})()).value == 5
