@@ -144,7 +144,7 @@ abm_status abm_select(abm_slab* s, const abm_pred* pred, int32_t* out_idx, int32
  * the row now in slot i. The first call allocates the sort's buffers (about
  * 16 bytes a slot plus one spare copy of the slab, kept until destroy); the
  * slab's arrays are replaced by the sorted copies (abm_slab_arrays changes).
- * LSD radix sort: four passes over the key bytes and one over the live flag. */
+ * LSD radix sort of the live slots, one pass per key byte that varies. */
 abm_status abm_sort(abm_slab* s, int32_t field, int32_t* out_perm, void* stream);
 
 /* ========================================================================== */
@@ -248,7 +248,7 @@ abm_status abm_selective_update(abm_slab* s, uint32_t step, uint32_t threshold,
  * or 512) and `ctas_per_sm` CTAs per SM (threads * ctas_per_sm <= 2048).
  * Results never depend on it; the autotuner picks it. Default 256 threads and
  * 4 or 8 CTAs per SM, by the number of records. Sets of up to 262,144 slots run
- * in one launch of their own shape. */
+ * in one launch of their own shape where they do not move too many records. */
 abm_status abm_slab_tune(abm_slab* s, int32_t threads, int32_t ctas_per_sm, void* stream);
 
 /* Fill out[k][F] (device int32) with record j field f = word f%4 of

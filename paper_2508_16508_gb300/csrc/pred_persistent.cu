@@ -48,9 +48,8 @@ __device__ __forceinline__ void red_release_add(u32* p, u32 v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// A grid barrier in two halves, so that independent work can run between
-// them: grid_arrive counts this CTA in (after its threads meet), grid_wait
-// waits for the whole grid.
+// The barrier's two halves: grid_arrive counts this CTA in (after its threads
+// meet), grid_wait waits for the whole grid.
 __device__ __forceinline__ void grid_arrive(u32* bar, u32& target, u32 expected = 0) {
   target += expected == 0 ? gridDim.x : expected;
   __syncthreads();
@@ -214,7 +213,7 @@ __device__ __forceinline__ int4 move_one(const WorldDev& w, int t, int slot, int
   return ag;
 }
 
-// phase 1/4: move every live agent; claims for the cell's grass (sheep) or
+// P1 (sheep), P3 (wolves): move every live agent; claims for the cell's grass (sheep) or
 // the cell's victim (wolves)
 // A world whose units fit in one round leaves the round's list, live words and
 // moved records in shared memory; `carried` = the list's length (-1 if not). A
@@ -316,7 +315,7 @@ __device__ __forceinline__ bool eat_rank_matched(const WorldDev& w, int t, int s
   return false;
 }
 
-// one live agent of phase 2/5: eat if it won its cell, then die (energy
+// one live agent of P2 (sheep) or P4 (wolves): eat if it won its cell, then die (energy
 // below zero) or be drawn as a parent. Returns bit 0 = parent, bit 1 = died,
 // bit 2 = ate.
 template <int S>
@@ -361,7 +360,7 @@ __device__ __forceinline__ u32 count_one(const WorldDev& w, int t, int slot, int
   return r;
 }
 
-// phase 2/5: eat, select parents, kill the starving. Units are dealt and
+// P2 (sheep), P4 (wolves): eat, select parents, kill the starving. Units are dealt and
 // their live agents listed as for the moves. Each unit then writes its free /
 // parent bits into the bit-planes (word = 32 slots = 8 lanes x 4 slots) and
 // its two counts, which are also summed per run of kseg units (the CTA
@@ -551,7 +550,7 @@ __device__ __forceinline__ void rank_unit(const WorldDev& w, int base, int ext, 
   }
 }
 
-// phase 3/6: ranks -> parent list (all) and free list (ranks below P only).
+// Wolf ranks (P1 of the next step) -> parent list (all) and free list (ranks below P only).
 // CTA b owns units [b*kseg, (b+1)*kseg); the unit ranks are the segment's
 // prefix plus a block scan of the unit counts; inside a unit, a warp scan.
 template <int S>

@@ -6,7 +6,7 @@
 // persistent kernel spends its time in that chain's round trips to L2 and in
 // its grid barriers, whatever the number of CTAs (40 x 40 cells: 14.5 us a step
 // with 1 to 152 CTAs). Here the chain runs in shared memory and the barrier is
-// the CTA's: the same world takes 3.8 us a step. The state is read once
+// the CTA's: the same world takes 3.2 us a step. The state is read once
 // and written back once per launch.
 //
 // The phases, their hazards and the results are those of k_persistent

@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count(ScanArgs a) {
 // the third depend on the call alone. mask_pair_consts works them out on the
 // host (round r: (hi(M1 c2) ^ c1 ^ k0, lo(M1 c2), hi(M0 c0) ^ c3 ^ k1,
 // lo(M0 c0)), M0 = 0xD2511F53, M1 = 0xCD9E8D57, round keys k = rk); the
-// device finishes the block from them. Same outputs as philox_rk.
+// device finishes the block from them. Same outputs as philox.
 static void mask_pair_consts(u32 step, const u32 (&rk)[20], u32 (&mk)[5]) {
   const auto wide = [](u32 m, u32 x, u32& hi, u32& lo) {
     const uint64_t p = (uint64_t)m * (uint64_t)x;
@@ -428,12 +428,6 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count_fused(ScanArg
   }
 }
 
-// Pass 2: ranks from the CTA prefix + warp prefix + a warp scan per step.
-// Each 512-slot step of a warp stages its flagged slots in shared memory in
-// rank order (each lane writes its own, 16 slots at most) and the warp copies
-// them out coalesced; steps with no rank below the limit are skipped. The add
-// passes also write the final live flags of every 16-slot group that receives
-// a new agent, whole (0/1), so no flag sector is written in part.
 // The selective-update call's records moved by the pass that ranks them: the
 // staged slots (offsets from slot0) take records r0 + i, i < n (ADDROW: added to
 // the row, wrapping), U 32-byte rows per lane in flight. Ranks are consecutive
@@ -494,9 +488,15 @@ __device__ __forceinline__ void stage_bits(S* stage, u32 m, u32 pos, u32 end, in
   }
 }
 
+// Pass 2: ranks from the CTA prefix + warp prefix + a warp scan per step.
+// Each 512-slot step of a warp stages its flagged slots in shared memory in
+// rank order (each lane writes its own, 16 slots at most) and the warp copies
+// them out coalesced; steps with no rank below the limit are skipped. The add
+// passes also write the final live flags of every 16-slot group that receives
+// a new agent, whole (0/1), so no flag sector is written in part.
 // MOVE (selective-update call, 8 fields, 32-byte aligned records): the pass
 // moves the records itself instead of writing the rank-ordered slot lists, and
-// no apply pass follows.
+// no apply pass follows. LATE (selective-update call): see k_count_fused.
 template <int OP, int THREADS, bool MOVE = false, bool LATE = false>
 __global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(ScanArgs a) {
   constexpr int WARPS = THREADS / 32;

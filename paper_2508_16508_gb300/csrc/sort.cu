@@ -5,11 +5,10 @@
 // The live slots are first packed, in slot order, as (key, slot) pairs, key =
 // the field with its sign bit flipped (so unsigned order is signed order);
 // placeholders need no sorting, so they are only listed. The packing pass also
-// counts all four key bytes, which gives every digit's first position and shows
-// which bytes hold one value only (the high bytes of cells, ids and ages):
-// their passes are left out. An LSD radix sort of the pairs then runs one pass
-// per byte that is left: per-chunk digit counts, a scan over the chunks, and a
-// stable scatter. Finally every agent's row (fields + live flag) is gathered
+// collects the keys' set and cleared bits, which shows which bytes hold one value
+// only (the high bytes of cells, ids and ages): their passes are left out. An LSD
+// radix sort of the pairs then runs one pass per byte that is left: digit counts
+// per chunk and in all, a scan over the chunks, and a stable scatter. Finally every agent's row (fields + live flag) is gathered
 // into spare arrays, which then become the slab's arrays.
 //
 // Every pass splits the pairs over the same number of CTAs, a contiguous chunk
@@ -376,8 +375,8 @@ __global__ void __launch_bounds__(kSortThreads, kSortCtasPerSm) k_sort_scatter(S
 
 // Small sets: pack and sort in one CTA, pairs in shared memory, every pass with
 // the pairs in registers in between. Leaves the values in val[0] (as k_sort_pack
-// does) with no pass left to run, for the gather. (Seventeen launches of the
-// passes above take 78 us for 3000 slots.)
+// does) with no pass left to run, for the gather. (With the
+// memset and the fourteen launches that it takes the place of 78 us for 3000 slots, now 46.)
 constexpr int kOneThreads = 1024;
 constexpr int kOneWarps = kOneThreads / 32;
 constexpr int kOneMax = kOneThreads * kSortItems;
