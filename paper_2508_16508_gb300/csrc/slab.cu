@@ -126,6 +126,7 @@ struct ScanArgs {
   const int32_t* list_base;  // OP_SELECT: device offset added to every rank (nullable)
   int* crowded;              // OP_FUSED: the slab's word (nullable)
   int crowded_known;         // its value at the launch
+  int wave;                  // slots of the first wave of a ranking pass that moves records
   u32 div1, div4;            // one launch: 65536 / units of a row, rounded up, in words and in 16 bytes
 };
 
@@ -436,6 +437,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_count_fused(ScanArg
 // kMoveShare for what that is worth).
 constexpr int kMoveBatch = 128;
 constexpr int kMoveStage = kMoveBatch + kWarpStep;
+// CTAs of such a pass resident on an SM (126 registers a thread).
+template <int THREADS>
+constexpr int move_resident() {
+  return 512 / THREADS;
+}
 
 template <bool ADDROW>
 __device__ __forceinline__ void move_staged(const ScanArgs& a, const unsigned short* stage, int slot0, u32 n, u32 r0,
@@ -498,7 +504,7 @@ __device__ __forceinline__ void stage_bits(S* stage, u32 m, u32 pos, u32 end, in
 // moves the records itself instead of writing the rank-ordered slot lists, and
 // no apply pass follows. LATE (selective-update call): see k_count_fused.
 template <int OP, int THREADS, bool MOVE = false, bool LATE = false>
-__global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(ScanArgs a) {
+__global__ void __launch_bounds__(THREADS, MOVE ? move_resident<THREADS>() : 1) k_scatter(ScanArgs a) {
   constexpr int WARPS = THREADS / 32;
   __shared__ u64 s_red[WARPS];
   __shared__ int s_stage[MOVE ? 1 : WARPS * kWarpStep];
@@ -548,6 +554,12 @@ __global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(S
   const int nrec = (OP == OP_UPDATE && a.use_rec_idx) ? s.counters[3] : a.k;
   const u32 limit = (u32)(OP == OP_UPDATE ? nrec : (OP == OP_SELECT || OP == OP_ARRAY ? 0x7FFFFFFF : a.k));
   const u32 limit_b = (u32)a.k;
+  if (OP == OP_FUSED && a.crowded && blockIdx.x == (unsigned)(a.wave / a.chunk) && threadIdx.x == 0) {
+    // (pa: the free slots in front of this CTA) adds reach the slots of a second wave and leave much free
+    const u32 added = min(limit, ta);
+    const int crowded = pa < added && 2 * (u64)ta > 5 * (u64)added;
+    if (crowded != a.crowded_known) *reinterpret_cast<volatile int*>(a.crowded) = crowded;
+  }
   // ranks land at list_a + *list_base (the permutation's second half)
   int32_t* const list_a = a.list_a + (OP == OP_SELECT && a.list_base ? *a.list_base : 0);
   int* const stage = s_stage + (MOVE ? 0 : warp * kWarpStep);
@@ -688,8 +700,6 @@ __global__ void __launch_bounds__(THREADS, MOVE ? 512 / THREADS : 1) k_scatter(S
         a.out_count[1] = added;
         a.out_count[2] = min(a.k, B);
       }
-      const int crowded = 2 * (u64)(u32)A > 5 * (u64)(u32)added;
-      if (a.crowded && crowded != a.crowded_known) *reinterpret_cast<volatile int*>(a.crowded) = crowded;
     }
     __threadfence();
   }
@@ -1448,7 +1458,7 @@ static abm_status slab_alloc(int capacity, int n_fields, u32 seed, u32 model, in
             cudaMalloc(&s->ctrl, sizeof(u32) * 8) == cudaSuccess;
   if (ok && n_fields == 8 && capacity > kSmallMax) {
     ok = cudaHostAlloc(&s->crowded, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess;
-    if (ok) *s->crowded = 1;
+    if (ok) *s->crowded = 0;
   }
   if (!ok) {
     cudaGetLastError();
@@ -1647,11 +1657,15 @@ static int apply_grid() {
 // sets of 2^24 slots: p = 0.01 57.8 us against 67, 0.0157 62 and 62, 0.02 68 and 66, 0.03 79 and
 // 76, 0.05 101 and 93, 0.1 145 and 126, 0.3 246 and 192. What is left at p = 0.05 is the draws
 // (30 us) and random 32-byte rows, of which DRAM moves 64 bytes each way. While a set fills
-// up, the adds that refill no removed slot go to the lowest free ones, to a few CTAs that
-// run on alone, where an apply pass spreads them: p = 0.02 after 20 and 60 calls 62 and 64 us
-// against 73 and 81, 0.03 71 and 77 against 85 and 89, 0.05 94 and 100 against 101 and 103, 0.1
-// 141 and 145 against 132 and 126. So from kMoveShare on records are moved at once when the
-// last call left at most 1.5 times its adds free, from kMoveAlways on always.
+// up, the adds that refill no removed slot go to the lowest free ones, to a few CTAs with much
+// to do, where an apply pass spreads them. That costs little while these are in the first
+// wave of CTAs, and much once they are in the second and run on alone: 2^24 slots at p = 0.03
+// after 12, 20 and 60 calls 69, 84 and 90 us moved and 70, 71 and 77 with lists, 0.05 after 3,
+// 9 and 20 calls 75, 94 and 102 against 81, 85 and 94 (1.4 times the adds left free from call
+// 40 on: 104 and 100), 0.1 after 4, 20 and 60 calls 123, 132 and 126 against 121, 141 and
+// 145. Sets of one wave (2^20 slots: 13 to 15 us) never lose. So from kMoveShare on records
+// are moved at once unless the last call filled slots of a second wave and left more than 1.5
+// times its adds free, from kMoveAlways on always.
 constexpr int kMoveShare = 64;
 constexpr int kMoveAlways = 12;
 constexpr int kLateShare = 256;
@@ -1659,7 +1673,7 @@ constexpr int kMoveCtasPerSm = 4;
 static bool fused_moves(const abm_slab* s, const ScanArgs& a) {
   if (s->d.F != 8 || s->d.Fp != 8 || ((((uintptr_t)a.rec) | ((uintptr_t)a.rec2)) & 31) != 0) return false;
   if ((long long)a.k * kMoveAlways >= (long long)s->d.cap) return true;
-  return (long long)a.k * kMoveShare >= (long long)s->d.cap && a.crowded && !a.crowded_known;
+  return (long long)a.k * kMoveShare >= (long long)s->d.cap && !a.crowded_known;
 }
 
 // Where one cluster is faster than the passes, for a call on n slots that moves up to k
@@ -1749,15 +1763,22 @@ static abm_status launch_scan(abm_slab* s, const ScanArgs& a, bool aux, cudaStre
       case 16: return launch_small<OP, 16>(b, st);
     }
   }
+  const auto chunk_at = [&](int ctas) {
+    const int target = std::max(1, std::min(num_sms() * ctas, s->max_ctas));
+    const long per = ((long)b.n + target - 1) / target;
+    return (int)(((per + SUB - 1) / SUB) * SUB);
+  };
   if (OP == OP_FUSED && s->crowded) {
-    b.crowded = s->crowded;
-    b.crowded_known = *reinterpret_cast<volatile int*>(s->crowded);
+    const long wave = (long)chunk_at(ctas_per_sm ? ctas_per_sm : kMoveCtasPerSm) * num_sms() * move_resident<THREADS>();
+    if (wave < b.n) {
+      b.wave = (int)wave;
+      b.crowded = s->crowded;
+      b.crowded_known = *reinterpret_cast<volatile int*>(s->crowded);
+    }
   }
   const bool move = OP == OP_FUSED && fused_moves(s, b);
   if (ctas_per_sm == 0) ctas_per_sm = move ? kMoveCtasPerSm : 8;
-  const int target = std::max(1, std::min(num_sms() * ctas_per_sm, s->max_ctas));
-  const long per = ((long)b.n + target - 1) / target;
-  b.chunk = (int)(((per + SUB - 1) / SUB) * SUB);
+  b.chunk = chunk_at(ctas_per_sm);
   b.G = (int)(((long)b.n + b.chunk - 1) / b.chunk);
   // the next passes may launch while the previous one drains; they wait on
   // it (griddepcontrol) before reading its results

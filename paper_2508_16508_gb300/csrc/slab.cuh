@@ -38,8 +38,9 @@ struct abm_slab {
   int max_ctas;
   // shape of the fused selective-update pass (abm_slab_tune)
   int fused_threads, fused_ctas_per_sm;
-  // large sets of 8 fields: 1 while the last selective-update call left many slots free, which chooses the launches of the
-  // next ones (never their results). Pinned host word, written by a call that finds it otherwise.
+  // large sets of 8 fields: 1 while the last selective-update call filled slots far up and left many free, which
+  // chooses the launches of the next ones (never their results). Pinned host word, written by a call that finds it
+  // otherwise.
   int* crowded;
   abm::SortScratch* sort;  // buffers of abm_sort, allocated by its first call
   int view;                // 1: active / fields belong to a predation world (abm_world_slab)

@@ -616,6 +616,12 @@ def test_selective_update_while_the_set_fills(eng, n, p):
     s.check()
 
 
+@pytest.mark.parametrize("n,p", [(2_400_003, 0.06)])
+def test_selective_update_fills_the_second_wave(eng, n, p):
+    """The same in sets whose ranking pass takes more than one wave of CTAs."""
+    test_selective_update_while_the_set_fills(eng, n, p)
+
+
 @pytest.mark.parametrize("threads,ctas", [(128, 16), (256, 2), (512, 4)])
 @pytest.mark.parametrize("F,p", [(8, 0.002), (8, 0.008), (8, 0.1), (5, 0.002), (5, 0.008), (5, 0.1)])
 def test_selective_update_shapes(eng, threads, ctas, F, p):
