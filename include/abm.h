@@ -408,8 +408,9 @@ abm_status abm_step_profiled(abm_world* w, int32_t nsteps, abm_step_stats* stats
  * requested steps in one launch: a cooperative one of at most `ctas_per_sm` CTAs
  * per SM with bounded grid barriers between the phases, or, while the extents
  * are small enough for that to be faster, of one CTA per SM, of one cluster, or
- * of one CTA that holds the world in shared memory; ABM_ENGINE_KERNELS runs six
- * kernels per step (and is what abm_step_profiled, energy statistics and
+ * of one CTA that holds the world in shared memory (calls of 128 steps or more
+ * that the population may outgrow are two launches, the second of which takes
+ * over where it does); ABM_ENGINE_KERNELS runs six kernels per step (and is what abm_step_profiled, energy statistics and
  * abm_step_graph use). Results are identical. */
 #define ABM_ENGINE_PERSISTENT 0
 #define ABM_ENGINE_KERNELS 1

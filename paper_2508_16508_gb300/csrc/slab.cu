@@ -1677,10 +1677,10 @@ static bool fused_moves(const abm_slab* s, const ScanArgs& a) {
 }
 
 // Where one cluster is faster than the passes, for a call on n slots that moves up to k
-// records of F fields (16-byte units where `quads`): its SMs are at most sixteen, and the slots of a lane leave that much less time for records. What a CTA
-// moves at most, in ns, against lines drawn from 1 to 16 fields and k from 0.002 to 0.5 n
-// (adds to half-live and nearly full sets, updates of the first slots and of slots spread
-// over the set). 131,072 slots, us of the passes and of the cluster: adds of 0.1 n to a
+// records of F fields (16-byte units where `quads`): its SMs are at most sixteen, and the
+// more slots a lane has, the less time is left for records. What a CTA moves at most, in ns,
+// against lines drawn from 1 to 16 fields and k from 0.002 to 0.5 n (adds to half-live and
+// nearly full sets, updates of the first slots and of slots spread over the set). 131,072 slots, us of the passes and of the cluster: adds of 0.1 n to a
 // half-live set, 5 fields 10.5 and 8.3, 11 fields 11.9 and 9.3, of 0.5 n 8 fields 10.9 and
 // 9.0, 16 fields 12.4 and 11.4 (its updates 10.7 and 13.1), 11 fields 12.9 and 14.1; 262,144
 // slots: adds of 0.03 n 10.7 and 10.3 (1 field), 10.0 and 10.3 (8), 12.2 and 11.0 (11), of
